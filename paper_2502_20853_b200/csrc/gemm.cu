@@ -120,33 +120,32 @@ __device__ __forceinline__ uint32_t idesc_mxf4(int n, uint32_t a_sf_id, uint32_t
            (a_sf_id << 29);
 }
 
-// bias[0 .. ncols) (bf16, ncols a multiple of 8, at most N) added to v[0 .. N)
-template <int N>
-__device__ __forceinline__ void add_bias(float (&v)[N], const __nv_bfloat16 *bias, int ncols)
+// The bias of one 32-column chunk, for a warp whose lanes hold one accumulator row each: lane l keeps columns 2 (l & 15) and
+// 2 (l & 15) + 1 as a bf16 pair (zero beyond N, where nothing is stored), the warp passes them round with shuffles, and the
+// mixed-precision add takes the bf16 value as it is.  The pairs are fetched before the wait for the accumulator.  (Every lane
+// loading the whole chunk's bias by itself, four dependent 16-byte loads per chunk behind that wait, cost 500 cycles per chunk:
+// 50432 x 4096 x 1024 took 161 us with a bias against 110 without; now 111.)
+__device__ __forceinline__ uint32_t load_bias_pair(const __nv_bfloat16 *bias, int64_t col, int64_t N, int lane)
+{
+    const int64_t c = col + 2 * (lane & 15);
+    return bias != nullptr && c < N ? __ldg(reinterpret_cast<const uint32_t *>(bias + c)) : 0u;
+}
+__device__ __forceinline__ void add_bias_chunk(uint32_t (&r)[32], uint32_t pair)
 {
 #pragma unroll
-    for (int j = 0; j < N; j += 8) {
-        if (j >= ncols) break;
-        const uint4 b = __ldg(reinterpret_cast<const uint4 *>(bias + j));
-        const uint32_t bw[4] = {b.x, b.y, b.z, b.w};
-#pragma unroll
-        for (int t = 0; t < 4; t++) {
-            v[j + 2 * t] += bf16lo(bw[t]);
-            v[j + 2 * t + 1] += bf16hi(bw[t]);
-        }
+    for (int j = 0; j < 16; j++) {
+        const uint32_t b = __shfl_sync(0xFFFFFFFFu, pair, j);
+        asm("{\n\t.reg .b16 l, h;\n\tmov.b32 {l, h}, %4;\n\tadd.rn.f32.bf16 %0, l, %2;\n\tadd.rn.f32.bf16 %1, h, %3;\n\t}"
+            : "=&r"(r[2 * j]), "=&r"(r[2 * j + 1]) : "r"(r[2 * j]), "r"(r[2 * j + 1]), "r"(b));
     }
 }
 
 // 32 accumulator columns of one row -> 32 bf16 in 16 words
-__device__ __forceinline__ void pack_row_bf16(const uint32_t (&r)[32], const __nv_bfloat16 *bias, int ncols, uint32_t (&w)[16])
+__device__ __forceinline__ void pack_row_bf16(const uint32_t (&r)[32], uint32_t (&w)[16])
 {
-    float v[32];
-#pragma unroll
-    for (int j = 0; j < 32; j++) v[j] = __uint_as_float(r[j]);
-    if (bias) add_bias<32>(v, bias, ncols);
 #pragma unroll
     for (int j = 0; j < 16; j++) {
-        __nv_bfloat162 h = __floats2bfloat162_rn(v[2 * j], v[2 * j + 1]);
+        __nv_bfloat162 h = __floats2bfloat162_rn(__uint_as_float(r[2 * j]), __uint_as_float(r[2 * j + 1]));
         w[j] = *reinterpret_cast<uint32_t *>(&h);
     }
 }
@@ -192,7 +191,7 @@ __device__ __forceinline__ void mbar_arrive_remote(uint32_t cluster_addr)
 template <int BN, int BUFS, bool REMOTE = false>
 __device__ __forceinline__ void epilogue_tile(const CUtensorMap *map_d, const CUtensorMap *map_w, const GemmParams &p, uint32_t taddr,
                                               int row0, int colbase, int split, uint8_t *staging, uint32_t &sbuf, int lane,
-                                              uint32_t acc_empty_bar)
+                                              uint32_t acc_empty_bar, const uint32_t (&bias)[BN / 64])
 {
     constexpr int kHalfCols = BN / 2;
     constexpr int kChunks = kHalfCols / 32;
@@ -230,7 +229,8 @@ __device__ __forceinline__ void epilogue_tile(const CUtensorMap *map_d, const CU
                 uint32_t r[32];
                 tc_ld32(taddr + cc * 32, r);
                 tc_wait_ld();
-                pack_row_bf16(r, use_bias ? p.bias + col : nullptr, (int)min((int64_t)32, p.N - col), pk[cc]);
+                if (use_bias) add_bias_chunk(r, bias[cc]);
+                pack_row_bf16(r, pk[cc]);
             }
         }
         release_acc();
@@ -291,14 +291,7 @@ __device__ __forceinline__ void epilogue_tile(const CUtensorMap *map_d, const CU
             if (cc == kChunks - 1) release_acc();
             if (!live) continue;
             const int ncols = (int)min((int64_t)32, p.N - col);
-            if (use_bias) {
-                float v[32];
-#pragma unroll
-                for (int j = 0; j < 32; j++) v[j] = __uint_as_float(r[j]);
-                add_bias<32>(v, p.bias + col, ncols);
-#pragma unroll
-                for (int j = 0; j < 32; j++) r[j] = __float_as_uint(v[j]);
-            }
+            if (use_bias) add_bias_chunk(r, load_bias_pair(p.bias, col, p.N, lane));
             store_box(r, col);
             if (ncols > 16) store_box(r + 16, col + 16);
         }
@@ -510,13 +503,16 @@ k_gemm_mxf4(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
         for (int item = blockIdx.x; item < items && alive; item += gridDim.x) {
             const int split = item % p.splits, tile = item / p.splits;
             const int mb = tile / p.tiles_n, nb = tile % p.tiles_n;
+            uint32_t bias[kHalfCols / 32];
+#pragma unroll
+            for (int cc = 0; cc < kHalfCols / 32; cc++) bias[cc] = load_bias_pair(p.bias, (int64_t)nb * BN + chalf * kHalfCols + cc * 32, p.N, lane);
             if (!mbar_wait(bar_acc_full + 8 * acc, acc_phase, abort_flag, p.dev_status, p.spin_limit)) { alive = false; break; }
             tc_fence_after();
             const int row0 = mb * kBM + quarter * 32;
             const int colbase = nb * BN + chalf * kHalfCols;
             const uint32_t taddr = tmem_base + ((uint32_t)(quarter * 32) << 16) + acc * BN + chalf * kHalfCols;
             epilogue_tile<BN, C::kStagingBufs>(&map_d, p.out_fp32 ? nullptr : &map_dw, p, taddr, row0, colbase, split, staging, sbuf, lane,
-                                               bar_acc_empty + 8 * acc);
+                                               bar_acc_empty + 8 * acc, bias);
             if (++acc == C::kAccStages) { acc = 0; acc_phase ^= 1u; }
         }
         if (lane == 0) bulk_wait0();   // all stores of this warp have completed before the CTA may exit
@@ -680,6 +676,7 @@ k_gemm_mxf4_q(const __grid_constant__ CUtensorMap map_a, const __grid_constant__
         for (int item = blockIdx.x; item < items; item += gridDim.x, it++) {
             const int mb = item / p.tiles_n, nb = item % p.tiles_n;
             const int row0 = mb * kBM, col0 = nb * BN;
+            const uint32_t bias[2] = {load_bias_pair(p.bias, col0 + chalf * 64, N, lane), load_bias_pair(p.bias, col0 + chalf * 64 + 32, N, lane)};
             bool ok = mbar_wait(bar_acc_full + 8 * acc, acc_phase, abort_flag, p.dev_status, p.spin_limit);
             if (aux_tma) ok = mbar_wait(bar_aux, (uint32_t)it & 1u, abort_flag, p.dev_status, p.spin_limit) && ok;
             if (epi_any(!ok)) break;      // a wait ran out in one of the eight warps: all of them leave together
@@ -702,16 +699,9 @@ k_gemm_mxf4_q(const __grid_constant__ CUtensorMap map_a, const __grid_constant__
                     __syncwarp();
                     if (lane == 0) mbar_arrive(bar_acc_empty + 8 * acc);   // the accumulator goes back to the MMA issuer
                 }
-                float v[32];
-#pragma unroll
-                for (int j = 0; j < 32; j++) v[j] = __uint_as_float(r[j]);
-                if (use_bias && live) add_bias<32>(v, p.bias + col, 32);
+                if (use_bias) add_bias_chunk(r, bias[cc]);
                 uint32_t yw[16];
-#pragma unroll
-                for (int j = 0; j < 16; j++) {
-                    const __nv_bfloat162 h = __floats2bfloat162_rn(v[2 * j], v[2 * j + 1]);
-                    yw[j] = *reinterpret_cast<const uint32_t *>(&h);
-                }
+                pack_row_bf16(r, yw);
                 if (WITH_Y && e.store_y) {
 #pragma unroll
                     for (int j = 0; j < 4; j++)
@@ -1036,13 +1026,16 @@ k_gemm_mxf4_bs(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
         uint32_t acc = 0, acc_phase = 0;
         for (int t = t0; t < t1; t++) {
             const int mb = t % p.tiles_m, nb = t / p.tiles_m;
+            uint32_t bias[kHalfCols / 32];
+#pragma unroll
+            for (int cc = 0; cc < kHalfCols / 32; cc++) bias[cc] = load_bias_pair(p.bias, (int64_t)nb * BN + chalf * kHalfCols + cc * 32, p.N, lane);
             if (!mbar_wait(bar_acc_full + 8 * acc, acc_phase, abort_flag, p.dev_status, p.spin_limit)) break;
             tc_fence_after();
             const int row0 = mb * kBM + quarter * 32;
             const int colbase = nb * BN + chalf * kHalfCols;
             const uint32_t taddr = tmem_base + ((uint32_t)(quarter * 32) << 16) + acc * BN + chalf * kHalfCols;
             epilogue_tile<BN, C::kStagingBufs>(&map_d, p.out_fp32 ? nullptr : &map_dw, p, taddr, row0, colbase, 0, staging, sbuf, lane,
-                                               bar_acc_empty + 8 * acc);
+                                               bar_acc_empty + 8 * acc, bias);
             if (++acc == 2) { acc = 0; acc_phase ^= 1u; }
         }
         if (lane == 0) bulk_wait0();   // all stores of this warp have completed before the CTA may exit
@@ -1710,6 +1703,9 @@ k_gemm_mxf4_pair(const __grid_constant__ CUtensorMap map_a, const __grid_constan
         for (int item = cluster_id; item < items && alive; item += num_clusters) {
             const int split = item % p.splits, tile = item / p.splits;
             const int mb = (tiles_m2 - 1 - tile / p.tiles_n) * 2 + (int)rank, nb = tile % p.tiles_n;
+            uint32_t bias[kHalfCols / 32];
+#pragma unroll
+            for (int cc = 0; cc < kHalfCols / 32; cc++) bias[cc] = load_bias_pair(p.bias, (int64_t)nb * BN + chalf * kHalfCols + cc * 32, p.N, lane);
             if (!mbar_wait_warp(bar_acc_full, acc_phase, abort_flag, p.dev_status, p.spin_limit)) { alive = false; break; }
             tc_fence_after();
             const int row0 = mb * kBM + quarter * 32;
@@ -1743,7 +1739,8 @@ k_gemm_mxf4_pair(const __grid_constant__ CUtensorMap map_a, const __grid_constan
                         uint32_t r[32];
                         tc_ld32(taddr + cc * 32, r);
                         tc_wait_ld();
-                        pack_row_bf16(r, use_bias ? p.bias + col : nullptr, (int)min((int64_t)32, p.N - col), pk[cc]);
+                        if (use_bias) add_bias_chunk(r, bias[cc]);
+                        pack_row_bf16(r, pk[cc]);
                     }
                 }
                 release_acc();
@@ -1782,14 +1779,7 @@ k_gemm_mxf4_pair(const __grid_constant__ CUtensorMap map_a, const __grid_constan
                     if (cc == kChunks - 1) release_acc();
                     if (!live) continue;
                     const int ncols = (int)min((int64_t)32, p.N - col);
-                    if (use_bias) {
-                        float v[32];
-#pragma unroll
-                        for (int j = 0; j < 32; j++) v[j] = __uint_as_float(r[j]);
-                        add_bias<32>(v, p.bias + col, ncols);
-#pragma unroll
-                        for (int j = 0; j < 32; j++) r[j] = __float_as_uint(v[j]);
-                    }
+                    if (use_bias) add_bias_chunk(r, load_bias_pair(p.bias, col, p.N, lane));
                     store_box(r, col);
                     if (ncols > 16) store_box(r + 16, col + 16);
                 }
@@ -2093,13 +2083,16 @@ k_gemm_mxf4_pbs(const __grid_constant__ CUtensorMap map_a, const __grid_constant
         for (int t = t0; t < t1; t++) {
             const PbsTile x = pbs_tile(walk, t);
             const int mb = x.mb2 * 2 + (int)rank, nb = x.nb;
+            uint32_t bias[kHalfCols / 32];
+#pragma unroll
+            for (int cc = 0; cc < kHalfCols / 32; cc++) bias[cc] = load_bias_pair(p.bias, (int64_t)nb * BN + chalf * kHalfCols + cc * 32, p.N, lane);
             if (!mbar_wait(bar_acc_full + 8 * acc, acc_phase, abort_flag, p.dev_status, p.spin_limit)) break;
             tc_fence_after();
             const int row0 = mb * kBM + quarter * 32;
             const int colbase = nb * BN + chalf * kHalfCols;
             const uint32_t taddr = tmem_base + ((uint32_t)(quarter * 32) << 16) + acc * BN + chalf * kHalfCols;
             epilogue_tile<BN, C::kStagingBufs, true>(&map_d, p.out_fp32 ? nullptr : &map_dw, p, taddr, row0, colbase, 0, staging, sbuf, lane,
-                                                     map_to_cta(bar_acc_empty + 8 * acc, 0));
+                                                     map_to_cta(bar_acc_empty + 8 * acc, 0), bias);
             if (++acc == 2) { acc = 0; acc_phase ^= 1u; }
         }
         if (lane == 0) bulk_wait0();   // all stores of this warp have completed before the CTA may exit

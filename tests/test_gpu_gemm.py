@@ -167,6 +167,13 @@ def test_gemm_bias_and_strided_output(mx, M, N, K, out_dtype):
     _bias_case(mx, M, N, K, out_dtype)
 
 
+@pytest.mark.parametrize("M,N,K", [(1, 8, 32), (197, 200, 384), (300, 264, 2600 // 32 * 32), (130, 40, 1056), (4100, 1752, 768)])
+@pytest.mark.parametrize("out_dtype", [0, 1])
+def test_gemm_bias_ragged_edges(mx, M, N, K, out_dtype):
+    """Bias pairs at the edges: a last chunk of 8 columns, one row, a partial last row tile, in every epilogue."""
+    _bias_case(mx, M, N, K, out_dtype)
+
+
 def test_gemm_argument_errors(mx):
     a, b = mx.QMat(128, 64), mx.QMat(128, 96)
     with pytest.raises(mx.MxError) as e:
