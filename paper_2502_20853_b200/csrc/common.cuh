@@ -48,7 +48,7 @@ __host__ __device__ __forceinline__ size_t scale_offset(int64_t row, int64_t blk
 // (mantissa + 63) >> 7 is 1 exactly when the 7-bit mantissa exceeds 0x40.
 __device__ __forceinline__ uint32_t scale_byte_from_amax(uint32_t amax_bits, uint32_t tf_add)
 {
-    const int b = (int)(amax_bits >> 7) - 2 + (int)(((amax_bits & 0x7Fu) + tf_add) >> 7);
+    const int b = (int)((amax_bits + tf_add) >> 7) - 2;   // the carry out of the mantissa is the increment
     return amax_bits ? (uint32_t)max(b, 0) : 98u;
 }
 __device__ __forceinline__ uint32_t tf_add_of(int scale_mode) { return scale_mode == MXFP4_SCALE_FLOOR ? 0u : 63u; }
@@ -110,19 +110,22 @@ __device__ __forceinline__ uint32_t mul_bf16x2(uint32_t a, uint32_t b)
     asm("mul.rn.bf16x2 %0, %1, %2;" : "=r"(d) : "r"(a), "r"(b));
     return d;
 }
+// A bf16 pair times a bf16 power of two each -> two FP32 latent values, by the mixed-precision FMA of sm_100: one full-rate
+// instruction per element (1.05 cycles per warp) does what a packed bf16 multiply (half rate: 2.0 cycles per pair) and an
+// unpack on the ALU pipe (2 cycles per element) did.  The addend -0 keeps the sign of a zero.  Exact: the product of two
+// bf16 values fits FP32.
+__device__ __forceinline__ void scale_pair(uint32_t w, uint32_t inv2, float &lo, float &hi)
+{
+    asm("{\n\t.reg .b16 a, b, c, d;\n\tmov.b32 {a, b}, %2;\n\tmov.b32 {c, d}, %3;\n\t"
+        "fma.rn.f32.bf16 %0, a, c, %4;\n\tfma.rn.f32.bf16 %1, b, d, %4;\n\t}"
+        : "=&f"(lo), "=&f"(hi) : "r"(w), "r"(inv2), "f"(-0.0f));
+}
 // 2^-s in both halves for s = byte - 127 (byte <= 253)
 __device__ __forceinline__ uint32_t inv_scale_bf16x2(uint32_t byte) { return ((254u - byte) << 7) * 0x00010001u; }
-// 2^s in both halves (byte 0 gives the subnormal 2^-127)
-__device__ __forceinline__ uint32_t scale_bf16x2(uint32_t byte) { return (byte ? (byte << 7) : 0x0040u) * 0x00010001u; }
 
-// Eight E2M1 codes (one word, code 0 in the lowest nibble) times the bf16 pair `sc2` (the same power of two in both
-// halves, or NaN) -> eight bf16 values in four words.  Exact: the products have at most two significant bits.
-__device__ __forceinline__ void dequant_x8(uint32_t codes, uint32_t sc2, uint32_t (&o)[4])
+// Four f16 pairs that hold E2M1 values, times the bf16 pair sc2 -> four bf16 pairs.
+__device__ __forceinline__ void scale_f16_pairs(const uint32_t (&h)[4], uint32_t sc2, uint32_t (&o)[4])
 {
-    uint32_t h[4];
-    asm("{\n\t.reg .b8 b0, b1, b2, b3;\n\tmov.b32 {b0, b1, b2, b3}, %4;\n\t"
-        "cvt.rn.f16x2.e2m1x2 %0, b0;\n\tcvt.rn.f16x2.e2m1x2 %1, b1;\n\tcvt.rn.f16x2.e2m1x2 %2, b2;\n\tcvt.rn.f16x2.e2m1x2 %3, b3;\n\t}"
-        : "=r"(h[0]), "=r"(h[1]), "=r"(h[2]), "=r"(h[3]) : "r"(codes));
 #pragma unroll
     for (int j = 0; j < 4; j++) {
         const float2 f = __half22float2(*reinterpret_cast<const __half2 *>(&h[j]));
@@ -132,22 +135,40 @@ __device__ __forceinline__ void dequant_x8(uint32_t codes, uint32_t sc2, uint32_
     }
 }
 
+// Eight E2M1 codes (one word, code 0 in the lowest nibble) times the bf16 pair `sc2` (the same power of two in both
+// halves, or NaN) -> eight bf16 values in four words.  Exact: the products have at most two significant bits.
+// The bytes are taken out of the word by way of its halves: ptxas 12.9 loses the upper half when a word that was packed from
+// four conversions (rne_x8) is unpacked into four bytes right away.
+__device__ __forceinline__ void dequant_x8(uint32_t codes, uint32_t sc2, uint32_t (&o)[4])
+{
+    uint32_t h[4];
+    asm("{\n\t.reg .b8 b0, b1, b2, b3;\n\t.reg .b16 c0, c1, c2, c3;\n\t.reg .b32 t;\n\t"
+        "shr.u32 t, %4, 16;\n\tmov.b32 {c0, c2}, %4;\n\tmov.b32 {c1, c3}, t;\n\tmov.b16 {b0, b1}, c0;\n\tmov.b16 {b2, b3}, c1;\n\t"
+        "cvt.rn.f16x2.e2m1x2 %0, b0;\n\tcvt.rn.f16x2.e2m1x2 %1, b1;\n\tcvt.rn.f16x2.e2m1x2 %2, b2;\n\tcvt.rn.f16x2.e2m1x2 %3, b3;\n\t}"
+        : "=r"(h[0]), "=r"(h[1]), "=r"(h[2]), "=r"(h[3]) : "r"(codes));
+    scale_f16_pairs(h, sc2, o);
+}
+
 // Stochastic rounding (Sec. 3.2: q2 iff v + xi >= midpoint, xi = D (u - 1/2)  <=>  f + u >= 1, f the
-// fraction of the way from the lower to the upper grid neighbour, u = u16 * 2^-16) of four consecutive
-// latent values with the sm_100a stochastic-rounding convert.  `w` is the random word of these four
+// fraction of the way from the lower to the upper grid neighbour, u = u16 * 2^-16) of consecutive
+// latent values, four at a time, with the sm_100a stochastic-rounding convert.  `w` is the random word of these four
 // elements: its low half is the 16-bit draw of the pair (v0, v1), its high half that of (v2, v3); within a
 // pair the second element reads the draw with its bit order reversed.  The result has the code of v0 in
 // its low nibble.  Magnitudes above 6 saturate; the sign of the source is kept, also on zero.
 // The convert adds the 16 random bits below the last kept bit and truncates, which is exactly f + u >= 1.
 // It expects the draw of the first pair in bytes 2 (high) and 0 (low) of its operand and that of the second
 // pair in bytes 3 and 1, hence the byte permutation.
-__device__ __forceinline__ uint32_t sr4(float v0, float v1, float v2, float v3, uint32_t w)
+// Eight values in one go: the two 16-bit results are merged once.
+__device__ __forceinline__ uint32_t sr_x8(float v0, float v1, float v2, float v3, float v4, float v5, float v6, float v7, uint32_t w0, uint32_t w1)
 {
-    uint32_t rb;
-    asm("prmt.b32 %0, %1, %1, 0x3120;" : "=r"(rb) : "r"(w));
-    uint16_t d;
-    asm("cvt.rs.satfinite.e2m1x4.f32 %0, {%1, %2, %3, %4}, %5;" : "=h"(d) : "f"(v3), "f"(v2), "f"(v1), "f"(v0), "r"(rb));
-    return (uint32_t)d;
+    uint32_t d;
+    asm("{\n\t.reg .b32 r0, r1;\n\t.reg .b16 d0, d1;\n\t"
+        "prmt.b32 r0, %9, %9, 0x3120;\n\tprmt.b32 r1, %10, %10, 0x3120;\n\t"
+        "cvt.rs.satfinite.e2m1x4.f32 d0, {%4, %3, %2, %1}, r0;\n\t"
+        "cvt.rs.satfinite.e2m1x4.f32 d1, {%8, %7, %6, %5}, r1;\n\t"
+        "mov.b32 %0, {d0, d1};\n\t}"
+        : "=r"(d) : "f"(v0), "f"(v1), "f"(v2), "f"(v3), "f"(v4), "f"(v5), "f"(v6), "f"(v7), "r"(w0), "r"(w1));
+    return d;
 }
 
 // ---- Philox4x32-10 ----------------------------------------------------------------------------
@@ -156,10 +177,12 @@ __device__ __forceinline__ uint32_t sr4(float v0, float v1, float v2, float v3, 
 struct SrStream {
     uint32_t k[20];      // k[2i] = seed_lo + i * 0x9E3779B9, k[2i+1] = seed_hi + i * 0xBB67AE85
     uint32_t stream_id;  // third counter word
-    uint32_t pad;
+    uint32_t wide;       // the output has more than 2^36 elements: the second counter word is not always zero
+    uint32_t x0, x2, c3; // with a second counter word of zero, the parts of the first two rounds that depend on the seed alone
 };
 
-inline SrStream make_sr_stream(uint64_t seed, uint32_t stream_id)
+// elements: of the quantizer's output
+inline SrStream make_sr_stream(uint64_t seed, uint32_t stream_id, int64_t elements)
 {
     SrStream s;
     uint32_t k0 = (uint32_t)seed, k1 = (uint32_t)(seed >> 32);
@@ -170,17 +193,38 @@ inline SrStream make_sr_stream(uint64_t seed, uint32_t stream_id)
         k1 += 0xBB67AE85u;
     }
     s.stream_id = stream_id;
-    s.pad = 0;
+    s.wide = elements > (1ll << 36) ? 1u : 0u;
+    const uint64_t p1 = (uint64_t)0xCD9E8D57u * stream_id;                          // round 0
+    const uint64_t p0 = (uint64_t)0xD2511F53u * ((uint32_t)(p1 >> 32) ^ s.k[0]);   // round 1
+    s.x0 = (uint32_t)p1 ^ s.k[2];
+    s.x2 = (uint32_t)(p0 >> 32) ^ s.k[3];
+    s.c3 = (uint32_t)p0;
     return s;
 }
 
 // The random words of elements 16q .. 16q+15 of a quantizer's output (counter = (q, stream_id, 0)):
-// elements 4k .. 4k+3 use word k (see sr4).
+// elements 4k .. 4k+3 use word k (see sr_x8).
+// A wide multiply holds its pipe for four cycles per warp, and the 20 of a call are what bounds it.  Unless the output has
+// more than 2^36 elements (WIDE) the second counter word is zero, and everything in the first two rounds that does not depend
+// on the first one is made on the host (two products, two XORs): a call has 18 products and takes 80 cycles per warp and SM
+// quarter.  (The high halves by FP64 FMAs beside a low multiply were slower: 87 to 96 cycles.)
+template <bool WIDE>
 __device__ __forceinline__ uint4 sr_words(const SrStream &s, uint64_t q)
 {
-    uint32_t c0 = (uint32_t)q, c1 = (uint32_t)(q >> 32), c2 = s.stream_id, c3 = 0u;
+    uint32_t c0, c1, c2, c3;
+    if (WIDE) {
+        c0 = (uint32_t)q, c1 = (uint32_t)(q >> 32), c2 = s.stream_id, c3 = 0u;
+    } else {
+        const uint64_t p0 = (uint64_t)0xD2511F53u * (uint32_t)q;               // round 0
+        c2 = (uint32_t)(p0 >> 32) ^ s.k[1];
+        const uint64_t p1 = (uint64_t)0xCD9E8D57u * c2;                        // round 1
+        c0 = (uint32_t)(p1 >> 32) ^ s.x0;
+        c1 = (uint32_t)p1;
+        c2 = (uint32_t)p0 ^ s.x2;
+        c3 = s.c3;
+    }
 #pragma unroll
-    for (int i = 0; i < 10; i++) {
+    for (int i = WIDE ? 0 : 2; i < 10; i++) {
         const uint64_t p0 = (uint64_t)0xD2511F53u * c0;
         const uint64_t p1 = (uint64_t)0xCD9E8D57u * c2;
         c0 = (uint32_t)(p1 >> 32) ^ c1 ^ s.k[2 * i];
@@ -189,6 +233,12 @@ __device__ __forceinline__ uint4 sr_words(const SrStream &s, uint64_t q)
         c3 = (uint32_t)p0;
     }
     return make_uint4(c0, c1, c2, c3);
+}
+// Two calls, by the width of the counter (a launch-uniform branch).
+__device__ __forceinline__ void sr_words_two(const SrStream &s, uint64_t qa, uint64_t qb, uint4 &ra, uint4 &rb)
+{
+    if (s.wide) ra = sr_words<true>(s, qa), rb = sr_words<true>(s, qb);
+    else ra = sr_words<false>(s, qa), rb = sr_words<false>(s, qb);
 }
 
 // ---- small helpers ------------------------------------------------------------------------------

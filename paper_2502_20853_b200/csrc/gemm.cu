@@ -652,9 +652,9 @@ k_gemm_mxf4_q(const __grid_constant__ CUtensorMap map_a, const __grid_constant__
         // ================= quantizing epilogue (warps 4..11 = 256 threads) =================
         const int et = (int)threadIdx.x - 32 * kEpiWarp0;
         const int quarter = warp & 3, chalf = (warp - kEpiWarp0) >> 2;
-        const QsGeom g = qs_geom(et);
         const int M = (int)p.M, N = (int)p.N;
-        const uint32_t tfa_r = tf_add_of(e.rw.scale_mode), tfa_t2 = tf_add_of(e.tr.scale_mode) * 0x00010001u;
+        const QsGeom g = qs_geom(et, M, N, e.rw.packed);
+        const uint32_t tfa_r2 = tf_add_of(e.rw.scale_mode) * 0x00010001u, tfa_t2 = tf_add_of(e.tr.scale_mode) * 0x00010001u;
         const uint32_t t_base = smem_base + C::kTileOff, t2_base = smem_base + C::kTile2Off, ty_base = smem_base + C::kTileYOff;
         const int trow = quarter * 32 + lane;                        // this thread's row of the tile
         const uint32_t row_off = (uint32_t)(chalf * (kTileBytes / 2) + trow * 128);
@@ -762,9 +762,8 @@ k_gemm_mxf4_q(const __grid_constant__ CUtensorMap map_a, const __grid_constant__
                 bulk_commit();
                 if (aux_tma && item + (int)gridDim.x < items) issue_aux(item + gridDim.x);
             }
-            if (e.emit_row) qs_row_pass<SR_ROW, DQ>(g, t_base, t2_base, row0, col0, M, N, e.rw, tfa_r, s_sc_row, nonfinite);
-            if (DQ) __syncwarp();                         // the column pass reads what the row pass of the same warp wrote
-            if (e.emit_t) qs_col_pass<SR_T>(g, DQ ? t2_base : t_base, row0, col0, M, N, e.tr, tfa_t2, staging, s_sc_t, nonfinite);
+            qs_tile<SR_ROW, SR_T, DQ>(g, t_base, t2_base, row0, col0, M, N, e.emit_row, e.emit_t, e.rw, e.tr, tfa_r2, tfa_t2, staging, s_sc_row, s_sc_t,
+                                      nonfinite);
             fence_async_smem();
             if (et == 0) bulk_wait_read<0>();             // Z has left the tile, the previous tile's codes their staging buffer
             epi_sync();
@@ -2494,7 +2493,7 @@ static QuantSide make_quant_side(const mxfp4_mat_t &m, const mxfp4_qparams_t &qp
     s.scales = m.scales;
     s.nblk4 = (int)ceil_div(m.cols / 32, 4);
     s.scale_mode = qp.scale_mode;
-    s.sr = make_sr_stream(qp.seed, qp.stream_id);
+    s.sr = make_sr_stream(qp.seed, qp.stream_id, m.rows * m.cols);
     return s;
 }
 

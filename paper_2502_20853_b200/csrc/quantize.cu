@@ -66,7 +66,8 @@ __global__ void __launch_bounds__(256) k_quantize_rows(const __nv_bfloat16 *__re
             out = make_uint4(rne8(q[0], inv), rne8(q[1], inv), rne8(q[2], inv), rne8(q[3], inv));
         } else {
             const uint64_t q0 = ((uint64_t)row * ((uint64_t)nblk * 32) + (uint64_t)blk * 32) >> 4;
-            const uint4 ra = sr_words(sr, q0), rb = sr_words(sr, q0 + 1);
+            uint4 ra, rb;
+            sr_words_two(sr, q0, q0 + 1, ra, rb);
             out.x = sr8(q[0], inv, ra.x, ra.y);
             out.y = sr8(q[1], inv, ra.z, ra.w);
             out.z = sr8(q[2], inv, rb.x, rb.y);
@@ -89,7 +90,7 @@ __global__ void __launch_bounds__(256) k_quantize_rows(const __nv_bfloat16 *__re
 constexpr int kPitch = 2 * kTile + 16;   // bytes per staged row (16-byte skew against bank conflicts)
 
 template <bool SR_T>
-__global__ void __launch_bounds__(256, 4) k_requantize_tile(const void *__restrict__ src, const uint8_t *__restrict__ src_scales,
+__global__ void __launch_bounds__(256, 3) k_requantize_tile(const void *__restrict__ src, const uint8_t *__restrict__ src_scales,
                                                             int src_nblk4, int rows, int cols, const __grid_constant__ QuantSide tr,
                                                             uint32_t *dev_status)
 {
@@ -120,7 +121,7 @@ __global__ void __launch_bounds__(256, 4) k_requantize_tile(const void *__restri
                 w[0] = q.x; w[1] = q.y; w[2] = q.z; w[3] = q.w;
                 const uint32_t sb = sc_chunk[(r & 31) * 16 + (r >> 5) * 4 + g];
                 // a 0xFF scale marks a non-finite group of the first quantizer: propagate NaN
-                sc2 = sb == 0xFFu ? 0x7FC07FC0u : scale_bf16x2(sb);
+                sc2 = sb == 0xFFu ? 0x7FC07FC0u : (sb ? sb << 7 : 0x0040u) * 0x00010001u;   // byte 0: 2^-127
             }
 #pragma unroll
             for (int j = 0; j < 4; j++) {
@@ -153,41 +154,43 @@ __global__ void __launch_bounds__(256, 4) k_requantize_tile(const void *__restri
         // rows come in groups of 32 and columns in blocks of 32: a thread's 16 x 4 patch is inside the matrix or outside it
         if (row0 + r < rows && col0 + c < cols) {
             const uint32_t tfa2 = tf_add_of(tr.scale_mode) * 0x00010001u;
-            const uint32_t b01 = scale_bytes_x2(am0, tfa2), b23 = scale_bytes_x2(am1, tfa2);
             // element index of (column, first row) in the transposed output, in units of 16
             const uint64_t qi = ((uint64_t)(col0 + c) * (uint64_t)rows + (uint64_t)(row0 + r)) >> 4;
 #pragma unroll
             for (int jp = 0; jp < 2; jp++) {      // columns c + 2 jp and c + 2 jp + 1 share a word of every row
-                const uint32_t b2 = jp ? b23 : b01;
-                const uint32_t nfm = __vcmpeq2(b2, 0x00FF00FFu);                 // 0xFFFF in the half of a non-finite group
+                const uint32_t am = jp ? am1 : am0;
+                uint32_t m2, inv2;
+                group_scales_x2(am, tfa2, m2, inv2);
+                const uint32_t nfm = (am + 0x00800080u) & 0x80008000u;   // bit 15 of the half of a non-finite group
                 nonfinite |= (uint32_t)(nfm != 0u);
-                const uint32_t inv2 = (0x00FE00FEu - ((b2 & ~nfm) | (nfm & 0x007F007Fu))) << 7;   // 2^-s of both columns as bf16
-                uint32_t lo0, hi0, lo1, hi1;   // codes of rows 0..7 / 8..15 of the two columns
-                uint32_t x[16];
-#pragma unroll
-                for (int i = 0; i < 16; i++) x[i] = mul_bf16x2(jp ? v[i].y : v[i].x, inv2);
+                uint32_t out[2][2];            // codes of rows 0..7 / 8..15 of the two columns
+                uint4 ra, rb;
                 if (SR_T) {
-                    const uint4 ra = sr_words(tr.sr, qi + (uint64_t)(2 * jp) * (uint64_t)(rows >> 4));
-                    const uint4 rb = sr_words(tr.sr, qi + (uint64_t)(2 * jp + 1) * (uint64_t)(rows >> 4));
-                    lo0 = sr4(bf16lo(x[0]), bf16lo(x[1]), bf16lo(x[2]), bf16lo(x[3]), ra.x) | (sr4(bf16lo(x[4]), bf16lo(x[5]), bf16lo(x[6]), bf16lo(x[7]), ra.y) << 16);
-                    hi0 = sr4(bf16lo(x[8]), bf16lo(x[9]), bf16lo(x[10]), bf16lo(x[11]), ra.z) | (sr4(bf16lo(x[12]), bf16lo(x[13]), bf16lo(x[14]), bf16lo(x[15]), ra.w) << 16);
-                    lo1 = sr4(bf16hi(x[0]), bf16hi(x[1]), bf16hi(x[2]), bf16hi(x[3]), rb.x) | (sr4(bf16hi(x[4]), bf16hi(x[5]), bf16hi(x[6]), bf16hi(x[7]), rb.y) << 16);
-                    hi1 = sr4(bf16hi(x[8]), bf16hi(x[9]), bf16hi(x[10]), bf16hi(x[11]), rb.z) | (sr4(bf16hi(x[12]), bf16hi(x[13]), bf16hi(x[14]), bf16hi(x[15]), rb.w) << 16);
-                } else {
-                    lo0 = rne_x8(bf16lo(x[0]), bf16lo(x[1]), bf16lo(x[2]), bf16lo(x[3]), bf16lo(x[4]), bf16lo(x[5]), bf16lo(x[6]), bf16lo(x[7]));
-                    hi0 = rne_x8(bf16lo(x[8]), bf16lo(x[9]), bf16lo(x[10]), bf16lo(x[11]), bf16lo(x[12]), bf16lo(x[13]), bf16lo(x[14]), bf16lo(x[15]));
-                    lo1 = rne_x8(bf16hi(x[0]), bf16hi(x[1]), bf16hi(x[2]), bf16hi(x[3]), bf16hi(x[4]), bf16hi(x[5]), bf16hi(x[6]), bf16hi(x[7]));
-                    hi1 = rne_x8(bf16hi(x[8]), bf16hi(x[9]), bf16hi(x[10]), bf16hi(x[11]), bf16hi(x[12]), bf16hi(x[13]), bf16hi(x[14]), bf16hi(x[15]));
+                    const uint64_t qa = qi + (uint64_t)(2 * jp) * (uint64_t)(rows >> 4);
+                    sr_words_two(tr.sr, qa, qa + (uint64_t)(rows >> 4), ra, rb);
                 }
-                if (nfm & 0x0000FFFFu) lo0 = hi0 = 0u;
-                if (nfm & 0xFFFF0000u) lo1 = hi1 = 0u;
+#pragma unroll
+                for (int k = 0; k < 2; k++) {
+                    float a[8], b[8];
+#pragma unroll
+                    for (int i = 0; i < 8; i++) scale_pair(jp ? v[8 * k + i].y : v[8 * k + i].x, inv2, a[i], b[i]);
+                    if (SR_T) {
+                        out[0][k] = sr_x8(a[0], a[1], a[2], a[3], a[4], a[5], a[6], a[7], k ? ra.z : ra.x, k ? ra.w : ra.y);
+                        out[1][k] = sr_x8(b[0], b[1], b[2], b[3], b[4], b[5], b[6], b[7], k ? rb.z : rb.x, k ? rb.w : rb.y);
+                    } else {
+                        out[0][k] = rne_x8(a[0], a[1], a[2], a[3], a[4], a[5], a[6], a[7]);
+                        out[1][k] = rne_x8(b[0], b[1], b[2], b[3], b[4], b[5], b[6], b[7]);
+                    }
+                }
+                if (nfm & 0x8000u) out[0][0] = out[0][1] = 0u;
+                if (nfm >> 31) out[1][0] = out[1][1] = 0u;
                 // output row c + j, bytes 16 rg + 8 h .. + 7: slot 2 rg + h, swizzled by the column quad
                 const int j0 = 2 * jp;
-                s_out[(c + j0) * 8 + ((2 * rg + h) ^ (cl & 7))] = make_uint2(lo0, hi0);
-                s_out[(c + j0 + 1) * 8 + ((2 * rg + h) ^ (cl & 7))] = make_uint2(lo1, hi1);
+                s_out[(c + j0) * 8 + ((2 * rg + h) ^ (cl & 7))] = make_uint2(out[0][0], out[0][1]);
+                s_out[(c + j0 + 1) * 8 + ((2 * rg + h) ^ (cl & 7))] = make_uint2(out[1][0], out[1][1]);
                 if (h == 0) {
-                    s_sc_t[((c + j0) & 31) * 16 + ((c + j0) >> 5) * 4 + rg] = (uint8_t)(b2 & 0xFFu);
-                    s_sc_t[((c + j0 + 1) & 31) * 16 + ((c + j0 + 1) >> 5) * 4 + rg] = (uint8_t)(b2 >> 16);
+                    s_sc_t[((c + j0) & 31) * 16 + ((c + j0) >> 5) * 4 + rg] = (uint8_t)((nfm & 0x8000u) ? 0xFFu : (am & 0xFFFFu) ? m2 - 2u : 98u);
+                    s_sc_t[((c + j0 + 1) & 31) * 16 + ((c + j0 + 1) >> 5) * 4 + rg] = (uint8_t)((nfm >> 31) ? 0xFFu : am >= 0x10000u ? (m2 >> 16) - 2u : 98u);
                 }
             }
         }
@@ -270,8 +273,8 @@ k_quantize_stream(const __grid_constant__ CUtensorMap map_src, const __grid_cons
     }
     __syncthreads();
 
-    const QsGeom g = qs_geom(tid);
-    const uint32_t tfa_r = tf_add_of(rw.scale_mode), tfa_t2 = tf_add_of(tr.scale_mode) * 0x00010001u;
+    const QsGeom g = qs_geom(tid, rows, cols, rw.packed);
+    const uint32_t tfa_r2 = tf_add_of(rw.scale_mode) * 0x00010001u, tfa_t2 = tf_add_of(tr.scale_mode) * 0x00010001u;
     uint32_t nonfinite = 0;
     // tile coordinates advance by the grid size without a division per tile
     const int step_y = (int)gridDim.x / ntx, step_x = (int)gridDim.x - step_y * ntx;
@@ -284,12 +287,9 @@ k_quantize_stream(const __grid_constant__ CUtensorMap map_src, const __grid_cons
         uint8_t *staging = smem + 2 * kTileBytes + stage * kQsStagingBytes;
         uint8_t *s_sc_row = staging + kTile * 64, *s_sc_t = s_sc_row + 512;
 
-        const bool ok = mbar_wait(bar_full + 8 * stage, (uint32_t)(it >> 1) & 1u, abort_flag, dev_status, spin_limit);
-
-        if (EMIT_ROW && ok) qs_row_pass<SR_ROW, DQ>(g, st_base, st_base, row0, col0, rows, cols, rw, tfa_r, s_sc_row, nonfinite);
-        if (DQ) __syncwarp();      // the column pass reads what the row pass of the SAME warp wrote back
-
-        if (ok) qs_col_pass<SR_T>(g, st_base, row0, col0, rows, cols, tr, tfa_t2, staging, s_sc_t, nonfinite);
+        const bool ok = mbar_wait_warp(bar_full + 8 * stage, (uint32_t)(it >> 1) & 1u, abort_flag, dev_status, spin_limit);
+        if (ok)
+            qs_tile<SR_ROW, SR_T, DQ>(g, st_base, st_base, row0, col0, rows, cols, EMIT_ROW, true, rw, tr, tfa_r2, tfa_t2, staging, s_sc_row, s_sc_t, nonfinite);
 
         // ---- hand the tile's results to the copy engine, refill the ring ----
         fence_async_smem();                       // this thread's staging writes, before the asynchronous reads
@@ -518,11 +518,11 @@ mxfp4_status_t quantize_rows(const void *src, int64_t rows, int64_t cols, int64_
     if (qp->rounding == MXFP4_ROUND_STOCHASTIC)
         k_quantize_rows<MXFP4_ROUND_STOCHASTIC><<<blocks, 256, 0, st>>>(
             static_cast<const __nv_bfloat16 *>(src), rows, nblk, ld, static_cast<uint8_t *>(dst.data), dst.scales, nblk4,
-            qp->scale_mode, make_sr_stream(qp->seed, qp->stream_id), dev_status);
+            qp->scale_mode, make_sr_stream(qp->seed, qp->stream_id, rows * cols), dev_status);
     else
         k_quantize_rows<MXFP4_ROUND_NEAREST><<<blocks, 256, 0, st>>>(
             static_cast<const __nv_bfloat16 *>(src), rows, nblk, ld, static_cast<uint8_t *>(dst.data), dst.scales, nblk4,
-            qp->scale_mode, make_sr_stream(qp->seed, qp->stream_id), dev_status);
+            qp->scale_mode, make_sr_stream(qp->seed, qp->stream_id, rows * cols), dev_status);
     MX_CHECK_LAUNCH();
     return MXFP4_OK;
 }
@@ -534,7 +534,7 @@ static QuantSide make_side(const mxfp4_mat_t &m, const mxfp4_qparams_t *qp)
     s.scales = m.scales;
     s.nblk4 = (int)ceil_div(m.cols / 32, 4);
     s.scale_mode = qp->scale_mode;
-    s.sr = make_sr_stream(qp->seed, qp->stream_id);
+    s.sr = make_sr_stream(qp->seed, qp->stream_id, m.rows * m.cols);
     return s;
 }
 

@@ -91,3 +91,39 @@ def test_product_with_8194_row_tiles(mx, big):
     pb, sb = wq.data.cpu().numpy(), wq.scales_linear().cpu().numpy()
     dref, tref = orc.gemm(pa, sa, pb, sb)
     check_gemm_bound(rows_of(y, rows, as_float=True), dref, tref, True, "Y on sampled rows of 1048736")
+
+
+def test_quantizing_epilogue_beyond_2_to_36_elements(mx):
+    """Outputs with more than 2^36 elements: the random counters (one per 16 elements) pass 2^32 and take the quantizer's
+    passes through their wide-counter form, along the rows and along the columns."""
+    M, N, K = (1 << 23) + 160, 8224, 32
+    assert M * N > 1 << 36
+    torch.cuda.empty_cache()
+    free, _ = torch.cuda.mem_get_info()
+    if free < 84 << 30:
+        pytest.skip("needs 84 GB of free device memory")
+    g = torch.Generator(device="cuda").manual_seed(36)
+    a = mx.quantize(torch.randn((M, K), device="cuda", generator=g).to(torch.bfloat16))
+    b = mx.quantize(torch.randn((N, K), device="cuda", generator=g).to(torch.bfloat16))
+    new = lambda r, c: mx.QMat(r, c, data=torch.empty((r, c // 2), dtype=torch.uint8, device="cuda"),  # noqa: E731
+                               scales=torch.empty(mx.scale_bytes(r, c), dtype=torch.uint8, device="cuda"))
+    zq, zq_t = new(M, N), new(N, M)
+    st, seed = mx.new_status(), 0x5EED0000 + 36
+    mx.gemm_quant(a, b, mx.Epilogue(zq=zq, qp_row=(0, 1, seed, 3), zq_t=zq_t, qp_t=(0, 1, seed, 5)), dev_status=st)
+    torch.cuda.synchronize()
+    assert int(st.item()) == 0
+    bf = mx.dequantize(b)
+    for r0, c0 in [(0, 0), (M - 32, N - 32), (M - 32, 0), (M - 192, N - 64)]:
+        rows = torch.arange(r0, r0 + 32, device="cuda")
+        sa = torch.stack([a.scales[mx.scale_offset(r, 0, K)] for r in range(r0, r0 + 32)])
+        codes = a.data[rows].cpu().numpy()
+        z = torch.from_numpy(orc.dequantize(codes, sa.cpu().numpy().reshape(32, 1))).cuda().double() @ bf[c0:c0 + 32].double().t()
+        z = z.to(torch.bfloat16).float().cpu().numpy()          # 32 exact products per element: one rounding
+        p, s, _ = orc.quantize(z, rounding=1, seed=seed, stream_id=3, out_row0=r0, out_col0=c0, out_ld=N)
+        got = torch.stack([zq.scales[mx.scale_offset(r, c0 // 32, N)] for r in range(r0, r0 + 32)]).cpu().numpy()
+        assert (got == s[:, 0]).all() and (zq.data[rows, c0 // 2:c0 // 2 + 16].cpu().numpy() == p).all(), (r0, c0)
+        p, s, _ = orc.quantize(z, transpose=True, rounding=1, seed=seed, stream_id=5, out_row0=c0, out_col0=r0, out_ld=M)
+        got = torch.stack([zq_t.scales[mx.scale_offset(c, r0 // 32, M)] for c in range(c0, c0 + 32)]).cpu().numpy()
+        assert (got == s[:, 0]).all() and (zq_t.data[c0:c0 + 32, r0 // 2:r0 // 2 + 16].cpu().numpy() == p).all(), (r0, c0)
+    del zq, zq_t, a
+    torch.cuda.empty_cache()

@@ -103,6 +103,30 @@ def test_chain_equals_quantize_then_double_quantization(mx, rounding):
         assert_qmat_equal(qt, p2, s2, "chain: double quantization")
 
 
+@pytest.mark.parametrize("shape", [(160, 96), (256, 288)])
+@pytest.mark.parametrize("rounding", [0, 1])
+def test_two_axis_passes_over_every_scale(mx, shape, rounding):
+    """Groups at every scale from bf16's subnormals to its largest values, all-zero groups and isolated Inf / NaN, through
+    both passes of the tile quantizer, plain and chained (the rare groups are put right after the pass)."""
+    rng = np.random.default_rng(shape[0] + rounding)
+    e = rng.integers(-132, 126, (shape[0] // 32, shape[1] // 32)).repeat(32, 0).repeat(32, 1)
+    e[:, ::40] = rng.integers(-132, 126, e[:, ::40].shape)      # single columns far from their neighbours
+    with np.errstate(over="ignore"):
+        x = workloads.round_to_bf16(np.ldexp(rng.standard_normal(shape).clip(-1.9, 1.9), e).astype(np.float32))
+    x[32:64, 32:64] = 0.0
+    x[64:96, 5] = 0.0
+    x[7, 70], x[40, 3], x[130, 33], x[131, 32] = np.inf, np.nan, -np.inf, np.nan
+    for sm in (0, 1):
+        want = orc.quantize(x, scale_mode=sm, rounding=rounding, seed=3, stream_id=3)
+        q, qt = mx.quantize_2axis(to_dev_bf16(x), (sm, rounding, 3, 3), (sm, rounding, 3, 5))
+        assert_qmat_equal(q, *want[:2], "row pass")
+        assert_qmat_equal(qt, *orc.quantize(x, transpose=True, scale_mode=sm, rounding=rounding, seed=3, stream_id=5)[:2], "column pass")
+        q, qt = mx.quantize_chain(to_dev_bf16(x), seed=3, scale_mode=sm, rounding=rounding, stream_id=3, rounding_t=rounding)
+        assert_qmat_equal(q, *want[:2], "chain: row pass")
+        want_t = orc.quantize(orc.dequantize(*want[:2]), transpose=True, scale_mode=sm, rounding=rounding, seed=3, stream_id=6)
+        assert_qmat_equal(qt, *want_t[:2], "chain: column pass")
+
+
 def test_double_quantization_and_dequantize(mx):
     rng = np.random.default_rng(7)
     x = rand_bf16(rng, (160, 224))
