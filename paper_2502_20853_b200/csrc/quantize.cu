@@ -8,33 +8,10 @@
 namespace mx {
 
 // ------------------------------------------------------------------------------------------------
-// Fill the padding entries (rows beyond `rows` up to a multiple of 128, blocks beyond `nblk` up to
-// a multiple of 4) of a tiled scale buffer with 0x7F (= scale 1).
-// ------------------------------------------------------------------------------------------------
-__global__ void k_fill_scale_padding(uint8_t *scales, int64_t rows, int64_t nblk, int64_t nblk4)
-{
-    const int64_t rows_pad = ceil_div(rows, 128) * 128;
-    const int64_t nb_pad = nblk4 * 4;
-    const int64_t total = rows_pad * nb_pad;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t r = i / nb_pad, b = i - r * nb_pad;
-        if (r >= rows || b >= nblk) scales[scale_offset(r, b, nblk4)] = 0x7F;
-    }
-}
-
-static void fill_padding_if_needed(uint8_t *scales, int64_t rows, int64_t cols, cudaStream_t st)
-{
-    const int64_t nblk = cols / 32, nblk4 = ceil_div(nblk, 4);
-    if (rows % 128 == 0 && nblk % 4 == 0) return;
-    const int64_t total = ceil_div(rows, 128) * 128 * nblk4 * 4;
-    int64_t nb = ceil_div(total, 256);
-    int blocks = (int)(nb < 1184 ? nb : 1184);
-    k_fill_scale_padding<<<blocks, 256, 0, st>>>(scales, rows, nblk, nblk4);
-    MX_LAUNCHED();
-}
-
-// ------------------------------------------------------------------------------------------------
-// Row-wise quantizer: one thread per 32-element group (Eq. 1 with 1x32 groups).
+// Row-wise quantizer: one thread per 32-element group (Eq. 1 with 1x32 groups).  The grid covers the scale buffer, rows up to
+// a multiple of 128 and blocks up to a multiple of 4: a thread outside the matrix writes the padding entry 0x7F (= scale 1),
+// so that ragged shapes take one launch (a launch of its own for the padding took 1.6 us at 197 rows and 3.1 us at 19700 x 768
+// of the 12 and 15 us of the whole quantization with the gaps around it).
 // ------------------------------------------------------------------------------------------------
 template <int ROUNDING>
 __global__ void __launch_bounds__(256) k_quantize_rows(const __nv_bfloat16 *__restrict__ src, int64_t rows, int nblk,
@@ -42,10 +19,14 @@ __global__ void __launch_bounds__(256) k_quantize_rows(const __nv_bfloat16 *__re
                                                        uint8_t *__restrict__ scales, int nblk4, int scale_mode,
                                                        const SrStream sr, uint32_t *dev_status)
 {
-    const int64_t gid = blockIdx.x * (int64_t)256 + threadIdx.x;
-    if (gid >= rows * nblk) return;
-    const int64_t row = gid / nblk;
-    const int blk = (int)(gid - row * nblk);
+    const uint64_t gid = blockIdx.x * (uint64_t)256 + threadIdx.x;
+    const uint32_t nb_pad = (uint32_t)nblk4 * 4u;
+    const int64_t row = (gid >> 32) ? (int64_t)(gid / nb_pad) : (int64_t)((uint32_t)gid / nb_pad);
+    const int blk = (int)(gid - (uint64_t)row * nb_pad);
+    if (row >= rows || blk >= nblk) {
+        scales[scale_offset(row, blk, nblk4)] = 0x7F;
+        return;
+    }
     const uint4 *p = reinterpret_cast<const uint4 *>(src + row * ld + blk * 32);
     uint4 q[4];
 #pragma unroll
@@ -355,20 +336,24 @@ __device__ __forceinline__ float qema_target(float v, float ve)
     return __uint_as_float(__float_as_uint(t) | (vb & 0x80000000u));
 }
 
-// Four consecutive lanes share a 32-element group: a thread owns 8 consecutive elements (the weight is contiguous).
+// Four consecutive lanes share a 32-element group: a thread owns 8 consecutive elements (the weight is contiguous).  The grid
+// covers the scale buffer with its padding entries, as in the row-wise quantizer.
 template <bool OSC>
 __global__ void __launch_bounds__(256) k_qema(const __nv_bfloat16 *__restrict__ w, float *__restrict__ ema, float beta,
                                               int update_ema, int64_t n, int nblk, uint8_t *__restrict__ packed,
                                               uint8_t *__restrict__ scales, int nblk4, int scale_mode, OscPtrs osc,
                                               uint32_t *dev_status)
 {
-    const int64_t total = n * nblk * 4;                       // threads with work (a multiple of 4)
-    const int64_t gid = blockIdx.x * (int64_t)256 + threadIdx.x;
-    const bool active = gid < total;
-    const int64_t cid = active ? gid : 0;                     // idle lanes of the last warp shadow chunk 0 and store nothing
-    const int64_t e0 = cid * 8;
-    const int64_t grp = cid >> 2, row = grp / nblk;
-    const int blk = (int)(grp - row * nblk);
+    const uint64_t gid = blockIdx.x * (uint64_t)256 + threadIdx.x, grp_pad = gid >> 2;
+    const uint32_t nb_pad = (uint32_t)nblk4 * 4u;
+    const int64_t row_pad = (grp_pad >> 32) ? (int64_t)(grp_pad / nb_pad) : (int64_t)((uint32_t)grp_pad / nb_pad);
+    const int blk_pad = (int)(grp_pad - (uint64_t)row_pad * nb_pad);
+    // the lanes of a padding entry shadow group 0 and store that entry only; without padding blocks the weight is addressed
+    // without waiting for the division
+    const bool active = (int)nb_pad == nblk ? gid < (uint64_t)n * nblk * 4 : row_pad < n && blk_pad < nblk;
+    const int64_t row = row_pad;
+    const int blk = blk_pad;
+    const int64_t cid = !active ? (int64_t)(gid & 3) : (int)nb_pad == nblk ? (int64_t)gid : (row * nblk + blk) * 4 + (int64_t)(gid & 3), e0 = cid * 8;
     const float omb = __fsub_rn(1.0f, beta);
 
     const uint4 q = *reinterpret_cast<const uint4 *>(w + e0);
@@ -416,7 +401,13 @@ __global__ void __launch_bounds__(256) k_qema(const __nv_bfloat16 *__restrict__ 
         for (int i = 0; i < 8; i++) z[i] = qema_target(wv[i] * inv, ev[i] * inv);
         out = rne_x8(z[0], z[1], z[2], z[3], z[4], z[5], z[6], z[7]);
     }
-    if (!active) return;
+    if (!active) {
+        if ((gid & 3) == 0) {
+            scales[scale_offset(row_pad, blk_pad, nblk4)] = 0x7F;
+            if (OSC) osc.s_prev[scale_offset(row_pad, blk_pad, nblk4)] = 0x7F;
+        }
+        return;
+    }
 
     const int64_t pk = row * ((int64_t)nblk * 16) + blk * 16 + (cid & 3) * 4;   // this thread's 4 bytes of codes
     if (OSC) {
@@ -512,9 +503,7 @@ mxfp4_status_t quantize_rows(const void *src, int64_t rows, int64_t cols, int64_
     if (!aligned16(src) || ld % 8 != 0) return MXFP4_MISALIGNED;
     if (rows == 0 || cols == 0) return MXFP4_OK;
     const int nblk = (int)(cols / 32), nblk4 = (nblk + 3) / 4;
-    fill_padding_if_needed(dst.scales, rows, cols, st);
-    const int64_t groups = rows * nblk;
-    const unsigned blocks = (unsigned)ceil_div(groups, 256);
+    const unsigned blocks = (unsigned)(ceil_div(rows, 128) * nblk4 * 2);   // a thread per scale entry, padding included: 512 per chunk
     if (qp->rounding == MXFP4_ROUND_STOCHASTIC)
         k_quantize_rows<MXFP4_ROUND_STOCHASTIC><<<blocks, 256, 0, st>>>(
             static_cast<const __nv_bfloat16 *>(src), rows, nblk, ld, static_cast<uint8_t *>(dst.data), dst.scales, nblk4,
@@ -547,7 +536,7 @@ static bool make_src_map(CUtensorMap *map, const void *src, int64_t rows, int64_
     cuuint64_t gstride[1] = {(cuuint64_t)ld * 2};
     cuuint32_t box[2] = {64, (cuuint32_t)kTile};
     cuuint32_t estr[2] = {1, 1};
-    return encode_tiled_cached(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void *>(src), gdim, gstride, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+    return fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void *>(src), gdim, gstride, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
               CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
@@ -560,7 +549,7 @@ static bool make_packed_t_map(CUtensorMap *map, void *packed, int64_t rows, int6
     cuuint64_t gstride[1] = {(cuuint64_t)(rows / 2)};
     cuuint32_t box[2] = {64, (cuuint32_t)kTile};
     cuuint32_t estr[2] = {1, 1};
-    return encode_tiled_cached(map, CU_TENSOR_MAP_DATA_TYPE_UINT8, 2, packed, gdim, gstride, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+    return fn(map, CU_TENSOR_MAP_DATA_TYPE_UINT8, 2, packed, gdim, gstride, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
               CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
@@ -734,9 +723,7 @@ mxfp4_status_t mxfp4_qema_quantize(const void *w_bf16, float *ema, float beta, i
     }
     if (n == 0 || k == 0) return MXFP4_OK;
     const int nblk = (int)(k / 32), nblk4 = (nblk + 3) / 4;
-    fill_padding_if_needed(dst.scales, n, k, st);
-    if (osc) fill_padding_if_needed(osc->wq_prev.scales, n, k, st);
-    const unsigned blocks = (unsigned)ceil_div(n * nblk * 4, 256);
+    const unsigned blocks = (unsigned)(ceil_div(n, 128) * nblk4 * 8);   // four threads per scale entry
     if (osc)
         k_qema<true><<<blocks, 256, 0, st>>>(static_cast<const __nv_bfloat16 *>(w_bf16), ema, beta, update_ema, n, nblk,
                                              static_cast<uint8_t *>(dst.data), dst.scales, nblk4, scale_mode, op, dev_status);

@@ -273,3 +273,27 @@ def test_config_tensors_all_quantizers(mx, config, layer):
     assert_qmat_equal(dyq_t, *ops["dyq_t"], "Q5")
     assert_qmat_equal(mx.quantize_t(wq, rounding=1, seed=seed, stream_id=4), *ops["wq_t"], "Q4")
     assert_qmat_equal(mx.quantize_t(xq, rounding=1, seed=seed, stream_id=6), *ops["xq_t"], "Q6")
+
+
+@pytest.mark.parametrize("shape", [(1, 32), (127, 96), (128, 128), (129, 4128), (300, 160)])
+def test_padding_entries_of_the_scale_buffer(mx, shape):
+    """Rows up to a multiple of 128 and blocks up to a multiple of 4 beyond the matrix hold 0x7F (scale 1), whatever was there
+    before, in every buffer of the row-wise quantizers."""
+    rows, cols = shape
+    x = to_dev_bf16(rand_bf16(np.random.default_rng(rows), shape))
+    inside = {mx.scale_offset(r, b, cols) for r in range(rows) for b in range(cols // 32)}
+    pad = torch.tensor([i for i in range(mx.scale_bytes(rows, cols)) if i not in inside], dtype=torch.int64, device="cuda")
+
+    def fresh():
+        q = mx.QMat(rows, cols)
+        q.scales.fill_(0x11)
+        return q
+
+    prev = mx.OscState(x.clone(), fresh(), torch.zeros(shape, device="cuda"), torch.zeros(shape, device="cuda"))
+    mx.quantize(x, out=prev.wq_prev)
+    prev.wq_prev.scales[pad] = 0x22
+    outs = [mx.quantize(x, out=fresh()), mx.quantize(x, rounding=1, seed=1, out=fresh()), mx.qema_quantize(x, x.float(), out=fresh()),
+            mx.qema_quantize(x, x.float(), osc=prev, out=fresh()), prev.wq_prev]
+    for q in outs:
+        assert bool((q.scales[pad] == 0x7F).all())
+        assert bool((q.scales_linear() != 0x11).all())
