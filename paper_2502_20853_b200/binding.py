@@ -37,6 +37,9 @@ class CMat(C.Structure):
     _fields_ = [("data", C.c_void_p), ("scales", C.c_void_p), ("rows", C.c_int64), ("cols", C.c_int64)]
 
 
+_NO_MAT = CMat(None, None, 0, 0)
+
+
 class CQParams(C.Structure):
     _fields_ = [("scale_mode", C.c_int32), ("rounding", C.c_int32), ("seed", C.c_uint64),
                 ("stream_id", C.c_uint32), ("reserved", C.c_uint32)]
@@ -148,11 +151,12 @@ def _check(fn, status):
 
 
 def _stream():
-    return C.c_void_p(torch.cuda.current_stream().cuda_stream)
+    # the raw handle of the current stream, without the Stream object that torch.cuda.current_stream() builds (3 us)
+    return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
 
 
 def _ptr(t):
-    return C.c_void_p(t.data_ptr()) if t is not None else C.c_void_p(0)
+    return t.data_ptr() if t is not None else None
 
 
 def launch_count():
@@ -168,17 +172,74 @@ def scale_offset(row, block, cols):
     return int(lib().mxfp4_scale_offset(row, block, cols))
 
 
+def _align256(n):
+    return (n + 255) & ~255
+
+
 class QMat:
-    """A quantized matrix in device memory: packed E2M1 codes + E8M0 scales in tiled order."""
+    """A quantized matrix in device memory: packed E2M1 codes + E8M0 scales in tiled order.  Codes and scales that the
+    binding allocates itself share one buffer (an allocation costs a call 2.4 us); ``data`` and ``scales`` are views of it,
+    made when they are asked for."""
+
+    __slots__ = ("rows", "cols", "_buf", "_at", "_data", "_scales", "_c")
 
     def __init__(self, rows, cols, device="cuda", data=None, scales=None):
         self.rows, self.cols = int(rows), int(cols)
-        self.data = data if data is not None else _new((self.rows, self.cols // 2), torch.uint8, device)
+        if data is None and scales is None and ALLOC_HOOK is None:
+            self._place(torch.empty(QMat._bytes(self.rows, self.cols), dtype=torch.uint8, device=device), 0)
+            return
+        self._buf = None
+        self._data = data if data is not None else _new((self.rows, self.cols // 2), torch.uint8, device)
         nbytes = max(scale_bytes(self.rows, self.cols), 16)
-        self.scales = scales if scales is not None else _new((nbytes,), torch.uint8, device)
+        self._scales = scales if scales is not None else _new((nbytes,), torch.uint8, device)
+        self._c = CMat(self._data.data_ptr(), self._scales.data_ptr(), self.rows, self.cols)
+
+    @staticmethod
+    def _bytes(rows, cols):
+        """Bytes of codes and scales in one buffer, both on 256-byte boundaries."""
+        return _align256(rows * (cols // 2)) + max(((rows + 127) >> 7) * ((cols + 127) >> 7) * 512, 256)
+
+    def _place(self, buf, at):
+        self._buf, self._at, self._data, self._scales = buf, at, None, None
+        p = buf.data_ptr() + at
+        self._c = CMat(p, p + _align256(self.rows * (self.cols // 2)), self.rows, self.cols)
+
+    @staticmethod
+    def several(shapes, device):
+        """QMats of the given shapes in one buffer: operands that live and die together."""
+        if ALLOC_HOOK is not None:
+            return [QMat(r, c, device) for r, c in shapes]
+        sizes = [QMat._bytes(r, c) for r, c in shapes]
+        buf = torch.empty(sum(sizes), dtype=torch.uint8, device=device)
+        out, at = [], 0
+        for (r, c), n in zip(shapes, sizes):
+            q = QMat.__new__(QMat)
+            q.rows, q.cols = r, c
+            q._place(buf, at)
+            out.append(q)
+            at += n
+        return out
+
+    @property
+    def device(self):
+        return (self._buf if self._buf is not None else self._data).device
+
+    @property
+    def data(self):
+        if self._data is None:
+            n = self.rows * (self.cols // 2)
+            self._data = self._buf[self._at:self._at + n].view(self.rows, self.cols // 2)
+        return self._data
+
+    @property
+    def scales(self):
+        if self._scales is None:
+            at = self._at + _align256(self.rows * (self.cols // 2))
+            self._scales = self._buf[at:at + max(scale_bytes(self.rows, self.cols), 16)]
+        return self._scales
 
     def c(self):
-        return CMat(self.data.data_ptr(), self.scales.data_ptr(), self.rows, self.cols)
+        return self._c
 
     def scales_linear(self):
         """Scale bytes gathered into [rows, cols/32] order (index arithmetic only; for inspection)."""
@@ -220,7 +281,7 @@ def quantize_t(src, scale_mode=SCALE_TRUNCATION_FREE, rounding=ROUND_NEAREST, se
     qp = _qp(scale_mode, rounding, seed, stream_id)
     if isinstance(src, QMat):
         rows, cols = src.rows, src.cols
-        out = out if out is not None else QMat(cols, rows, src.data.device)
+        out = out if out is not None else QMat(cols, rows, src.device)
         cm = src.c()
         st = lib().mxfp4_quantize_t(None, C.byref(cm), rows, cols, cols, out.c(), C.byref(qp), _ptr(dev_status), _stream())
     else:
@@ -281,7 +342,7 @@ def qema_quantize(w, ema, beta=0.998, update_ema=True, scale_mode=SCALE_TRUNCATI
 
 
 def dequantize(q):
-    out = _new((q.rows, q.cols), torch.float32, q.data.device)
+    out = _new((q.rows, q.cols), torch.float32, q.device)
     _check("mxfp4_dequantize", lib().mxfp4_dequantize(q.c(), _ptr(out), q.cols, _stream()))
     return out
 
@@ -302,10 +363,10 @@ def linear_workspace_bytes(m, k, n):
 def gemm(a, b, out_dtype=OUT_BF16, bias=None, out=None, workspace=None, dev_status=None):
     """D[M, N] = deq(a)[M, kc] @ deq(b)[N, kc]^T."""
     dt = torch.float32 if out_dtype == OUT_FP32 else torch.bfloat16
-    out = out if out is not None else _new((a.rows, b.rows), dt, a.data.device)
+    out = out if out is not None else _new((a.rows, b.rows), dt, a.device)
     need = gemm_workspace_bytes(a.rows, b.rows, a.cols)
     if workspace is None and need:
-        workspace = _new((need,), torch.uint8, a.data.device)
+        workspace = _new((need,), torch.uint8, a.device)
     _check("mxfp4_gemm", lib().mxfp4_gemm(a.c(), b.c(), _ptr(out), out.stride(0), out_dtype, _ptr(bias), _ptr(workspace),
                                           workspace.numel() if workspace is not None else 0, _ptr(dev_status), _stream()))
     return out
@@ -320,7 +381,7 @@ class Epilogue:
         self.hook, self.aux, self.y, self.z, self.zq, self.qp_row, self.zq_t, self.qp_t, self.chain = hook, aux, y, z, zq, qp_row, zq_t, qp_t, chain
 
     def c(self):
-        none = CMat(None, None, 0, 0)
+        none = _NO_MAT
         return CEpilogue(self.hook, int(bool(self.chain)),
                          self.aux.data_ptr() if self.aux is not None else None, self.aux.stride(0) if self.aux is not None else 0,
                          self.y.data_ptr() if self.y is not None else None, self.y.stride(0) if self.y is not None else 0,
@@ -342,9 +403,9 @@ def gemm_wait_selftest(a, b, dev_status, out_dtype=OUT_BF16, spin_limit=2048):
     ``spin_limit`` polls: the waits run out, DEV_TIMEOUT is raised in ``dev_status`` and the kernels drain and return.
     The output is undefined and is thrown away."""
     dt = torch.float32 if out_dtype == OUT_FP32 else torch.bfloat16
-    out = _new((a.rows, b.rows), dt, a.data.device)
+    out = _new((a.rows, b.rows), dt, a.device)
     need = gemm_workspace_bytes(a.rows, b.rows, a.cols)
-    ws = _new((max(need, 16),), torch.uint8, a.data.device)
+    ws = _new((max(need, 16),), torch.uint8, a.device)
     _check("mxfp4_gemm_wait_selftest", lib().mxfp4_gemm_wait_selftest(a.c(), b.c(), _ptr(out), out.stride(0), out_dtype, _ptr(ws), ws.numel(),
                                                                       spin_limit, _ptr(dev_status), _stream()))
 
@@ -380,7 +441,7 @@ class LinearCtx:
         self.xq, self.wq, self.xq_t, self.seed, self.wq_t = xq, wq, xq_t, seed, wq_t
 
     def c(self):
-        none = CMat(None, None, 0, 0)
+        none = _NO_MAT
         t = self.xq_t.c() if self.xq_t is not None else none
         wt = self.wq_t.c() if self.wq_t is not None else none
         sd = self.seed & 0xFFFFFFFFFFFFFFFF
@@ -400,13 +461,22 @@ def linear_fwd(x, w=None, wq=None, bias=None, scale_mode=SCALE_TRUNCATION_FREE, 
         dev = x.device
     else:
         m, k = ctx.xq.rows, ctx.xq.cols
-        dev = ctx.xq.data.device
+        dev = ctx.xq.device
     if ctx is None:
         if wq is None:
-            wq = QMat(w.shape[0], k, dev)
-        ctx = LinearCtx(QMat(m, k, dev), wq)
+            n = w.shape[0]
+            if bwd_seed is not None and n % 32 == 0:
+                # Q4 of the backward pass comes with Q2, from the one pass over W
+                wq, wq_t = QMat.several([(n, k), (k, n)], dev)
+            else:
+                wq, wq_t = QMat(n, k, dev), None
+        else:
+            wq_t = None
         if bwd_seed is not None:
-            ctx.xq_t, ctx.seed = QMat(k, m, dev), bwd_seed
+            xq, xq_t = QMat.several([(m, k), (k, m)], dev)
+            ctx = LinearCtx(xq, wq, xq_t, bwd_seed, wq_t)
+        else:
+            ctx = LinearCtx(QMat(m, k, dev), wq)
     elif bwd_seed is not None:
         ctx.seed = bwd_seed
         if ctx.xq_t is None:
@@ -433,7 +503,7 @@ def linear_bwd(dy, ctx, seed, scale_mode=SCALE_TRUNCATION_FREE, dw_dtype=OUT_FP3
     ``epi_dx`` (an Epilogue): the input-gradient product runs with that quantizing epilogue; the first return value is
     then ``epi_dx``."""
     m, k, n = ctx.xq.rows, ctx.xq.cols, ctx.wq.rows
-    dev = ctx.xq.data.device
+    dev = ctx.xq.device
     if dy is not None:
         dy = _bf16_2d(dy)
     if epi_dx is None:
@@ -491,7 +561,7 @@ def quant_conf_hist(w, bins=20, scale_mode=SCALE_TRUNCATION_FREE, out=None):
 def change_sums(cur, prev, out=None):
     """(sum (cur - prev)^2, sum prev^2) as a float64[2] device tensor (added to ``out``): one term of the rate of change of
     App. A.3.  cur / prev: two bf16 tensors of one shape, or two QMat of one shape."""
-    dev = cur.data.device if isinstance(cur, QMat) else cur.device
+    dev = cur.device if isinstance(cur, QMat) else cur.device
     res = out if out is not None else torch.zeros(2, dtype=torch.float64, device=dev)
     if isinstance(cur, QMat):
         _check("mxfp4_change_sums_q", lib().mxfp4_change_sums_q(cur.c(), prev.c(), _ptr(res), _stream()))
