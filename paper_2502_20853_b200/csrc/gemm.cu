@@ -128,7 +128,9 @@ __device__ __forceinline__ uint32_t idesc_mxf4(int n, uint32_t a_sf_id, uint32_t
 __device__ __forceinline__ uint32_t load_bias_pair(const __nv_bfloat16 *bias, int64_t col, int64_t N, int lane)
 {
     const int64_t c = col + 2 * (lane & 15);
-    return bias != nullptr && c < N ? __ldg(reinterpret_cast<const uint32_t *>(bias + c)) : 0u;
+    uint32_t v = 0u;
+    if (bias != nullptr && c < N) asm volatile("ld.global.nc.u32 %0, [%1];" : "=r"(v) : "l"(bias + c));
+    return v;
 }
 __device__ __forceinline__ void add_bias_chunk(uint32_t (&r)[32], uint32_t pair)
 {
@@ -484,6 +486,7 @@ k_gemm_mxf4(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem_base = *tmem_slot;
+    pdl_wait();
 
     const int items = p.tiles_m * p.tiles_n * p.splits;
 
@@ -645,6 +648,7 @@ k_gemm_mxf4_q(const __grid_constant__ CUtensorMap map_a, const __grid_constant__
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem_base = *tmem_slot;
+    pdl_wait();
 
     if (warp < kEpiWarp0) {
         gemm_feed_roles<C, BN>(warp, smem_base, bar_full, bar_sf_full, bar_empty, bar_acc_full, bar_acc_empty, tmem_base, abort_flag, map_a, map_b, p);
@@ -867,6 +871,7 @@ k_gemm_mxf4_bs(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem_base = *tmem_slot;
+    pdl_wait();
 
     // tiles are numbered column by column: t = nb * tiles_m + mb; this CTA owns [t0, t1)
     const int64_t total = (int64_t)p.tiles_m * p.tiles_n;
@@ -1147,6 +1152,7 @@ k_gemm_mxf4_ck(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem_base = *tmem_slot;
+    pdl_wait();
 
     // the cluster's tile and this CTA's part of the contraction
     const int tile = (int)(blockIdx.x / S);
@@ -1532,6 +1538,7 @@ k_gemm_mxf4_pair(const __grid_constant__ CUtensorMap map_a, const __grid_constan
     extern __shared__ __align__(1024) uint8_t smem_aligned[];
     uint8_t *smem = smem_aligned;
     if (smem_u32(smem) & 1023u) {   // the swizzled operand tiles need it; nothing has been set up yet, so everybody just leaves
+        pdl_wait();
         if (threadIdx.x == 0 && p.dev_status) atomicOr(p.dev_status, MXFP4_DEV_SMEM_LAYOUT);
         return;
     }
@@ -1570,6 +1577,7 @@ k_gemm_mxf4_pair(const __grid_constant__ CUtensorMap map_a, const __grid_constan
     cluster_sync_all();     // both CTAs have their barriers and TMEM before anyone signals across
     tc_fence_after();
     const uint32_t tmem_base = *tmem_slot;
+    pdl_wait();
 
     const int tiles_m2 = (p.tiles_m + 1) >> 1;
     const int items = tiles_m2 * p.tiles_n * p.splits;
@@ -1914,6 +1922,7 @@ k_gemm_mxf4_pbs(const __grid_constant__ CUtensorMap map_a, const __grid_constant
     cluster_sync_all();     // both CTAs have their barriers and TMEM before anyone signals across
     tc_fence_after();
     const uint32_t tmem_base = *tmem_slot;
+    pdl_wait();
 
     // pair tiles (256 rows x 192 columns) are numbered column by column: t = nb * tiles_m2 + mb2; this pair owns [t0, t1)
     // and walks it as pbs_tile says
@@ -2112,6 +2121,9 @@ __global__ void __launch_bounds__(256) k_splitk_reduce(const float *__restrict__
                                                        void *__restrict__ d, int64_t ldd, int out_fp32,
                                                        const __nv_bfloat16 *__restrict__ bias)
 {
+    pdl_launch_dependents();
+    pdl_wait();
+    part = after_wait(part), bias = after_wait(bias);
     const int64_t total4 = M * N / 4;
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < total4; i += (int64_t)gridDim.x * blockDim.x) {
         const int64_t e = i * 4, row = e / N, col = e - row * N;
@@ -2301,8 +2313,7 @@ static mxfp4_status_t launch_gemm_pair(const CUtensorMap &ma, const CUtensorMap 
     using C = Gemm2Cfg<DEEP>;
     static bool attr_set[kMaxDevices];
     MX_CHECK_CUDA(set_smem_once(attr_set, k_gemm_mxf4_pair<DEEP>, C::kSmemBytes));
-    k_gemm_mxf4_pair<DEEP><<<grid, kGemmThreads, C::kSmemBytes, st>>>(ma, mb, msa, msb, md, p);
-    MX_CHECK_LAUNCH();
+    MX_CHECK_CUDA(launch_pdl(k_gemm_mxf4_pair<DEEP>, (unsigned)grid, 1, kGemmThreads, C::kSmemBytes, st, ma, mb, msa, msb, md, p));
     return MXFP4_OK;
 }
 
@@ -2314,8 +2325,7 @@ static mxfp4_status_t launch_gemm_pbs(const CUtensorMap &ma, const CUtensorMap &
     if (p.kt_total > KT) return MXFP4_INVALID_ARG;   // the resident block holds KT K tiles
     static bool attr_set[kMaxDevices];
     MX_CHECK_CUDA(set_smem_once(attr_set, k_gemm_mxf4_pbs<KT, AS>, C::kSmemBytes));
-    k_gemm_mxf4_pbs<KT, AS><<<grid, kGemmThreads, C::kSmemBytes, st>>>(ma, mb, msa, msb, md, mdw, p);
-    MX_CHECK_LAUNCH();
+    MX_CHECK_CUDA(launch_pdl(k_gemm_mxf4_pbs<KT, AS>, (unsigned)grid, 1, kGemmThreads, C::kSmemBytes, st, ma, mb, msa, msb, md, mdw, p));
     return MXFP4_OK;
 }
 
@@ -2326,8 +2336,7 @@ static mxfp4_status_t launch_gemm_bs(const CUtensorMap &ma, const CUtensorMap &m
     using C = GemmBsCfg<BN, KT, AS>;
     static bool attr_set[kMaxDevices];
     MX_CHECK_CUDA(set_smem_once(attr_set, k_gemm_mxf4_bs<BN, KT, AS>, C::kSmemBytes));
-    k_gemm_mxf4_bs<BN, KT, AS><<<grid, kGemmThreads, C::kSmemBytes, st>>>(ma, mb, md, mdw, p);
-    MX_CHECK_LAUNCH();
+    MX_CHECK_CUDA(launch_pdl(k_gemm_mxf4_bs<BN, KT, AS>, (unsigned)grid, 1, kGemmThreads, C::kSmemBytes, st, ma, mb, md, mdw, p));
     return MXFP4_OK;
 }
 
@@ -2342,13 +2351,15 @@ static mxfp4_status_t launch_gemm_ck(const CUtensorMap &ma, const CUtensorMap &m
     cfg.blockDim = dim3(kGemmThreads);
     cfg.dynamicSmemBytes = C::kSmemBytes;
     cfg.stream = st;
-    cudaLaunchAttribute attr[1];
+    cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeClusterDimension;
     attr[0].val.clusterDim.x = (unsigned)cluster;
     attr[0].val.clusterDim.y = 1;
     attr[0].val.clusterDim.z = 1;
+    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = 2;
     MX_CHECK_CUDA(cudaLaunchKernelEx(&cfg, k_gemm_mxf4_ck, ma, mb, p));
     MX_LAUNCHED();
     return MXFP4_OK;
@@ -2361,8 +2372,7 @@ static mxfp4_status_t launch_gemm(const CUtensorMap &ma, const CUtensorMap &mb, 
     using C = GemmCfg<BN, DEEP>;
     static bool attr_set[kMaxDevices];
     MX_CHECK_CUDA(set_smem_once(attr_set, k_gemm_mxf4<BN, DEEP>, C::kSmemBytes));
-    k_gemm_mxf4<BN, DEEP><<<grid, kGemmThreads, C::kSmemBytes, st>>>(ma, mb, md, mdw, p);
-    MX_CHECK_LAUNCH();
+    MX_CHECK_CUDA(launch_pdl(k_gemm_mxf4<BN, DEEP>, (unsigned)grid, 1, kGemmThreads, C::kSmemBytes, st, ma, mb, md, mdw, p));
     return MXFP4_OK;
 }
 
@@ -2446,9 +2456,8 @@ static mxfp4_status_t gemm_impl(mxfp4_mat_t a, mxfp4_mat_t b, void *d, int64_t l
         const int64_t total4 = M * N / 4;
         const int64_t nb4 = ceil_div(total4, 256);
         const int blocks = (int)(nb4 < (int64_t)sms * 8 ? nb4 : (int64_t)sms * 8);
-        k_splitk_reduce<<<blocks, 256, 0, st>>>(static_cast<const float *>(workspace), g.splits, M, N, d, ldd,
-                                                out_dtype == MXFP4_OUT_FP32, static_cast<const __nv_bfloat16 *>(bias));
-        MX_CHECK_LAUNCH();
+        MX_CHECK_CUDA(launch_pdl(k_splitk_reduce, (unsigned)blocks, 1, 256, 0, st, static_cast<const float *>(workspace), g.splits, M, N, d, ldd,
+                                 (int)(out_dtype == MXFP4_OUT_FP32), static_cast<const __nv_bfloat16 *>(bias)));
     }
     return MXFP4_OK;
 }
@@ -2505,8 +2514,7 @@ static mxfp4_status_t launch_gemm_q(const CUtensorMap &ma, const CUtensorMap &mb
     using C = GemmQCfg<WITH_Y>;
     static bool attr_set[kMaxDevices];
     MX_CHECK_CUDA(set_smem_once(attr_set, k_gemm_mxf4_q<SR_ROW, SR_T, DQ, WITH_Y>, C::kSmemBytes));
-    k_gemm_mxf4_q<SR_ROW, SR_T, DQ, WITH_Y><<<grid, kGemmThreads, C::kSmemBytes, st>>>(ma, mb, my, mz, mx_, mt, p, e);
-    MX_CHECK_LAUNCH();
+    MX_CHECK_CUDA(launch_pdl(k_gemm_mxf4_q<SR_ROW, SR_T, DQ, WITH_Y>, (unsigned)grid, 1, kGemmThreads, C::kSmemBytes, st, ma, mb, my, mz, mx_, mt, p, e));
     return MXFP4_OK;
 }
 

@@ -27,6 +27,9 @@ __global__ void __launch_bounds__(256) k_qramp_detect(const float *__restrict__ 
 {
     // a fixed number of blocks walks the array, so that the count of oscillating elements costs one atomic per block
     __shared__ uint32_t s_osc[8];
+    pdl_launch_dependents();
+    pdl_wait();
+    dist_w = after_wait(dist_w), dist_q = after_wait(dist_q);
     uint32_t osc = 0;
     const int64_t octs = (count + 7) / 8;     // eight elements per thread and turn: 64 bytes of loads in flight
     for (int64_t q = blockIdx.x * (int64_t)256 + threadIdx.x; q < octs; q += (int64_t)gridDim.x * 256) {
@@ -90,6 +93,9 @@ __global__ void __launch_bounds__(256) k_qramp_adamw(float *__restrict__ w, __nv
                                                      float *__restrict__ acc, uint8_t *__restrict__ cnt,
                                                      const uint8_t *__restrict__ n_w, int64_t count, const AdamW h)
 {
+    pdl_launch_dependents();
+    pdl_wait();
+    grad = after_wait(grad), n_w = after_wait(n_w);
     const int64_t i0 = (blockIdx.x * (int64_t)256 + threadIdx.x) * 4;
     if (i0 + 3 < count) {
         float4 W = *reinterpret_cast<const float4 *>(w + i0), G = *reinterpret_cast<const float4 *>(grad + i0);
@@ -153,8 +159,7 @@ mxfp4_status_t mxfp4_qramp_detect(const float *dist_w, const float *dist_q, int6
     const float inv_k1 = (frexpf(k1, &e) == 0.5f && e > -100 && e < 100) ? 1.0f / k1 : 0.0f;   // exact only for powers of two
     const int64_t want = ceil_div(ceil_div(count, 8), 256);
     const unsigned blocks = (unsigned)(want < (int64_t)sms * 8 ? want : (int64_t)sms * 8);
-    k_qramp_detect<<<blocks, 256, 0, static_cast<cudaStream_t>(stream)>>>(dist_w, dist_q, count, k1, inv_k1, k2, n_max, n_w, oscillating);
-    MX_CHECK_LAUNCH();
+    MX_CHECK_CUDA(launch_pdl(k_qramp_detect, blocks, 1, 256, 0, static_cast<cudaStream_t>(stream), dist_w, dist_q, count, k1, inv_k1, k2, n_max, n_w, oscillating));
     return MXFP4_OK;
 }
 
@@ -172,9 +177,7 @@ mxfp4_status_t mxfp4_qramp_adamw(float *w, void *w_bf16, const float *grad, floa
         return MXFP4_MISALIGNED;
     const AdamW h = {hp->lr, hp->beta1, hp->beta2, hp->eps, hp->weight_decay, hp->bias_corr1, hp->bias_corr2};
     const unsigned blocks = (unsigned)ceil_div(ceil_div(count, 4), 256);
-    k_qramp_adamw<<<blocks, 256, 0, static_cast<cudaStream_t>(stream)>>>(w, static_cast<__nv_bfloat16 *>(w_bf16), grad, m, v, acc, cnt,
-                                                                        n_w, count, h);
-    MX_CHECK_LAUNCH();
+    MX_CHECK_CUDA(launch_pdl(k_qramp_adamw, blocks, 1, 256, 0, static_cast<cudaStream_t>(stream), w, static_cast<__nv_bfloat16 *>(w_bf16), grad, m, v, acc, cnt, n_w, count, h));
     return MXFP4_OK;
 }
 

@@ -19,6 +19,8 @@ __global__ void __launch_bounds__(256) k_quantize_rows(const __nv_bfloat16 *__re
                                                        uint8_t *__restrict__ scales, int nblk4, int scale_mode,
                                                        const SrStream sr, uint32_t *dev_status)
 {
+    pdl_launch_dependents();
+    pdl_wait();
     const uint64_t gid = blockIdx.x * (uint64_t)256 + threadIdx.x;
     const uint32_t nb_pad = (uint32_t)nblk4 * 4u;
     const int64_t row = (gid >> 32) ? (int64_t)(gid / nb_pad) : (int64_t)((uint32_t)gid / nb_pad);
@@ -79,6 +81,7 @@ __global__ void __launch_bounds__(256, 3) k_requantize_tile(const void *__restri
     __shared__ __align__(16) uint2 s_out[kTile * 8];          // [output row = source column][8-byte slot], slots XOR-swizzled
     __shared__ __align__(16) uint8_t s_sc_t[512];
 
+    pdl_launch_dependents();
     const int tid = threadIdx.x;
     const int row0 = blockIdx.y * kTile, col0 = blockIdx.x * kTile;
     uint32_t nonfinite = 0;
@@ -88,8 +91,9 @@ __global__ void __launch_bounds__(256, 3) k_requantize_tile(const void *__restri
     // ---- stage the tile ----
     {
         // packed source: one thread per (row, 32-element group): 16 bytes of codes + 1 scale byte
-        const uint8_t *s = static_cast<const uint8_t *>(src);
-        const uint8_t *sc_chunk = src_scales + ((size_t)(row0 >> 7) * src_nblk4 + (col0 >> 7)) * 512;
+        pdl_wait();
+        const uint8_t *s = after_wait(static_cast<const uint8_t *>(src));
+        const uint8_t *sc_chunk = after_wait(src_scales) + ((size_t)(row0 >> 7) * src_nblk4 + (col0 >> 7)) * 512;
 #pragma unroll
         for (int it = 0; it < 2; it++) {
             const int item = it * 256 + tid;
@@ -231,6 +235,7 @@ k_quantize_stream(const __grid_constant__ CUtensorMap map_src, const __grid_cons
     const uint32_t bar_full = smem_base + kQsBarOff;
     volatile uint32_t *abort_flag = reinterpret_cast<volatile uint32_t *>(smem + kQsBarOff + 32);
 
+    pdl_launch_dependents();
     const int tid = threadIdx.x;
     const int ntx = (cols + kTile - 1) / kTile, nty = (rows + kTile - 1) / kTile;
     const int total = ntx * nty;
@@ -248,6 +253,9 @@ k_quantize_stream(const __grid_constant__ CUtensorMap map_src, const __grid_cons
         mbar_init(bar_full + 8, 1);
         *abort_flag = 0u;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    pdl_wait();
+    if (tid == 0) {
         // withhold_loads (self-test of the drain path): nothing is ever loaded, so the first bounded wait runs out
         for (int s = 0; s < 2; s++)
             if (!withhold_loads && (int)blockIdx.x + s * (int)gridDim.x < total) issue_load(blockIdx.x + s * gridDim.x, s);
@@ -344,6 +352,9 @@ __global__ void __launch_bounds__(256) k_qema(const __nv_bfloat16 *__restrict__ 
                                               uint8_t *__restrict__ scales, int nblk4, int scale_mode, OscPtrs osc,
                                               uint32_t *dev_status)
 {
+    pdl_launch_dependents();
+    pdl_wait();
+    w = after_wait(w);
     const uint64_t gid = blockIdx.x * (uint64_t)256 + threadIdx.x, grp_pad = gid >> 2;
     const uint32_t nb_pad = (uint32_t)nblk4 * 4u;
     const int64_t row_pad = (grp_pad >> 32) ? (int64_t)(grp_pad / nb_pad) : (int64_t)((uint32_t)grp_pad / nb_pad);
@@ -449,6 +460,9 @@ __global__ void __launch_bounds__(256) k_qema(const __nv_bfloat16 *__restrict__ 
 __global__ void __launch_bounds__(256) k_dequantize(const uint8_t *__restrict__ packed, const uint8_t *__restrict__ scales,
                                                     int64_t rows, int nblk, int nblk4, float *__restrict__ dst, int64_t ld)
 {
+    pdl_launch_dependents();
+    pdl_wait();
+    packed = after_wait(packed), scales = after_wait(scales);
     const int64_t gid = blockIdx.x * (int64_t)256 + threadIdx.x;
     if (gid >= rows * nblk) return;
     const int64_t row = gid / nblk;
@@ -504,15 +518,9 @@ mxfp4_status_t quantize_rows(const void *src, int64_t rows, int64_t cols, int64_
     if (rows == 0 || cols == 0) return MXFP4_OK;
     const int nblk = (int)(cols / 32), nblk4 = (nblk + 3) / 4;
     const unsigned blocks = (unsigned)(ceil_div(rows, 128) * nblk4 * 2);   // a thread per scale entry, padding included: 512 per chunk
-    if (qp->rounding == MXFP4_ROUND_STOCHASTIC)
-        k_quantize_rows<MXFP4_ROUND_STOCHASTIC><<<blocks, 256, 0, st>>>(
-            static_cast<const __nv_bfloat16 *>(src), rows, nblk, ld, static_cast<uint8_t *>(dst.data), dst.scales, nblk4,
-            qp->scale_mode, make_sr_stream(qp->seed, qp->stream_id, rows * cols), dev_status);
-    else
-        k_quantize_rows<MXFP4_ROUND_NEAREST><<<blocks, 256, 0, st>>>(
-            static_cast<const __nv_bfloat16 *>(src), rows, nblk, ld, static_cast<uint8_t *>(dst.data), dst.scales, nblk4,
-            qp->scale_mode, make_sr_stream(qp->seed, qp->stream_id, rows * cols), dev_status);
-    MX_CHECK_LAUNCH();
+    MX_CHECK_CUDA(launch_pdl(qp->rounding == MXFP4_ROUND_STOCHASTIC ? k_quantize_rows<MXFP4_ROUND_STOCHASTIC> : k_quantize_rows<MXFP4_ROUND_NEAREST>,
+                             blocks, 1, 256, 0, st, static_cast<const __nv_bfloat16 *>(src), rows, nblk, ld, static_cast<uint8_t *>(dst.data),
+                             dst.scales, nblk4, qp->scale_mode, make_sr_stream(qp->seed, qp->stream_id, rows * cols), dev_status));
     return MXFP4_OK;
 }
 
@@ -562,8 +570,8 @@ static mxfp4_status_t launch_stream(cudaStream_t st, const CUtensorMap &ms, cons
     const int64_t tiles = ceil_div(rows, kTile) * ceil_div(cols, kTile);
     const int64_t cap = kQsCtasPerSm * (int64_t)sm_count();
     const int grid = (int)(tiles < cap ? tiles : cap);
-    k_quantize_stream<EMIT_ROW, SR_ROW, SR_T, DQ><<<grid, kQsThreads, kQsSmemBytes, st>>>(ms, mt, rows, cols, rw, tr, dev_status, spin_limit, withhold_loads);
-    MX_CHECK_LAUNCH();
+    MX_CHECK_CUDA(launch_pdl(k_quantize_stream<EMIT_ROW, SR_ROW, SR_T, DQ>, (unsigned)grid, 1, kQsThreads, kQsSmemBytes, st, ms, mt, rows, cols, rw, tr,
+                             dev_status, spin_limit, withhold_loads));
     return MXFP4_OK;
 }
 
@@ -603,8 +611,8 @@ static mxfp4_status_t quantize_tile_ex(const void *src_bf16, const mxfp4_mat_t *
     const int r = (int)rows, c = (int)cols;
     if (src_q) {
         const int nb4 = (int)ceil_div(cols / 32, 4);
-        if (sr_t) k_requantize_tile<true><<<grid, 256, 0, st>>>(src_q->data, src_q->scales, nb4, r, c, tr, dev_status);
-        else k_requantize_tile<false><<<grid, 256, 0, st>>>(src_q->data, src_q->scales, nb4, r, c, tr, dev_status);
+        MX_CHECK_CUDA(launch_pdl(sr_t ? k_requantize_tile<true> : k_requantize_tile<false>, grid.x, grid.y, 256, 0, st, src_q->data, src_q->scales, nb4, r, c, tr,
+                                 dev_status));
     } else {
         // bf16 source: the streaming kernel
         if (ceil_div(rows, kTile) * ceil_div(cols, kTile) > 0x7FFFFFFF) return MXFP4_BAD_SHAPE;
@@ -626,7 +634,6 @@ static mxfp4_status_t quantize_tile_ex(const void *src_bf16, const mxfp4_mat_t *
         default: return launch_stream<true, true, true, true>(st, ms, mt, r, c, rw, tr, dev_status, spin_limit, withhold_loads);
         }
     }
-    MX_CHECK_LAUNCH();
     return MXFP4_OK;
 }
 
@@ -724,13 +731,8 @@ mxfp4_status_t mxfp4_qema_quantize(const void *w_bf16, float *ema, float beta, i
     if (n == 0 || k == 0) return MXFP4_OK;
     const int nblk = (int)(k / 32), nblk4 = (nblk + 3) / 4;
     const unsigned blocks = (unsigned)(ceil_div(n, 128) * nblk4 * 8);   // four threads per scale entry
-    if (osc)
-        k_qema<true><<<blocks, 256, 0, st>>>(static_cast<const __nv_bfloat16 *>(w_bf16), ema, beta, update_ema, n, nblk,
-                                             static_cast<uint8_t *>(dst.data), dst.scales, nblk4, scale_mode, op, dev_status);
-    else
-        k_qema<false><<<blocks, 256, 0, st>>>(static_cast<const __nv_bfloat16 *>(w_bf16), ema, beta, update_ema, n, nblk,
-                                              static_cast<uint8_t *>(dst.data), dst.scales, nblk4, scale_mode, op, dev_status);
-    MX_CHECK_LAUNCH();
+    MX_CHECK_CUDA(launch_pdl(osc ? k_qema<true> : k_qema<false>, blocks, 1, 256, 0, st, static_cast<const __nv_bfloat16 *>(w_bf16), ema, beta, update_ema, n, nblk,
+                             static_cast<uint8_t *>(dst.data), dst.scales, nblk4, scale_mode, op, dev_status));
     return MXFP4_OK;
 }
 
@@ -744,9 +746,8 @@ mxfp4_status_t mxfp4_dequantize(mxfp4_mat_t src, float *dst, int64_t ld, void *s
     if (src.rows == 0 || src.cols == 0) return MXFP4_OK;
     const int nblk = (int)(src.cols / 32), nblk4 = (nblk + 3) / 4;
     const unsigned blocks = (unsigned)ceil_div(src.rows * nblk, 256);
-    k_dequantize<<<blocks, 256, 0, static_cast<cudaStream_t>(stream)>>>(static_cast<const uint8_t *>(src.data), src.scales,
-                                                                        src.rows, nblk, nblk4, dst, ld);
-    MX_CHECK_LAUNCH();
+    MX_CHECK_CUDA(launch_pdl(k_dequantize, blocks, 1, 256, 0, static_cast<cudaStream_t>(stream), static_cast<const uint8_t *>(src.data), src.scales, src.rows, nblk,
+                             nblk4, dst, ld));
     return MXFP4_OK;
 }
 

@@ -231,3 +231,41 @@ def test_mlp_pair_with_the_quantizations_fused_into_the_products(mx):
     assert_qmat_equal(dyq1_t, *b1["dyq_t"], "Q5 of fc1's output gradient, made by fc2's epilogue")
     check_gemm_bound(dx1.float().cpu().numpy(), b1["dx"], b1["tdx"], True, "dX1")
     check_gemm_bound(dw1.cpu().numpy(), b1["dw"], b1["tdw"], False, "dW1")
+
+
+@pytest.mark.parametrize("rows", [32, 224, 2048])
+def test_chained_launches_see_each_other(mx, rows):
+    """The kernels of a step are placed while the one before them drains and wait for it themselves: many steps queued without
+    a synchronisation, on two streams, over buffers that are overwritten from step to step, give the results of steps that
+    are waited for one by one."""
+    L, x, w, dy = workloads.make_layer(2, 0, rows=rows)
+    xs = [to_dev_bf16(np.roll(x, i, axis=0)) for i in range(4)]
+    wd, dyd, bias = to_dev_bf16(w), to_dev_bf16(dy), to_dev_bf16(w[:, :1].T.copy()).reshape(-1)
+
+    def buffers():
+        return dict(ctx=mx.LinearCtx(mx.QMat(rows, L.K), mx.QMat(L.N, L.K), xq_t=mx.QMat(L.K, rows), seed=5, wq_t=mx.QMat(L.K, L.N)),
+                    y=torch.empty((rows, L.N), dtype=torch.bfloat16, device="cuda"), dx=torch.empty((rows, L.K), dtype=torch.bfloat16, device="cuda"),
+                    dw=torch.empty((L.N, L.K), device="cuda"), ws=torch.empty(mx.linear_workspace_bytes(rows, L.K, L.N), dtype=torch.uint8, device="cuda"))
+
+    def step(b, i):
+        mx.linear_fwd(xs[i % 4], wd, bias=bias, ctx=b["ctx"], out=b["y"], bwd_seed=5)
+        mx.linear_bwd(dyd, b["ctx"], 5, dx=b["dx"], dw=b["dw"], workspace=b["ws"])
+        return [b["y"], b["dx"], b["dw"], b["ctx"].xq_t.data]
+
+    b = buffers()
+    want = []
+    for i in range(4):
+        want.append([t.clone() for t in step(b, i)])
+        torch.cuda.synchronize()
+    streams, bufs, got = [torch.cuda.Stream(), torch.cuda.Stream()], [buffers(), buffers()], []
+    torch.cuda.synchronize()
+    for i in range(24):
+        for s, b in zip(streams, bufs):
+            with torch.cuda.stream(s):
+                r = step(b, i)
+                if i >= 20:
+                    got.append((i, [t.clone() for t in r]))
+    torch.cuda.synchronize()
+    for i, r in got:
+        for a, c in zip(r, want[i % 4]):
+            assert torch.equal(a, c), "step %d" % i
