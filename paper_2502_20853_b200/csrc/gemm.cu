@@ -565,24 +565,6 @@ struct GemmQCfg {
     static_assert(kSmemBytes <= 232448, "shared memory budget");
 };
 
-// GELU (0.5 y (1 + erf(y / sqrt 2))) in FP32.  erf by the rational form of Abramowitz & Stegun 7.1.26 (absolute error
-// below 1.5e-7), one exponential and one reciprocal: the result is rounded to bf16, for which this is ample.
-__device__ __forceinline__ float gelu_f32(float y)
-{
-    const float x = fabsf(y) * 0.70710678118654752f;
-    float t, ex;
-    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(t) : "f"(fmaf(0.3275911f, x, 1.0f)));
-    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(ex) : "f"(x * x * -1.4426950408889634f));
-    float poly = fmaf(1.061405429f, t, -1.453152027f);
-    poly = fmaf(poly, t, 1.421413741f);
-    poly = fmaf(poly, t, -0.284496736f);
-    poly = fmaf(poly, t, 0.254829592f);
-    const float erfc_abs = poly * t * ex;                         // 1 - erf(|y| / sqrt 2)
-    const float half_y = 0.5f * y;
-    // y >= 0: 0.5 y (2 - erfc) ; y < 0: 0.5 y erfc
-    return half_y * (y >= 0.0f ? 2.0f - erfc_abs : erfc_abs);
-}
-
 struct QuantEpilogue {
     QuantSide rw, tr;             // row-wise result [M, N] and transposed result [N, M]
     int emit_row, emit_t;
@@ -715,11 +697,7 @@ k_gemm_mxf4_q(const __grid_constant__ CUtensorMap map_a, const __grid_constant__
                 uint32_t zw[16];
                 if (e.hook == MXFP4_HOOK_GELU) {
 #pragma unroll
-                    for (int j = 0; j < 16; j++) {
-                        const float a = bf16lo(yw[j]), b = bf16hi(yw[j]);
-                        const __nv_bfloat162 h = __floats2bfloat162_rn(gelu_f32(a), gelu_f32(b));
-                        zw[j] = *reinterpret_cast<const uint32_t *>(&h);
-                    }
+                    for (int j = 0; j < 16; j++) zw[j] = gelu_bf16x2(yw[j]);
                 } else if (e.hook == MXFP4_HOOK_MULTIPLY) {
                     uint4 aw[4] = {make_uint4(0, 0, 0, 0), make_uint4(0, 0, 0, 0), make_uint4(0, 0, 0, 0), make_uint4(0, 0, 0, 0)};
                     if (aux_tma) {
@@ -2555,6 +2533,21 @@ mxfp4_status_t gemm_quant_check(mxfp4_mat_t a, mxfp4_mat_t b, const void *bias, 
     return MXFP4_OK;
 }
 
+mxfp4_status_t quantize_gelu_chain(const void *y_bf16, int64_t rows, int64_t cols, int64_t ldy, void *z_bf16, int64_t ldz, mxfp4_mat_t dst,
+                                   const mxfp4_qparams_t *qp_row, mxfp4_mat_t dst_t, const mxfp4_qparams_t *qp_t, uint32_t *dev_status, cudaStream_t st);
+
+// Whether the product and the quantization run as two kernels: when the epilogue is GELU with the double-quantization chain,
+// Y is stored anyway, and there are at least four 128 x 128 tiles per SM.  The fused epilogue has eight warps per SM for the
+// cast, the hook and both passes, and they are the bottleneck; the two kernels read Y back (2 of 5 bytes per element more)
+// but run at the product's and the tile quantizer's own rates: fused / two kernels 84 / 66.3 us at 25216 x 1536 x 384,
+// 396 / 314 at 50432 x 4096 x 1024, 305 / 237 at 401408 x 384 x 96, 33.6 / 31.7 at 8192 x 1536 x 384 (5.2 tiles per SM), but
+// 20.6 / 22.5 at 4096 x 1536 x 384 (2.6) and 12.3 / 15.3 at 1024 x 768 x 192, where a second launch costs more.
+static bool two_pass(const mxfp4_epilogue_t *epi, int64_t M, int64_t N)
+{
+    return epi->hook == MXFP4_HOOK_GELU && epi->chain && epi->y_bf16 && epi->y_bf16 != epi->z_bf16 &&
+           ceil_div(M, kBM) * ceil_div(N, 128) >= 4 * (int64_t)sm_count();
+}
+
 mxfp4_status_t gemm_quant(mxfp4_mat_t a, mxfp4_mat_t b, const void *bias, const mxfp4_epilogue_t *epi, uint32_t *dev_status, cudaStream_t st)
 {
     const mxfp4_status_t chk = gemm_quant_check(a, b, bias, epi);
@@ -2562,6 +2555,12 @@ mxfp4_status_t gemm_quant(mxfp4_mat_t a, mxfp4_mat_t b, const void *bias, const 
     const int64_t M = a.rows, N = b.rows, Kc = a.cols;
     if (M == 0 || N == 0) return MXFP4_OK;
     const bool row = epi->zq.data != nullptr, tr = epi->zq_t.data != nullptr;
+    if (two_pass(epi, M, N)) {
+        // Y by the product's own kernels (the contraction is not split), then the tile quantizer reads it back
+        mxfp4_status_t s = gemm(a, b, epi->y_bf16, epi->ldy, MXFP4_OUT_BF16, bias, nullptr, 0, dev_status, st, false);
+        if (s) return s;
+        return quantize_gelu_chain(epi->y_bf16, M, N, epi->ldy, epi->z_bf16, epi->ldz, epi->zq, &epi->qp_row, epi->zq_t, &epi->qp_t, dev_status, st);
+    }
     CUtensorMap ma, mb, my, mz, mx_, mt;
     if (!make_operand_map(&ma, a.data, M, Kc, kBM) || !make_operand_map(&mb, b.data, N, Kc, 128)) return MXFP4_CUDA_ERROR;
     my = mz = mx_ = mt = ma;   // placeholders when the tensors they describe are not asked for

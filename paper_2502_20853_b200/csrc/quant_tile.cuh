@@ -91,6 +91,48 @@ __device__ __forceinline__ uint32_t absmax_u4(uint32_t acc, const uint4 &q)
 }
 
 
+// Two FP32 values in one 64-bit register: an FMA of such pairs takes one issue slot (the passes are bound by issue).
+__device__ __forceinline__ uint64_t f32x2(float a, float b)
+{
+    uint64_t r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+    return r;
+}
+__device__ __forceinline__ uint64_t fma_f32x2(uint64_t a, uint64_t b, float c)
+{
+    uint64_t r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(f32x2(c, c)));
+    return r;
+}
+
+// GELU (0.5 y (1 + erf(y / sqrt 2))) of a bf16 pair in FP32, rounded to bf16: h + |h| erf with h = y / 2 and
+// erf(|y| / sqrt 2) = 1 - 2^P(|y|).  P is a minimax fit (linear programming over [0, 6.2], weighted by erfc) of
+// log2 erfc(|y| / sqrt 2) without a constant term, degree 8; its leading coefficient makes it fall for ever beyond.  Error below
+// 1e-7 |y|, by eight packed multiply-adds and one ex2 each.  (The rational form of Abramowitz & Stegun 7.1.26 that stood here
+// has the same error and a reciprocal more, on a unit with a quarter of the rate: 88 against 84 us for the fused product at
+// 25216 x 1536 x 384.)
+__device__ __forceinline__ uint32_t gelu_bf16x2(uint32_t w)
+{
+    float h0, h1, a0, a1, p0, p1, e0, e1;
+    scale_pair(w, 0x3F003F00u, h0, h1);
+    scale_pair(w & 0x7FFF7FFFu, 0x3F803F80u, a0, a1);
+    const uint64_t a = f32x2(a0, a1);
+    uint64_t p = fma_f32x2(f32x2(-2.4936796307883924e-06f, -2.4936796307883924e-06f), a, 3.588577965274453e-05f);
+    p = fma_f32x2(p, a, -1.7219783330801874e-04f);
+    p = fma_f32x2(p, a, -1.6490205598529428e-04f);
+    p = fma_f32x2(p, a, 7.092964835464954e-03f);
+    p = fma_f32x2(p, a, -5.251217260956764e-02f);
+    p = fma_f32x2(p, a, -4.592042863368988e-01f);
+    p = fma_f32x2(p, a, -1.151105523109436e+00f);
+    asm("mul.rn.f32x2 %0, %0, %1;" : "+l"(p) : "l"(a));
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(p0), "=f"(p1) : "l"(p));
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e0) : "f"(p0));
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e1) : "f"(p1));
+    uint32_t r;
+    asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(r) : "f"(fmaf(fabsf(h1), 1.0f - e1, h1)), "f"(fmaf(fabsf(h0), 1.0f - e0, h0)));
+    return r;
+}
+
 // Per-thread geometry of the two passes (the same for every tile of a launch).
 //   row pass   : warps 0-3 take the left 64 columns, warps 4-7 the right; a lane pair shares a row (its two groups);
 //                a thread handles rows r_row0 and r_row0 + 16
@@ -139,9 +181,11 @@ __device__ __forceinline__ QsGeom qs_geom(int tid, int rows, int cols, uint8_t *
 // The passes are bound by the instructions they issue (about 1.6 cycles each), so groups that hold Inf / NaN are quantized
 // like any others and put right afterwards, behind one vote per pass (handling them in line cost 24 instructions per group,
 // a tenth of the kernel's time).
-template <bool SR_ROW, bool DQ, bool WIDE>
+// GELU: the tile holds Y and what is quantized is Z = bf16(GELU(Y)) (needs DQ: the column pass must not read the tile as it
+// was); Z is stored too if hook_out is not null (bf16, leading dimension hook_ld).
+template <bool SR_ROW, bool DQ, bool WIDE, bool GELU>
 __device__ __forceinline__ void qs_row_pass(const QsGeom &g, uint32_t st_base, uint32_t dq_base, int row0, int col0, int rows, int cols,
-                                            const QuantSide &rw, uint32_t tfa_r2, uint8_t *s_sc_row, uint32_t &nonfinite)
+                                            const QuantSide &rw, uint32_t tfa_r2, uint8_t *s_sc_row, uint32_t &nonfinite, __nv_bfloat16 *hook_out, int64_t hook_ld)
 {
     uint8_t *out = g.r_out + ((int64_t)row0 * (cols >> 1) + (col0 >> 1));
     const uint64_t tile_q = (uint64_t)row0 * (uint64_t)(cols >> 4) + (uint64_t)(col0 >> 4);
@@ -154,6 +198,15 @@ __device__ __forceinline__ void qs_row_pass(const QsGeom &g, uint32_t st_base, u
         for (int j = 0; j < 4; j++)
             asm volatile("ld.shared.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(q[j].x), "=r"(q[j].y), "=r"(q[j].z), "=r"(q[j].w)
                          : "r"(st_base + g.r_off[j] + (uint32_t)(item * 16 * 128)));
+        if (GELU) {
+#pragma unroll
+            for (int j = 0; j < 4; j++) q[j] = make_uint4(gelu_bf16x2(q[j].x), gelu_bf16x2(q[j].y), gelu_bf16x2(q[j].z), gelu_bf16x2(q[j].w));
+            if (hook_out != nullptr && rows_left > item * 16) {
+                uint4 *z = reinterpret_cast<uint4 *>(hook_out + (int64_t)(row0 + g.r_row0 + item * 16) * hook_ld + col0 + g.r_col);
+#pragma unroll
+                for (int j = 0; j < 4; j++) z[j] = q[j];
+            }
+        }
         uint32_t am4[4];
 #pragma unroll
         for (int j = 0; j < 4; j++) am4[j] = absmax_fold(absmax_fold(q[j].x, q[j].y), absmax_fold(q[j].z, q[j].w));
@@ -265,24 +318,27 @@ __device__ __forceinline__ void qs_col_pass(const QsGeom &g, uint32_t st_base, i
 
 // Both passes over a tile, by the width of the random streams' counters (a launch-uniform branch around the whole tile).
 // With DQ the column pass reads what the row pass of the SAME warp wrote to dq_base.
-template <bool SR_ROW, bool SR_T, bool DQ, bool WIDE>
+template <bool SR_ROW, bool SR_T, bool DQ, bool WIDE, bool GELU>
 __device__ __forceinline__ void qs_tile_w(const QsGeom &g, uint32_t st_base, uint32_t dq_base, int row0, int col0, int rows, int cols, bool emit_row,
                                           bool emit_t, const QuantSide &rw, const QuantSide &tr, uint32_t tfa_r2, uint32_t tfa_t2, uint8_t *staging,
-                                          uint8_t *s_sc_row, uint8_t *s_sc_t, uint32_t &nonfinite)
+                                          uint8_t *s_sc_row, uint8_t *s_sc_t, uint32_t &nonfinite, __nv_bfloat16 *hook_out, int64_t hook_ld)
 {
-    if (emit_row) qs_row_pass<SR_ROW, DQ, WIDE>(g, st_base, dq_base, row0, col0, rows, cols, rw, tfa_r2, s_sc_row, nonfinite);
+    if (emit_row)
+        qs_row_pass<SR_ROW, DQ, WIDE, GELU>(g, st_base, dq_base, row0, col0, rows, cols, rw, tfa_r2, s_sc_row, nonfinite, hook_out, hook_ld);
     if (DQ) __syncwarp();
     if (emit_t) qs_col_pass<SR_T, WIDE>(g, DQ ? dq_base : st_base, row0, col0, rows, cols, tr, tfa_t2, staging, s_sc_t, nonfinite);
 }
-template <bool SR_ROW, bool SR_T, bool DQ>
+template <bool SR_ROW, bool SR_T, bool DQ, bool GELU = false>
 __device__ __forceinline__ void qs_tile(const QsGeom &g, uint32_t st_base, uint32_t dq_base, int row0, int col0, int rows, int cols, bool emit_row,
                                         bool emit_t, const QuantSide &rw, const QuantSide &tr, uint32_t tfa_r2, uint32_t tfa_t2, uint8_t *staging,
-                                        uint8_t *s_sc_row, uint8_t *s_sc_t, uint32_t &nonfinite)
+                                        uint8_t *s_sc_row, uint8_t *s_sc_t, uint32_t &nonfinite, __nv_bfloat16 *hook_out = nullptr, int64_t hook_ld = 0)
 {
     if ((SR_ROW || SR_T) && (rw.sr.wide | tr.sr.wide))
-        qs_tile_w<SR_ROW, SR_T, DQ, true>(g, st_base, dq_base, row0, col0, rows, cols, emit_row, emit_t, rw, tr, tfa_r2, tfa_t2, staging, s_sc_row, s_sc_t, nonfinite);
+        qs_tile_w<SR_ROW, SR_T, DQ, true, GELU>(g, st_base, dq_base, row0, col0, rows, cols, emit_row, emit_t, rw, tr, tfa_r2, tfa_t2, staging, s_sc_row, s_sc_t,
+                                                nonfinite, hook_out, hook_ld);
     else
-        qs_tile_w<SR_ROW, SR_T, DQ, false>(g, st_base, dq_base, row0, col0, rows, cols, emit_row, emit_t, rw, tr, tfa_r2, tfa_t2, staging, s_sc_row, s_sc_t, nonfinite);
+        qs_tile_w<SR_ROW, SR_T, DQ, false, GELU>(g, st_base, dq_base, row0, col0, rows, cols, emit_row, emit_t, rw, tr, tfa_r2, tfa_t2, staging, s_sc_row, s_sc_t,
+                                                 nonfinite, hook_out, hook_ld);
 }
 
 }  // namespace mx

@@ -223,11 +223,12 @@ constexpr int kQsBarOff = 2 * kTileBytes + 2 * kQsStagingBytes;
 constexpr int kQsSmemBytes = kQsBarOff + 64 + 1024 /*align*/;
 constexpr int kQsCtasPerSm = 2;
 
-template <bool EMIT_ROW, bool SR_ROW, bool SR_T, bool DQ>
+// GELU: the source is a product's result Y, quantized behind the activation (see qs_row_pass).
+template <bool EMIT_ROW, bool SR_ROW, bool SR_T, bool DQ, bool GELU>
 __global__ void __launch_bounds__(kQsThreads, kQsCtasPerSm)
 k_quantize_stream(const __grid_constant__ CUtensorMap map_src, const __grid_constant__ CUtensorMap map_t, int rows, int cols,
                   const __grid_constant__ QuantSide rw, const __grid_constant__ QuantSide tr, uint32_t *dev_status, uint32_t spin_limit,
-                  int withhold_loads)
+                  int withhold_loads, __nv_bfloat16 *hook_out, int64_t hook_ld)
 {
     extern __shared__ uint8_t qs_smem_raw[];
     uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(qs_smem_raw) + 1023) & ~(uintptr_t)1023);
@@ -278,7 +279,8 @@ k_quantize_stream(const __grid_constant__ CUtensorMap map_src, const __grid_cons
 
         const bool ok = mbar_wait_warp(bar_full + 8 * stage, (uint32_t)(it >> 1) & 1u, abort_flag, dev_status, spin_limit);
         if (ok)
-            qs_tile<SR_ROW, SR_T, DQ>(g, st_base, st_base, row0, col0, rows, cols, EMIT_ROW, true, rw, tr, tfa_r2, tfa_t2, staging, s_sc_row, s_sc_t, nonfinite);
+            qs_tile<SR_ROW, SR_T, DQ, GELU>(g, st_base, st_base, row0, col0, rows, cols, EMIT_ROW, true, rw, tr, tfa_r2, tfa_t2, staging, s_sc_row, s_sc_t, nonfinite,
+                                            hook_out, hook_ld);
 
         // ---- hand the tile's results to the copy engine, refill the ring ----
         fence_async_smem();                       // this thread's staging writes, before the asynchronous reads
@@ -561,17 +563,18 @@ static bool make_packed_t_map(CUtensorMap *map, void *packed, int64_t rows, int6
               CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-template <bool EMIT_ROW, bool SR_ROW, bool SR_T, bool DQ>
+template <bool EMIT_ROW, bool SR_ROW, bool SR_T, bool DQ, bool GELU = false>
 static mxfp4_status_t launch_stream(cudaStream_t st, const CUtensorMap &ms, const CUtensorMap &mt, int rows, int cols, const QuantSide &rw,
-                                    const QuantSide &tr, uint32_t *dev_status, uint32_t spin_limit = kWaitSpinLimit, int withhold_loads = 0)
+                                    const QuantSide &tr, uint32_t *dev_status, uint32_t spin_limit = kWaitSpinLimit, int withhold_loads = 0,
+                                    __nv_bfloat16 *hook_out = nullptr, int64_t hook_ld = 0)
 {
     static bool attr_set[kMaxDevices];
-    MX_CHECK_CUDA(set_smem_once(attr_set, k_quantize_stream<EMIT_ROW, SR_ROW, SR_T, DQ>, kQsSmemBytes));
+    MX_CHECK_CUDA(set_smem_once(attr_set, k_quantize_stream<EMIT_ROW, SR_ROW, SR_T, DQ, GELU>, kQsSmemBytes));
     const int64_t tiles = ceil_div(rows, kTile) * ceil_div(cols, kTile);
     const int64_t cap = kQsCtasPerSm * (int64_t)sm_count();
     const int grid = (int)(tiles < cap ? tiles : cap);
-    MX_CHECK_CUDA(launch_pdl(k_quantize_stream<EMIT_ROW, SR_ROW, SR_T, DQ>, (unsigned)grid, 1, kQsThreads, kQsSmemBytes, st, ms, mt, rows, cols, rw, tr,
-                             dev_status, spin_limit, withhold_loads));
+    MX_CHECK_CUDA(launch_pdl(k_quantize_stream<EMIT_ROW, SR_ROW, SR_T, DQ, GELU>, (unsigned)grid, 1, kQsThreads, kQsSmemBytes, st, ms, mt, rows, cols, rw, tr,
+                             dev_status, spin_limit, withhold_loads, hook_out, hook_ld));
     return MXFP4_OK;
 }
 
@@ -642,6 +645,24 @@ mxfp4_status_t quantize_tile(const void *src_bf16, const mxfp4_mat_t *src_q, int
                              const mxfp4_qparams_t *qp_t, uint32_t *dev_status, cudaStream_t st, bool chain)
 {
     return quantize_tile_ex(src_bf16, src_q, rows, cols, ld, dst, qp_row, dst_t, qp_t, dev_status, st, chain, kWaitSpinLimit, 0);
+}
+
+// The second half of mxfp4_gemm_quant with GELU and the double-quantization chain: Z = bf16(GELU(Y)) and its quantizations from
+// one read of Y.  The caller has checked every argument.
+mxfp4_status_t quantize_gelu_chain(const void *y_bf16, int64_t rows, int64_t cols, int64_t ldy, void *z_bf16, int64_t ldz, mxfp4_mat_t dst,
+                                   const mxfp4_qparams_t *qp_row, mxfp4_mat_t dst_t, const mxfp4_qparams_t *qp_t, uint32_t *dev_status, cudaStream_t st)
+{
+    CUtensorMap ms, mt;
+    if (!make_src_map(&ms, y_bf16, rows, cols, ldy) || !make_packed_t_map(&mt, dst_t.data, rows, cols)) return MXFP4_CUDA_ERROR;
+    const QuantSide rw = make_side(dst, qp_row), tr = make_side(dst_t, qp_t);
+    __nv_bfloat16 *z = static_cast<__nv_bfloat16 *>(z_bf16);
+    const int r = (int)rows, c = (int)cols;
+    const bool sr_r = qp_row->rounding == MXFP4_ROUND_STOCHASTIC, sr_t = qp_t->rounding == MXFP4_ROUND_STOCHASTIC;
+    if (sr_r)
+        return sr_t ? launch_stream<true, true, true, true, true>(st, ms, mt, r, c, rw, tr, dev_status, kWaitSpinLimit, 0, z, ldz)
+                    : launch_stream<true, true, false, true, true>(st, ms, mt, r, c, rw, tr, dev_status, kWaitSpinLimit, 0, z, ldz);
+    return sr_t ? launch_stream<true, false, true, true, true>(st, ms, mt, r, c, rw, tr, dev_status, kWaitSpinLimit, 0, z, ldz)
+                : launch_stream<true, false, false, true, true>(st, ms, mt, r, c, rw, tr, dev_status, kWaitSpinLimit, 0, z, ldz);
 }
 
 std::atomic<unsigned long long> g_launches{0};

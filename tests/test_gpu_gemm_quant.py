@@ -106,6 +106,39 @@ def test_quantizing_epilogue_gelu_with_bias_keeps_y(mx):
     assert_qmat_equal(epi.zq_t, pt, s_t, "Q6 of the next layer")
 
 
+@pytest.mark.parametrize("M,N,with_z", [(4128, 2336, True), (18944, 512, False), (18912, 512, False)])
+def test_gelu_chain_of_many_tiles(mx, M, N, with_z):
+    """From four tiles per SM on the product and the quantization behind GELU run as two kernels: sizes on both sides of that
+    line (592 and 591 tiles of the 592 on 148 SMs) and partial tiles, Y with a leading dimension of its own."""
+    K = 64
+    ops, a, b = operands(mx, M, N, K, 11)
+    big = torch.full((M, N + 16), 7.0, dtype=torch.bfloat16, device="cuda")
+    y = big[:, :N]
+    z = torch.empty((M, N), dtype=torch.bfloat16, device="cuda") if with_z else None
+    epi = mx.Epilogue(hook=mx.HOOK_GELU, y=y, z=z, zq=mx.QMat(M, N), zq_t=mx.QMat(N, M), qp_t=(0, 1, 5, 6), chain=True)
+    st = mx.new_status()
+    mx.gemm_quant(a, b, epi, dev_status=st)
+    torch.cuda.synchronize()
+    assert int(st.item()) == 0 and bool((big[:, N:] == 7.0).all())
+    assert torch.equal(y, mx.gemm(a, b))
+    yd = y.double()
+    g = 0.5 * yd * (1.0 + torch.erf(yd / math.sqrt(2.0)))
+    if with_z:
+        assert bool(((z.double() - g).abs() <= g.abs() * 2.0 ** -8 + yd.abs() * 2.0 ** -20).all())
+    else:   # the codes of Z stand for it: dequantized, they are within half a step of the group's grid (6 * 2^s >= the maximum)
+        gm = g.abs().reshape(M, N // 32, 32).amax(2, keepdim=True)
+        d = (mx.dequantize(epi.zq).double() - g).abs().reshape(M, N // 32, 32)
+        assert bool((d <= gm * (1.01 / 3)).all())
+        z = None
+    if z is not None:
+        q, qt = mx.quantize_chain(z, seed=5)
+        for got, want in ((epi.zq, q), (epi.zq_t, qt)):
+            assert torch.equal(got.data, want.data) and torch.equal(got.scales_linear(), want.scales_linear())
+    else:
+        qt = mx.quantize_t(epi.zq, rounding=1, seed=5, stream_id=6)
+        assert torch.equal(epi.zq_t.data, qt.data) and torch.equal(epi.zq_t.scales_linear(), qt.scales_linear())
+
+
 def test_quantizing_epilogue_multiply_is_exact(mx):
     """dX times the derivative of the activation, then Q3 / Q5 of the previous layer: the product of two bf16 values is
     exact in FP32, so Z = bf16(Y * aux) is reproducible bit for bit from the Y the kernel emitted."""
