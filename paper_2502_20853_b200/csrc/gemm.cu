@@ -46,7 +46,8 @@ struct GemmCfg {
     static constexpr int kTmemCols = 512;
     static constexpr int kStagingOff = kStages * kStageBytes;           // multiple of 1024
     static constexpr int kBarOff = kStagingOff + kEpiWarps * kStagingBufs * kStagingBytes;
-    static constexpr int kSmemBytes = kBarOff + 1024 /*align*/ + 256 /*barriers*/;
+    static constexpr int kBiasOff = kBarOff + 256;                      // a line of BN / 2 bf16 per epilogue warp
+    static constexpr int kSmemBytes = kBiasOff + kEpiWarps * BN + 1024 /*align*/;
     static_assert(kSfCol + kStages * kSfSlot <= 512, "TMEM budget");
     static_assert(kStageBytes % 1024 == 0, "stage alignment");
     static_assert(kSmemBytes <= 232448, "shared memory budget");
@@ -120,11 +121,44 @@ __device__ __forceinline__ uint32_t idesc_mxf4(int n, uint32_t a_sf_id, uint32_t
            (a_sf_id << 29);
 }
 
-// The bias of one 32-column chunk, for a warp whose lanes hold one accumulator row each: lane l keeps columns 2 (l & 15) and
-// 2 (l & 15) + 1 as a bf16 pair (zero beyond N, where nothing is stored), the warp passes them round with shuffles, and the
-// mixed-precision add takes the bf16 value as it is.  The pairs are fetched before the wait for the accumulator.  (Every lane
-// loading the whole chunk's bias by itself, four dependent 16-byte loads per chunk behind that wait, cost 500 cycles per chunk:
-// 50432 x 4096 x 1024 took 161 us with a bias against 110 without; now 111.)
+// The bias of a warp's share of a tile.  The lanes hold one accumulator row each, so every lane needs every column's value: they
+// fetch it together, a bf16 pair per lane and turn, before the wait for the accumulator (bias_fetch; zero beyond N, where
+// nothing is stored), put it into the warp's own line of shared memory (bias_stage), and read it back as broadcasts, 16 bytes
+// at a time, for the mixed-precision add, which takes bf16 values as they are (add_bias_chunk).  50432 x 4096 x 1024, back to
+// back: 107.6 us without a bias, MEASURED with it; passing the pairs round with shuffles instead took 125 us, every lane
+// fetching every value by itself behind the wait 160.
+template <int COLS>
+__device__ __forceinline__ void bias_fetch(uint32_t (&w)[(COLS + 63) / 64], const __nv_bfloat16 *bias, int64_t col, int64_t N, int lane)
+{
+#pragma unroll
+    for (int i = 0; i < (COLS + 63) / 64; i++) {
+        const int64_t c = col + 64 * i + 2 * lane;
+        w[i] = 0u;
+        if (bias != nullptr && c < N) asm volatile("ld.global.nc.u32 %0, [%1];" : "=r"(w[i]) : "l"(bias + c));
+    }
+}
+template <int COLS>
+__device__ __forceinline__ void bias_stage(const uint32_t (&w)[(COLS + 63) / 64], uint32_t line, int lane)
+{
+#pragma unroll
+    for (int i = 0; i < (COLS + 63) / 64; i++)
+        if (64 * i + 2 * lane < COLS) asm volatile("st.shared.u32 [%0], %1;" ::"r"(line + (uint32_t)(128 * i + 4 * lane)), "r"(w[i]) : "memory");
+    __syncwarp();
+}
+__device__ __forceinline__ void add_bias_chunk(uint32_t (&r)[32], uint32_t line)
+{
+#pragma unroll
+    for (int j = 0; j < 4; j++) {
+        uint32_t b[4];
+        asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(b[0]), "=r"(b[1]), "=r"(b[2]), "=r"(b[3]) : "r"(line + 16u * j));
+#pragma unroll
+        for (int t = 0; t < 4; t++)
+            asm("{\n\t.reg .b16 l, h;\n\tmov.b32 {l, h}, %4;\n\tadd.rn.f32.bf16 %0, l, %2;\n\tadd.rn.f32.bf16 %1, h, %3;\n\t}"
+                : "=&r"(r[8 * j + 2 * t]), "=&r"(r[8 * j + 2 * t + 1]) : "r"(r[8 * j + 2 * t]), "r"(r[8 * j + 2 * t + 1]), "r"(b[t]));
+    }
+}
+// The same without a line of shared memory (the streaming pair kernel has none to spare, and its long K loops hide it): each
+// lane keeps columns 2 (l & 15) and 2 (l & 15) + 1 of a 32-column chunk, the warp passes the pairs round with shuffles.
 __device__ __forceinline__ uint32_t load_bias_pair(const __nv_bfloat16 *bias, int64_t col, int64_t N, int lane)
 {
     const int64_t c = col + 2 * (lane & 15);
@@ -132,7 +166,7 @@ __device__ __forceinline__ uint32_t load_bias_pair(const __nv_bfloat16 *bias, in
     if (bias != nullptr && c < N) asm volatile("ld.global.nc.u32 %0, [%1];" : "=r"(v) : "l"(bias + c));
     return v;
 }
-__device__ __forceinline__ void add_bias_chunk(uint32_t (&r)[32], uint32_t pair)
+__device__ __forceinline__ void add_bias_chunk_shfl(uint32_t (&r)[32], uint32_t pair)
 {
 #pragma unroll
     for (int j = 0; j < 16; j++) {
@@ -189,11 +223,12 @@ __device__ __forceinline__ void mbar_arrive_remote(uint32_t cluster_addr)
     asm volatile("mbarrier.arrive.shared::cluster.b64 _, [%0];" ::"r"(cluster_addr) : "memory");
 }
 
+// `bias_line`: the share's bias in shared memory (bias_stage).
 // REMOTE: `acc_empty_bar` is a shared::cluster address (the barrier lives in the leader of a CTA pair).
 template <int BN, int BUFS, bool REMOTE = false>
 __device__ __forceinline__ void epilogue_tile(const CUtensorMap *map_d, const CUtensorMap *map_w, const GemmParams &p, uint32_t taddr,
                                               int row0, int colbase, int split, uint8_t *staging, uint32_t &sbuf, int lane,
-                                              uint32_t acc_empty_bar, const uint32_t (&bias)[BN / 64])
+                                              uint32_t acc_empty_bar, uint32_t bias_line)
 {
     constexpr int kHalfCols = BN / 2;
     constexpr int kChunks = kHalfCols / 32;
@@ -231,7 +266,7 @@ __device__ __forceinline__ void epilogue_tile(const CUtensorMap *map_d, const CU
                 uint32_t r[32];
                 tc_ld32(taddr + cc * 32, r);
                 tc_wait_ld();
-                if (use_bias) add_bias_chunk(r, bias[cc]);
+                if (use_bias) add_bias_chunk(r, bias_line + 64u * cc);
                 pack_row_bf16(r, pk[cc]);
             }
         }
@@ -293,7 +328,7 @@ __device__ __forceinline__ void epilogue_tile(const CUtensorMap *map_d, const CU
             if (cc == kChunks - 1) release_acc();
             if (!live) continue;
             const int ncols = (int)min((int64_t)32, p.N - col);
-            if (use_bias) add_bias_chunk(r, load_bias_pair(p.bias, col, p.N, lane));
+            if (use_bias) add_bias_chunk(r, bias_line + 64u * cc);
             store_box(r, col);
             if (ncols > 16) store_box(r + 16, col + 16);
         }
@@ -498,6 +533,7 @@ k_gemm_mxf4(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
         const int quarter = warp & 3;            // TMEM lanes 32*quarter .. +31 are the ones this warp may read
         const int chalf = ew >> 2;               // which half of the tile's columns this warp stores
         uint8_t *staging = smem + C::kStagingOff + ew * C::kStagingBufs * kStagingBytes;
+        const uint32_t bias_line = smem_base + C::kBiasOff + ew * (BN / 2) * 2;
         uint32_t sbuf = 0;                       // staging buffer of the next box (round robin)
         constexpr int kHalfCols = BN / 2;
         constexpr int kChunks = kHalfCols / 32;
@@ -506,16 +542,16 @@ k_gemm_mxf4(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
         for (int item = blockIdx.x; item < items && alive; item += gridDim.x) {
             const int split = item % p.splits, tile = item / p.splits;
             const int mb = tile / p.tiles_n, nb = tile % p.tiles_n;
-            uint32_t bias[kHalfCols / 32];
-#pragma unroll
-            for (int cc = 0; cc < kHalfCols / 32; cc++) bias[cc] = load_bias_pair(p.bias, (int64_t)nb * BN + chalf * kHalfCols + cc * 32, p.N, lane);
+            uint32_t bias[(kHalfCols + 63) / 64];
+            bias_fetch<kHalfCols>(bias, p.bias, (int64_t)nb * BN + chalf * kHalfCols, p.N, lane);
             if (!mbar_wait(bar_acc_full + 8 * acc, acc_phase, abort_flag, p.dev_status, p.spin_limit)) { alive = false; break; }
             tc_fence_after();
             const int row0 = mb * kBM + quarter * 32;
             const int colbase = nb * BN + chalf * kHalfCols;
             const uint32_t taddr = tmem_base + ((uint32_t)(quarter * 32) << 16) + acc * BN + chalf * kHalfCols;
+            if (p.bias != nullptr) bias_stage<kHalfCols>(bias, bias_line, lane);
             epilogue_tile<BN, C::kStagingBufs>(&map_d, p.out_fp32 ? nullptr : &map_dw, p, taddr, row0, colbase, split, staging, sbuf, lane,
-                                               bar_acc_empty + 8 * acc, bias);
+                                               bar_acc_empty + 8 * acc, bias_line);
             if (++acc == C::kAccStages) { acc = 0; acc_phase ^= 1u; }
         }
         if (lane == 0) bulk_wait0();   // all stores of this warp have completed before the CTA may exit
@@ -559,7 +595,8 @@ struct GemmQCfg {
     static constexpr int kStagingOff = kTileYOff + (WITH_Y ? kTileBytes : 0);   // 2 x (transposed codes 8 KB + two scale chunks)
     static constexpr int kStagingBytes = kTile * 64 + 1024;
     static constexpr int kBarOff = kStagingOff + 2 * kStagingBytes;
-    static constexpr int kSmemBytes = kBarOff + 1024 /*align*/ + 256 /*barriers*/;
+    static constexpr int kBiasOff = kBarOff + 256;                   // a line of 64 bf16 per epilogue warp
+    static constexpr int kSmemBytes = kBiasOff + kEpiWarps * 128 + 1024 /*align*/;
     static_assert(kSfCol + kStages * kSfSlot <= 512, "TMEM budget");
     static_assert(kStageBytes % 1024 == 0 && kStagingBytes % 1024 == 0, "alignment");
     static_assert(kSmemBytes <= 232448, "shared memory budget");
@@ -655,6 +692,7 @@ k_gemm_mxf4_q(const __grid_constant__ CUtensorMap map_a, const __grid_constant__
         };
         if (aux_tma && et == 0 && !p.withhold_loads && (int)blockIdx.x < p.tiles_m * p.tiles_n) issue_aux(blockIdx.x);
         const bool use_bias = p.bias != nullptr;
+        const uint32_t bias_line = smem_base + C::kBiasOff + (warp - kEpiWarp0) * 128;
         uint32_t nonfinite = 0;
         uint32_t acc = 0, acc_phase = 0;
         const int items = p.tiles_m * p.tiles_n;
@@ -662,11 +700,13 @@ k_gemm_mxf4_q(const __grid_constant__ CUtensorMap map_a, const __grid_constant__
         for (int item = blockIdx.x; item < items; item += gridDim.x, it++) {
             const int mb = item / p.tiles_n, nb = item % p.tiles_n;
             const int row0 = mb * kBM, col0 = nb * BN;
-            const uint32_t bias[2] = {load_bias_pair(p.bias, col0 + chalf * 64, N, lane), load_bias_pair(p.bias, col0 + chalf * 64 + 32, N, lane)};
+            uint32_t bias[1];
+            bias_fetch<64>(bias, p.bias, col0 + chalf * 64, N, lane);
             bool ok = mbar_wait(bar_acc_full + 8 * acc, acc_phase, abort_flag, p.dev_status, p.spin_limit);
             if (aux_tma) ok = mbar_wait(bar_aux, (uint32_t)it & 1u, abort_flag, p.dev_status, p.spin_limit) && ok;
             if (epi_any(!ok)) break;      // a wait ran out in one of the eight warps: all of them leave together
             tc_fence_after();
+            if (use_bias) bias_stage<64>(bias, bias_line, lane);
             uint8_t *staging = smem + C::kStagingOff + (it & 1) * C::kStagingBytes;
             uint8_t *s_sc_row = staging + kTile * 64, *s_sc_t = s_sc_row + 512;
             const uint32_t taddr = tmem_base + ((uint32_t)(quarter * 32) << 16) + acc * BN + chalf * 64;
@@ -685,7 +725,7 @@ k_gemm_mxf4_q(const __grid_constant__ CUtensorMap map_a, const __grid_constant__
                     __syncwarp();
                     if (lane == 0) mbar_arrive(bar_acc_empty + 8 * acc);   // the accumulator goes back to the MMA issuer
                 }
-                if (use_bias) add_bias_chunk(r, bias[cc]);
+                if (use_bias) add_bias_chunk(r, bias_line + 64u * cc);
                 uint32_t yw[16];
                 pack_row_bf16(r, yw);
                 if (WITH_Y && e.store_y) {
@@ -791,7 +831,8 @@ struct GemmBsCfg {
     static constexpr int kSfaOff = kSfbOff + KT * kSfbBytes;
     static constexpr int kStagingOff = kSfaOff + AS * kSfaBytes;
     static constexpr int kBarOff = kStagingOff + kEpiWarps * kStagingBufs * kStagingBytes;
-    static constexpr int kSmemBytes = kBarOff + 1024 /*align*/ + 256 /*barriers*/;
+    static constexpr int kBiasOff = kBarOff + 256;             // a line of BN / 2 bf16 per epilogue warp
+    static constexpr int kSmemBytes = kBiasOff + kEpiWarps * BN + 1024 /*align*/;
     static constexpr int kSfbCol = 2 * BN;                     // TMEM columns: two accumulators, resident SFB (8 kRB per K tile), SFA ring (8 per stage)
     static constexpr int kSfaCol = kSfbCol + KT * 8 * kRB;
     static constexpr int kTmemCols = 512;
@@ -1003,21 +1044,22 @@ k_gemm_mxf4_bs(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
         const int quarter = warp & 3;
         const int chalf = ew >> 2;
         uint8_t *staging = smem + C::kStagingOff + ew * C::kStagingBufs * kStagingBytes;
+        const uint32_t bias_line = smem_base + C::kBiasOff + ew * (BN / 2) * 2;
         uint32_t sbuf = 0;
         constexpr int kHalfCols = BN / 2;
         uint32_t acc = 0, acc_phase = 0;
         for (int t = t0; t < t1; t++) {
             const int mb = t % p.tiles_m, nb = t / p.tiles_m;
-            uint32_t bias[kHalfCols / 32];
-#pragma unroll
-            for (int cc = 0; cc < kHalfCols / 32; cc++) bias[cc] = load_bias_pair(p.bias, (int64_t)nb * BN + chalf * kHalfCols + cc * 32, p.N, lane);
+            uint32_t bias[(kHalfCols + 63) / 64];
+            bias_fetch<kHalfCols>(bias, p.bias, (int64_t)nb * BN + chalf * kHalfCols, p.N, lane);
             if (!mbar_wait(bar_acc_full + 8 * acc, acc_phase, abort_flag, p.dev_status, p.spin_limit)) break;
             tc_fence_after();
             const int row0 = mb * kBM + quarter * 32;
             const int colbase = nb * BN + chalf * kHalfCols;
             const uint32_t taddr = tmem_base + ((uint32_t)(quarter * 32) << 16) + acc * BN + chalf * kHalfCols;
+            if (p.bias != nullptr) bias_stage<kHalfCols>(bias, bias_line, lane);
             epilogue_tile<BN, C::kStagingBufs>(&map_d, p.out_fp32 ? nullptr : &map_dw, p, taddr, row0, colbase, 0, staging, sbuf, lane,
-                                               bar_acc_empty + 8 * acc, bias);
+                                               bar_acc_empty + 8 * acc, bias_line);
             if (++acc == 2) { acc = 0; acc_phase ^= 1u; }
         }
         if (lane == 0) bulk_wait0();   // all stores of this warp have completed before the CTA may exit
@@ -1724,7 +1766,7 @@ k_gemm_mxf4_pair(const __grid_constant__ CUtensorMap map_a, const __grid_constan
                         uint32_t r[32];
                         tc_ld32(taddr + cc * 32, r);
                         tc_wait_ld();
-                        if (use_bias) add_bias_chunk(r, bias[cc]);
+                        if (use_bias) add_bias_chunk_shfl(r, bias[cc]);
                         pack_row_bf16(r, pk[cc]);
                     }
                 }
@@ -1764,7 +1806,7 @@ k_gemm_mxf4_pair(const __grid_constant__ CUtensorMap map_a, const __grid_constan
                     if (cc == kChunks - 1) release_acc();
                     if (!live) continue;
                     const int ncols = (int)min((int64_t)32, p.N - col);
-                    if (use_bias) add_bias_chunk(r, load_bias_pair(p.bias, col, p.N, lane));
+                    if (use_bias) add_bias_chunk_shfl(r, load_bias_pair(p.bias, col, p.N, lane));
                     store_box(r, col);
                     if (ncols > 16) store_box(r + 16, col + 16);
                 }
@@ -1837,13 +1879,14 @@ struct GemmPbsCfg {
     static constexpr int kSfaOff = kSfbOff + KT * kSfbBytes;
     static constexpr int kStagingOff = kSfaOff + AS * kSfaBytes;
     static constexpr int kBarOff = kStagingOff + kEpiWarps * kStagingBufs * kStagingBytes;
-    static constexpr int kSmemBytes = kBarOff + 1024 /*align*/ + 512 /*barriers*/;
+    static constexpr int kBiasOff = kBarOff + 256;              // a line of BN / 2 bf16 per epilogue warp
+    static constexpr int kSmemBytes = kBiasOff + kEpiWarps * BN + 1024 /*align*/;
     static constexpr int kSfbCol = 2 * BN;                      // TMEM columns: two accumulators, resident SFB (16 per K tile), SFA ring (8 per stage)
     static constexpr int kSfaCol = kSfbCol + KT * 16;
     static constexpr int kTmemCols = 512;
     static_assert(kSfaCol + AS * 8 <= 512, "TMEM budget");
     static_assert(kAOff % 1024 == 0 && kStagingOff % 1024 == 0, "alignment");
-    static_assert((3 * AS + 7) * 8 + 8 <= 512, "barrier slots");
+    static_assert((3 * AS + 7) * 8 + 8 <= 256, "barrier slots");
     static_assert(kSmemBytes <= 232448, "shared memory budget");
 };
 
@@ -2063,22 +2106,23 @@ k_gemm_mxf4_pbs(const __grid_constant__ CUtensorMap map_a, const __grid_constant
         const int quarter = warp & 3;
         const int chalf = ew >> 2;
         uint8_t *staging = smem + C::kStagingOff + ew * C::kStagingBufs * kStagingBytes;
+        const uint32_t bias_line = smem_base + C::kBiasOff + ew * (BN / 2) * 2;
         uint32_t sbuf = 0;
         constexpr int kHalfCols = BN / 2;
         uint32_t acc = 0, acc_phase = 0;
         for (int t = t0; t < t1; t++) {
             const PbsTile x = pbs_tile(walk, t);
             const int mb = x.mb2 * 2 + (int)rank, nb = x.nb;
-            uint32_t bias[kHalfCols / 32];
-#pragma unroll
-            for (int cc = 0; cc < kHalfCols / 32; cc++) bias[cc] = load_bias_pair(p.bias, (int64_t)nb * BN + chalf * kHalfCols + cc * 32, p.N, lane);
+            uint32_t bias[(kHalfCols + 63) / 64];
+            bias_fetch<kHalfCols>(bias, p.bias, (int64_t)nb * BN + chalf * kHalfCols, p.N, lane);
             if (!mbar_wait(bar_acc_full + 8 * acc, acc_phase, abort_flag, p.dev_status, p.spin_limit)) break;
             tc_fence_after();
             const int row0 = mb * kBM + quarter * 32;
             const int colbase = nb * BN + chalf * kHalfCols;
             const uint32_t taddr = tmem_base + ((uint32_t)(quarter * 32) << 16) + acc * BN + chalf * kHalfCols;
+            if (p.bias != nullptr) bias_stage<kHalfCols>(bias, bias_line, lane);
             epilogue_tile<BN, C::kStagingBufs, true>(&map_d, p.out_fp32 ? nullptr : &map_dw, p, taddr, row0, colbase, 0, staging, sbuf, lane,
-                                                     map_to_cta(bar_acc_empty + 8 * acc, 0), bias);
+                                                     map_to_cta(bar_acc_empty + 8 * acc, 0), bias_line);
             if (++acc == 2) { acc = 0; acc_phase ^= 1u; }
         }
         if (lane == 0) bulk_wait0();   // all stores of this warp have completed before the CTA may exit
