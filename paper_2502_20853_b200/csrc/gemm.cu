@@ -125,7 +125,7 @@ __device__ __forceinline__ uint32_t idesc_mxf4(int n, uint32_t a_sf_id, uint32_t
 // fetch it together, a bf16 pair per lane and turn, before the wait for the accumulator (bias_fetch; zero beyond N, where
 // nothing is stored), put it into the warp's own line of shared memory (bias_stage), and read it back as broadcasts, 16 bytes
 // at a time, for the mixed-precision add, which takes bf16 values as they are (add_bias_chunk).  50432 x 4096 x 1024, back to
-// back: 107.6 us without a bias, MEASURED with it; passing the pairs round with shuffles instead took 125 us, every lane
+// back: 109 us without a bias, 120 with it; passing the pairs round with shuffles instead took 123 to 125 us, every lane
 // fetching every value by itself behind the wait 160.
 template <int COLS>
 __device__ __forceinline__ void bias_fetch(uint32_t (&w)[(COLS + 63) / 64], const __nv_bfloat16 *bias, int64_t col, int64_t N, int lane)
