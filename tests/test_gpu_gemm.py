@@ -174,6 +174,14 @@ def test_gemm_bias_ragged_edges(mx, M, N, K, out_dtype):
     _bias_case(mx, M, N, K, out_dtype)
 
 
+@pytest.mark.parametrize("M,N,K", [(128, 96, 128 * 1024), (24, 8, 8192), (256, 248, 16384), (256, 264, 16384)])
+@pytest.mark.parametrize("out_dtype", [0, 1])
+def test_gemm_many_splits_of_a_small_output(mx, M, N, K, out_dtype):
+    """Up to 64 partial sums, reduced by eight threads per output (below 64 blocks' worth of outputs) or by one."""
+    assert mx.gemm_workspace_bytes(M, N, K) >= 8 * M * N * 4
+    _bias_case(mx, M, N, K, out_dtype)
+
+
 def test_gemm_argument_errors(mx):
     a, b = mx.QMat(128, 64), mx.QMat(128, 96)
     with pytest.raises(mx.MxError) as e:
