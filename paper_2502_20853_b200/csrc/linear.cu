@@ -8,6 +8,9 @@ mxfp4_status_t quantize_rows(const void *src, int64_t rows, int64_t cols, int64_
 mxfp4_status_t quantize_tile(const void *src_bf16, const mxfp4_mat_t *src_q, int64_t rows, int64_t cols, int64_t ld,
                              const mxfp4_mat_t *dst, const mxfp4_qparams_t *qp_row, mxfp4_mat_t dst_t,
                              const mxfp4_qparams_t *qp_t, uint32_t *dev_status, cudaStream_t st, bool chain);
+mxfp4_status_t quantize_chain_two(const void *x_bf16, int64_t m, int64_t k, int64_t ldx, const mxfp4_mat_t &xq, const mxfp4_mat_t &xq_t, const mxfp4_qparams_t *q6,
+                                  const void *w_bf16, int64_t n, const mxfp4_mat_t &wq, const mxfp4_mat_t &wq_t, const mxfp4_qparams_t *q4,
+                                  const mxfp4_qparams_t *rne, uint32_t *dev_status, cudaStream_t st);
 mxfp4_status_t gemm(mxfp4_mat_t a, mxfp4_mat_t b, void *d, int64_t ldd, int out_dtype, const void *bias, void *workspace,
                     size_t workspace_bytes, uint32_t *dev_status, cudaStream_t st, bool allow_split);
 mxfp4_status_t gemm_check(mxfp4_mat_t a, mxfp4_mat_t b, const void *d, int64_t ldd, int out_dtype, const void *bias,
@@ -85,22 +88,21 @@ mxfp4_status_t mxfp4_linear_fwd_ex(const void *x_bf16, int64_t ldx, int64_t m, i
         if (!ctx->wq_t.scales) return MXFP4_INVALID_ARG;
         if ((reinterpret_cast<uintptr_t>(ctx->wq_t.data) | reinterpret_cast<uintptr_t>(ctx->wq_t.scales)) & 15u) return MXFP4_MISALIGNED;
     }
-    if (x_bf16 && ctx->xq_t.data) {
-        // Q1 and, from its dequantized result, Q6 (stream 6 of the seed the backward pass will use) in one pass over X
-        const mxfp4_qparams_t q6 = {scale_mode, MXFP4_ROUND_STOCHASTIC, ctx->xq_t_seed, 6, 0};
-        s = quantize_tile(x_bf16, nullptr, m, k, ldx, &ctx->xq, &qp, ctx->xq_t, &q6, dev_status, st, true);
+    // Q1 and, from its dequantized result, Q6 (stream 6 of the seed the backward pass will use) come from one pass over X,
+    // Q2 and Q4 (stream 4) likewise from one over W; both together in one launch
+    const mxfp4_qparams_t q6 = {scale_mode, MXFP4_ROUND_STOCHASTIC, ctx->xq_t_seed, 6, 0};
+    const mxfp4_qparams_t q4 = {scale_mode, MXFP4_ROUND_STOCHASTIC, ctx->wq_t_seed, 4, 0};
+    const bool make_q6 = x_bf16 && ctx->xq_t.data;
+    if (make_q6 && make_q4 && m > 0 && n > 0 && k > 0) {
+        if (scale_mode != MXFP4_SCALE_TRUNCATION_FREE && scale_mode != MXFP4_SCALE_FLOOR) return MXFP4_INVALID_ARG;
+        s = quantize_chain_two(x_bf16, m, k, ldx, ctx->xq, ctx->xq_t, &q6, w_bf16, n, ctx->wq, ctx->wq_t, &q4, &qp, dev_status, st);
         if (s) return s;
-    } else if (x_bf16) {
-        s = quantize_rows(x_bf16, m, k, ldx, ctx->xq, &qp, dev_status, st);  // Q1
+    } else {
+        if (make_q6) s = quantize_tile(x_bf16, nullptr, m, k, ldx, &ctx->xq, &qp, ctx->xq_t, &q6, dev_status, st, true);
+        else s = x_bf16 ? quantize_rows(x_bf16, m, k, ldx, ctx->xq, &qp, dev_status, st) : MXFP4_OK;
         if (s) return s;
-    }
-    if (make_q4) {
-        // Q2 and, from its dequantized result, Q4 (stream 4 of the seed the backward pass will use)
-        const mxfp4_qparams_t q4 = {scale_mode, MXFP4_ROUND_STOCHASTIC, ctx->wq_t_seed, 4, 0};
-        s = quantize_tile(w_bf16, nullptr, n, k, k, &ctx->wq, &qp, ctx->wq_t, &q4, dev_status, st, true);
-        if (s) return s;
-    } else if (w_bf16) {
-        s = quantize_rows(w_bf16, n, k, k, ctx->wq, &qp, dev_status, st);  // Q2
+        if (make_q4) s = quantize_tile(w_bf16, nullptr, n, k, k, &ctx->wq, &qp, ctx->wq_t, &q4, dev_status, st, true);
+        else s = w_bf16 ? quantize_rows(w_bf16, n, k, k, ctx->wq, &qp, dev_status, st) : MXFP4_OK;
         if (s) return s;
     }
     if (epi) return gemm_quant(ctx->xq, ctx->wq, bias_bf16, epi, dev_status, st);

@@ -223,54 +223,28 @@ constexpr int kQsBarOff = 2 * kTileBytes + 2 * kQsStagingBytes;
 constexpr int kQsSmemBytes = kQsBarOff + 64 + 1024 /*align*/;
 constexpr int kQsCtasPerSm = 2;
 
-// GELU: the source is a product's result Y, quantized behind the activation (see qs_row_pass).
-template <bool EMIT_ROW, bool SR_ROW, bool SR_T, bool DQ, bool GELU>
-__global__ void __launch_bounds__(kQsThreads, kQsCtasPerSm)
-k_quantize_stream(const __grid_constant__ CUtensorMap map_src, const __grid_constant__ CUtensorMap map_t, int rows, int cols,
-                  const __grid_constant__ QuantSide rw, const __grid_constant__ QuantSide tr, uint32_t *dev_status, uint32_t spin_limit,
-                  int withhold_loads, __nv_bfloat16 *hook_out, int64_t hook_ld)
+// One source matrix of a launch and its results.
+struct QsJob {
+    CUtensorMap map_src, map_t;
+    QuantSide rw, tr;
+    int rows, cols;
+};
+struct QsNone {};
+
+// The walk of a CTA over the tiles of one matrix.  The tiles of a launch are numbered through: this matrix has the numbers
+// [first, end), and `tile` and the ring's turn `it` run on from one matrix to the next.  load(tile, stage) starts the load of
+// any tile of the launch.
+template <bool EMIT_ROW, bool SR_ROW, bool SR_T, bool DQ, bool GELU, class Load>
+__device__ __forceinline__ bool qs_walk(const QsJob &job, const QsGeom &g, int first, int end, int all, int &tile, int &it, uint8_t *smem, uint32_t smem_base,
+                                        uint32_t bar_full, volatile uint32_t *abort_flag, uint32_t *dev_status, uint32_t spin_limit, uint32_t &nonfinite,
+                                        __nv_bfloat16 *hook_out, int64_t hook_ld, const Load &load)
 {
-    extern __shared__ uint8_t qs_smem_raw[];
-    uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(qs_smem_raw) + 1023) & ~(uintptr_t)1023);
-    const uint32_t smem_base = smem_u32(smem);
-    const uint32_t bar_full = smem_base + kQsBarOff;
-    volatile uint32_t *abort_flag = reinterpret_cast<volatile uint32_t *>(smem + kQsBarOff + 32);
-
-    pdl_launch_dependents();
-    const int tid = threadIdx.x;
-    const int ntx = (cols + kTile - 1) / kTile, nty = (rows + kTile - 1) / kTile;
-    const int total = ntx * nty;
-
-    auto issue_load = [&](int tile, int stage) {
-        const int ty = tile / ntx, tx = tile - ty * ntx;
-        const uint32_t bar = bar_full + 8 * stage, dst = smem_base + stage * kTileBytes;
-        mbar_expect_tx(bar, kTileBytes);
-        tma_load_2d(dst, &map_src, tx * kTile, ty * kTile, bar);
-        tma_load_2d(dst + kTileBytes / 2, &map_src, tx * kTile + 64, ty * kTile, bar);
-    };
-
-    if (tid == 0) {
-        mbar_init(bar_full, 1);
-        mbar_init(bar_full + 8, 1);
-        *abort_flag = 0u;
-        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    }
-    pdl_wait();
-    if (tid == 0) {
-        // withhold_loads (self-test of the drain path): nothing is ever loaded, so the first bounded wait runs out
-        for (int s = 0; s < 2; s++)
-            if (!withhold_loads && (int)blockIdx.x + s * (int)gridDim.x < total) issue_load(blockIdx.x + s * gridDim.x, s);
-    }
-    __syncthreads();
-
-    const QsGeom g = qs_geom(tid, rows, cols, rw.packed);
-    const uint32_t tfa_r2 = tf_add_of(rw.scale_mode) * 0x00010001u, tfa_t2 = tf_add_of(tr.scale_mode) * 0x00010001u;
-    uint32_t nonfinite = 0;
+    const int rows = job.rows, cols = job.cols, ntx = (cols + kTile - 1) / kTile;
+    const uint32_t tfa_r2 = tf_add_of(job.rw.scale_mode) * 0x00010001u, tfa_t2 = tf_add_of(job.tr.scale_mode) * 0x00010001u;
     // tile coordinates advance by the grid size without a division per tile
     const int step_y = (int)gridDim.x / ntx, step_x = (int)gridDim.x - step_y * ntx;
-    int ty = (int)blockIdx.x / ntx, tx = (int)blockIdx.x - ty * ntx;
-    int it = 0;
-    for (int tile = blockIdx.x; tile < total; tile += gridDim.x, it++) {
+    int ty = (tile - first) / ntx, tx = (tile - first) - ty * ntx;
+    for (; tile < end; tile += gridDim.x, it++) {
         const int stage = it & 1;
         const int row0 = ty * kTile, col0 = tx * kTile;
         const uint32_t st_base = smem_base + stage * kTileBytes;
@@ -279,26 +253,90 @@ k_quantize_stream(const __grid_constant__ CUtensorMap map_src, const __grid_cons
 
         const bool ok = mbar_wait_warp(bar_full + 8 * stage, (uint32_t)(it >> 1) & 1u, abort_flag, dev_status, spin_limit);
         if (ok)
-            qs_tile<SR_ROW, SR_T, DQ, GELU>(g, st_base, st_base, row0, col0, rows, cols, EMIT_ROW, true, rw, tr, tfa_r2, tfa_t2, staging, s_sc_row, s_sc_t, nonfinite,
-                                            hook_out, hook_ld);
+            qs_tile<SR_ROW, SR_T, DQ, GELU>(g, st_base, st_base, row0, col0, rows, cols, EMIT_ROW, true, job.rw, job.tr, tfa_r2, tfa_t2, staging, s_sc_row, s_sc_t,
+                                            nonfinite, hook_out, hook_ld);
 
         // ---- hand the tile's results to the copy engine, refill the ring ----
         fence_async_smem();                       // this thread's staging writes, before the asynchronous reads
-        if (tid == 0) bulk_wait_read<0>();        // the previous tile's stores have left the other staging buffer
-        if (__syncthreads_or(!ok)) break;          // a bounded wait ran out somewhere in the CTA: everybody leaves
-        if (tid == 0) {
-            tma_store_2d(&map_t, row0 >> 1, col0, smem_u32(staging));
-            bulk_store(tr.scales + ((size_t)(col0 >> 7) * tr.nblk4 + (row0 >> 7)) * 512, smem_u32(s_sc_t), 512);
-            if (EMIT_ROW) bulk_store(rw.scales + ((size_t)(row0 >> 7) * rw.nblk4 + (col0 >> 7)) * 512, smem_u32(s_sc_row), 512);
+        if (threadIdx.x == 0) bulk_wait_read<0>();   // the previous tile's stores have left the other staging buffer
+        if (__syncthreads_or(!ok)) return false;   // a bounded wait ran out somewhere in the CTA: everybody leaves
+        if (threadIdx.x == 0) {
+            tma_store_2d(&job.map_t, row0 >> 1, col0, smem_u32(staging));
+            bulk_store(job.tr.scales + ((size_t)(col0 >> 7) * job.tr.nblk4 + (row0 >> 7)) * 512, smem_u32(s_sc_t), 512);
+            if (EMIT_ROW) bulk_store(job.rw.scales + ((size_t)(row0 >> 7) * job.rw.nblk4 + (col0 >> 7)) * 512, smem_u32(s_sc_row), 512);
             bulk_commit();
             const int next = tile + 2 * (int)gridDim.x;
-            if (next < total) issue_load(next, stage);
+            if (next < all) load(next, stage);
         }
         tx += step_x;
         ty += step_y;
         if (tx >= ntx) { tx -= ntx; ty++; }
     }
-    if (tid == 0) bulk_wait0();                   // every store has completed before the shared memory goes away
+    return true;
+}
+
+// GELU: the source is a product's result Y, quantized behind the activation (see qs_row_pass).
+// Job2 = QsJob: a second matrix with the same roundings follows in the same launch (its tiles fill the tail of the first:
+// activations and weight of a forward pass); QsNone: there is none.
+template <bool EMIT_ROW, bool SR_ROW, bool SR_T, bool DQ, bool GELU, class Job2>
+__global__ void __launch_bounds__(kQsThreads, kQsCtasPerSm)
+k_quantize_stream(const __grid_constant__ QsJob job, const __grid_constant__ Job2 job2, uint32_t *dev_status, uint32_t spin_limit, int withhold_loads,
+                  __nv_bfloat16 *hook_out, int64_t hook_ld)
+{
+    constexpr bool kTwo = sizeof(Job2) == sizeof(QsJob);
+    extern __shared__ uint8_t qs_smem_raw[];
+    uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(qs_smem_raw) + 1023) & ~(uintptr_t)1023);
+    const uint32_t smem_base = smem_u32(smem);
+    const uint32_t bar_full = smem_base + kQsBarOff;
+    volatile uint32_t *abort_flag = reinterpret_cast<volatile uint32_t *>(smem + kQsBarOff + 32);
+
+    pdl_launch_dependents();
+    const int ntx = (job.cols + kTile - 1) / kTile, total = ntx * ((job.rows + kTile - 1) / kTile);
+    int ntx2 = 1, all = total;
+    if constexpr (kTwo) {
+        ntx2 = (job2.cols + kTile - 1) / kTile;
+        all += ntx2 * ((job2.rows + kTile - 1) / kTile);
+    }
+    auto load = [&](int tile, int stage) {
+        const uint32_t bar = bar_full + 8 * stage, dst = smem_base + stage * kTileBytes;
+        mbar_expect_tx(bar, kTileBytes);
+        const CUtensorMap *map = &job.map_src;
+        int n = ntx;
+        if constexpr (kTwo) {
+            if (tile >= total) map = &job2.map_src, n = ntx2, tile -= total;
+        }
+        const int ty = tile / n, tx = tile - ty * n;
+        tma_load_2d(dst, map, tx * kTile, ty * kTile, bar);
+        tma_load_2d(dst + kTileBytes / 2, map, tx * kTile + 64, ty * kTile, bar);
+    };
+
+    if (threadIdx.x == 0) {
+        mbar_init(bar_full, 1);
+        mbar_init(bar_full + 8, 1);
+        *abort_flag = 0u;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    const QsGeom g = qs_geom(threadIdx.x, job.rows, job.cols, job.rw.packed);
+    pdl_wait();
+    if (threadIdx.x == 0) {
+        // withhold_loads (self-test of the drain path): nothing is ever loaded, so the first bounded wait runs out
+        for (int s = 0; s < 2; s++)
+            if (!withhold_loads && (int)blockIdx.x + s * (int)gridDim.x < all) load(blockIdx.x + s * gridDim.x, s);
+    }
+    __syncthreads();
+
+    uint32_t nonfinite = 0;
+    int tile = blockIdx.x, it = 0;
+    const bool alive = qs_walk<EMIT_ROW, SR_ROW, SR_T, DQ, GELU>(job, g, 0, total, all, tile, it, smem, smem_base, bar_full, abort_flag, dev_status, spin_limit,
+                                                                 nonfinite, hook_out, hook_ld, load);
+    if constexpr (kTwo) {
+        if (alive && tile < all) {
+            const QsGeom g2 = qs_geom(threadIdx.x, job2.rows, job2.cols, job2.rw.packed);
+            qs_walk<EMIT_ROW, SR_ROW, SR_T, DQ, GELU>(job2, g2, total, all, all, tile, it, smem, smem_base, bar_full, abort_flag, dev_status, spin_limit, nonfinite,
+                                                      hook_out, hook_ld, load);
+        }
+    }
+    if (threadIdx.x == 0) bulk_wait0();           // every store has completed before the shared memory goes away
     if (nonfinite && dev_status) atomicOr(dev_status, MXFP4_DEV_NONFINITE);
 }
 
@@ -563,18 +601,29 @@ static bool make_packed_t_map(CUtensorMap *map, void *packed, int64_t rows, int6
               CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-template <bool EMIT_ROW, bool SR_ROW, bool SR_T, bool DQ, bool GELU = false>
-static mxfp4_status_t launch_stream(cudaStream_t st, const CUtensorMap &ms, const CUtensorMap &mt, int rows, int cols, const QuantSide &rw,
-                                    const QuantSide &tr, uint32_t *dev_status, uint32_t spin_limit = kWaitSpinLimit, int withhold_loads = 0,
-                                    __nv_bfloat16 *hook_out = nullptr, int64_t hook_ld = 0)
+static int64_t qs_tiles(int64_t rows, int64_t cols) { return ceil_div(rows, kTile) * ceil_div(cols, kTile); }
+
+static bool make_job(QsJob *job, const void *src_bf16, int64_t rows, int64_t cols, int64_t ld, const mxfp4_mat_t *dst, const mxfp4_qparams_t *qp_row,
+                     const mxfp4_mat_t &dst_t, const mxfp4_qparams_t *qp_t)
+{
+    job->tr = make_side(dst_t, qp_t);
+    job->rw = dst ? make_side(*dst, qp_row) : job->tr;
+    job->rows = (int)rows;
+    job->cols = (int)cols;
+    return make_src_map(&job->map_src, src_bf16, rows, cols, ld) && make_packed_t_map(&job->map_t, dst_t.data, rows, cols);
+}
+
+template <bool EMIT_ROW, bool SR_ROW, bool SR_T, bool DQ, bool GELU = false, class Job2 = QsNone>
+static mxfp4_status_t launch_stream(cudaStream_t st, const QsJob &job, uint32_t *dev_status, uint32_t spin_limit = kWaitSpinLimit, int withhold_loads = 0,
+                                    __nv_bfloat16 *hook_out = nullptr, int64_t hook_ld = 0, const Job2 &job2 = Job2(), int64_t tiles2 = 0)
 {
     static bool attr_set[kMaxDevices];
-    MX_CHECK_CUDA(set_smem_once(attr_set, k_quantize_stream<EMIT_ROW, SR_ROW, SR_T, DQ, GELU>, kQsSmemBytes));
-    const int64_t tiles = ceil_div(rows, kTile) * ceil_div(cols, kTile);
+    MX_CHECK_CUDA(set_smem_once(attr_set, k_quantize_stream<EMIT_ROW, SR_ROW, SR_T, DQ, GELU, Job2>, kQsSmemBytes));
+    const int64_t tiles = qs_tiles(job.rows, job.cols) + tiles2;
     const int64_t cap = kQsCtasPerSm * (int64_t)sm_count();
-    const int grid = (int)(tiles < cap ? tiles : cap);
-    MX_CHECK_CUDA(launch_pdl(k_quantize_stream<EMIT_ROW, SR_ROW, SR_T, DQ, GELU>, (unsigned)grid, 1, kQsThreads, kQsSmemBytes, st, ms, mt, rows, cols, rw, tr,
-                             dev_status, spin_limit, withhold_loads, hook_out, hook_ld));
+    const unsigned grid = (unsigned)(tiles < cap ? tiles : cap);
+    MX_CHECK_CUDA(launch_pdl(k_quantize_stream<EMIT_ROW, SR_ROW, SR_T, DQ, GELU, Job2>, grid, 1, kQsThreads, kQsSmemBytes, st, job, job2, dev_status, spin_limit,
+                             withhold_loads, hook_out, hook_ld));
     return MXFP4_OK;
 }
 
@@ -607,34 +656,31 @@ static mxfp4_status_t quantize_tile_ex(const void *src_bf16, const mxfp4_mat_t *
     // every tile writes its whole 512-byte scale chunk(s), padding entries included
     const dim3 grid((unsigned)ceil_div(cols, kTile), (unsigned)ceil_div(rows, kTile));
     if (src_q && grid.y > 65535u) return MXFP4_BAD_SHAPE;
-    const QuantSide tr = make_side(dst_t, qp_t);
-    const QuantSide rw = dst ? make_side(*dst, qp_row) : tr;
     const bool sr_t = qp_t->rounding == MXFP4_ROUND_STOCHASTIC;
     const bool sr_r = dst && qp_row->rounding == MXFP4_ROUND_STOCHASTIC;
-    const int r = (int)rows, c = (int)cols;
     if (src_q) {
         const int nb4 = (int)ceil_div(cols / 32, 4);
-        MX_CHECK_CUDA(launch_pdl(sr_t ? k_requantize_tile<true> : k_requantize_tile<false>, grid.x, grid.y, 256, 0, st, src_q->data, src_q->scales, nb4, r, c, tr,
-                                 dev_status));
+        MX_CHECK_CUDA(launch_pdl(sr_t ? k_requantize_tile<true> : k_requantize_tile<false>, grid.x, grid.y, 256, 0, st, src_q->data, src_q->scales, nb4, (int)rows,
+                                 (int)cols, make_side(dst_t, qp_t), dev_status));
     } else {
         // bf16 source: the streaming kernel
-        if (ceil_div(rows, kTile) * ceil_div(cols, kTile) > 0x7FFFFFFF) return MXFP4_BAD_SHAPE;
-        CUtensorMap ms, mt;
-        if (!make_src_map(&ms, src_bf16, rows, cols, ld) || !make_packed_t_map(&mt, dst_t.data, rows, cols)) return MXFP4_CUDA_ERROR;
+        if (qs_tiles(rows, cols) > 0x7FFFFFFF) return MXFP4_BAD_SHAPE;
+        QsJob job;
+        if (!make_job(&job, src_bf16, rows, cols, ld, dst, qp_row, dst_t, qp_t)) return MXFP4_CUDA_ERROR;
         if (!dst) {
-            return sr_t ? launch_stream<false, false, true, false>(st, ms, mt, r, c, rw, tr, dev_status, spin_limit, withhold_loads)
-                        : launch_stream<false, false, false, false>(st, ms, mt, r, c, rw, tr, dev_status, spin_limit, withhold_loads);
+            return sr_t ? launch_stream<false, false, true, false>(st, job, dev_status, spin_limit, withhold_loads)
+                        : launch_stream<false, false, false, false>(st, job, dev_status, spin_limit, withhold_loads);
         }
         const int sel = (chain ? 4 : 0) | (sr_r ? 2 : 0) | (sr_t ? 1 : 0);
         switch (sel) {
-        case 0: return launch_stream<true, false, false, false>(st, ms, mt, r, c, rw, tr, dev_status, spin_limit, withhold_loads);
-        case 1: return launch_stream<true, false, true, false>(st, ms, mt, r, c, rw, tr, dev_status, spin_limit, withhold_loads);
-        case 2: return launch_stream<true, true, false, false>(st, ms, mt, r, c, rw, tr, dev_status, spin_limit, withhold_loads);
-        case 3: return launch_stream<true, true, true, false>(st, ms, mt, r, c, rw, tr, dev_status, spin_limit, withhold_loads);
-        case 4: return launch_stream<true, false, false, true>(st, ms, mt, r, c, rw, tr, dev_status, spin_limit, withhold_loads);
-        case 5: return launch_stream<true, false, true, true>(st, ms, mt, r, c, rw, tr, dev_status, spin_limit, withhold_loads);
-        case 6: return launch_stream<true, true, false, true>(st, ms, mt, r, c, rw, tr, dev_status, spin_limit, withhold_loads);
-        default: return launch_stream<true, true, true, true>(st, ms, mt, r, c, rw, tr, dev_status, spin_limit, withhold_loads);
+        case 0: return launch_stream<true, false, false, false>(st, job, dev_status, spin_limit, withhold_loads);
+        case 1: return launch_stream<true, false, true, false>(st, job, dev_status, spin_limit, withhold_loads);
+        case 2: return launch_stream<true, true, false, false>(st, job, dev_status, spin_limit, withhold_loads);
+        case 3: return launch_stream<true, true, true, false>(st, job, dev_status, spin_limit, withhold_loads);
+        case 4: return launch_stream<true, false, false, true>(st, job, dev_status, spin_limit, withhold_loads);
+        case 5: return launch_stream<true, false, true, true>(st, job, dev_status, spin_limit, withhold_loads);
+        case 6: return launch_stream<true, true, false, true>(st, job, dev_status, spin_limit, withhold_loads);
+        default: return launch_stream<true, true, true, true>(st, job, dev_status, spin_limit, withhold_loads);
         }
     }
     return MXFP4_OK;
@@ -652,17 +698,28 @@ mxfp4_status_t quantize_tile(const void *src_bf16, const mxfp4_mat_t *src_q, int
 mxfp4_status_t quantize_gelu_chain(const void *y_bf16, int64_t rows, int64_t cols, int64_t ldy, void *z_bf16, int64_t ldz, mxfp4_mat_t dst,
                                    const mxfp4_qparams_t *qp_row, mxfp4_mat_t dst_t, const mxfp4_qparams_t *qp_t, uint32_t *dev_status, cudaStream_t st)
 {
-    CUtensorMap ms, mt;
-    if (!make_src_map(&ms, y_bf16, rows, cols, ldy) || !make_packed_t_map(&mt, dst_t.data, rows, cols)) return MXFP4_CUDA_ERROR;
-    const QuantSide rw = make_side(dst, qp_row), tr = make_side(dst_t, qp_t);
+    QsJob job;
+    if (!make_job(&job, y_bf16, rows, cols, ldy, &dst, qp_row, dst_t, qp_t)) return MXFP4_CUDA_ERROR;
     __nv_bfloat16 *z = static_cast<__nv_bfloat16 *>(z_bf16);
-    const int r = (int)rows, c = (int)cols;
     const bool sr_r = qp_row->rounding == MXFP4_ROUND_STOCHASTIC, sr_t = qp_t->rounding == MXFP4_ROUND_STOCHASTIC;
     if (sr_r)
-        return sr_t ? launch_stream<true, true, true, true, true>(st, ms, mt, r, c, rw, tr, dev_status, kWaitSpinLimit, 0, z, ldz)
-                    : launch_stream<true, true, false, true, true>(st, ms, mt, r, c, rw, tr, dev_status, kWaitSpinLimit, 0, z, ldz);
-    return sr_t ? launch_stream<true, false, true, true, true>(st, ms, mt, r, c, rw, tr, dev_status, kWaitSpinLimit, 0, z, ldz)
-                : launch_stream<true, false, false, true, true>(st, ms, mt, r, c, rw, tr, dev_status, kWaitSpinLimit, 0, z, ldz);
+        return sr_t ? launch_stream<true, true, true, true, true>(st, job, dev_status, kWaitSpinLimit, 0, z, ldz)
+                    : launch_stream<true, true, false, true, true>(st, job, dev_status, kWaitSpinLimit, 0, z, ldz);
+    return sr_t ? launch_stream<true, false, true, true, true>(st, job, dev_status, kWaitSpinLimit, 0, z, ldz)
+                : launch_stream<true, false, false, true, true>(st, job, dev_status, kWaitSpinLimit, 0, z, ldz);
+}
+
+// The forward pass's two chains in one launch: Q1 + Q6 of x [m, k] and Q2 + Q4 of w [n, k] (round to nearest along the rows,
+// then stochastic double quantization).  The caller has checked every argument; m, n and k are multiples of 32.
+mxfp4_status_t quantize_chain_two(const void *x_bf16, int64_t m, int64_t k, int64_t ldx, const mxfp4_mat_t &xq, const mxfp4_mat_t &xq_t, const mxfp4_qparams_t *q6,
+                                  const void *w_bf16, int64_t n, const mxfp4_mat_t &wq, const mxfp4_mat_t &wq_t, const mxfp4_qparams_t *q4,
+                                  const mxfp4_qparams_t *rne, uint32_t *dev_status, cudaStream_t st)
+{
+    if (m == 0 || n == 0 || k == 0) return MXFP4_BAD_SHAPE;
+    if (qs_tiles(m, k) + qs_tiles(n, k) > 0x7FFFFFFF || m > 0x7FFFFF80 || n > 0x7FFFFF80 || k > 0x7FFFFF80) return MXFP4_BAD_SHAPE;
+    QsJob x, w;
+    if (!make_job(&x, x_bf16, m, k, ldx, &xq, rne, xq_t, q6) || !make_job(&w, w_bf16, n, k, k, &wq, rne, wq_t, q4)) return MXFP4_CUDA_ERROR;
+    return launch_stream<true, false, true, true, false, QsJob>(st, x, dev_status, kWaitSpinLimit, 0, nullptr, 0, w, qs_tiles(n, k));
 }
 
 std::atomic<unsigned long long> g_launches{0};

@@ -269,3 +269,21 @@ def test_chained_launches_see_each_other(mx, rows):
     for i, r in got:
         for a, c in zip(r, want[i % 4]):
             assert torch.equal(a, c), "step %d" % i
+
+
+@pytest.mark.parametrize("M,K,N", [(32, 32, 32), (160, 96, 288), (64, 4096, 4096), (40032, 96, 64), (19008, 256, 160)])
+def test_forward_quantizes_activations_and_weight_in_one_launch(mx, M, K, N):
+    """Q1 + Q6 of X and Q2 + Q4 of W share a launch: the tiles of W follow those of X (fewer tiles than blocks, W alone filling
+    the blocks, the change of matrix in the middle of a block's walk, non-finite groups in one of the two)."""
+    g = torch.Generator(device="cuda").manual_seed(M + K + N)
+    x = torch.randn((M, K), generator=g, device="cuda").to(torch.bfloat16)
+    w = (torch.randn((N, K), generator=g, device="cuda") * 0.02).to(torch.bfloat16)
+    w[N // 2, K // 2] = float("inf")
+    before = mx.launch_count()
+    st = mx.new_status()
+    _, ctx = mx.linear_fwd(x, w, bwd_seed=77, dev_status=st)
+    assert mx.launch_count() - before == 2
+    torch.cuda.synchronize()
+    assert int(st.item()) == mx.DEV_NONFINITE
+    for got, want in zip((ctx.xq, ctx.xq_t, ctx.wq, ctx.wq_t), mx.quantize_chain(x, seed=77) + mx.quantize_chain(w, seed=77, stream_id_t=4)):
+        assert torch.equal(got.data, want.data) and torch.equal(got.scales, want.scales)
