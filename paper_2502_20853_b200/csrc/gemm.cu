@@ -1445,26 +1445,31 @@ __global__ void __launch_bounds__(128, 1) k_mma_ceiling(int iters, uint32_t *dev
 // Roles per CTA are those of the single-CTA kernel, except that only the leader (rank 0) issues scale copies and MMAs
 // (both act on the shared memory and TMEM of both CTAs), and warp 2 of the peer relays "my stage has landed" to the
 // leader.  Stage and accumulator releases reach both CTAs through multicast commits.
-template <bool DEEP>
+// BN = 192: 256 x 192 tiles for output widths that are multiples of 192 but not of 256.  Narrower stages (31 KB), two
+// accumulators (the next tile's K loop runs under the epilogue), which leaves TMEM columns for the scales of five stages.
+template <bool DEEP, int BN>
 struct Gemm2Cfg {
     static constexpr int kABytes = kBM * kBKBytes;                      // 16 KB: this CTA's 128 rows of A
-    static constexpr int kBBytes = 128 * kBKBytes;                      // 16 KB: this CTA's half of the 256 B rows
+    static constexpr int kBBytes = (BN / 2) * kBKBytes;                 // this CTA's half of the B rows
     static constexpr int kSfaBytes = 2 * kSfChunk;
-    static constexpr int kSfbBytes = 2 * kSfChunk * 2;                  // all 256 B rows
-    static constexpr int kStageBytes = kABytes + kBBytes + kSfaBytes + kSfbBytes;   // 35 KB
+    static constexpr int kSfbBytes = 2 * kSfChunk * 2;                  // all B rows: the two 128-row blocks a tile touches
+    static constexpr int kStageBytes = kABytes + kBBytes + kSfaBytes + kSfbBytes;   // 35 KB / 31 KB
     // The loop is bound by operand bytes in flight over load latency, so every stage counts: six stages and a single
     // staging buffer per epilogue warp for long K loops (177 against 187 us at 8192^3), and no slack for aligning the
     // window: the kernel declares its window 1024-byte aligned and checks that it is.
-    static constexpr int kStages = DEEP ? 4 : 6;
-    static constexpr int kStagingBufs = DEEP ? 4 : 1;
-    static constexpr int kSfCol = 256;                                  // TMEM: accumulator, then per ring stage SFA (8) + SFB (16)
+    static constexpr int kStages = BN == 192 ? 5 : DEEP ? 4 : 6;
+    static constexpr int kStagingBufs = BN == 192 ? 3 : DEEP ? 4 : 1;
+    static constexpr int kAccStages = BN == 192 ? 2 : 1;
+    static constexpr int kSfCol = kAccStages * BN;                      // TMEM: accumulators, then per ring stage SFA (8) + SFB (16)
     static constexpr int kSfSlot = 24;
     static constexpr int kTmemCols = 512;
     static constexpr int kStagingOff = kStages * kStageBytes;
     static constexpr int kBarOff = kStagingOff + kEpiWarps * kStagingBufs * kStagingBytes;
-    static constexpr int kSmemBytes = kBarOff + 256 /*barriers*/;
+    static constexpr int kBiasOff = kBarOff + 256;                      // BN = 192: a line of BN / 2 bf16 per epilogue warp
+    static constexpr int kSmemBytes = kBiasOff + (BN == 192 ? kEpiWarps * BN : 0);
     static_assert(kSfCol + kStages * kSfSlot <= 512, "TMEM budget");
     static_assert(kStageBytes % 1024 == 0 && kStagingOff % 1024 == 0, "alignment");
+    static_assert((3 * kStages + 2 * kAccStages + 1) * 8 <= 256, "barrier slots");
     static_assert(kSmemBytes <= 232448, "shared memory budget");
 };
 
@@ -1547,14 +1552,13 @@ __device__ __forceinline__ uint32_t idesc_mxf4_pair(uint32_t a_sf_id, uint32_t b
     return (b_sf_id << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(n >> 3) << 17) | (1u << 23) | ((uint32_t)(256 >> 4) << 24) | (a_sf_id << 29);
 }
 
-template <bool DEEP>
+template <bool DEEP, int BN>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kGemmThreads, 1)
 k_gemm_mxf4_pair(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b,
                  const __grid_constant__ CUtensorMap map_sfa, const __grid_constant__ CUtensorMap map_sfb,
-                 const __grid_constant__ CUtensorMap map_d, const GemmParams p)
+                 const __grid_constant__ CUtensorMap map_d, const __grid_constant__ CUtensorMap map_dw, const GemmParams p)
 {
-    using C = Gemm2Cfg<DEEP>;
-    constexpr int BN = 256;
+    using C = Gemm2Cfg<DEEP, BN>;
     extern __shared__ __align__(1024) uint8_t smem_aligned[];
     uint8_t *smem = smem_aligned;
     if (smem_u32(smem) & 1023u) {   // the swizzled operand tiles need it; nothing has been set up yet, so everybody just leaves
@@ -1569,8 +1573,8 @@ k_gemm_mxf4_pair(const __grid_constant__ CUtensorMap map_a, const __grid_constan
     const uint32_t bar_sf_full = bar_full + 8 * C::kStages;
     const uint32_t bar_empty = bar_sf_full + 8 * C::kStages;
     const uint32_t bar_acc_full = bar_empty + 8 * C::kStages;
-    const uint32_t bar_acc_empty = bar_acc_full + 8;
-    uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(bars + 4 * C::kStages + 2);
+    const uint32_t bar_acc_empty = bar_acc_full + 8 * C::kAccStages;
+    uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(bars + 3 * C::kStages + 2 * C::kAccStages);
     volatile uint32_t *abort_flag = tmem_slot + 1;
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -1583,8 +1587,10 @@ k_gemm_mxf4_pair(const __grid_constant__ CUtensorMap map_a, const __grid_constan
             mbar_init(bar_sf_full + 8 * s, 1);
             mbar_init(bar_empty + 8 * s, 1);
         }
-        mbar_init(bar_acc_full, 1);
-        mbar_init(bar_acc_empty, 2 * kEpiWarps);   // the epilogue warps of both CTAs hand the accumulator back to the leader
+        for (int a = 0; a < C::kAccStages; a++) {
+            mbar_init(bar_acc_full + 8 * a, 1);
+            mbar_init(bar_acc_empty + 8 * a, 2 * kEpiWarps);   // the epilogue warps of both CTAs hand an accumulator back to the leader
+        }
         *abort_flag = 0u;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
@@ -1628,12 +1634,12 @@ k_gemm_mxf4_pair(const __grid_constant__ CUtensorMap map_a, const __grid_constan
                 if (leader && operands) {
                     if (rank == 0) mbar_expect_tx(bar_full + 8 * stage, 2u * (uint32_t)C::kStageBytes);
                     tma2_load_2d(sA, &map_a, ktr * kBKBytes, mb * kBM, full);
-                    tma2_load_2d(sB, &map_b, ktr * kBKBytes, nb * BN + (int)rank * 128, full);
+                    tma2_load_2d(sB, &map_b, ktr * kBKBytes, nb * BN + (int)rank * (BN / 2), full);
                 }
                 if (leader && !operands) {
                     // scale rows are 128-row blocks, 256 words (two 512-byte chunks) per stage; blocks beyond the matrix read as zero
                     tma2_load_2d(sSFA, &map_sfa, ktr * 256, mb, full);
-                    tma2_load_2d(sSFB, &map_sfb, ktr * 256, nb * 2, full);
+                    tma2_load_2d(sSFB, &map_sfb, ktr * 256, (nb * BN) >> 7, full);
                 }
                 __syncwarp();
                 if (++stage == C::kStages) { stage = 0; phase ^= 1u; }
@@ -1677,20 +1683,23 @@ k_gemm_mxf4_pair(const __grid_constant__ CUtensorMap map_a, const __grid_constan
         // ================= MMA issuer (leader CTA only) =================
         if (rank == 0) {
             const bool leader = elect_one();
-            uint32_t stage = 0, phase = 0, acc_phase = 0;
+            uint32_t stage = 0, phase = 0, acc = 0, acc_phase = 0;
             bool alive = true;
             for (int item = cluster_id; item < items && alive; item += num_clusters) {
                 const int split = item % p.splits;
                 const int kt0 = split * p.kt_per_split;
                 const int kt1 = min(kt0 + p.kt_per_split, p.kt_total);
-                if (!mbar_wait_cluster_warp(bar_acc_empty, acc_phase ^ 1u, abort_flag, p.dev_status, p.spin_limit)) { alive = false; break; }
+                // scale columns hold 32 rows each: a tile that starts 64 rows into a 128-row block starts 2 columns in
+                const uint32_t sfb_shift = BN == 192 ? (uint32_t)((((item / p.splits) % p.tiles_n) * BN & 127) >> 5) : 0u;
+                const uint32_t d_tmem = tmem_base + acc * BN;
+                if (!mbar_wait_cluster_warp(bar_acc_empty + 8 * acc, acc_phase ^ 1u, abort_flag, p.dev_status, p.spin_limit)) { alive = false; break; }
                 tc_fence_after();
                 for (int kt = kt0; kt < kt1; kt++) {
                     if (!mbar_wait_warp(bar_sf_full + 8 * stage, phase, abort_flag, p.dev_status, p.spin_limit)) { alive = false; break; }
                     tc_fence_after();
                     const uint32_t sA = smem_base + stage * C::kStageBytes;
                     const uint32_t sB = sA + C::kABytes;
-                    const uint32_t t_sfa = tmem_base + C::kSfCol + stage * C::kSfSlot, t_sfb = t_sfa + 8;
+                    const uint32_t t_sfa = tmem_base + C::kSfCol + stage * C::kSfSlot, t_sfb = t_sfa + 8 + sfb_shift;
                     const int64_t kleft = p.Kc - (int64_t)(kt1 - 1 - (kt - kt0)) * kBKElems;
                     const int krem = kleft < kBKElems ? (int)kleft : kBKElems;
                     const int nmma = (krem + 63) / 64;
@@ -1700,8 +1709,8 @@ k_gemm_mxf4_pair(const __grid_constant__ CUtensorMap map_a, const __grid_constan
                         for (int k = 0; k < 4; k++) {
                             if (k < nmma) {
                                 const uint32_t sf_id = (uint32_t)(k & 1) * 2u;
-                                tc2_mma_mxf4(tmem_base, adesc + (uint64_t)(k * (kMmaKBytes >> 4)), bdesc + (uint64_t)(k * (kMmaKBytes >> 4)),
-                                             idesc_mxf4_pair(sf_id, sf_id), t_sfa + 4 * (k >> 1), t_sfb + 8 * (k >> 1),
+                                tc2_mma_mxf4(d_tmem, adesc + (uint64_t)(k * (kMmaKBytes >> 4)), bdesc + (uint64_t)(k * (kMmaKBytes >> 4)),
+                                             idesc_mxf4_pair(sf_id, sf_id, BN), t_sfa + 4 * (k >> 1), t_sfb + 8 * (k >> 1),
                                              (kt > kt0 || k > 0) ? 1u : 0u);
                             }
                         }
@@ -1710,13 +1719,13 @@ k_gemm_mxf4_pair(const __grid_constant__ CUtensorMap map_a, const __grid_constan
                     __syncwarp();
                     if (++stage == C::kStages) { stage = 0; phase ^= 1u; }
                 }
-                if (alive && leader) tc2_commit_both(bar_acc_full);   // both CTAs' accumulators are complete
+                if (alive && leader) tc2_commit_both(bar_acc_full + 8 * acc);   // both CTAs' accumulators are complete
                 __syncwarp();
-                acc_phase ^= 1u;
+                if (++acc == C::kAccStages) { acc = 0; acc_phase ^= 1u; }
             }
         }
     } else if (warp >= kEpiWarp0) {
-        // ================= epilogue (warps 4..11 of both CTAs: own 128 rows x 256 columns) =================
+        // ================= epilogue (warps 4..11 of both CTAs: own 128 rows x BN columns) =================
         const int ew = warp - kEpiWarp0;
         const int quarter = warp & 3;
         const int chalf = ew >> 2;
@@ -1724,6 +1733,23 @@ k_gemm_mxf4_pair(const __grid_constant__ CUtensorMap map_a, const __grid_constan
         uint32_t sbuf = 0;
         constexpr int kHalfCols = BN / 2;
         constexpr int kChunks = kHalfCols / 32;
+        if constexpr (BN == 192) {
+            const uint32_t bias_line = smem_base + C::kBiasOff + ew * (BN / 2) * 2;
+            uint32_t acc = 0, acc_phase = 0;
+            for (int item = cluster_id; item < items; item += num_clusters) {
+                const int split = item % p.splits, tile = item / p.splits;
+                const int mb = (tiles_m2 - 1 - tile / p.tiles_n) * 2 + (int)rank, nb = tile % p.tiles_n;
+                uint32_t bias[(kHalfCols + 63) / 64];
+                bias_fetch<kHalfCols>(bias, p.bias, (int64_t)nb * BN + chalf * kHalfCols, p.N, lane);
+                if (!mbar_wait_warp(bar_acc_full + 8 * acc, acc_phase, abort_flag, p.dev_status, p.spin_limit)) break;
+                tc_fence_after();
+                if (p.bias != nullptr) bias_stage<kHalfCols>(bias, bias_line, lane);
+                epilogue_tile<BN, C::kStagingBufs, true>(&map_d, p.out_fp32 ? nullptr : &map_dw, p,
+                                                         tmem_base + ((uint32_t)(quarter * 32) << 16) + acc * BN + chalf * kHalfCols, mb * kBM + quarter * 32,
+                                                         nb * BN + chalf * kHalfCols, split, staging, sbuf, lane, map_to_cta(bar_acc_empty + 8 * acc, 0), bias_line);
+                if (++acc == C::kAccStages) { acc = 0; acc_phase ^= 1u; }
+            }
+        } else {
         const uint32_t acc_empty_leader = map_to_cta(bar_acc_empty, 0);
         uint32_t acc_phase = 0;
         bool alive = true;
@@ -1812,6 +1838,7 @@ k_gemm_mxf4_pair(const __grid_constant__ CUtensorMap map_a, const __grid_constan
                 }
             }
             acc_phase ^= 1u;
+        }
         }
         if (lane == 0) bulk_wait0();
     }
@@ -2325,6 +2352,16 @@ static GemmPlan plan_gemm(int64_t m, int64_t n, int64_t kc, int sms, bool allow_
     else if (kc <= 1024 || n < 256 || (kc <= 2304 && n % 256 != 0 && n % 192 == 0)) g.bn = 192;
     else g.bn = 256;
     g.pair = g.bn == 256 && m > 128 && sms >= 2;
+    // 256 x 192 tiles on pairs, for widths that 256-wide tiles waste a quarter of or more, when K is split (1536 x 384 x 25216
+    // 16.7 -> 15.8 us, 384 x 384 x 25216 12.1 -> 11.0, 512 x 384 x 4096 9.5 -> 8.8), and in place of the single-CTA 192-wide
+    // kernel from four tiles per pair on (50432 x 1152 x 1280 53.7 -> 46.1; with 2.7 tiles per pair, 25216 x 384 x 1536, both
+    // take 15.6).  For long K loops that fill the machine the 256-wide pair with its sixth stage is faster even with the
+    // waste (50432 x 960 x 4096: 82 against 96 us).
+    if (m > 128 && n % 192 == 0 && n % 256 != 0 && kc > 1024 && sms >= 2) {
+        const int64_t pairs = sms / 2, tm2 = ceil_div(ceil_div(m, kBM), 2);
+        const bool split = allow_split && g.kt_total >= 8 && tm2 * ceil_div(n, 256) * 2 <= pairs;
+        if ((split && n <= 576) || (g.bn == 192 && tm2 * (n / 192) >= 4 * pairs)) g.pair = true, g.bn = 192;
+    }
     g.tiles_m = (int)ceil_div(m, kBM);
     g.tiles_n = (int)ceil_div(n, g.bn);
     const int units = (g.pair ? (g.tiles_m + 1) / 2 : g.tiles_m) * g.tiles_n;   // work items before splitting K
@@ -2353,14 +2390,14 @@ static bool ensure_device_ok()
     return ok[dev] == 1;
 }
 
-template <bool DEEP>
+template <bool DEEP, int BN>
 static mxfp4_status_t launch_gemm_pair(const CUtensorMap &ma, const CUtensorMap &mb, const CUtensorMap &msa, const CUtensorMap &msb,
-                                       const CUtensorMap &md, const GemmParams &p, int grid, cudaStream_t st)
+                                       const CUtensorMap &md, const CUtensorMap &mdw, const GemmParams &p, int grid, cudaStream_t st)
 {
-    using C = Gemm2Cfg<DEEP>;
+    using C = Gemm2Cfg<DEEP, BN>;
     static bool attr_set[kMaxDevices];
-    MX_CHECK_CUDA(set_smem_once(attr_set, k_gemm_mxf4_pair<DEEP>, C::kSmemBytes));
-    MX_CHECK_CUDA(launch_pdl(k_gemm_mxf4_pair<DEEP>, (unsigned)grid, 1, kGemmThreads, C::kSmemBytes, st, ma, mb, msa, msb, md, p));
+    MX_CHECK_CUDA(set_smem_once(attr_set, k_gemm_mxf4_pair<DEEP, BN>, C::kSmemBytes));
+    MX_CHECK_CUDA(launch_pdl(k_gemm_mxf4_pair<DEEP, BN>, (unsigned)grid, 1, kGemmThreads, C::kSmemBytes, st, ma, mb, msa, msb, md, mdw, p));
     return MXFP4_OK;
 }
 
@@ -2463,7 +2500,7 @@ static mxfp4_status_t gemm_impl(mxfp4_mat_t a, mxfp4_mat_t b, void *d, int64_t l
 
     const bool store_fp32 = g.splits > 1 || out_dtype == MXFP4_OUT_FP32;
     CUtensorMap ma, mb, md;
-    if (!make_operand_map(&ma, a.data, M, Kc, kBM) || !make_operand_map(&mb, b.data, N, Kc, g.pbs ? 96 : g.pair ? 128 : g.bn)) return MXFP4_CUDA_ERROR;
+    if (!make_operand_map(&ma, a.data, M, Kc, kBM) || !make_operand_map(&mb, b.data, N, Kc, g.pbs ? 96 : g.pair ? g.bn / 2 : g.bn)) return MXFP4_CUDA_ERROR;
     if (!make_output_map(&md, g.splits > 1 ? workspace : d, M, N, g.splits > 1 ? N : ldd, g.splits, store_fp32)) return MXFP4_CUDA_ERROR;
 
     GemmParams p;
@@ -2494,7 +2531,8 @@ static mxfp4_status_t gemm_impl(mxfp4_mat_t a, mxfp4_mat_t b, void *d, int64_t l
     if (!store_fp32 && !make_output_map_wide(&mdw, d, M, N, ldd)) return MXFP4_CUDA_ERROR;
     mxfp4_status_t s = g.pbs         ? launch_gemm_pbs<4, 8>(ma, mb, msa, msb, md, mdw, p, grid, st)
                        : g.bs == 1   ? launch_gemm_bs<192, 2, 7>(ma, mb, md, mdw, p, grid, st)
-                       : g.pair      ? (g.deep ? launch_gemm_pair<true>(ma, mb, msa, msb, md, p, grid, st) : launch_gemm_pair<false>(ma, mb, msa, msb, md, p, grid, st))
+                       : g.pair && g.bn == 192 ? launch_gemm_pair<false, 192>(ma, mb, msa, msb, md, mdw, p, grid, st)
+                       : g.pair      ? (g.deep ? launch_gemm_pair<true, 256>(ma, mb, msa, msb, md, mdw, p, grid, st) : launch_gemm_pair<false, 256>(ma, mb, msa, msb, md, mdw, p, grid, st))
                        : g.bn == 256 ? (g.deep ? launch_gemm<256, true>(ma, mb, md, mdw, p, grid, st) : launch_gemm<256, false>(ma, mb, md, mdw, p, grid, st))
                        : g.bn == 192 ? launch_gemm<192, false>(ma, mb, md, mdw, p, grid, st)
                                      : (g.deep ? launch_gemm<128, true>(ma, mb, md, mdw, p, grid, st) : launch_gemm<128, false>(ma, mb, md, mdw, p, grid, st));

@@ -174,6 +174,14 @@ def test_gemm_bias_ragged_edges(mx, M, N, K, out_dtype):
     _bias_case(mx, M, N, K, out_dtype)
 
 
+@pytest.mark.parametrize("M,N,K", [(384, 384, 8192), (300, 192, 2080), (136, 576, 4128), (38000, 576, 1056)])
+@pytest.mark.parametrize("out_dtype", [0, 1])
+def test_gemm_pairs_of_192_columns(mx, M, N, K, out_dtype):
+    """256 x 192 tiles on CTA pairs: split K with a ragged last K tile and a last pair of one row tile, and many tiles per pair
+    with both accumulators in turn."""
+    _bias_case(mx, M, N, K, out_dtype)
+
+
 @pytest.mark.parametrize("M,N,K", [(128, 96, 128 * 1024), (24, 8, 8192), (256, 248, 16384), (256, 264, 16384)])
 @pytest.mark.parametrize("out_dtype", [0, 1])
 def test_gemm_many_splits_of_a_small_output(mx, M, N, K, out_dtype):
