@@ -53,6 +53,22 @@ struct GemmCfg {
     static_assert(kSmemBytes <= 232448, "shared memory budget");
 };
 
+// Division by a number known at launch: the quotient of n < 2^31 by a multiplication (the roles of a kernel find their tile's
+// coordinates once per tile in the middle of their chains; the compiler's division is a chain of about 150 cycles, and a role
+// needed up to four).
+struct FastDiv {
+    uint32_t d, m, s;
+    __device__ __forceinline__ int div(int n) const { return (int)((__umulhi((uint32_t)n, m) + (uint32_t)n) >> s); }
+    __device__ __forceinline__ int mod(int n) const { return n - div(n) * (int)d; }
+};
+static FastDiv fast_div(int64_t d)
+{
+    FastDiv f = {(uint32_t)d, 0u, 0u};
+    while ((1ll << f.s) < d) f.s++;
+    f.m = (uint32_t)((((1ull << f.s) - (uint64_t)d) << 32) / (uint64_t)d + 1u);
+    return f;
+}
+
 struct GemmParams {
     const uint8_t *sfa;   // scales of A, tiled order
     const uint8_t *sfb;
@@ -60,6 +76,9 @@ struct GemmParams {
     int nblk4;            // ceil(Kc/32/4): 512-byte chunks per 128-row block
     int rbA, rbB;         // 128-row scale blocks present in A / B buffers
     int tiles_m, tiles_n, splits, kt_total, kt_per_split;
+    FastDiv by_splits, by_tiles_n, by_tiles_m, by_tiles_m2, by_period;   // tiles_m2: row tiles of a CTA pair; period: see PbsWalk
+    FastDiv by_workers;   // kernels that give a block (pair) a contiguous range of tiles: `share` each and `extra` more, spread evenly
+    int share, extra;
     int out_fp32;         // element type of the stored tile (FP32 also for split-K partials)
     const __nv_bfloat16 *bias;   // applied only when splits == 1 (and by the cluster kernel, whose sum is complete)
     uint32_t *dev_status;
@@ -68,6 +87,10 @@ struct GemmParams {
     uint32_t spin_limit;  // polls after which a bounded wait gives up (kWaitSpinLimit in normal use)
     int withhold_loads;   // self-test of the drain path: the producers issue nothing, so every wait runs out
 };
+
+// First tile of worker w's contiguous range, floor(total w / workers).  The workers with one tile more are spread evenly: with
+// the first `extra` ones the ranges start at a constant stride in memory and 401408 x 384 x 96 took 82 us instead of 76.
+__device__ __forceinline__ int range_start(const GemmParams &p, int w) { return w * p.share + p.by_workers.div(w * p.extra); }
 
 // ---- PTX wrappers of the tensor-core instructions (mbarrier, TMA and elect wrappers: tma.cuh) ----
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
@@ -352,9 +375,10 @@ __device__ __forceinline__ void gemm_feed_roles(int warp, uint32_t smem_base, ui
             const bool operands = warp == 0;
             uint32_t stage = 0, phase = 0;
             bool alive = true;
+            pdl_wait();        // the roles that touch global memory wait for the preceding kernel: the producers and the epilogue
             for (int item = blockIdx.x; item < items && alive; item += gridDim.x) {
-                const int split = item % p.splits, tile = item / p.splits;
-                const int mb = tile / p.tiles_n, nb = tile % p.tiles_n;
+                const int tile = p.by_splits.div(item), split = item - tile * p.splits;
+                const int mb = p.by_tiles_n.div(tile), nb = tile - mb * p.tiles_n;
                 const int kt0 = split * p.kt_per_split;
                 const int kt1 = min(kt0 + p.kt_per_split, p.kt_total);
                 // 128-row scale blocks of B that this tile touches (a 192-wide tile starts in the middle of one every other time)
@@ -397,7 +421,7 @@ __device__ __forceinline__ void gemm_feed_roles(int warp, uint32_t smem_base, ui
             uint32_t stage = 0, phase = 0;
             bool alive = true;
             for (int item = blockIdx.x; item < items && alive; item += gridDim.x) {
-                const int split = item % p.splits;
+                const int split = p.by_splits.mod(item);
                 const int kt0 = split * p.kt_per_split;
                 const int kt1 = min(kt0 + p.kt_per_split, p.kt_total);
                 for (int kt = kt0; kt < kt1; kt++) {
@@ -438,8 +462,8 @@ __device__ __forceinline__ void gemm_feed_roles(int warp, uint32_t smem_base, ui
             bool ready = false;   // the current stage's scales (hence operands) are known to be in place
             bool alive = true;
             for (int item = blockIdx.x; item < items && alive; item += gridDim.x) {
-                const int split = item % p.splits, tile = item / p.splits;
-                const int nb = tile % p.tiles_n;
+                const int tile = p.by_splits.div(item), split = item - tile * p.splits;
+                const int nb = p.by_tiles_n.mod(tile);
                 const int kt0 = split * p.kt_per_split;
                 const int kt1 = min(kt0 + p.kt_per_split, p.kt_total);
                 // scale columns hold 32 rows each: a tile that starts 64 rows into a 128-row block starts 2 columns in
@@ -500,6 +524,7 @@ k_gemm_mxf4(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const uint32_t smem_base = smem_u32(smem);
 
+    if (threadIdx.x == 32 * 3) { prefetch_map(&map_a); prefetch_map(&map_b); prefetch_map(&map_d); prefetch_map(&map_dw); }
     if (threadIdx.x == 0) {
         for (int s = 0; s < C::kStages; s++) {
             mbar_init(bar_full + 8 * s, 1);
@@ -521,7 +546,6 @@ k_gemm_mxf4(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem_base = *tmem_slot;
-    pdl_wait();
 
     const int items = p.tiles_m * p.tiles_n * p.splits;
 
@@ -529,6 +553,7 @@ k_gemm_mxf4(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
         gemm_feed_roles<C, BN>(warp, smem_base, bar_full, bar_sf_full, bar_empty, bar_acc_full, bar_acc_empty, tmem_base, abort_flag, map_a, map_b, p);
     } else if (warp >= kEpiWarp0) {
         // ================= epilogue (warps 4..11) =================
+        pdl_wait();
         const int ew = warp - kEpiWarp0;
         const int quarter = warp & 3;            // TMEM lanes 32*quarter .. +31 are the ones this warp may read
         const int chalf = ew >> 2;               // which half of the tile's columns this warp stores
@@ -540,8 +565,8 @@ k_gemm_mxf4(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
         uint32_t acc = 0, acc_phase = 0;
         bool alive = true;
         for (int item = blockIdx.x; item < items && alive; item += gridDim.x) {
-            const int split = item % p.splits, tile = item / p.splits;
-            const int mb = tile / p.tiles_n, nb = tile % p.tiles_n;
+            const int tile = p.by_splits.div(item), split = item - tile * p.splits;
+            const int mb = p.by_tiles_n.div(tile), nb = tile - mb * p.tiles_n;
             uint32_t bias[(kHalfCols + 63) / 64];
             bias_fetch<kHalfCols>(bias, p.bias, (int64_t)nb * BN + chalf * kHalfCols, p.N, lane);
             if (!mbar_wait(bar_acc_full + 8 * acc, acc_phase, abort_flag, p.dev_status, p.spin_limit)) { alive = false; break; }
@@ -554,7 +579,7 @@ k_gemm_mxf4(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
                                                bar_acc_empty + 8 * acc, bias_line);
             if (++acc == C::kAccStages) { acc = 0; acc_phase ^= 1u; }
         }
-        if (lane == 0) bulk_wait0();   // all stores of this warp have completed before the CTA may exit
+        if (lane == 0) bulk_wait_read<0>();   // the stores of this warp have read their staging buffers: the shared memory may go
     }
 
     tc_fence_before();
@@ -645,6 +670,7 @@ k_gemm_mxf4_q(const __grid_constant__ CUtensorMap map_a, const __grid_constant__
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const uint32_t smem_base = smem_u32(smem);
 
+    if (threadIdx.x == 32 * 3) { prefetch_map(&map_a); prefetch_map(&map_b); prefetch_map(&map_z); prefetch_map(&map_t); }
     if (threadIdx.x == 0) {
         for (int s = 0; s < C::kStages; s++) {
             mbar_init(bar_full + 8 * s, 1);
@@ -667,12 +693,12 @@ k_gemm_mxf4_q(const __grid_constant__ CUtensorMap map_a, const __grid_constant__
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem_base = *tmem_slot;
-    pdl_wait();
 
     if (warp < kEpiWarp0) {
         gemm_feed_roles<C, BN>(warp, smem_base, bar_full, bar_sf_full, bar_empty, bar_acc_full, bar_acc_empty, tmem_base, abort_flag, map_a, map_b, p);
     } else {
         // ================= quantizing epilogue (warps 4..11 = 256 threads) =================
+        pdl_wait();
         const int et = (int)threadIdx.x - 32 * kEpiWarp0;
         const int quarter = warp & 3, chalf = (warp - kEpiWarp0) >> 2;
         const int M = (int)p.M, N = (int)p.N;
@@ -685,7 +711,7 @@ k_gemm_mxf4_q(const __grid_constant__ CUtensorMap map_a, const __grid_constant__
         // the hook's second factor travels by TMA into the second tile one tile ahead (that tile is free unless DQ uses it)
         const bool aux_tma = e.hook == MXFP4_HOOK_MULTIPLY && e.aux_tma && !DQ;
         auto issue_aux = [&](int item) {
-            const int mb = item / p.tiles_n, nb = item % p.tiles_n;
+            const int mb = p.by_tiles_n.div(item), nb = item - mb * p.tiles_n;
             mbar_expect_tx(bar_aux, kTileBytes);
             tma_load_2d(t2_base, &map_aux, nb * BN, mb * kBM, bar_aux);
             tma_load_2d(t2_base + kTileBytes / 2, &map_aux, nb * BN + 64, mb * kBM, bar_aux);
@@ -698,7 +724,7 @@ k_gemm_mxf4_q(const __grid_constant__ CUtensorMap map_a, const __grid_constant__
         const int items = p.tiles_m * p.tiles_n;
         int it = 0;
         for (int item = blockIdx.x; item < items; item += gridDim.x, it++) {
-            const int mb = item / p.tiles_n, nb = item % p.tiles_n;
+            const int mb = p.by_tiles_n.div(item), nb = item - mb * p.tiles_n;
             const int row0 = mb * kBM, col0 = nb * BN;
             uint32_t bias[1];
             bias_fetch<64>(bias, p.bias, col0 + chalf * 64, N, lane);
@@ -799,7 +825,7 @@ k_gemm_mxf4_q(const __grid_constant__ CUtensorMap map_a, const __grid_constant__
             }
             if (++acc == C::kAccStages) { acc = 0; acc_phase ^= 1u; }
         }
-        if (et == 0) bulk_wait0();
+        if (et == 0) bulk_wait_read<0>();
         if (nonfinite && p.dev_status) atomicOr(p.dev_status, MXFP4_DEV_NONFINITE);
     }
 
@@ -866,6 +892,7 @@ k_gemm_mxf4_bs(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const uint32_t smem_base = smem_u32(smem);
 
+    if (threadIdx.x == 32 * 3) { prefetch_map(&map_a); prefetch_map(&map_b); prefetch_map(&map_d); prefetch_map(&map_dw); }
     if (threadIdx.x == 0) {
         for (int s = 0; s < AS; s++) {
             mbar_init(bar_a_full + 8 * s, 1);
@@ -890,11 +917,9 @@ k_gemm_mxf4_bs(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem_base = *tmem_slot;
-    pdl_wait();
 
     // tiles are numbered column by column: t = nb * tiles_m + mb; this CTA owns [t0, t1)
-    const int64_t total = (int64_t)p.tiles_m * p.tiles_n;
-    const int t0 = (int)(total * blockIdx.x / gridDim.x), t1 = (int)(total * (blockIdx.x + 1) / gridDim.x);
+    const int t0 = range_start(p, blockIdx.x), t1 = range_start(p, blockIdx.x + 1);
     const int ktn = p.kt_total;
 
     if (warp == 0) {
@@ -902,8 +927,9 @@ k_gemm_mxf4_bs(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
         const bool leader = elect_one() && !p.withhold_loads;
         uint32_t stage = 0, phase = 0;
         bool alive = true;
+        pdl_wait();
         for (int t = t0; t < t1 && alive; t++) {
-            const int mb = t % p.tiles_m;
+            const int mb = p.by_tiles_m.mod(t);
             for (int kt = 0; kt < ktn; kt++) {
                 if (!mbar_wait_warp(bar_a_empty + 8 * stage, phase ^ 1u, abort_flag, p.dev_status, p.spin_limit)) { alive = false; break; }
                 const int nch = min(2, p.nblk4 - 2 * kt);
@@ -922,8 +948,9 @@ k_gemm_mxf4_bs(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
         // ================= B producer: the block of a column, once per run of tiles in that column =================
         const bool leader = elect_one() && !p.withhold_loads;
         uint32_t runs = 0;
+        pdl_wait();
         for (int t = t0; t < t1;) {
-            const int nb = t / p.tiles_m;
+            const int nb = p.by_tiles_m.div(t);
             // the MMAs of the previous column have finished reading the block
             if (runs > 0 && !mbar_wait_warp(bar_b_empty, (runs - 1u) & 1u, abort_flag, p.dev_status, p.spin_limit)) break;
             const int rb0 = (nb * BN) >> 7;
@@ -952,7 +979,7 @@ k_gemm_mxf4_bs(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
         int cur_nb = -1;
         bool alive = true;
         for (int t = t0; t < t1 && alive; t++) {
-            const int nb = t / p.tiles_m;
+            const int nb = p.by_tiles_m.div(t);
             if (nb != cur_nb) {
                 if (!mbar_wait_warp(bar_b_full, runs & 1u, abort_flag, p.dev_status, p.spin_limit)) break;
                 tc_fence_after();
@@ -996,8 +1023,8 @@ k_gemm_mxf4_bs(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
         bool ready = false;
         bool alive = true;
         for (int t = t0; t < t1 && alive; t++) {
-            const int nb = t / p.tiles_m;
-            const bool last_of_run = (t + 1 == t1) || ((t + 1) / p.tiles_m != nb);
+            const int nb = p.by_tiles_m.div(t);
+            const bool last_of_run = (t + 1 == t1) || (t + 1 == (nb + 1) * p.tiles_m);
             if (nb != cur_nb) {
                 // the block of this column and its scales are in place (the copier saw the block land before it copied)
                 if (!mbar_wait_warp(bar_b_sf_full, runs & 1u, abort_flag, p.dev_status, p.spin_limit)) break;
@@ -1040,6 +1067,7 @@ k_gemm_mxf4_bs(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
         }
     } else if (warp >= kEpiWarp0) {
         // ================= epilogue (warps 4..11) =================
+        pdl_wait();
         const int ew = warp - kEpiWarp0;
         const int quarter = warp & 3;
         const int chalf = ew >> 2;
@@ -1049,7 +1077,7 @@ k_gemm_mxf4_bs(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
         constexpr int kHalfCols = BN / 2;
         uint32_t acc = 0, acc_phase = 0;
         for (int t = t0; t < t1; t++) {
-            const int mb = t % p.tiles_m, nb = t / p.tiles_m;
+            const int nb = p.by_tiles_m.div(t), mb = t - nb * p.tiles_m;
             uint32_t bias[(kHalfCols + 63) / 64];
             bias_fetch<kHalfCols>(bias, p.bias, (int64_t)nb * BN + chalf * kHalfCols, p.N, lane);
             if (!mbar_wait(bar_acc_full + 8 * acc, acc_phase, abort_flag, p.dev_status, p.spin_limit)) break;
@@ -1062,7 +1090,7 @@ k_gemm_mxf4_bs(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
                                                bar_acc_empty + 8 * acc, bias_line);
             if (++acc == 2) { acc = 0; acc_phase ^= 1u; }
         }
-        if (lane == 0) bulk_wait0();   // all stores of this warp have completed before the CTA may exit
+        if (lane == 0) bulk_wait_read<0>();   // the stores of this warp have read their staging buffers: the shared memory may go
     }
 
     tc_fence_before();
@@ -1154,6 +1182,7 @@ k_gemm_mxf4_ck(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
     const uint32_t smem_base = smem_u32(smem);
     const uint32_t rank = ck_cluster_rank(), S = ck_cluster_size();
 
+    if (threadIdx.x == 32 * 3) { prefetch_map(&map_a); prefetch_map(&map_b); }
     if (threadIdx.x == 0) {
         for (int s = 0; s < C::kStages; s++) {
             mbar_init(bar_full + 8 * s, 1);
@@ -1581,6 +1610,7 @@ k_gemm_mxf4_pair(const __grid_constant__ CUtensorMap map_a, const __grid_constan
     const uint32_t smem_base = smem_u32(smem);
     const uint32_t rank = cluster_rank();
 
+    if (threadIdx.x == 32 * 3) { prefetch_map(&map_a); prefetch_map(&map_b); prefetch_map(&map_sfa); prefetch_map(&map_sfb); prefetch_map(&map_d); }
     if (threadIdx.x == 0) {
         for (int s = 0; s < C::kStages; s++) {
             mbar_init(bar_full + 8 * s, 1);
@@ -1603,7 +1633,6 @@ k_gemm_mxf4_pair(const __grid_constant__ CUtensorMap map_a, const __grid_constan
     cluster_sync_all();     // both CTAs have their barriers and TMEM before anyone signals across
     tc_fence_after();
     const uint32_t tmem_base = *tmem_slot;
-    pdl_wait();
 
     const int tiles_m2 = (p.tiles_m + 1) >> 1;
     const int items = tiles_m2 * p.tiles_n * p.splits;
@@ -1618,9 +1647,10 @@ k_gemm_mxf4_pair(const __grid_constant__ CUtensorMap map_a, const __grid_constan
         const bool operands = warp == 0;
         uint32_t stage = 0, phase = 0;
         bool alive = true;
+        pdl_wait();
         for (int item = cluster_id; item < items && alive; item += num_clusters) {
-            const int split = item % p.splits, tile = item / p.splits;
-            const int mb = (tiles_m2 - 1 - tile / p.tiles_n) * 2 + (int)rank, nb = tile % p.tiles_n;
+            const int tile = p.by_splits.div(item), split = item - tile * p.splits;
+            const int tm = p.by_tiles_n.div(tile), mb = (tiles_m2 - 1 - tm) * 2 + (int)rank, nb = tile - tm * p.tiles_n;
             const int kt0 = split * p.kt_per_split;
             const int kt1 = min(kt0 + p.kt_per_split, p.kt_total);
             for (int kt = kt0; kt < kt1; kt++) {
@@ -1652,7 +1682,7 @@ k_gemm_mxf4_pair(const __grid_constant__ CUtensorMap map_a, const __grid_constan
             uint32_t stage = 0, phase = 0;
             bool alive = true;
             for (int item = cluster_id; item < items && alive; item += num_clusters) {
-                const int split = item % p.splits;
+                const int split = p.by_splits.mod(item);
                 const int kt0 = split * p.kt_per_split;
                 const int kt1 = min(kt0 + p.kt_per_split, p.kt_total);
                 for (int kt = kt0; kt < kt1; kt++) {
@@ -1686,11 +1716,11 @@ k_gemm_mxf4_pair(const __grid_constant__ CUtensorMap map_a, const __grid_constan
             uint32_t stage = 0, phase = 0, acc = 0, acc_phase = 0;
             bool alive = true;
             for (int item = cluster_id; item < items && alive; item += num_clusters) {
-                const int split = item % p.splits;
+                const int split = p.by_splits.mod(item);
                 const int kt0 = split * p.kt_per_split;
                 const int kt1 = min(kt0 + p.kt_per_split, p.kt_total);
                 // scale columns hold 32 rows each: a tile that starts 64 rows into a 128-row block starts 2 columns in
-                const uint32_t sfb_shift = BN == 192 ? (uint32_t)((((item / p.splits) % p.tiles_n) * BN & 127) >> 5) : 0u;
+                const uint32_t sfb_shift = BN == 192 ? (uint32_t)((p.by_tiles_n.mod(p.by_splits.div(item)) * BN & 127) >> 5) : 0u;
                 const uint32_t d_tmem = tmem_base + acc * BN;
                 if (!mbar_wait_cluster_warp(bar_acc_empty + 8 * acc, acc_phase ^ 1u, abort_flag, p.dev_status, p.spin_limit)) { alive = false; break; }
                 tc_fence_after();
@@ -1726,6 +1756,7 @@ k_gemm_mxf4_pair(const __grid_constant__ CUtensorMap map_a, const __grid_constan
         }
     } else if (warp >= kEpiWarp0) {
         // ================= epilogue (warps 4..11 of both CTAs: own 128 rows x BN columns) =================
+        pdl_wait();
         const int ew = warp - kEpiWarp0;
         const int quarter = warp & 3;
         const int chalf = ew >> 2;
@@ -1737,8 +1768,8 @@ k_gemm_mxf4_pair(const __grid_constant__ CUtensorMap map_a, const __grid_constan
             const uint32_t bias_line = smem_base + C::kBiasOff + ew * (BN / 2) * 2;
             uint32_t acc = 0, acc_phase = 0;
             for (int item = cluster_id; item < items; item += num_clusters) {
-                const int split = item % p.splits, tile = item / p.splits;
-                const int mb = (tiles_m2 - 1 - tile / p.tiles_n) * 2 + (int)rank, nb = tile % p.tiles_n;
+                const int tile = p.by_splits.div(item), split = item - tile * p.splits;
+                const int tm = p.by_tiles_n.div(tile), mb = (tiles_m2 - 1 - tm) * 2 + (int)rank, nb = tile - tm * p.tiles_n;
                 uint32_t bias[(kHalfCols + 63) / 64];
                 bias_fetch<kHalfCols>(bias, p.bias, (int64_t)nb * BN + chalf * kHalfCols, p.N, lane);
                 if (!mbar_wait_warp(bar_acc_full + 8 * acc, acc_phase, abort_flag, p.dev_status, p.spin_limit)) break;
@@ -1754,8 +1785,8 @@ k_gemm_mxf4_pair(const __grid_constant__ CUtensorMap map_a, const __grid_constan
         uint32_t acc_phase = 0;
         bool alive = true;
         for (int item = cluster_id; item < items && alive; item += num_clusters) {
-            const int split = item % p.splits, tile = item / p.splits;
-            const int mb = (tiles_m2 - 1 - tile / p.tiles_n) * 2 + (int)rank, nb = tile % p.tiles_n;
+            const int tile = p.by_splits.div(item), split = item - tile * p.splits;
+            const int tm = p.by_tiles_n.div(tile), mb = (tiles_m2 - 1 - tm) * 2 + (int)rank, nb = tile - tm * p.tiles_n;
             uint32_t bias[kHalfCols / 32];
 #pragma unroll
             for (int cc = 0; cc < kHalfCols / 32; cc++) bias[cc] = load_bias_pair(p.bias, (int64_t)nb * BN + chalf * kHalfCols + cc * 32, p.N, lane);
@@ -1840,7 +1871,7 @@ k_gemm_mxf4_pair(const __grid_constant__ CUtensorMap map_a, const __grid_constan
             acc_phase ^= 1u;
         }
         }
-        if (lane == 0) bulk_wait0();
+        if (lane == 0) bulk_wait_read<0>();
     }
 
     // neither CTA may leave (or free TMEM) while the other can still reach its shared memory, barriers or TMEM
@@ -1870,7 +1901,8 @@ k_gemm_mxf4_pair(const __grid_constant__ CUtensorMap map_a, const __grid_constan
 // from L2 (in rising order an A tile of 50432 x 4096 x 1024 was read from DRAM about four times; 116 -> 109 us).  The
 // single-CTA B-stationary kernel (short contractions, small A operands) gains nothing from the same walk.
 struct PbsWalk {
-    int tiles_m2, t0, t1, period;
+    int tiles_m2, t0, t1;
+    FastDiv by_tiles_m2, by_period;
 };
 struct PbsTile {
     int nb, mb2;
@@ -1879,11 +1911,11 @@ struct PbsTile {
 __device__ __forceinline__ PbsTile pbs_tile(const PbsWalk &w, int t)
 {
     PbsTile x;
-    x.nb = t / w.tiles_m2;
+    x.nb = w.by_tiles_m2.div(t);
     const int c0 = x.nb * w.tiles_m2;
     const int lo = max(w.t0, c0), hi = min(w.t1, c0 + w.tiles_m2);   // this pair's run in the column
     const int len = hi - lo, ra = lo - c0;
-    const int s = ((ra + w.period - 1) / w.period) * w.period;         // first multiple of the period at or after the run's first row
+    const int period = (int)w.by_period.d, s = w.by_period.div(ra + period - 1) * period;         // first multiple of the period at or after the run's first row
     const int rot = s < ra + len ? s - ra : 0;
     int o = t - lo + rot;
     if (o >= len) o -= len;
@@ -1945,6 +1977,7 @@ k_gemm_mxf4_pbs(const __grid_constant__ CUtensorMap map_a, const __grid_constant
     const uint32_t smem_base = smem_u32(smem);
     const uint32_t rank = cluster_rank();
 
+    if (threadIdx.x == 32 * 3) { prefetch_map(&map_a); prefetch_map(&map_b); prefetch_map(&map_sfa); prefetch_map(&map_sfb); prefetch_map(&map_d); }
     if (threadIdx.x == 0) {
         for (int s = 0; s < AS; s++) {
             mbar_init(bar_a_full + 8 * s, 1);
@@ -1970,16 +2003,14 @@ k_gemm_mxf4_pbs(const __grid_constant__ CUtensorMap map_a, const __grid_constant
     cluster_sync_all();     // both CTAs have their barriers and TMEM before anyone signals across
     tc_fence_after();
     const uint32_t tmem_base = *tmem_slot;
-    pdl_wait();
 
     // pair tiles (256 rows x 192 columns) are numbered column by column: t = nb * tiles_m2 + mb2; this pair owns [t0, t1)
     // and walks it as pbs_tile says
     const int tiles_m2 = (p.tiles_m + 1) >> 1;
-    const int64_t total = (int64_t)tiles_m2 * p.tiles_n;
-    const int cluster_id = blockIdx.x >> 1, num_clusters = gridDim.x >> 1;
-    const int t0 = (int)(total * cluster_id / num_clusters), t1 = (int)(total * (cluster_id + 1) / num_clusters);
+    const int cluster_id = blockIdx.x >> 1;
+    const int t0 = range_start(p, cluster_id), t1 = range_start(p, cluster_id + 1);
     const int ktn = p.kt_total;
-    const PbsWalk walk = {tiles_m2, t0, t1, max(1, (int)((total + num_clusters - 1) / num_clusters))};
+    const PbsWalk walk = {tiles_m2, t0, t1, p.by_tiles_m2, p.by_period};
 
     if (warp == 0) {
         // ===== producer (both CTAs): own 128 rows of A and their scales per stage; own half of a column's B block and all
@@ -1987,6 +2018,7 @@ k_gemm_mxf4_pbs(const __grid_constant__ CUtensorMap map_a, const __grid_constant
         const bool leader = elect_one() && !p.withhold_loads;
         uint32_t stage = 0, phase = 0, runs = 0;
         int nb = 0;
+        pdl_wait();
         bool alive = true;
         auto load_block = [&]() -> bool {
             // the MMAs of the previous column have finished reading the block (multicast commits reach both CTAs)
@@ -2129,6 +2161,7 @@ k_gemm_mxf4_pbs(const __grid_constant__ CUtensorMap map_a, const __grid_constant
         }
     } else if (warp >= kEpiWarp0) {
         // ===== epilogue (warps 4..11 of both CTAs: own 128 rows x 192 columns) =====
+        pdl_wait();
         const int ew = warp - kEpiWarp0;
         const int quarter = warp & 3;
         const int chalf = ew >> 2;
@@ -2152,7 +2185,7 @@ k_gemm_mxf4_pbs(const __grid_constant__ CUtensorMap map_a, const __grid_constant
                                                      map_to_cta(bar_acc_empty + 8 * acc, 0), bias_line);
             if (++acc == 2) { acc = 0; acc_phase ^= 1u; }
         }
-        if (lane == 0) bulk_wait0();   // all stores of this warp have completed before the CTA may exit
+        if (lane == 0) bulk_wait_read<0>();   // the stores of this warp have read their staging buffers: the shared memory may go
     }
 
     // neither CTA may leave (or free TMEM) while the other can still reach its shared memory, barriers or TMEM
@@ -2486,6 +2519,22 @@ mxfp4_status_t gemm_check(mxfp4_mat_t a, mxfp4_mat_t b, const void *d, int64_t l
     return MXFP4_OK;
 }
 
+// The divisors of the tile numbering and, for `workers` blocks or pairs of them that take contiguous ranges of the column-by-column
+// numbering, their shares (pairs: of 256-row tiles; only the kernels that walk that way read them).
+static void set_walk(GemmParams &p, int workers, bool pairs = false)
+{
+    const int tiles_m2 = (p.tiles_m + 1) / 2;
+    const int64_t total = (int64_t)(pairs ? tiles_m2 : p.tiles_m) * p.tiles_n;
+    p.by_splits = fast_div(p.splits);
+    p.by_tiles_n = fast_div(p.tiles_n);
+    p.by_tiles_m = fast_div(p.tiles_m);
+    p.by_tiles_m2 = fast_div(tiles_m2);
+    p.by_workers = fast_div(workers ? workers : 1);
+    p.share = workers ? (int)(total / workers) : 0;
+    p.extra = workers ? (int)(total % workers) : 0;
+    p.by_period = fast_div(p.share + (p.extra > 0 ? 1 : 0) > 0 ? p.share + (p.extra > 0 ? 1 : 0) : 1);
+}
+
 // spin_limit / withhold_loads: see GemmParams (normal use: kWaitSpinLimit, 0).
 static mxfp4_status_t gemm_impl(mxfp4_mat_t a, mxfp4_mat_t b, void *d, int64_t ldd, int out_dtype, const void *bias, void *workspace,
                                 size_t workspace_bytes, uint32_t *dev_status, cudaStream_t st, bool allow_split, uint32_t spin_limit,
@@ -2517,6 +2566,7 @@ static mxfp4_status_t gemm_impl(mxfp4_mat_t a, mxfp4_mat_t b, void *d, int64_t l
     p.ldd = ldd;
     p.spin_limit = spin_limit;
     p.withhold_loads = withhold_loads;
+    set_walk(p, 0);
     if (g.ck) {
         p.splits = g.ck;
         p.out_fp32 = out_dtype == MXFP4_OUT_FP32;
@@ -2525,6 +2575,7 @@ static mxfp4_status_t gemm_impl(mxfp4_mat_t a, mxfp4_mat_t b, void *d, int64_t l
     const bool paired = g.pair || g.pbs;
     const int items = (paired ? (g.tiles_m + 1) / 2 : g.tiles_m) * g.tiles_n * g.splits;
     const int grid = paired ? 2 * min(items, sms / 2) : min(items, sms);
+    set_walk(p, paired ? grid / 2 : grid, paired);
     CUtensorMap msa, msb;
     if (paired && (!make_scale_map(&msa, a.scales, M, Kc, 1) || !make_scale_map(&msb, b.scales, N, Kc, 2))) return MXFP4_CUDA_ERROR;
     CUtensorMap mdw = md;
@@ -2688,6 +2739,7 @@ mxfp4_status_t gemm_quant(mxfp4_mat_t a, mxfp4_mat_t b, const void *bias, const 
     p.ldd = 0;
     p.spin_limit = kWaitSpinLimit;
     p.withhold_loads = 0;
+    set_walk(p, 0);
 
     QuantEpilogue e;
     const mxfp4_qparams_t none = {MXFP4_SCALE_TRUNCATION_FREE, MXFP4_ROUND_NEAREST, 0, 0, 0};

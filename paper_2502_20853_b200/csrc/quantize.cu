@@ -315,6 +315,8 @@ k_quantize_stream(const __grid_constant__ QsJob job, const __grid_constant__ Job
         mbar_init(bar_full + 8, 1);
         *abort_flag = 0u;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        prefetch_map(&job.map_src);
+        prefetch_map(&job.map_t);
     }
     const QsGeom g = qs_geom(threadIdx.x, job.rows, job.cols, job.rw.packed);
     pdl_wait();
@@ -336,7 +338,7 @@ k_quantize_stream(const __grid_constant__ QsJob job, const __grid_constant__ Job
                                                       hook_out, hook_ld, load);
         }
     }
-    if (threadIdx.x == 0) bulk_wait0();           // every store has completed before the shared memory goes away
+    if (threadIdx.x == 0) bulk_wait_read<0>();    // every store has read its staging buffer: the shared memory may go
     if (nonfinite && dev_status) atomicOr(dev_status, MXFP4_DEV_NONFINITE);
 }
 
