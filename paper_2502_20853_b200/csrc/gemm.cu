@@ -76,9 +76,10 @@ struct GemmParams {
     int nblk4;            // ceil(Kc/32/4): 512-byte chunks per 128-row block
     int rbA, rbB;         // 128-row scale blocks present in A / B buffers
     int tiles_m, tiles_n, splits, kt_total, kt_per_split;
-    FastDiv by_splits, by_tiles_n, by_tiles_m, by_tiles_m2, by_period;   // tiles_m2: row tiles of a CTA pair; period: see PbsWalk
-    FastDiv by_workers;   // kernels that give a block (pair) a contiguous range of tiles: `share` each and `extra` more, spread evenly
-    int share, extra;
+    FastDiv by_splits, by_tiles_n;
+    // the walk of the B-stationary kernels, see Walk
+    FastDiv by_rest_rows, by_rest_workers;
+    int abreast, rounds, rows, rest_row0, share, extra;
     int out_fp32;         // element type of the stored tile (FP32 also for split-K partials)
     const __nv_bfloat16 *bias;   // applied only when splits == 1 (and by the cluster kernel, whose sum is complete)
     uint32_t *dev_status;
@@ -88,9 +89,57 @@ struct GemmParams {
     int withhold_loads;   // self-test of the drain path: the producers issue nothing, so every wait runs out
 };
 
-// First tile of worker w's contiguous range, floor(total w / workers).  The workers with one tile more are spread evenly: with
-// the first `extra` ones the ranges start at a constant stride in memory and 401408 x 384 x 96 took 82 us instead of 76.
-__device__ __forceinline__ int range_start(const GemmParams &p, int w) { return w * p.share + p.by_workers.div(w * p.extra); }
+// How the workers (CTAs, or pairs of them) of the B-stationary kernels share the tiles.  A worker keeps the B block of its tile
+// column for as long as it can, and all workers write the same stretch of the output at the same time: stores to many distant
+// places are slow here (a kernel that does nothing but store, 384 bytes of a row at a time: 4.7-5.1 TB/s with a far-away
+// stretch of rows for each SM, 5.5-5.8 TB/s when all SMs fill the same rows).  So `abreast` workers go down each column,
+// taking its row tiles in turn, and at any moment all columns are near the same rows (the columns ask for an A tile at about
+// the same time, too, and it comes from L2).  Workers that are left over because the columns do not divide
+// their number take the last rows: contiguous ranges, of equal length, of those rows' tiles, numbered column by column.  With
+// more columns than workers everything is shared that way.
+// Against contiguous ranges of all tiles, in us: 401408 x 384 x 96 75.7 -> 64.9, 100352 x 1536 x 384 87 -> 58, 25216 x 1536 x 384
+// 19.8 -> 18.1; on pairs 100352 x 1536 x 768 75.9 -> 66.4, 50432 x 4096 x 1024 106 -> 101, 50432 x 2304 x 768 52 -> 50.
+struct Walk {
+    int count;            // tiles of this worker
+    int col, row, step;   // step > 0: rows row, row + step, .. of the column; 0: the tiles t0, t0 + 1, .. of the last rows
+    int t0;
+};
+struct WalkItem {
+    int col, row;
+    bool first, last;   // of this worker's run in the column
+};
+__device__ __forceinline__ Walk walk_begin(const GemmParams &p, int w)
+{
+    Walk x;
+    const int r = p.by_tiles_n.div(w);
+    x.step = r < p.abreast ? p.abreast : 0;
+    x.row = r;
+    x.col = w - r * p.tiles_n;
+    w -= p.abreast * p.tiles_n;
+    // floor(tiles w / workers): the workers with one tile more are spread evenly (at a constant stride between the ranges their
+    // stores meet in the same parts of the memory: 401408 x 384 x 96 took 82 us instead of 76)
+    x.t0 = w * p.share + p.by_rest_workers.div(w * p.extra);
+    x.count = x.step ? p.rounds - (r + (p.rounds - 1) * p.abreast >= p.rows) : (w + 1) * p.share + p.by_rest_workers.div((w + 1) * p.extra) - x.t0;
+    return x;
+}
+__device__ __forceinline__ WalkItem walk_item(const GemmParams &p, const Walk &w, int i)
+{
+    WalkItem x;
+    x.first = i == 0;
+    x.last = i == w.count - 1;
+    if (w.step) {
+        x.col = w.col;
+        x.row = w.row + i * w.step;
+    } else {
+        const int rows = (int)p.by_rest_rows.d;
+        x.col = p.by_rest_rows.div(w.t0 + i);
+        const int r = w.t0 + i - x.col * rows;
+        x.first |= r == 0;
+        x.last |= r == rows - 1;
+        x.row = p.rest_row0 + r;
+    }
+    return x;
+}
 
 // ---- PTX wrappers of the tensor-core instructions (mbarrier, TMA and elect wrappers: tma.cuh) ----
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
@@ -840,10 +889,9 @@ k_gemm_mxf4_q(const __grid_constant__ CUtensorMap map_a, const __grid_constant__
 // ---- the B-stationary kernel --------------------------------------------------------------------------
 // For contraction lengths of a few K tiles (the forward and input-gradient products of the layers: Kc = 384 .. 1536)
 // the ring of the kernel above carries, per stage, a B tile that the CTA has loaded many times before, and its rate
-// is ring bytes in flight over load latency.  Here a CTA walks DOWN a column of tiles: the whole B block of the
+// is ring bytes in flight over load latency.  Here a CTA walks DOWN a column of tiles (see Walk): the whole B block of the
 // column (BN rows x Kc, with its scales in TMEM) stays resident, and the ring carries A alone, so that the same
-// shared memory holds two to three times as many tiles in flight.  Tiles are numbered column by column and each CTA
-// takes a contiguous range; B is reloaded where the range crosses into the next column.
+// shared memory holds two to three times as many tiles in flight.
 template <int BN, int KT, int AS>   // KT: K tiles the resident B block can hold; AS: stages of the A ring
 struct GemmBsCfg {
     static constexpr int kRB = (BN + 127) / 128;
@@ -851,7 +899,7 @@ struct GemmBsCfg {
     static constexpr int kBBytes = BN * kBKBytes;              // one K tile of the B block
     static constexpr int kSfaBytes = 2 * kSfChunk;
     static constexpr int kSfbBytes = 2 * kSfChunk * kRB;       // per K tile
-    static constexpr int kStagingBufs = (BN == 192 && KT > 2) ? 2 : BN / 64;
+    static constexpr int kStagingBufs = BN / 64;
     static constexpr int kAOff = KT * kBBytes;
     static constexpr int kSfbOff = kAOff + AS * kABytes;
     static constexpr int kSfaOff = kSfbOff + KT * kSfbBytes;
@@ -918,8 +966,7 @@ k_gemm_mxf4_bs(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
     tc_fence_after();
     const uint32_t tmem_base = *tmem_slot;
 
-    // tiles are numbered column by column: t = nb * tiles_m + mb; this CTA owns [t0, t1)
-    const int t0 = range_start(p, blockIdx.x), t1 = range_start(p, blockIdx.x + 1);
+    const Walk walk = walk_begin(p, blockIdx.x);
     const int ktn = p.kt_total;
 
     if (warp == 0) {
@@ -928,8 +975,8 @@ k_gemm_mxf4_bs(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
         uint32_t stage = 0, phase = 0;
         bool alive = true;
         pdl_wait();
-        for (int t = t0; t < t1 && alive; t++) {
-            const int mb = p.by_tiles_m.mod(t);
+        for (int i = 0; i < walk.count && alive; i++) {
+            const int mb = walk_item(p, walk, i).row;
             for (int kt = 0; kt < ktn; kt++) {
                 if (!mbar_wait_warp(bar_a_empty + 8 * stage, phase ^ 1u, abort_flag, p.dev_status, p.spin_limit)) { alive = false; break; }
                 const int nch = min(2, p.nblk4 - 2 * kt);
@@ -949,8 +996,10 @@ k_gemm_mxf4_bs(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
         const bool leader = elect_one() && !p.withhold_loads;
         uint32_t runs = 0;
         pdl_wait();
-        for (int t = t0; t < t1;) {
-            const int nb = p.by_tiles_m.div(t);
+        for (int i = 0; i < walk.count; i++) {
+            const WalkItem x = walk_item(p, walk, i);
+            if (!x.first) continue;
+            const int nb = x.col;
             // the MMAs of the previous column have finished reading the block
             if (runs > 0 && !mbar_wait_warp(bar_b_empty, (runs - 1u) & 1u, abort_flag, p.dev_status, p.spin_limit)) break;
             const int rb0 = (nb * BN) >> 7;
@@ -970,17 +1019,15 @@ k_gemm_mxf4_bs(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
             }
             __syncwarp();
             runs++;
-            t = min(t1, (nb + 1) * p.tiles_m);
+            if (walk.step) break;   // its only run
         }
     } else if (warp == 2) {
         // ================= scale copier: B scales once per column, A scales per stage =================
         const bool leader = elect_one();
         uint32_t stage = 0, phase = 0, runs = 0;
-        int cur_nb = -1;
         bool alive = true;
-        for (int t = t0; t < t1 && alive; t++) {
-            const int nb = p.by_tiles_m.div(t);
-            if (nb != cur_nb) {
+        for (int i = 0; i < walk.count && alive; i++) {
+            if (walk_item(p, walk, i).first) {
                 if (!mbar_wait_warp(bar_b_full, runs & 1u, abort_flag, p.dev_status, p.spin_limit)) break;
                 tc_fence_after();
                 if (leader) {
@@ -996,7 +1043,6 @@ k_gemm_mxf4_bs(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
                     tc_commit(bar_b_sf_full);
                 }
                 __syncwarp();
-                cur_nb = nb;
                 runs++;
             }
             for (int kt = 0; kt < ktn; kt++) {
@@ -1019,16 +1065,14 @@ k_gemm_mxf4_bs(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
         const bool leader = elect_one();
         uint32_t stage = 0, phase = 0, acc = 0, acc_phase = 0, runs = 0;
         const int nmma_last = (int)((p.Kc - (int64_t)(ktn - 1) * kBKElems + 63) / 64);   // MMAs of the last K tile
-        int cur_nb = -1;
         bool ready = false;
         bool alive = true;
-        for (int t = t0; t < t1 && alive; t++) {
-            const int nb = p.by_tiles_m.div(t);
-            const bool last_of_run = (t + 1 == t1) || (t + 1 == (nb + 1) * p.tiles_m);
-            if (nb != cur_nb) {
+        for (int i = 0; i < walk.count && alive; i++) {
+            const WalkItem x = walk_item(p, walk, i);
+            const int nb = x.col;
+            if (x.first) {
                 // the block of this column and its scales are in place (the copier saw the block land before it copied)
                 if (!mbar_wait_warp(bar_b_sf_full, runs & 1u, abort_flag, p.dev_status, p.spin_limit)) break;
-                cur_nb = nb;
                 runs++;
             }
             const uint32_t sfb_shift = (uint32_t)(((nb * BN) & 127) >> 5);
@@ -1060,7 +1104,7 @@ k_gemm_mxf4_bs(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
             }
             if (alive && leader) {
                 tc_commit(bar_acc_full + 8 * acc);            // accumulator complete
-                if (last_of_run) tc_commit(bar_b_empty);      // and the resident block may be replaced
+                if (x.last) tc_commit(bar_b_empty);           // and the resident block may be replaced
             }
             __syncwarp();
             if (++acc == 2) { acc = 0; acc_phase ^= 1u; }
@@ -1076,8 +1120,9 @@ k_gemm_mxf4_bs(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
         uint32_t sbuf = 0;
         constexpr int kHalfCols = BN / 2;
         uint32_t acc = 0, acc_phase = 0;
-        for (int t = t0; t < t1; t++) {
-            const int nb = p.by_tiles_m.div(t), mb = t - nb * p.tiles_m;
+        for (int i = 0; i < walk.count; i++) {
+            const WalkItem x = walk_item(p, walk, i);
+            const int nb = x.col, mb = x.row;
             uint32_t bias[(kHalfCols + 63) / 64];
             bias_fetch<kHalfCols>(bias, p.bias, (int64_t)nb * BN + chalf * kHalfCols, p.N, lane);
             if (!mbar_wait(bar_acc_full + 8 * acc, acc_phase, abort_flag, p.dev_status, p.spin_limit)) break;
@@ -1894,37 +1939,6 @@ k_gemm_mxf4_pair(const __grid_constant__ CUtensorMap map_a, const __grid_constan
 // epilogue of one tile run under the K loop of the next.  Per stage and SM the port sees 16 KB written and 16 + 12 KB read for a 128 x 192 x 256
 // block of the product, less than the tensor pipe needs for it.  Roles, barriers and the cross-CTA signalling are those
 // of the two kernels this combines (k_gemm_mxf4_pair, k_gemm_mxf4_bs).
-// The walk of one CTA pair over its range [t0, t1) of the column-by-column numbering.  Inside a column the pair does not
-// take its rows in rising order but rotated so that it starts at a multiple of `period` (the range length, the same for
-// every pair): all pairs then work on rows of the same residue at the same time, i.e. the pairs that need an A tile (one
-// per column) ask for it within a few microseconds of one another instead of spread over the whole kernel, and it comes
-// from L2 (in rising order an A tile of 50432 x 4096 x 1024 was read from DRAM about four times; 116 -> 109 us).  The
-// single-CTA B-stationary kernel (short contractions, small A operands) gains nothing from the same walk.
-struct PbsWalk {
-    int tiles_m2, t0, t1;
-    FastDiv by_tiles_m2, by_period;
-};
-struct PbsTile {
-    int nb, mb2;
-    bool first, last;   // of this pair's run in the column nb
-};
-__device__ __forceinline__ PbsTile pbs_tile(const PbsWalk &w, int t)
-{
-    PbsTile x;
-    x.nb = w.by_tiles_m2.div(t);
-    const int c0 = x.nb * w.tiles_m2;
-    const int lo = max(w.t0, c0), hi = min(w.t1, c0 + w.tiles_m2);   // this pair's run in the column
-    const int len = hi - lo, ra = lo - c0;
-    const int period = (int)w.by_period.d, s = w.by_period.div(ra + period - 1) * period;         // first multiple of the period at or after the run's first row
-    const int rot = s < ra + len ? s - ra : 0;
-    int o = t - lo + rot;
-    if (o >= len) o -= len;
-    x.mb2 = ra + o;
-    x.first = t == lo;
-    x.last = t == hi - 1;
-    return x;
-}
-
 template <int KT, int AS>   // KT: K tiles the resident B block can hold; AS: stages of the A ring
 struct GemmPbsCfg {
     static constexpr int BN = 192;
@@ -2004,13 +2018,8 @@ k_gemm_mxf4_pbs(const __grid_constant__ CUtensorMap map_a, const __grid_constant
     tc_fence_after();
     const uint32_t tmem_base = *tmem_slot;
 
-    // pair tiles (256 rows x 192 columns) are numbered column by column: t = nb * tiles_m2 + mb2; this pair owns [t0, t1)
-    // and walks it as pbs_tile says
-    const int tiles_m2 = (p.tiles_m + 1) >> 1;
-    const int cluster_id = blockIdx.x >> 1;
-    const int t0 = range_start(p, cluster_id), t1 = range_start(p, cluster_id + 1);
+    const Walk walk = walk_begin(p, blockIdx.x >> 1);   // pair tiles: 256 rows x 192 columns
     const int ktn = p.kt_total;
-    const PbsWalk walk = {tiles_m2, t0, t1, p.by_tiles_m2, p.by_period};
 
     if (warp == 0) {
         // ===== producer (both CTAs): own 128 rows of A and their scales per stage; own half of a column's B block and all
@@ -2036,13 +2045,13 @@ k_gemm_mxf4_pbs(const __grid_constant__ CUtensorMap map_a, const __grid_constant
             runs++;
             return true;
         };
-        for (int t = t0; t < t1 && alive; t++) {
+        for (int i = 0; i < walk.count && alive; i++) {
             // the first block before anything else; later ones after the A stages of the column's first tile, which need
             // nothing from the new block and keep the ring full while the old column drains
-            const PbsTile x = pbs_tile(walk, t);
-            nb = x.nb;
-            if (t == t0 && !load_block()) break;
-            const int mb = x.mb2 * 2 + (int)rank;
+            const WalkItem x = walk_item(p, walk, i);
+            nb = x.col;
+            if (i == 0 && !load_block()) break;
+            const int mb = x.row * 2 + (int)rank;
             for (int kt = 0; kt < ktn; kt++) {
                 if (!mbar_wait_warp(bar_a_empty + 8 * stage, phase ^ 1u, abort_flag, p.dev_status, p.spin_limit)) { alive = false; break; }
                 if (leader) {
@@ -2054,7 +2063,7 @@ k_gemm_mxf4_pbs(const __grid_constant__ CUtensorMap map_a, const __grid_constant
                 __syncwarp();
                 if (++stage == AS) { stage = 0; phase ^= 1u; }
             }
-            if (alive && t != t0 && x.first && !load_block()) break;
+            if (alive && i > 0 && x.first && !load_block()) break;
         }
     } else if (warp == 2) {
         // ===== scale copier (leader only; each copy acts on both CTAs): B scales once per column, A scales per stage =====
@@ -2062,8 +2071,8 @@ k_gemm_mxf4_pbs(const __grid_constant__ CUtensorMap map_a, const __grid_constant
             const bool leader = elect_one();
             uint32_t stage = 0, phase = 0, runs = 0;
             bool alive = true;
-            for (int t = t0; t < t1 && alive; t++) {
-                if (pbs_tile(walk, t).first) {
+            for (int i = 0; i < walk.count && alive; i++) {
+                if (walk_item(p, walk, i).first) {
                     if (!mbar_wait_warp(bar_b_full, runs & 1u, abort_flag, p.dev_status, p.spin_limit)) break;
                     tc_fence_after();
                     if (leader) {
@@ -2111,11 +2120,10 @@ k_gemm_mxf4_pbs(const __grid_constant__ CUtensorMap map_a, const __grid_constant
             const int nmma_last = (int)((p.Kc - (int64_t)(ktn - 1) * kBKElems + 63) / 64);   // MMAs of the last K tile
             const uint32_t d_tmem = tmem_base + me * BN;
             bool alive = true;
-            for (int t = t0; t < t1 && alive; t++) {
-                const bool mine = (uint32_t)((t - t0) & 1) == me;
-                const PbsTile x = pbs_tile(walk, t);
-                const int nb = x.nb;
-                const bool last_of_run = x.last;
+            for (int i = 0; i < walk.count && alive; i++) {
+                const bool mine = (uint32_t)(i & 1) == me;
+                const WalkItem x = walk_item(p, walk, i);
+                const int nb = x.col;
                 if (x.first) {
                     // the block of this column and its scales are in place in both CTAs (the copier saw them land before it copied)
                     if (!mbar_wait_warp(bar_b_sf_full, runs & 1u, abort_flag, p.dev_status, p.spin_limit)) break;
@@ -2154,7 +2162,7 @@ k_gemm_mxf4_pbs(const __grid_constant__ CUtensorMap map_a, const __grid_constant
                 }
                 if (alive && leader) {
                     if (mine) tc2_commit_both(bar_acc_full + 8 * me);   // both CTAs' accumulators are complete
-                    if (last_of_run) tc2_commit_both(bar_b_empty);      // this warp's MMAs on the resident blocks are complete
+                    if (x.last) tc2_commit_both(bar_b_empty);      // this warp's MMAs on the resident blocks are complete
                 }
                 __syncwarp();
             }
@@ -2170,9 +2178,9 @@ k_gemm_mxf4_pbs(const __grid_constant__ CUtensorMap map_a, const __grid_constant
         uint32_t sbuf = 0;
         constexpr int kHalfCols = BN / 2;
         uint32_t acc = 0, acc_phase = 0;
-        for (int t = t0; t < t1; t++) {
-            const PbsTile x = pbs_tile(walk, t);
-            const int mb = x.mb2 * 2 + (int)rank, nb = x.nb;
+        for (int i = 0; i < walk.count; i++) {
+            const WalkItem x = walk_item(p, walk, i);
+            const int mb = x.row * 2 + (int)rank, nb = x.col;
             uint32_t bias[(kHalfCols + 63) / 64];
             bias_fetch<kHalfCols>(bias, p.bias, (int64_t)nb * BN + chalf * kHalfCols, p.N, lane);
             if (!mbar_wait(bar_acc_full + 8 * acc, acc_phase, abort_flag, p.dev_status, p.spin_limit)) break;
@@ -2356,7 +2364,8 @@ static GemmPlan plan_gemm(int64_t m, int64_t n, int64_t kc, int sms, bool allow_
     if (g.kt_total >= 3 && g.kt_total <= 4 && n >= 192 && m >= 2048 && sms >= 2 &&
         ceil_div(ceil_div(m, kBM), 2) * ceil_div(n, 192) >= sms) {
         // short contraction, tall output: pairs of CTAs walk down columns of 256 x 192 tiles with the column's B block resident
-        // (with one or two K tiles the single-CTA B-stationary kernel below measured 4-10 % faster; with fewer than two pair
+        // (with one or two K tiles the single-CTA B-stationary kernel below is faster: 401408 x 384 x 96 65.1 against 67.4 us,
+        // 25216 x 1152 x 384 14.6 against 16.1, and even at 100352 x 1536 x 384, 58; with fewer than two pair
         // tiles per CTA pair the set-up of a column costs more than the kernel saves: 12.3 against 10.2 us at 2048 x 768 x 768)
         g.pbs = true;
         g.bn = 192;
@@ -2519,20 +2528,31 @@ mxfp4_status_t gemm_check(mxfp4_mat_t a, mxfp4_mat_t b, const void *d, int64_t l
     return MXFP4_OK;
 }
 
-// The divisors of the tile numbering and, for `workers` blocks or pairs of them that take contiguous ranges of the column-by-column
-// numbering, their shares (pairs: of 256-row tiles; only the kernels that walk that way read them).
-static void set_walk(GemmParams &p, int workers, bool pairs = false)
+// The divisors of the tile numbering and, for the B-stationary kernels, how `rows` row tiles (of one CTA or of a pair) are shared by
+// `workers`: the smallest number of rounds for which the rest, the rows behind those that the rounds reach, keeps the left-over
+// workers no longer than that.  A change of column costs them about a tile (with that left out, 50432 x 2304 x 768 took
+// 54 us, its two left-over pairs the last to finish; 49 with one round more and no rest).
+static void set_walk(GemmParams &p, int workers = 1, int rows = 1)
 {
-    const int tiles_m2 = (p.tiles_m + 1) / 2;
-    const int64_t total = (int64_t)(pairs ? tiles_m2 : p.tiles_m) * p.tiles_n;
     p.by_splits = fast_div(p.splits);
     p.by_tiles_n = fast_div(p.tiles_n);
-    p.by_tiles_m = fast_div(p.tiles_m);
-    p.by_tiles_m2 = fast_div(tiles_m2);
-    p.by_workers = fast_div(workers ? workers : 1);
-    p.share = workers ? (int)(total / workers) : 0;
-    p.extra = workers ? (int)(total % workers) : 0;
-    p.by_period = fast_div(p.share + (p.extra > 0 ? 1 : 0) > 0 ? p.share + (p.extra > 0 ? 1 : 0) : 1);
+    p.rows = rows;
+    p.abreast = workers / p.tiles_n;
+    const int rest_workers = workers - p.abreast * p.tiles_n;
+    int64_t rest = (int64_t)rows * p.tiles_n;
+    p.rounds = 0;
+    p.rest_row0 = 0;
+    if (p.abreast > 0) {
+        for (p.rounds = (int)((rest - 1) / workers); p.rest_row0 < rows; p.rounds++) {
+            p.rest_row0 = min(rows, (p.rounds + 1) * p.abreast);
+            rest = (int64_t)(rows - p.rest_row0) * p.tiles_n;
+            if (rest_workers > 0 && ceil_div(rest, rest_workers) + p.tiles_n / rest_workers - 1 <= p.rounds + 1) { p.rounds++; break; }
+        }
+    }
+    p.by_rest_rows = fast_div(max(1, rows - p.rest_row0));
+    p.by_rest_workers = fast_div(max(1, rest_workers));
+    p.share = rest_workers ? (int)(rest / rest_workers) : 0;
+    p.extra = rest_workers ? (int)(rest % rest_workers) : 0;
 }
 
 // spin_limit / withhold_loads: see GemmParams (normal use: kWaitSpinLimit, 0).
@@ -2566,16 +2586,16 @@ static mxfp4_status_t gemm_impl(mxfp4_mat_t a, mxfp4_mat_t b, void *d, int64_t l
     p.ldd = ldd;
     p.spin_limit = spin_limit;
     p.withhold_loads = withhold_loads;
-    set_walk(p, 0);
+    set_walk(p);
     if (g.ck) {
         p.splits = g.ck;
         p.out_fp32 = out_dtype == MXFP4_OUT_FP32;
         return launch_gemm_ck(ma, mb, p, g.tiles_m * g.tiles_n, g.ck, st);
     }
     const bool paired = g.pair || g.pbs;
-    const int items = (paired ? (g.tiles_m + 1) / 2 : g.tiles_m) * g.tiles_n * g.splits;
-    const int grid = paired ? 2 * min(items, sms / 2) : min(items, sms);
-    set_walk(p, paired ? grid / 2 : grid, paired);
+    const int rows = paired ? (g.tiles_m + 1) / 2 : g.tiles_m, workers = paired ? sms / 2 : sms;
+    const int items = min(workers, rows * g.tiles_n * g.splits), grid = paired ? 2 * items : items;
+    set_walk(p, items, rows);
     CUtensorMap msa, msb;
     if (paired && (!make_scale_map(&msa, a.scales, M, Kc, 1) || !make_scale_map(&msb, b.scales, N, Kc, 2))) return MXFP4_CUDA_ERROR;
     CUtensorMap mdw = md;
@@ -2739,7 +2759,7 @@ mxfp4_status_t gemm_quant(mxfp4_mat_t a, mxfp4_mat_t b, const void *bias, const 
     p.ldd = 0;
     p.spin_limit = kWaitSpinLimit;
     p.withhold_loads = 0;
-    set_walk(p, 0);
+    set_walk(p);
 
     QuantEpilogue e;
     const mxfp4_qparams_t none = {MXFP4_SCALE_TRUNCATION_FREE, MXFP4_ROUND_NEAREST, 0, 0, 0};

@@ -190,6 +190,14 @@ def test_gemm_many_splits_of_a_small_output(mx, M, N, K, out_dtype):
     _bias_case(mx, M, N, K, out_dtype)
 
 
+@pytest.mark.parametrize("M,N,K", [(6980, 1496, 96), (150, 28488, 96), (7224, 928, 544), (2100, 14248, 544)])
+@pytest.mark.parametrize("out_dtype", [0, 1])
+def test_gemm_b_stationary_walk(mx, M, N, K, out_dtype):
+    """The B-stationary kernels where (on 148 SMs) left-over workers take the last row tile of every column, and where there are
+    more tile columns than workers; single CTAs (K = 96) and pairs (K = 544)."""
+    _bias_case(mx, M, N, K, out_dtype)
+
+
 def test_gemm_argument_errors(mx):
     a, b = mx.QMat(128, 64), mx.QMat(128, 96)
     with pytest.raises(mx.MxError) as e:
