@@ -1,4 +1,5 @@
-"""ctypes binding of libmxfp4.so: argument marshalling only — every step runs in the CUDA kernels.
+"""Binding of libmxfp4.so: argument marshalling only — every step runs in the CUDA kernels.  The calls that a training or
+serving step makes are marshalled by the native module ``_host`` (csrc/host.cpp), all others by ctypes.
 
 torch is used for device memory and streams.  The library must be present (built in-tree by
 ``paper_2502_20853_b200.build``); there is no fallback path of any kind.
@@ -7,6 +8,13 @@ import ctypes as C
 import os
 
 import torch
+
+try:
+    from . import _host
+except ImportError:      # not built yet: it takes the host compiler alone, and the class QMat needs it
+    from .build import build_host
+    build_host()
+    from . import _host
 
 _HERE = os.path.dirname(os.path.abspath(__file__))
 LIB_PATH = os.path.join(_HERE, "libmxfp4.so")
@@ -143,6 +151,9 @@ def lib():
     L.mxfp4_qramp_detect.argtypes = [vp, vp, i64, C.c_float, i32, i32, vp, vp, vp]
     L.mxfp4_qramp_adamw.restype = i32
     L.mxfp4_qramp_adamw.argtypes = [vp, vp, vp, vp, vp, vp, vp, vp, i64, C.POINTER(CAdamW), vp]
+    # the entry points that _host calls
+    for name in ("linear_fwd_ex", "linear_bwd_ex", "quantize", "quantize_t", "qema_quantize"):
+        setattr(L, "at_" + name, C.cast(getattr(L, "mxfp4_" + name), C.c_void_p).value)
     _lib = L
     return L
 
@@ -178,49 +189,31 @@ def _align256(n):
     return (n + 255) & ~255
 
 
-class QMat:
+class QMat(_host.Mat):
     """A quantized matrix in device memory: packed E2M1 codes + E8M0 scales in tiled order.  Codes and scales that the
-    binding allocates itself share one buffer (an allocation costs a call 2.4 us); ``data`` and ``scales`` are views of it,
+    binding allocates itself share one buffer (an allocation costs a call 1.7 us); ``data`` and ``scales`` are views of it,
     made when they are asked for."""
 
-    __slots__ = ("rows", "cols", "_buf", "_at", "_data", "_scales", "_c")
+    __slots__ = ()
 
     def __init__(self, rows, cols, device="cuda", data=None, scales=None):
-        self.rows, self.cols = int(rows), int(cols)
+        rows, cols = int(rows), int(cols)
         if data is None and scales is None and ALLOC_HOOK is None:
-            self._place(torch.empty(QMat._bytes(self.rows, self.cols), dtype=torch.uint8, device=device), 0)
+            buf = torch.empty(_host.nbytes(rows, cols), dtype=torch.uint8, device=device)
+            _host.place(self, buf, buf.data_ptr(), rows, cols)
             return
-        self._buf = None
-        self._data = data if data is not None else _new((self.rows, self.cols // 2), torch.uint8, device)
-        nbytes = max(scale_bytes(self.rows, self.cols), 16)
-        self._scales = scales if scales is not None else _new((nbytes,), torch.uint8, device)
-        self._c = CMat(self._data.data_ptr(), self._scales.data_ptr(), self.rows, self.cols)
+        self.rows, self.cols = rows, cols
+        self._data = data if data is not None else _new((rows, cols // 2), torch.uint8, device)
+        self._scales = scales if scales is not None else _new((max(scale_bytes(rows, cols), 16),), torch.uint8, device)
+        self.data_addr, self.scales_addr = self._data.data_ptr(), self._scales.data_ptr()
 
     @staticmethod
-    def _bytes(rows, cols):
-        """Bytes of codes and scales in one buffer, both on 256-byte boundaries."""
-        return _align256(rows * (cols // 2)) + max(((rows + 127) >> 7) * ((cols + 127) >> 7) * 512, 256)
-
-    def _place(self, buf, at):
-        self._buf, self._at, self._data, self._scales = buf, at, None, None
-        p = buf.data_ptr() + at
-        self._c = CMat(p, p + _align256(self.rows * (self.cols // 2)), self.rows, self.cols)
-
-    @staticmethod
-    def several(shapes, device):
-        """QMats of the given shapes in one buffer: operands that live and die together."""
+    def two(r0, c0, r1, c1, device):
+        """Two QMats in one buffer: operands that live and die together."""
         if ALLOC_HOOK is not None:
-            return [QMat(r, c, device) for r, c in shapes]
-        sizes = [QMat._bytes(r, c) for r, c in shapes]
-        buf = torch.empty(sum(sizes), dtype=torch.uint8, device=device)
-        out, at = [], 0
-        for (r, c), n in zip(shapes, sizes):
-            q = QMat.__new__(QMat)
-            q.rows, q.cols = r, c
-            q._place(buf, at)
-            out.append(q)
-            at += n
-        return out
+            return QMat(r0, c0, device), QMat(r1, c1, device)
+        buf = torch.empty(_host.nbytes(r0, c0, r1, c1), dtype=torch.uint8, device=device)
+        return _host.place(QMat, buf, buf.data_ptr(), r0, c0, r1, c1)
 
     @property
     def device(self):
@@ -241,7 +234,7 @@ class QMat:
         return self._scales
 
     def c(self):
-        return self._c
+        return CMat(self.data_addr, self.scales_addr, self.rows, self.cols)
 
     def scales_linear(self):
         """Scale bytes gathered into [rows, cols/32] order (index arithmetic only; for inspection)."""
@@ -271,27 +264,23 @@ def quantize(x, scale_mode=SCALE_TRUNCATION_FREE, rounding=ROUND_NEAREST, seed=0
     x = _bf16_2d(x)
     rows, cols = x.shape
     out = out if out is not None else QMat(rows, cols, x.device)
-    qp = _qp(scale_mode, rounding, seed, stream_id)
-    _check("mxfp4_quantize", lib().mxfp4_quantize(_ptr(x), rows, cols, x.stride(0), out.c(), C.byref(qp),
-                                                  _ptr(dev_status), _stream()))
+    _check("mxfp4_quantize", _host.quantize(lib().at_quantize, x.data_ptr(), rows, cols, x.stride(0), out, scale_mode, rounding, seed, stream_id,
+                                            _ptr(dev_status), _stream()))
     return out
 
 
 def quantize_t(src, scale_mode=SCALE_TRUNCATION_FREE, rounding=ROUND_NEAREST, seed=0, stream_id=0, out=None,
                dev_status=None):
     """Quantize along rows, emit the transposed matrix.  ``src`` is a bf16 tensor or a QMat (double quantization)."""
-    qp = _qp(scale_mode, rounding, seed, stream_id)
     if isinstance(src, QMat):
-        rows, cols = src.rows, src.cols
-        out = out if out is not None else QMat(cols, rows, src.device)
-        cm = src.c()
-        st = lib().mxfp4_quantize_t(None, C.byref(cm), rows, cols, cols, out.c(), C.byref(qp), _ptr(dev_status), _stream())
+        x, q, rows, cols = None, src, src.rows, src.cols
+        ld = cols
     else:
-        x = _bf16_2d(src)
-        rows, cols = x.shape
-        out = out if out is not None else QMat(cols, rows, x.device)
-        st = lib().mxfp4_quantize_t(_ptr(x), None, rows, cols, x.stride(0), out.c(), C.byref(qp), _ptr(dev_status), _stream())
-    _check("mxfp4_quantize_t", st)
+        x, q = _bf16_2d(src).data_ptr(), None
+        (rows, cols), ld = src.shape, src.stride(0)
+    out = out if out is not None else QMat(cols, rows, src.device)
+    _check("mxfp4_quantize_t", _host.quantize_t(lib().at_quantize_t, x, q, rows, cols, ld, out, scale_mode, rounding, seed, stream_id,
+                                                _ptr(dev_status), _stream()))
     return out
 
 
@@ -326,9 +315,6 @@ class OscState:
     def __init__(self, w_prev, wq_prev, dist_w, dist_q):
         self.w_prev, self.wq_prev, self.dist_w, self.dist_q = w_prev, wq_prev, dist_w, dist_q
 
-    def c(self):
-        return COsc(self.w_prev.data_ptr(), self.wq_prev.c(), self.dist_w.data_ptr(), self.dist_q.data_ptr())
-
 
 def qema_quantize(w, ema, beta=0.998, update_ema=True, scale_mode=SCALE_TRUNCATION_FREE, osc=None, out=None,
                   dev_status=None):
@@ -336,10 +322,9 @@ def qema_quantize(w, ema, beta=0.998, update_ema=True, scale_mode=SCALE_TRUNCATI
     assert w.is_contiguous() and ema.is_cuda and ema.dtype == torch.float32 and ema.is_contiguous() and ema.shape == w.shape
     n, k = w.shape
     out = out if out is not None else QMat(n, k, w.device)
-    co = osc.c() if osc is not None else None
-    _check("mxfp4_qema_quantize",
-           lib().mxfp4_qema_quantize(_ptr(w), _ptr(ema), C.c_float(beta), int(bool(update_ema)), n, k, out.c(), scale_mode,
-                                     C.byref(co) if co is not None else None, _ptr(dev_status), _stream()))
+    o = (osc.w_prev.data_ptr(), osc.wq_prev, osc.dist_w.data_ptr(), osc.dist_q.data_ptr()) if osc is not None else (None, None, None, None)
+    _check("mxfp4_qema_quantize", _host.qema_quantize(lib().at_qema_quantize, w.data_ptr(), ema.data_ptr(), beta, bool(update_ema), n, k, out,
+                                                      scale_mode, *o, _ptr(dev_status), _stream()))
     return out
 
 
@@ -442,13 +427,6 @@ class LinearCtx:
     def __init__(self, xq, wq, xq_t=None, seed=0, wq_t=None):
         self.xq, self.wq, self.xq_t, self.seed, self.wq_t = xq, wq, xq_t, seed, wq_t
 
-    def c(self):
-        none = _NO_MAT
-        t = self.xq_t.c() if self.xq_t is not None else none
-        wt = self.wq_t.c() if self.wq_t is not None else none
-        sd = self.seed & 0xFFFFFFFFFFFFFFFF
-        return CCtx(self.xq.c(), self.wq.c(), t, sd, wt, sd)
-
 
 def linear_fwd(x, w=None, wq=None, bias=None, scale_mode=SCALE_TRUNCATION_FREE, ctx=None, out=None, dev_status=None,
                bwd_seed=None, epi=None):
@@ -469,13 +447,13 @@ def linear_fwd(x, w=None, wq=None, bias=None, scale_mode=SCALE_TRUNCATION_FREE, 
             n = w.shape[0]
             if bwd_seed is not None and n % 32 == 0:
                 # Q4 of the backward pass comes with Q2, from the one pass over W
-                wq, wq_t = QMat.several([(n, k), (k, n)], dev)
+                wq, wq_t = QMat.two(n, k, k, n, dev)
             else:
                 wq, wq_t = QMat(n, k, dev), None
         else:
             wq_t = None
         if bwd_seed is not None:
-            xq, xq_t = QMat.several([(m, k), (k, m)], dev)
+            xq, xq_t = QMat.two(m, k, k, m, dev)
             ctx = LinearCtx(xq, wq, xq_t, bwd_seed, wq_t)
         else:
             ctx = LinearCtx(QMat(m, k, dev), wq)
@@ -485,16 +463,17 @@ def linear_fwd(x, w=None, wq=None, bias=None, scale_mode=SCALE_TRUNCATION_FREE, 
             ctx.xq_t = QMat(k, m, dev)
     n = ctx.wq.rows
     if epi is None:
-        out = out if out is not None else _new((m, n), torch.bfloat16, dev)
-    cc = ctx.c()
+        y = out = out if out is not None else _new((m, n), torch.bfloat16, dev)
+        ce = None
+    else:
+        y, ce = None, epi.c()
     if w is not None:
         w = _bf16_2d(w)
         assert w.is_contiguous()
-    ce = epi.c() if epi is not None else None
-    _check("mxfp4_linear_fwd_ex", lib().mxfp4_linear_fwd_ex(_ptr(x), x.stride(0) if x is not None else 0, m, k, _ptr(w), n, _ptr(bias),
-                                                            _ptr(out) if epi is None else None, out.stride(0) if epi is None else 0,
-                                                            C.byref(cc), scale_mode, C.byref(ce) if ce is not None else None,
-                                                            _ptr(dev_status), _stream()))
+    _check("mxfp4_linear_fwd_ex",
+           _host.linear_fwd(lib().at_linear_fwd_ex, _ptr(x), x.stride(0) if x is not None else 0, m, k, _ptr(w), n, _ptr(bias), _ptr(y),
+                            y.stride(0) if y is not None else 0, ctx.xq, ctx.wq, ctx.xq_t, ctx.wq_t, ctx.seed, scale_mode,
+                            C.addressof(ce) if ce is not None else None, _ptr(dev_status), _stream()))
     return (epi if epi is not None else out), ctx
 
 
@@ -514,15 +493,14 @@ def linear_bwd(dy, ctx, seed, scale_mode=SCALE_TRUNCATION_FREE, dw_dtype=OUT_FP3
     dw = dw if dw is not None else _new((n, k), dwt, dev)
     if workspace is None:
         workspace = _new((linear_workspace_bytes(m, k, n),), torch.uint8, dev)
-    cc = ctx.c()
     ce = epi_dx.c() if epi_dx is not None else None
-    cq, cqt = (dyq.c(), dyq_t.c()) if dy is None else (None, None)
-    _check("mxfp4_linear_bwd_ex", lib().mxfp4_linear_bwd_ex(_ptr(dy), dy.stride(0) if dy is not None else 0,
-                                                            C.byref(cq) if cq is not None else None, C.byref(cqt) if cqt is not None else None,
-                                                            C.byref(cc), seed & 0xFFFFFFFFFFFFFFFF, scale_mode,
-                                                            _ptr(dx) if epi_dx is None else None, dx.stride(0) if epi_dx is None else 0,
-                                                            _ptr(dw), dw.stride(0), dw_dtype, C.byref(ce) if ce is not None else None,
-                                                            _ptr(workspace), workspace.numel(), _ptr(dev_status), _stream()))
+    if dy is not None:
+        dyq = dyq_t = None
+    _check("mxfp4_linear_bwd_ex",
+           _host.linear_bwd(lib().at_linear_bwd_ex, _ptr(dy), dy.stride(0) if dy is not None else 0, dyq, dyq_t, ctx.xq, ctx.wq, ctx.xq_t,
+                            ctx.wq_t, ctx.seed, seed, scale_mode, _ptr(dx) if ce is None else None, dx.stride(0) if ce is None else 0,
+                            dw.data_ptr(), dw.stride(0), dw_dtype, C.addressof(ce) if ce is not None else None, workspace.data_ptr(),
+                            workspace.numel(), _ptr(dev_status), _stream()))
     return (epi_dx if epi_dx is not None else dx), dw
 
 

@@ -1,7 +1,8 @@
-"""Compile the CUDA sources into the in-tree shared library libmxfp4.so (sm_100a only)."""
+"""Compile the CUDA sources into the in-tree shared library libmxfp4.so (sm_100a only) and the binding's host module _host.so."""
 import os
 import subprocess
 import sys
+import sysconfig
 from concurrent.futures import ThreadPoolExecutor
 
 _HERE = os.path.dirname(os.path.abspath(__file__))
@@ -12,6 +13,24 @@ NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", 
               "-Xcompiler", "-fPIC", "--expt-relaxed-constexpr"]
 
 
+HOST = os.path.join(_HERE, "_host.so")
+HOST_SOURCE = os.path.join(CSRC, "host.cpp")
+
+
+def build_host(force: bool = False) -> str:
+    """Build _host.so if missing or stale; return its path."""
+    header = os.path.join(os.path.dirname(_HERE), "include", "mxfp4.h")
+    if not force and os.path.exists(HOST) and os.path.getmtime(HOST) >= max(os.path.getmtime(HOST_SOURCE), os.path.getmtime(header)):
+        return HOST
+    tmp = HOST + ".tmp.%d" % os.getpid()
+    r = subprocess.run([os.environ.get("CXX", "g++"), "-std=c++17", "-O2", "-fPIC", "-shared", "-I", sysconfig.get_paths()["include"],
+                        "-o", tmp, HOST_SOURCE], capture_output=True, text=True)
+    if r.returncode != 0:
+        raise RuntimeError("the host module does not build:\n%s\n%s" % (r.stdout, r.stderr))
+    os.replace(tmp, HOST)
+    return HOST
+
+
 def _newest_source_mtime():
     paths = [os.path.join(CSRC, f) for f in os.listdir(CSRC)]
     paths.append(os.path.join(os.path.dirname(_HERE), "include", "mxfp4.h"))
@@ -19,7 +38,8 @@ def _newest_source_mtime():
 
 
 def build(force: bool = False, verbose: bool = False, extra_flags=()) -> str:
-    """Build libmxfp4.so if missing or stale; return its path.  nvcc cross-compiles without a GPU."""
+    """Build libmxfp4.so and _host.so if missing or stale; return the former's path.  nvcc cross-compiles without a GPU."""
+    build_host(force)
     if not force and os.path.exists(LIB) and os.path.getmtime(LIB) >= _newest_source_mtime():
         return LIB
     nvcc = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")

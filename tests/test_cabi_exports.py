@@ -53,3 +53,19 @@ def test_missing_library_fails_loudly(monkeypatch):
     monkeypatch.setattr(b, "LIB_PATH", "/nonexistent/libmxfp4.so")
     with pytest.raises(RuntimeError):
         b.lib()
+
+
+@pytest.mark.parametrize("rows,cols", [(1, 32), (127, 96), (128, 128), (129, 160), (197, 384)])
+def test_matrices_in_one_buffer(rows, cols):
+    import paper_2502_20853_b200 as mx
+    a, b = mx.QMat.two(rows, cols, cols, (rows + 31) // 32 * 32, "cpu")
+    at = a._buf.data_ptr()
+    for q in (a, b, mx.QMat(rows, cols, "cpu")):
+        at = at if q._buf is a._buf else q._buf.data_ptr()
+        assert q.data.data_ptr() == q.c().data == q.data_addr >= at and (q.data_addr - q._buf.data_ptr()) % 256 == 0
+        assert q.scales.data_ptr() == q.c().scales >= q.data_addr + q.data.numel() and (q.scales_addr - q._buf.data_ptr()) % 256 == 0
+        assert q.data.shape == (q.rows, q.cols // 2) and q.scales.numel() >= mx.scale_bytes(q.rows, q.cols)
+        at = q.scales_addr + q.scales.numel()
+        assert at <= q._buf.data_ptr() + q._buf.numel()
+    with pytest.raises(TypeError):
+        mx.binding._host.quantize(0, 0, 0, 0, 0, "no matrix", 0, 0, 0, 0, 0, 0)
