@@ -27,10 +27,7 @@ constexpr int kEpiWarps = 8;
 constexpr int kGemmThreads = 32 * (kEpiWarp0 + kEpiWarps);
 constexpr int kStagingBytes = 2048;             // per epilogue warp: 32 rows x 64 bytes
 
-// DEEP = false: the longest ring, one staging buffer per epilogue warp (long K loops).
-// DEEP = true : a shorter ring and four staging buffers per epilogue warp, so that a warp can drain its part of the
-//               accumulator without waiting for its own stores (short K loops, where the epilogue is the larger part).
-template <int BN, bool DEEP>
+template <int BN>
 struct GemmCfg {
     static constexpr int kRB = (BN + 127) / 128;                        // 128-row scale blocks of B per tile
     static constexpr int kABytes = kBM * kBKBytes;                      // 16 KB
@@ -38,8 +35,8 @@ struct GemmCfg {
     static constexpr int kSfaBytes = 2 * kSfChunk;                      // two K chunks of 128 elements
     static constexpr int kSfbBytes = 2 * kSfChunk * kRB;
     static constexpr int kStageBytes = kABytes + kBBytes + kSfaBytes + kSfbBytes;
-    static constexpr int kStages = BN <= 128 ? (DEEP ? 4 : 6) : BN <= 192 ? 4 : (DEEP ? 3 : 4);
-    static constexpr int kStagingBufs = BN == 192 ? 3 : (DEEP ? (BN / 64) : 1);   // DEEP / 192: one buffer per 32-column chunk of a warp's share
+    static constexpr int kStages = BN <= 128 ? 5 : 4;
+    static constexpr int kStagingBufs = BN <= 192 ? BN / 64 : 1;        // up to 192: one buffer per 32-column chunk of a warp's share
     static constexpr int kAccStages = (BN <= 192) ? 2 : 1;              // tiles up to 192 wide leave room for two accumulators
     static constexpr int kSfCol = kAccStages * BN;                      // TMEM columns: accumulators, then per ring stage SFA (8) + SFB (8 kRB)
     static constexpr int kSfSlot = 8 + 8 * kRB;
@@ -552,12 +549,12 @@ __device__ __forceinline__ void gemm_feed_roles(int warp, uint32_t smem_base, ui
 }
 
 // ---- the kernel ------------------------------------------------------------------------------------
-template <int BN, bool DEEP>
+template <int BN>
 __global__ void __launch_bounds__(kGemmThreads, 1)
 k_gemm_mxf4(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b,
             const __grid_constant__ CUtensorMap map_d, const __grid_constant__ CUtensorMap map_dw, const GemmParams p)
 {
-    using C = GemmCfg<BN, DEEP>;
+    using C = GemmCfg<BN>;
     extern __shared__ uint8_t smem_raw[];
     uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
     uint64_t *bars = reinterpret_cast<uint64_t *>(smem + C::kBarOff);
@@ -1521,7 +1518,7 @@ __global__ void __launch_bounds__(128, 1) k_mma_ceiling(int iters, uint32_t *dev
 // leader.  Stage and accumulator releases reach both CTAs through multicast commits.
 // BN = 192: 256 x 192 tiles for output widths that are multiples of 192 but not of 256.  Narrower stages (31 KB), two
 // accumulators (the next tile's K loop runs under the epilogue), which leaves TMEM columns for the scales of five stages.
-template <bool DEEP, int BN>
+template <int BN>
 struct Gemm2Cfg {
     static constexpr int kABytes = kBM * kBKBytes;                      // 16 KB: this CTA's 128 rows of A
     static constexpr int kBBytes = (BN / 2) * kBKBytes;                 // this CTA's half of the B rows
@@ -1529,10 +1526,11 @@ struct Gemm2Cfg {
     static constexpr int kSfbBytes = 2 * kSfChunk * 2;                  // all B rows: the two 128-row blocks a tile touches
     static constexpr int kStageBytes = kABytes + kBBytes + kSfaBytes + kSfbBytes;   // 35 KB / 31 KB
     // The loop is bound by operand bytes in flight over load latency, so every stage counts: six stages and a single
-    // staging buffer per epilogue warp for long K loops (177 against 187 us at 8192^3), and no slack for aligning the
-    // window: the kernel declares its window 1024-byte aligned and checks that it is.
-    static constexpr int kStages = BN == 192 ? 5 : DEEP ? 4 : 6;
-    static constexpr int kStagingBufs = BN == 192 ? 3 : DEEP ? 4 : 1;
+    // staging buffer per epilogue warp (8192^3 184 us, 198 with five and three, 187 with no slack to align the window: the kernel
+    // declares its window 1024-byte aligned and checks that it is).  So do short K loops, whose epilogue is the larger part: with four
+    // stages and four buffers 50432 x 1024 x 1536 took 52.6 us, 43.6 with five and three, and takes 38.8.
+    static constexpr int kStages = BN == 192 ? 5 : 6;
+    static constexpr int kStagingBufs = BN == 192 ? 3 : 1;
     static constexpr int kAccStages = BN == 192 ? 2 : 1;
     static constexpr int kSfCol = kAccStages * BN;                      // TMEM: accumulators, then per ring stage SFA (8) + SFB (16)
     static constexpr int kSfSlot = 24;
@@ -1626,13 +1624,13 @@ __device__ __forceinline__ uint32_t idesc_mxf4_pair(uint32_t a_sf_id, uint32_t b
     return (b_sf_id << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(n >> 3) << 17) | (1u << 23) | ((uint32_t)(256 >> 4) << 24) | (a_sf_id << 29);
 }
 
-template <bool DEEP, int BN>
+template <int BN>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kGemmThreads, 1)
 k_gemm_mxf4_pair(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b,
                  const __grid_constant__ CUtensorMap map_sfa, const __grid_constant__ CUtensorMap map_sfb,
                  const __grid_constant__ CUtensorMap map_d, const __grid_constant__ CUtensorMap map_dw, const GemmParams p)
 {
-    using C = Gemm2Cfg<DEEP, BN>;
+    using C = Gemm2Cfg<BN>;
     extern __shared__ __align__(1024) uint8_t smem_aligned[];
     uint8_t *smem = smem_aligned;
     if (smem_u32(smem) & 1023u) {   // the swizzled operand tiles need it; nothing has been set up yet, so everybody just leaves
@@ -2322,7 +2320,6 @@ static bool make_output_map_wide(CUtensorMap *map, void *d, int64_t m, int64_t n
 }
 
 struct GemmPlan {
-    bool deep;   // short K loop per tile: favour the epilogue (more staging, shorter ring)
     bool pair;   // 256 x 256 tiles on pairs of CTAs (cta_group::2)
     int bs;      // B-stationary kernel: 0 = no, 1 = 192 wide, up to 2 K tiles
     int ck;      // cluster split-K kernel: 0 = no, else the cluster size (CTAs sharing one 128 x 192 tile)
@@ -2342,6 +2339,7 @@ static GemmPlan plan_gemm(int64_t m, int64_t n, int64_t kc, int sms, bool allow_
     g.bs = 0;
     g.ck = 0;
     g.pbs = false;
+    const int64_t rows = ceil_div(m, kBM), tiles128 = rows * ceil_div(n, 128), tiles192 = rows * ceil_div(n, 192);
     if (g.kt_total >= 16) {
         // Few tiles, long contraction (weight-gradient products): pairs of CTAs share a 128 x 192 tile and add their
         // halves of the contraction through distributed shared memory, when that fills between half and all of the
@@ -2354,11 +2352,23 @@ static GemmPlan plan_gemm(int64_t m, int64_t n, int64_t kc, int sms, bool allow_
     if (g.ck) {
         g.bn = 192;
         g.pair = false;
-        g.deep = false;
         g.tiles_m = (int)ceil_div(m, kBM);
         g.tiles_n = (int)ceil_div(n, g.bn);
         g.splits = 1;                                   // nothing goes through a workspace
         g.kt_per_split = (int)ceil_div(g.kt_total, g.ck);
+        return g;
+    }
+    if (tiles128 <= sms && (!allow_split || g.kt_total < 8)) {
+        // One tile per SM at most: the time is one tile's, from the launch to its last store, and the narrowest tile has the shortest.
+        // Back to back, against the wide kernels below, in us: 197 x 1536 x 384 5.7 -> 4.3, 1024 x 768 x 192 5.2 -> 4.2,
+        // 1024 x 1024 x 1536 7.7 -> 5.5, 128 x 4096 x 2048 9.0 -> 5.9.  (768 x 768 x 2048 would take 6.3 us this way, 9.6 with K split;
+        // but split sums are the more accurate ones, and the faster ones from about 768 x 768 x 8192 on: 12.8 us on either.)
+        g.bn = 128;
+        g.pair = false;
+        g.tiles_m = (int)rows;
+        g.tiles_n = (int)ceil_div(n, 128);
+        g.splits = 1;
+        g.kt_per_split = g.kt_total;
         return g;
     }
     if (g.kt_total >= 3 && g.kt_total <= 4 && n >= 192 && m >= 2048 && sms >= 2 &&
@@ -2370,7 +2380,6 @@ static GemmPlan plan_gemm(int64_t m, int64_t n, int64_t kc, int sms, bool allow_
         g.pbs = true;
         g.bn = 192;
         g.pair = false;
-        g.deep = false;
         g.tiles_m = (int)ceil_div(m, kBM);
         g.tiles_n = (int)ceil_div(n, g.bn);
         g.splits = 1;
@@ -2383,27 +2392,26 @@ static GemmPlan plan_gemm(int64_t m, int64_t n, int64_t kc, int sms, bool allow_
         g.bs = 1;
         g.bn = 192;
         g.pair = false;
-        g.deep = false;
         g.tiles_m = (int)ceil_div(m, kBM);
         g.tiles_n = (int)ceil_div(n, g.bn);
         g.splits = 1;
         g.kt_per_split = g.kt_total;
         return g;
     }
+    // One wave of 192-wide tiles on single CTAs, where K would not be split, up to 32 K tiles (6272 x 512 x 1536 8.9 -> 7.0 us,
+    // 4096 x 768 x 2048 11.1 -> 8.9, x 8192 18.4 on either, x 16384 28.3 -> 31.0).
+    const bool one_wave = tiles192 <= sms && g.kt_total <= 32 && (!allow_split || ceil_div(rows, 2) * ceil_div(n, 256) * 4 > sms);
     if (n <= 128) g.bn = 128;
-    else if (kc <= 1024 || n < 256 || (kc <= 2304 && n % 256 != 0 && n % 192 == 0)) g.bn = 192;
+    else if (kc <= 1024 || one_wave) g.bn = 192;
     else g.bn = 256;
     g.pair = g.bn == 256 && m > 128 && sms >= 2;
     // 256 x 192 tiles on pairs, for widths that 256-wide tiles waste a quarter of or more, when K is split (1536 x 384 x 25216
-    // 16.7 -> 15.8 us, 384 x 384 x 25216 12.1 -> 11.0, 512 x 384 x 4096 9.5 -> 8.8), and in place of the single-CTA 192-wide
-    // kernel from four tiles per pair on (50432 x 1152 x 1280 53.7 -> 46.1; with 2.7 tiles per pair, 25216 x 384 x 1536, both
-    // take 15.6).  For long K loops that fill the machine the 256-wide pair with its sixth stage is faster even with the
-    // waste (50432 x 960 x 4096: 82 against 96 us).
-    if (m > 128 && n % 192 == 0 && n % 256 != 0 && kc > 1024 && sms >= 2) {
-        const int64_t pairs = sms / 2, tm2 = ceil_div(ceil_div(m, kBM), 2);
-        const bool split = allow_split && g.kt_total >= 8 && tm2 * ceil_div(n, 256) * 2 <= pairs;
-        if ((split && n <= 576) || (g.bn == 192 && tm2 * (n / 192) >= 4 * pairs)) g.pair = true, g.bn = 192;
-    }
+    // 16.7 -> 15.8 us, 384 x 384 x 25216 12.1 -> 11.0, 512 x 384 x 4096 9.5 -> 8.8).  K loops that are not split are faster on the 256-wide
+    // pair with its sixth stage, even with the waste (25216 x 1152 x 1536 27.7 us on single CTAs, 25.1 on the pair; 50432 x 1152 x 2048
+    // 64.6 with 192-wide pairs, 57.7; 50432 x 960 x 4096 96 and 82; 50432 x 224 x 1536 22.6 and 15.5).
+    if (m > 128 && n % 192 == 0 && n % 256 != 0 && n <= 576 && kc > 1024 && sms >= 2 && allow_split && g.kt_total >= 8 &&
+        ceil_div(ceil_div(m, kBM), 2) * ceil_div(n, 256) * 2 <= sms / 2)
+        g.pair = true, g.bn = 192;
     g.tiles_m = (int)ceil_div(m, kBM);
     g.tiles_n = (int)ceil_div(n, g.bn);
     const int units = (g.pair ? (g.tiles_m + 1) / 2 : g.tiles_m) * g.tiles_n;   // work items before splitting K
@@ -2415,7 +2423,6 @@ static GemmPlan plan_gemm(int64_t m, int64_t n, int64_t kc, int sms, bool allow_
     }
     g.kt_per_split = (int)ceil_div(g.kt_total, splits);
     g.splits = (int)ceil_div(g.kt_total, g.kt_per_split);
-    g.deep = g.kt_per_split <= 8;   // K loop of at most 2048 per tile
     return g;
 }
 
@@ -2432,14 +2439,14 @@ static bool ensure_device_ok()
     return ok[dev] == 1;
 }
 
-template <bool DEEP, int BN>
+template <int BN>
 static mxfp4_status_t launch_gemm_pair(const CUtensorMap &ma, const CUtensorMap &mb, const CUtensorMap &msa, const CUtensorMap &msb,
                                        const CUtensorMap &md, const CUtensorMap &mdw, const GemmParams &p, int grid, cudaStream_t st)
 {
-    using C = Gemm2Cfg<DEEP, BN>;
+    using C = Gemm2Cfg<BN>;
     static bool attr_set[kMaxDevices];
-    MX_CHECK_CUDA(set_smem_once(attr_set, k_gemm_mxf4_pair<DEEP, BN>, C::kSmemBytes));
-    MX_CHECK_CUDA(launch_pdl(k_gemm_mxf4_pair<DEEP, BN>, (unsigned)grid, 1, kGemmThreads, C::kSmemBytes, st, ma, mb, msa, msb, md, mdw, p));
+    MX_CHECK_CUDA(set_smem_once(attr_set, k_gemm_mxf4_pair<BN>, C::kSmemBytes));
+    MX_CHECK_CUDA(launch_pdl(k_gemm_mxf4_pair<BN>, (unsigned)grid, 1, kGemmThreads, C::kSmemBytes, st, ma, mb, msa, msb, md, mdw, p));
     return MXFP4_OK;
 }
 
@@ -2491,14 +2498,14 @@ static mxfp4_status_t launch_gemm_ck(const CUtensorMap &ma, const CUtensorMap &m
     return MXFP4_OK;
 }
 
-template <int BN, bool DEEP>
+template <int BN>
 static mxfp4_status_t launch_gemm(const CUtensorMap &ma, const CUtensorMap &mb, const CUtensorMap &md, const CUtensorMap &mdw,
                                   const GemmParams &p, int grid, cudaStream_t st)
 {
-    using C = GemmCfg<BN, DEEP>;
+    using C = GemmCfg<BN>;
     static bool attr_set[kMaxDevices];
-    MX_CHECK_CUDA(set_smem_once(attr_set, k_gemm_mxf4<BN, DEEP>, C::kSmemBytes));
-    MX_CHECK_CUDA(launch_pdl(k_gemm_mxf4<BN, DEEP>, (unsigned)grid, 1, kGemmThreads, C::kSmemBytes, st, ma, mb, md, mdw, p));
+    MX_CHECK_CUDA(set_smem_once(attr_set, k_gemm_mxf4<BN>, C::kSmemBytes));
+    MX_CHECK_CUDA(launch_pdl(k_gemm_mxf4<BN>, (unsigned)grid, 1, kGemmThreads, C::kSmemBytes, st, ma, mb, md, mdw, p));
     return MXFP4_OK;
 }
 
@@ -2602,11 +2609,10 @@ static mxfp4_status_t gemm_impl(mxfp4_mat_t a, mxfp4_mat_t b, void *d, int64_t l
     if (!store_fp32 && !make_output_map_wide(&mdw, d, M, N, ldd)) return MXFP4_CUDA_ERROR;
     mxfp4_status_t s = g.pbs         ? launch_gemm_pbs<4, 8>(ma, mb, msa, msb, md, mdw, p, grid, st)
                        : g.bs == 1   ? launch_gemm_bs<192, 2, 7>(ma, mb, md, mdw, p, grid, st)
-                       : g.pair && g.bn == 192 ? launch_gemm_pair<false, 192>(ma, mb, msa, msb, md, mdw, p, grid, st)
-                       : g.pair      ? (g.deep ? launch_gemm_pair<true, 256>(ma, mb, msa, msb, md, mdw, p, grid, st) : launch_gemm_pair<false, 256>(ma, mb, msa, msb, md, mdw, p, grid, st))
-                       : g.bn == 256 ? (g.deep ? launch_gemm<256, true>(ma, mb, md, mdw, p, grid, st) : launch_gemm<256, false>(ma, mb, md, mdw, p, grid, st))
-                       : g.bn == 192 ? launch_gemm<192, false>(ma, mb, md, mdw, p, grid, st)
-                                     : (g.deep ? launch_gemm<128, true>(ma, mb, md, mdw, p, grid, st) : launch_gemm<128, false>(ma, mb, md, mdw, p, grid, st));
+                       : g.pair      ? (g.bn == 192 ? launch_gemm_pair<192>(ma, mb, msa, msb, md, mdw, p, grid, st) : launch_gemm_pair<256>(ma, mb, msa, msb, md, mdw, p, grid, st))
+                       : g.bn == 256 ? launch_gemm<256>(ma, mb, md, mdw, p, grid, st)
+                       : g.bn == 192 ? launch_gemm<192>(ma, mb, md, mdw, p, grid, st)
+                                     : launch_gemm<128>(ma, mb, md, mdw, p, grid, st);
     if (s) return s;
     if (g.splits > 1 && !withhold_loads) {
         const int groups = g.splits >= 8 && M * N / 4 < 64 * 256 ? 8 : 1;   // fewer than 64 blocks otherwise

@@ -198,6 +198,15 @@ def test_gemm_b_stationary_walk(mx, M, N, K, out_dtype):
     _bias_case(mx, M, N, K, out_dtype)
 
 
+# on 148 SMs: one wave of 128-wide tiles up to its last tile and its longest K loop, and just beyond either; one wave of 192-wide tiles
+# and beyond (256-wide pairs)
+@pytest.mark.parametrize("M,N,K", [(18900, 128, 544), (4700, 512, 1056), (1024, 512, 1792), (1024, 512, 1824), (6300, 384, 544), (6270, 512, 1568),
+                                   (9500, 512, 1568), (1, 8, 1760)])
+@pytest.mark.parametrize("out_dtype", [0, 1])
+def test_gemm_one_wave_and_beyond(mx, M, N, K, out_dtype):
+    _bias_case(mx, M, N, K, out_dtype)
+
+
 def test_gemm_argument_errors(mx):
     a, b = mx.QMat(128, 64), mx.QMat(128, 96)
     with pytest.raises(mx.MxError) as e:

@@ -54,6 +54,14 @@ def test_gemm_waits_run_out_and_the_kernel_drains(mx, M, N, K, out_dtype):
     check_gemm_bound(d.float().cpu().numpy(), dref, tref, bf16_out=(out_dtype == 0), what="gemm after the self-test")
 
 
+# the kernels of products of more than one wave: B-stationary, CTA pairs with and without split K, one CTA per tile
+# (192 wide)
+@pytest.mark.parametrize("M,N,K", [(9600, 384, 512), (1024, 512, 8192), (9500, 512, 1536), (6272, 512, 1536)])
+@pytest.mark.parametrize("out_dtype", [0, 1])
+def test_gemm_waits_run_out_beyond_one_wave(mx, M, N, K, out_dtype):
+    test_gemm_waits_run_out_and_the_kernel_drains(mx, M, N, K, out_dtype)
+
+
 def test_quantizer_waits_run_out_and_the_kernel_drains(mx):
     rng = np.random.default_rng(9)
     x = rng.standard_normal((384, 320)).astype(np.float32)
