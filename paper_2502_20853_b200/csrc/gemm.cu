@@ -77,6 +77,7 @@ struct GemmParams {
     // the walk of the B-stationary kernels, see Walk
     FastDiv by_rest_rows, by_rest_workers;
     int abreast, rounds, rows, rest_row0, share, extra;
+    int head;             // second product of a launch of CTA pairs: see pair_item
     int out_fp32;         // element type of the stored tile (FP32 also for split-K partials)
     const __nv_bfloat16 *bias;   // applied only when splits == 1 (and by the cluster kernel, whose sum is complete)
     uint32_t *dev_status;
@@ -85,6 +86,16 @@ struct GemmParams {
     uint32_t spin_limit;  // polls after which a bounded wait gives up (kWaitSpinLimit in normal use)
     int withhold_loads;   // self-test of the drain path: the producers issue nothing, so every wait runs out
 };
+
+// One product of a launch, and the one or two products of a launch.
+struct GemmJob {
+    CUtensorMap a, b, d, dw;
+    GemmParams p;
+};
+struct PairJob : GemmJob {
+    CUtensorMap sfa, sfb;
+};
+struct NoJob {};
 
 // How the workers (CTAs, or pairs of them) of the B-stationary kernels share the tiles.  A worker keeps the B block of its tile
 // column for as long as it can, and all workers write the same stretch of the output at the same time: stores to many distant
@@ -409,7 +420,8 @@ __device__ __forceinline__ void epilogue_tile(const CUtensorMap *map_d, const CU
 template <class C, int BN>
 __device__ __forceinline__ void gemm_feed_roles(int warp, uint32_t smem_base, uint32_t bar_full, uint32_t bar_sf_full, uint32_t bar_empty,
                                                 uint32_t bar_acc_full, uint32_t bar_acc_empty, uint32_t tmem_base, volatile uint32_t *abort_flag,
-                                                const CUtensorMap &map_a, const CUtensorMap &map_b, const GemmParams &p)
+                                                const CUtensorMap &map_a, const CUtensorMap &map_b, const GemmParams &p, int block,
+                                                int blocks)
 {
     const int items = p.tiles_m * p.tiles_n * p.splits;
     if (warp == 0 || warp == 3) {
@@ -422,7 +434,7 @@ __device__ __forceinline__ void gemm_feed_roles(int warp, uint32_t smem_base, ui
             uint32_t stage = 0, phase = 0;
             bool alive = true;
             pdl_wait();        // the roles that touch global memory wait for the preceding kernel: the producers and the epilogue
-            for (int item = blockIdx.x; item < items && alive; item += gridDim.x) {
+            for (int item = block; item < items && alive; item += blocks) {
                 const int tile = p.by_splits.div(item), split = item - tile * p.splits;
                 const int mb = p.by_tiles_n.div(tile), nb = tile - mb * p.tiles_n;
                 const int kt0 = split * p.kt_per_split;
@@ -466,7 +478,7 @@ __device__ __forceinline__ void gemm_feed_roles(int warp, uint32_t smem_base, ui
             const bool leader = elect_one();
             uint32_t stage = 0, phase = 0;
             bool alive = true;
-            for (int item = blockIdx.x; item < items && alive; item += gridDim.x) {
+            for (int item = block; item < items && alive; item += blocks) {
                 const int split = p.by_splits.mod(item);
                 const int kt0 = split * p.kt_per_split;
                 const int kt1 = min(kt0 + p.kt_per_split, p.kt_total);
@@ -507,7 +519,7 @@ __device__ __forceinline__ void gemm_feed_roles(int warp, uint32_t smem_base, ui
             const int nmma_last = (int)((p.Kc - (int64_t)(p.kt_total - 1) * kBKElems + 63) / 64);   // MMAs of the last K tile
             bool ready = false;   // the current stage's scales (hence operands) are known to be in place
             bool alive = true;
-            for (int item = blockIdx.x; item < items && alive; item += gridDim.x) {
+            for (int item = block; item < items && alive; item += blocks) {
                 const int tile = p.by_splits.div(item), split = item - tile * p.splits;
                 const int nb = p.by_tiles_n.mod(tile);
                 const int kt0 = split * p.kt_per_split;
@@ -549,12 +561,17 @@ __device__ __forceinline__ void gemm_feed_roles(int warp, uint32_t smem_base, ui
 }
 
 // ---- the kernel ------------------------------------------------------------------------------------
-template <int BN>
+template <int BN, class Job2>   // Job2 = GemmJob: the blocks behind those of the first product's tiles make a second one; NoJob: there is none
 __global__ void __launch_bounds__(kGemmThreads, 1)
-k_gemm_mxf4(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b,
-            const __grid_constant__ CUtensorMap map_d, const __grid_constant__ CUtensorMap map_dw, const GemmParams p)
+k_gemm_mxf4(const __grid_constant__ GemmJob one, const __grid_constant__ Job2 two)
 {
     using C = GemmCfg<BN>;
+    constexpr bool kTwo = sizeof(Job2) == sizeof(GemmJob);
+    const int blocks1 = one.p.tiles_m * one.p.tiles_n;
+    const bool second = kTwo && (int)blockIdx.x >= blocks1;
+    const GemmJob &job = second ? reinterpret_cast<const GemmJob &>(two) : one;
+    const GemmParams &p = job.p;
+    const int block = (int)blockIdx.x - (second ? blocks1 : 0), blocks = !kTwo ? (int)gridDim.x : second ? (int)gridDim.x - blocks1 : blocks1;
     extern __shared__ uint8_t smem_raw[];
     uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
     uint64_t *bars = reinterpret_cast<uint64_t *>(smem + C::kBarOff);
@@ -570,7 +587,7 @@ k_gemm_mxf4(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const uint32_t smem_base = smem_u32(smem);
 
-    if (threadIdx.x == 32 * 3) { prefetch_map(&map_a); prefetch_map(&map_b); prefetch_map(&map_d); prefetch_map(&map_dw); }
+    if (threadIdx.x == 32 * 3) { prefetch_map(&job.a); prefetch_map(&job.b); prefetch_map(&job.d); prefetch_map(&job.dw); }
     if (threadIdx.x == 0) {
         for (int s = 0; s < C::kStages; s++) {
             mbar_init(bar_full + 8 * s, 1);
@@ -596,7 +613,7 @@ k_gemm_mxf4(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
     const int items = p.tiles_m * p.tiles_n * p.splits;
 
     if (warp < kEpiWarp0) {
-        gemm_feed_roles<C, BN>(warp, smem_base, bar_full, bar_sf_full, bar_empty, bar_acc_full, bar_acc_empty, tmem_base, abort_flag, map_a, map_b, p);
+        gemm_feed_roles<C, BN>(warp, smem_base, bar_full, bar_sf_full, bar_empty, bar_acc_full, bar_acc_empty, tmem_base, abort_flag, job.a, job.b, p, block, blocks);
     } else if (warp >= kEpiWarp0) {
         // ================= epilogue (warps 4..11) =================
         pdl_wait();
@@ -610,7 +627,7 @@ k_gemm_mxf4(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
         constexpr int kChunks = kHalfCols / 32;
         uint32_t acc = 0, acc_phase = 0;
         bool alive = true;
-        for (int item = blockIdx.x; item < items && alive; item += gridDim.x) {
+        for (int item = block; item < items && alive; item += blocks) {
             const int tile = p.by_splits.div(item), split = item - tile * p.splits;
             const int mb = p.by_tiles_n.div(tile), nb = tile - mb * p.tiles_n;
             uint32_t bias[(kHalfCols + 63) / 64];
@@ -621,7 +638,7 @@ k_gemm_mxf4(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
             const int colbase = nb * BN + chalf * kHalfCols;
             const uint32_t taddr = tmem_base + ((uint32_t)(quarter * 32) << 16) + acc * BN + chalf * kHalfCols;
             if (p.bias != nullptr) bias_stage<kHalfCols>(bias, bias_line, lane);
-            epilogue_tile<BN, C::kStagingBufs>(&map_d, p.out_fp32 ? nullptr : &map_dw, p, taddr, row0, colbase, split, staging, sbuf, lane,
+            epilogue_tile<BN, C::kStagingBufs>(&job.d, p.out_fp32 ? nullptr : &job.dw, p, taddr, row0, colbase, split, staging, sbuf, lane,
                                                bar_acc_empty + 8 * acc, bias_line);
             if (++acc == C::kAccStages) { acc = 0; acc_phase ^= 1u; }
         }
@@ -741,7 +758,8 @@ k_gemm_mxf4_q(const __grid_constant__ CUtensorMap map_a, const __grid_constant__
     const uint32_t tmem_base = *tmem_slot;
 
     if (warp < kEpiWarp0) {
-        gemm_feed_roles<C, BN>(warp, smem_base, bar_full, bar_sf_full, bar_empty, bar_acc_full, bar_acc_empty, tmem_base, abort_flag, map_a, map_b, p);
+        gemm_feed_roles<C, BN>(warp, smem_base, bar_full, bar_sf_full, bar_empty, bar_acc_full, bar_acc_empty, tmem_base, abort_flag, map_a, map_b, p, blockIdx.x,
+                               gridDim.x);
     } else {
         // ================= quantizing epilogue (warps 4..11 = 256 threads) =================
         pdl_wait();
@@ -1624,18 +1642,65 @@ __device__ __forceinline__ uint32_t idesc_mxf4_pair(uint32_t a_sf_id, uint32_t b
     return (b_sf_id << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(n >> 3) << 17) | (1u << 23) | ((uint32_t)(256 >> 4) << 24) | (a_sf_id << 29);
 }
 
-template <int BN>
+// The work items (tile, part of the contraction) of one CTA pair.  Two products in one launch (the weight gradient and the input
+// gradient of a layer): the first has the longer items.  The pairs take its items in turn; those that this leaves with one
+// item fewer start on the second product, `head` rounds ahead of the others.
+struct PairItem {
+    bool second, done;
+    int mb2, nb, split;
+};
+struct PairWalk {
+    int w, workers, items, items2;   // this pair, the pairs of the launch, the items of either product
+    int mine, full, ahead;           // this pair's items of the first; pairs with one item more, and with one fewer (all, when none has more)
+};
+__device__ __forceinline__ int pair_items(const GemmParams &p) { return ((p.tiles_m + 1) >> 1) * p.tiles_n * p.splits; }
+template <bool TWO> __device__ __forceinline__ PairWalk pair_walk(const GemmParams &p, const GemmParams &p2)
+{
+    PairWalk k;
+    k.w = blockIdx.x >> 1, k.workers = gridDim.x >> 1;
+    k.items = pair_items(p);
+    if (TWO) {
+        k.items2 = pair_items(p2);
+        k.mine = (k.items - k.w + k.workers - 1) / k.workers;
+        k.full = k.items % k.workers;
+        k.ahead = k.workers - k.full;
+    }
+    return k;
+}
+template <bool TWO> __device__ __forceinline__ PairItem pair_item(const GemmParams &p, const GemmParams &p2, const PairWalk &k, int i)
+{
+    PairItem x;
+    int item = k.w + i * k.workers;
+    x.second = false;
+    x.done = item >= k.items;
+    const GemmParams *q = &p;
+    if (TWO && x.done) {
+        const int j = i - k.mine, head = p2.head;
+        item = k.w >= k.full && j < head ? j * k.ahead + k.w - k.full : head * k.ahead + (k.w >= k.full ? j - head : j) * k.workers + k.w;
+        x.second = true;
+        x.done = item >= k.items2;
+        q = &p2;
+    }
+    const int tile = q->by_splits.div(item), tm = q->by_tiles_n.div(tile);
+    x.split = item - tile * q->splits;
+    x.mb2 = ((q->tiles_m + 1) >> 1) - 1 - tm;
+    x.nb = tile - tm * q->tiles_n;
+    return x;
+}
+
+template <int BN, class Job2>   // Job2 = PairJob: a second product follows; NoJob: there is none
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kGemmThreads, 1)
-k_gemm_mxf4_pair(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b,
-                 const __grid_constant__ CUtensorMap map_sfa, const __grid_constant__ CUtensorMap map_sfb,
-                 const __grid_constant__ CUtensorMap map_d, const __grid_constant__ CUtensorMap map_dw, const GemmParams p)
+k_gemm_mxf4_pair(const __grid_constant__ PairJob one, const __grid_constant__ Job2 two)
 {
     using C = Gemm2Cfg<BN>;
+    constexpr bool kTwo = sizeof(Job2) == sizeof(PairJob);
+    const PairJob *const job2 = kTwo ? reinterpret_cast<const PairJob *>(&two) : &one;
+    const GemmParams &p0 = one.p;   // what both products share: limits, status
     extern __shared__ __align__(1024) uint8_t smem_aligned[];
     uint8_t *smem = smem_aligned;
     if (smem_u32(smem) & 1023u) {   // the swizzled operand tiles need it; nothing has been set up yet, so everybody just leaves
         pdl_wait();
-        if (threadIdx.x == 0 && p.dev_status) atomicOr(p.dev_status, MXFP4_DEV_SMEM_LAYOUT);
+        if (threadIdx.x == 0 && p0.dev_status) atomicOr(p0.dev_status, MXFP4_DEV_SMEM_LAYOUT);
         return;
     }
     uint64_t *bars = reinterpret_cast<uint64_t *>(smem + C::kBarOff);
@@ -1653,7 +1718,7 @@ k_gemm_mxf4_pair(const __grid_constant__ CUtensorMap map_a, const __grid_constan
     const uint32_t smem_base = smem_u32(smem);
     const uint32_t rank = cluster_rank();
 
-    if (threadIdx.x == 32 * 3) { prefetch_map(&map_a); prefetch_map(&map_b); prefetch_map(&map_sfa); prefetch_map(&map_sfb); prefetch_map(&map_d); }
+    if (threadIdx.x == 32 * 3) { prefetch_map(&one.a); prefetch_map(&one.b); prefetch_map(&one.sfa); prefetch_map(&one.sfb); prefetch_map(&one.d); }
     if (threadIdx.x == 0) {
         for (int s = 0; s < C::kStages; s++) {
             mbar_init(bar_full + 8 * s, 1);
@@ -1677,27 +1742,28 @@ k_gemm_mxf4_pair(const __grid_constant__ CUtensorMap map_a, const __grid_constan
     tc_fence_after();
     const uint32_t tmem_base = *tmem_slot;
 
-    const int tiles_m2 = (p.tiles_m + 1) >> 1;
-    const int items = tiles_m2 * p.tiles_n * p.splits;
-    const int cluster_id = blockIdx.x >> 1, num_clusters = gridDim.x >> 1;
+    const PairWalk walk = pair_walk<kTwo>(one.p, job2->p);
 
     if (warp == 0 || warp == 3) {
         // ===== TMA producers (both CTAs: own rows of A and own half of B by warp 0; own SFA and all of SFB by warp 3) =====
         // All loads of both CTAs complete on the LEADER's full barrier (the cta_group::2 form of the load allows the
         // barrier to live in the other CTA of the pair), so the leader learns that a stage has landed in both shared
         // memories without any message between the CTAs.  The leader's warp 0 posts the byte count of both.
-        const bool leader = elect_one() && !p.withhold_loads;
+        const bool leader = elect_one() && !p0.withhold_loads;
         const bool operands = warp == 0;
         uint32_t stage = 0, phase = 0;
         bool alive = true;
         pdl_wait();
-        for (int item = cluster_id; item < items && alive; item += num_clusters) {
-            const int tile = p.by_splits.div(item), split = item - tile * p.splits;
-            const int tm = p.by_tiles_n.div(tile), mb = (tiles_m2 - 1 - tm) * 2 + (int)rank, nb = tile - tm * p.tiles_n;
-            const int kt0 = split * p.kt_per_split;
+        for (int i = 0; alive; i++) {
+            const PairItem x = pair_item<kTwo>(one.p, job2->p, walk, i);
+            if (x.done) break;
+            const PairJob &job = x.second ? *job2 : one;
+            const GemmParams &p = job.p;
+            const int mb = x.mb2 * 2 + (int)rank, nb = x.nb;
+            const int kt0 = x.split * p.kt_per_split;
             const int kt1 = min(kt0 + p.kt_per_split, p.kt_total);
             for (int kt = kt0; kt < kt1; kt++) {
-                if (!mbar_wait_warp(bar_empty + 8 * stage, phase ^ 1u, abort_flag, p.dev_status, p.spin_limit)) { alive = false; break; }
+                if (!mbar_wait_warp(bar_empty + 8 * stage, phase ^ 1u, abort_flag, p0.dev_status, p0.spin_limit)) { alive = false; break; }
                 const uint32_t sA = smem_base + stage * C::kStageBytes;
                 const uint32_t sB = sA + C::kABytes;
                 const uint32_t sSFA = sB + C::kBBytes;
@@ -1706,13 +1772,13 @@ k_gemm_mxf4_pair(const __grid_constant__ CUtensorMap map_a, const __grid_constan
                 const int ktr = kt1 - 1 - (kt - kt0);   // the K tiles are taken from the last to the first
                 if (leader && operands) {
                     if (rank == 0) mbar_expect_tx(bar_full + 8 * stage, 2u * (uint32_t)C::kStageBytes);
-                    tma2_load_2d(sA, &map_a, ktr * kBKBytes, mb * kBM, full);
-                    tma2_load_2d(sB, &map_b, ktr * kBKBytes, nb * BN + (int)rank * (BN / 2), full);
+                    tma2_load_2d(sA, &job.a, ktr * kBKBytes, mb * kBM, full);
+                    tma2_load_2d(sB, &job.b, ktr * kBKBytes, nb * BN + (int)rank * (BN / 2), full);
                 }
                 if (leader && !operands) {
                     // scale rows are 128-row blocks, 256 words (two 512-byte chunks) per stage; blocks beyond the matrix read as zero
-                    tma2_load_2d(sSFA, &map_sfa, ktr * 256, mb, full);
-                    tma2_load_2d(sSFB, &map_sfb, ktr * 256, (nb * BN) >> 7, full);
+                    tma2_load_2d(sSFA, &job.sfa, ktr * 256, mb, full);
+                    tma2_load_2d(sSFB, &job.sfb, ktr * 256, (nb * BN) >> 7, full);
                 }
                 __syncwarp();
                 if (++stage == C::kStages) { stage = 0; phase ^= 1u; }
@@ -1724,12 +1790,14 @@ k_gemm_mxf4_pair(const __grid_constant__ CUtensorMap map_a, const __grid_constan
             const bool leader = elect_one();
             uint32_t stage = 0, phase = 0;
             bool alive = true;
-            for (int item = cluster_id; item < items && alive; item += num_clusters) {
-                const int split = p.by_splits.mod(item);
-                const int kt0 = split * p.kt_per_split;
+            for (int i = 0; alive; i++) {
+                const PairItem x = pair_item<kTwo>(one.p, job2->p, walk, i);
+                if (x.done) break;
+                const GemmParams &p = x.second ? job2->p : one.p;
+                const int kt0 = x.split * p.kt_per_split;
                 const int kt1 = min(kt0 + p.kt_per_split, p.kt_total);
                 for (int kt = kt0; kt < kt1; kt++) {
-                    if (!mbar_wait_warp(bar_full + 8 * stage, phase, abort_flag, p.dev_status, p.spin_limit)) { alive = false; break; }
+                    if (!mbar_wait_warp(bar_full + 8 * stage, phase, abort_flag, p0.dev_status, p0.spin_limit)) { alive = false; break; }
                     tc_fence_after();
                     const uint32_t sSFA = smem_base + stage * C::kStageBytes + C::kABytes + C::kBBytes;
                     const uint32_t sSFB = sSFA + C::kSfaBytes;
@@ -1758,17 +1826,19 @@ k_gemm_mxf4_pair(const __grid_constant__ CUtensorMap map_a, const __grid_constan
             const bool leader = elect_one();
             uint32_t stage = 0, phase = 0, acc = 0, acc_phase = 0;
             bool alive = true;
-            for (int item = cluster_id; item < items && alive; item += num_clusters) {
-                const int split = p.by_splits.mod(item);
-                const int kt0 = split * p.kt_per_split;
+            for (int i = 0; alive; i++) {
+                const PairItem x = pair_item<kTwo>(one.p, job2->p, walk, i);
+                if (x.done) break;
+                const GemmParams &p = x.second ? job2->p : one.p;
+                const int kt0 = x.split * p.kt_per_split;
                 const int kt1 = min(kt0 + p.kt_per_split, p.kt_total);
                 // scale columns hold 32 rows each: a tile that starts 64 rows into a 128-row block starts 2 columns in
-                const uint32_t sfb_shift = BN == 192 ? (uint32_t)((p.by_tiles_n.mod(p.by_splits.div(item)) * BN & 127) >> 5) : 0u;
+                const uint32_t sfb_shift = BN == 192 ? (uint32_t)((x.nb * BN & 127) >> 5) : 0u;
                 const uint32_t d_tmem = tmem_base + acc * BN;
-                if (!mbar_wait_cluster_warp(bar_acc_empty + 8 * acc, acc_phase ^ 1u, abort_flag, p.dev_status, p.spin_limit)) { alive = false; break; }
+                if (!mbar_wait_cluster_warp(bar_acc_empty + 8 * acc, acc_phase ^ 1u, abort_flag, p0.dev_status, p0.spin_limit)) { alive = false; break; }
                 tc_fence_after();
                 for (int kt = kt0; kt < kt1; kt++) {
-                    if (!mbar_wait_warp(bar_sf_full + 8 * stage, phase, abort_flag, p.dev_status, p.spin_limit)) { alive = false; break; }
+                    if (!mbar_wait_warp(bar_sf_full + 8 * stage, phase, abort_flag, p0.dev_status, p0.spin_limit)) { alive = false; break; }
                     tc_fence_after();
                     const uint32_t sA = smem_base + stage * C::kStageBytes;
                     const uint32_t sB = sA + C::kABytes;
@@ -1810,36 +1880,42 @@ k_gemm_mxf4_pair(const __grid_constant__ CUtensorMap map_a, const __grid_constan
         if constexpr (BN == 192) {
             const uint32_t bias_line = smem_base + C::kBiasOff + ew * (BN / 2) * 2;
             uint32_t acc = 0, acc_phase = 0;
-            for (int item = cluster_id; item < items; item += num_clusters) {
-                const int tile = p.by_splits.div(item), split = item - tile * p.splits;
-                const int tm = p.by_tiles_n.div(tile), mb = (tiles_m2 - 1 - tm) * 2 + (int)rank, nb = tile - tm * p.tiles_n;
+            for (int i = 0;; i++) {
+                const PairItem x = pair_item<kTwo>(one.p, job2->p, walk, i);
+                if (x.done) break;
+                const PairJob &job = x.second ? *job2 : one;
+                const GemmParams &p = job.p;
+                const int mb = x.mb2 * 2 + (int)rank, nb = x.nb;
                 uint32_t bias[(kHalfCols + 63) / 64];
                 bias_fetch<kHalfCols>(bias, p.bias, (int64_t)nb * BN + chalf * kHalfCols, p.N, lane);
-                if (!mbar_wait_warp(bar_acc_full + 8 * acc, acc_phase, abort_flag, p.dev_status, p.spin_limit)) break;
+                if (!mbar_wait_warp(bar_acc_full + 8 * acc, acc_phase, abort_flag, p0.dev_status, p0.spin_limit)) break;
                 tc_fence_after();
                 if (p.bias != nullptr) bias_stage<kHalfCols>(bias, bias_line, lane);
-                epilogue_tile<BN, C::kStagingBufs, true>(&map_d, p.out_fp32 ? nullptr : &map_dw, p,
+                epilogue_tile<BN, C::kStagingBufs, true>(&job.d, p.out_fp32 ? nullptr : &job.dw, p,
                                                          tmem_base + ((uint32_t)(quarter * 32) << 16) + acc * BN + chalf * kHalfCols, mb * kBM + quarter * 32,
-                                                         nb * BN + chalf * kHalfCols, split, staging, sbuf, lane, map_to_cta(bar_acc_empty + 8 * acc, 0), bias_line);
+                                                         nb * BN + chalf * kHalfCols, x.split, staging, sbuf, lane, map_to_cta(bar_acc_empty + 8 * acc, 0), bias_line);
                 if (++acc == C::kAccStages) { acc = 0; acc_phase ^= 1u; }
             }
         } else {
         const uint32_t acc_empty_leader = map_to_cta(bar_acc_empty, 0);
         uint32_t acc_phase = 0;
         bool alive = true;
-        for (int item = cluster_id; item < items && alive; item += num_clusters) {
-            const int tile = p.by_splits.div(item), split = item - tile * p.splits;
-            const int tm = p.by_tiles_n.div(tile), mb = (tiles_m2 - 1 - tm) * 2 + (int)rank, nb = tile - tm * p.tiles_n;
+        for (int i = 0; alive; i++) {
+            const PairItem x = pair_item<kTwo>(one.p, job2->p, walk, i);
+            if (x.done) break;
+            const PairJob &job = x.second ? *job2 : one;
+            const GemmParams &p = job.p;
+            const int mb = x.mb2 * 2 + (int)rank, nb = x.nb;
             uint32_t bias[kHalfCols / 32];
 #pragma unroll
             for (int cc = 0; cc < kHalfCols / 32; cc++) bias[cc] = load_bias_pair(p.bias, (int64_t)nb * BN + chalf * kHalfCols + cc * 32, p.N, lane);
-            if (!mbar_wait_warp(bar_acc_full, acc_phase, abort_flag, p.dev_status, p.spin_limit)) { alive = false; break; }
+            if (!mbar_wait_warp(bar_acc_full, acc_phase, abort_flag, p0.dev_status, p0.spin_limit)) { alive = false; break; }
             tc_fence_after();
             const int row0 = mb * kBM + quarter * 32;
             const int colbase = nb * BN + chalf * kHalfCols;
             const uint32_t taddr = tmem_base + ((uint32_t)(quarter * 32) << 16) + chalf * kHalfCols;
             const bool use_bias = p.bias != nullptr && p.splits == 1;
-            auto store_box = [&](const uint32_t *w, int x) {
+            auto store_box = [&](const uint32_t *w, int col0) {
                 if (lane == 0) bulk_wait_read<C::kStagingBufs - 1>();
                 __syncwarp();
                 uint8_t *buf = staging + sbuf * kStagingBytes;
@@ -1847,7 +1923,7 @@ k_gemm_mxf4_pair(const __grid_constant__ CUtensorMap map_a, const __grid_constan
                 fence_async_smem();
                 __syncwarp();
                 if (lane == 0) {
-                    tma_store_3d(&map_d, x, row0, split, smem_u32(buf));
+                    tma_store_3d(&job.d, col0, row0, x.split, smem_u32(buf));
                     bulk_commit();
                 }
                 sbuf = (sbuf + 1) % C::kStagingBufs;
@@ -1883,7 +1959,7 @@ k_gemm_mxf4_pair(const __grid_constant__ CUtensorMap map_a, const __grid_constan
 #pragma unroll
                         for (int cc = 0; cc < kChunks; cc++)
                             if (colbase + cc * 32 < p.N && row0 < p.M)
-                                tma_store_3d(&map_d, colbase + cc * 32, row0, split, smem_u32(staging + cc * kStagingBytes));
+                                tma_store_3d(&job.d, colbase + cc * 32, row0, x.split, smem_u32(staging + cc * kStagingBytes));
                         bulk_commit();
                     }
                 } else {
@@ -2439,14 +2515,13 @@ static bool ensure_device_ok()
     return ok[dev] == 1;
 }
 
-template <int BN>
-static mxfp4_status_t launch_gemm_pair(const CUtensorMap &ma, const CUtensorMap &mb, const CUtensorMap &msa, const CUtensorMap &msb,
-                                       const CUtensorMap &md, const CUtensorMap &mdw, const GemmParams &p, int grid, cudaStream_t st)
+template <int BN, class Job2>
+static mxfp4_status_t launch_gemm_pair(const PairJob &one, const Job2 &two, int grid, cudaStream_t st)
 {
     using C = Gemm2Cfg<BN>;
     static bool attr_set[kMaxDevices];
-    MX_CHECK_CUDA(set_smem_once(attr_set, k_gemm_mxf4_pair<BN>, C::kSmemBytes));
-    MX_CHECK_CUDA(launch_pdl(k_gemm_mxf4_pair<BN>, (unsigned)grid, 1, kGemmThreads, C::kSmemBytes, st, ma, mb, msa, msb, md, mdw, p));
+    MX_CHECK_CUDA(set_smem_once(attr_set, k_gemm_mxf4_pair<BN, Job2>, C::kSmemBytes));
+    MX_CHECK_CUDA(launch_pdl(k_gemm_mxf4_pair<BN, Job2>, (unsigned)grid, 1, kGemmThreads, C::kSmemBytes, st, one, two));
     return MXFP4_OK;
 }
 
@@ -2498,14 +2573,13 @@ static mxfp4_status_t launch_gemm_ck(const CUtensorMap &ma, const CUtensorMap &m
     return MXFP4_OK;
 }
 
-template <int BN>
-static mxfp4_status_t launch_gemm(const CUtensorMap &ma, const CUtensorMap &mb, const CUtensorMap &md, const CUtensorMap &mdw,
-                                  const GemmParams &p, int grid, cudaStream_t st)
+template <int BN, class Job2>
+static mxfp4_status_t launch_gemm(const GemmJob &one, const Job2 &two, int grid, cudaStream_t st)
 {
     using C = GemmCfg<BN>;
     static bool attr_set[kMaxDevices];
-    MX_CHECK_CUDA(set_smem_once(attr_set, k_gemm_mxf4<BN>, C::kSmemBytes));
-    MX_CHECK_CUDA(launch_pdl(k_gemm_mxf4<BN>, (unsigned)grid, 1, kGemmThreads, C::kSmemBytes, st, ma, mb, md, mdw, p));
+    MX_CHECK_CUDA(set_smem_once(attr_set, k_gemm_mxf4<BN, Job2>, C::kSmemBytes));
+    MX_CHECK_CUDA(launch_pdl(k_gemm_mxf4<BN, Job2>, (unsigned)grid, 1, kGemmThreads, C::kSmemBytes, st, one, two));
     return MXFP4_OK;
 }
 
@@ -2563,29 +2637,20 @@ static void set_walk(GemmParams &p, int workers = 1, int rows = 1)
 }
 
 // spin_limit / withhold_loads: see GemmParams (normal use: kWaitSpinLimit, 0).
-static mxfp4_status_t gemm_impl(mxfp4_mat_t a, mxfp4_mat_t b, void *d, int64_t ldd, int out_dtype, const void *bias, void *workspace,
-                                size_t workspace_bytes, uint32_t *dev_status, cudaStream_t st, bool allow_split, uint32_t spin_limit,
-                                int withhold_loads)
+// The maps and parameters of one product with plan g.
+static bool make_job(PairJob &job, const GemmPlan &g, mxfp4_mat_t a, mxfp4_mat_t b, void *d, int64_t ldd, int out_dtype, const void *bias, void *workspace,
+                     uint32_t *dev_status, uint32_t spin_limit, int withhold_loads)
 {
-    const mxfp4_status_t chk = gemm_check(a, b, d, ldd, out_dtype, bias, workspace, workspace_bytes, allow_split);
-    if (chk) return chk;
     const int64_t M = a.rows, N = b.rows, Kc = a.cols;
-    if (M == 0 || N == 0) return MXFP4_OK;
-    const int sms = sm_count();
-    const GemmPlan g = plan_gemm(M, N, Kc, sms, allow_split);
-
     const bool store_fp32 = g.splits > 1 || out_dtype == MXFP4_OUT_FP32;
-    CUtensorMap ma, mb, md;
-    if (!make_operand_map(&ma, a.data, M, Kc, kBM) || !make_operand_map(&mb, b.data, N, Kc, g.pbs ? 96 : g.pair ? g.bn / 2 : g.bn)) return MXFP4_CUDA_ERROR;
-    if (!make_output_map(&md, g.splits > 1 ? workspace : d, M, N, g.splits > 1 ? N : ldd, g.splits, store_fp32)) return MXFP4_CUDA_ERROR;
-
-    GemmParams p;
+    GemmParams &p = job.p;
     p.sfa = a.scales; p.sfb = b.scales;
     p.M = M; p.N = N; p.Kc = Kc;
     p.nblk4 = (int)ceil_div(Kc / 32, 4);
     p.rbA = (int)ceil_div(M, 128); p.rbB = (int)ceil_div(N, 128);
     p.tiles_m = g.tiles_m; p.tiles_n = g.tiles_n; p.splits = g.splits;
     p.kt_total = g.kt_total; p.kt_per_split = g.kt_per_split;
+    p.head = 0;
     p.out_fp32 = store_fp32;
     p.bias = static_cast<const __nv_bfloat16 *>(bias);
     p.dev_status = dev_status;
@@ -2594,34 +2659,107 @@ static mxfp4_status_t gemm_impl(mxfp4_mat_t a, mxfp4_mat_t b, void *d, int64_t l
     p.spin_limit = spin_limit;
     p.withhold_loads = withhold_loads;
     set_walk(p);
+    if (!make_operand_map(&job.a, a.data, M, Kc, kBM) || !make_operand_map(&job.b, b.data, N, Kc, g.pbs ? 96 : g.pair ? g.bn / 2 : g.bn) ||
+        !make_output_map(&job.d, g.splits > 1 ? workspace : d, M, N, g.splits > 1 ? N : ldd, g.splits, store_fp32))
+        return false;
+    if ((g.pair || g.pbs) && (!make_scale_map(&job.sfa, a.scales, M, Kc, 1) || !make_scale_map(&job.sfb, b.scales, N, Kc, 2))) return false;
+    job.dw = job.d;
+    return store_fp32 || make_output_map_wide(&job.dw, d, M, N, ldd);
+}
+
+static mxfp4_status_t launch_splitk_reduce(const GemmPlan &g, const void *workspace, int64_t M, int64_t N, void *d, int64_t ldd, int out_dtype,
+                                           const void *bias, int sms, cudaStream_t st)
+{
+    const int groups = g.splits >= 8 && M * N / 4 < 64 * 256 ? 8 : 1;   // fewer than 64 blocks otherwise
+    const int64_t nb4 = ceil_div(M * N / 4, 256 / groups);
+    const unsigned blocks = (unsigned)(nb4 < (int64_t)sms * 8 ? nb4 : (int64_t)sms * 8);
+    MX_CHECK_CUDA(launch_pdl(groups == 8 ? k_splitk_reduce<8> : k_splitk_reduce<1>, blocks, 1, 256, 0, st, static_cast<const float *>(workspace),
+                             g.splits, M, N, d, ldd, (int)(out_dtype == MXFP4_OUT_FP32), static_cast<const __nv_bfloat16 *>(bias)));
+    return MXFP4_OK;
+}
+
+static mxfp4_status_t gemm_impl(mxfp4_mat_t a, mxfp4_mat_t b, void *d, int64_t ldd, int out_dtype, const void *bias, void *workspace,
+                                size_t workspace_bytes, uint32_t *dev_status, cudaStream_t st, bool allow_split, uint32_t spin_limit,
+                                int withhold_loads)
+{
+    const mxfp4_status_t chk = gemm_check(a, b, d, ldd, out_dtype, bias, workspace, workspace_bytes, allow_split);
+    if (chk) return chk;
+    const int64_t M = a.rows, N = b.rows;
+    if (M == 0 || N == 0) return MXFP4_OK;
+    const int sms = sm_count();
+    const GemmPlan g = plan_gemm(M, N, a.cols, sms, allow_split);
+    PairJob job;
+    if (!make_job(job, g, a, b, d, ldd, out_dtype, bias, workspace, dev_status, spin_limit, withhold_loads)) return MXFP4_CUDA_ERROR;
+    GemmParams &p = job.p;
     if (g.ck) {
         p.splits = g.ck;
-        p.out_fp32 = out_dtype == MXFP4_OUT_FP32;
-        return launch_gemm_ck(ma, mb, p, g.tiles_m * g.tiles_n, g.ck, st);
+        return launch_gemm_ck(job.a, job.b, p, g.tiles_m * g.tiles_n, g.ck, st);
     }
     const bool paired = g.pair || g.pbs;
     const int rows = paired ? (g.tiles_m + 1) / 2 : g.tiles_m, workers = paired ? sms / 2 : sms;
     const int items = min(workers, rows * g.tiles_n * g.splits), grid = paired ? 2 * items : items;
     set_walk(p, items, rows);
-    CUtensorMap msa, msb;
-    if (paired && (!make_scale_map(&msa, a.scales, M, Kc, 1) || !make_scale_map(&msb, b.scales, N, Kc, 2))) return MXFP4_CUDA_ERROR;
-    CUtensorMap mdw = md;
-    if (!store_fp32 && !make_output_map_wide(&mdw, d, M, N, ldd)) return MXFP4_CUDA_ERROR;
-    mxfp4_status_t s = g.pbs         ? launch_gemm_pbs<4, 8>(ma, mb, msa, msb, md, mdw, p, grid, st)
-                       : g.bs == 1   ? launch_gemm_bs<192, 2, 7>(ma, mb, md, mdw, p, grid, st)
-                       : g.pair      ? (g.bn == 192 ? launch_gemm_pair<192>(ma, mb, msa, msb, md, mdw, p, grid, st) : launch_gemm_pair<256>(ma, mb, msa, msb, md, mdw, p, grid, st))
-                       : g.bn == 256 ? launch_gemm<256>(ma, mb, md, mdw, p, grid, st)
-                       : g.bn == 192 ? launch_gemm<192>(ma, mb, md, mdw, p, grid, st)
-                                     : launch_gemm<128>(ma, mb, md, mdw, p, grid, st);
-    if (s) return s;
-    if (g.splits > 1 && !withhold_loads) {
-        const int groups = g.splits >= 8 && M * N / 4 < 64 * 256 ? 8 : 1;   // fewer than 64 blocks otherwise
-        const int64_t nb4 = ceil_div(M * N / 4, 256 / groups);
-        const unsigned blocks = (unsigned)(nb4 < (int64_t)sms * 8 ? nb4 : (int64_t)sms * 8);
-        MX_CHECK_CUDA(launch_pdl(groups == 8 ? k_splitk_reduce<8> : k_splitk_reduce<1>, blocks, 1, 256, 0, st, static_cast<const float *>(workspace),
-                                 g.splits, M, N, d, ldd, (int)(out_dtype == MXFP4_OUT_FP32), static_cast<const __nv_bfloat16 *>(bias)));
+    const mxfp4_status_t s = g.pbs         ? launch_gemm_pbs<4, 8>(job.a, job.b, job.sfa, job.sfb, job.d, job.dw, p, grid, st)
+                             : g.bs == 1   ? launch_gemm_bs<192, 2, 7>(job.a, job.b, job.d, job.dw, p, grid, st)
+                             : g.pair      ? (g.bn == 192 ? launch_gemm_pair<192>(job, NoJob{}, grid, st) : launch_gemm_pair<256>(job, NoJob{}, grid, st))
+                             : g.bn == 256 ? launch_gemm<256>(job, NoJob{}, grid, st)
+                             : g.bn == 192 ? launch_gemm<192>(job, NoJob{}, grid, st)
+                                           : launch_gemm<128>(job, NoJob{}, grid, st);
+    if (s || g.splits == 1 || withhold_loads) return s;
+    return launch_splitk_reduce(g, workspace, M, N, d, ldd, out_dtype, bias, sms, st);
+}
+
+// The two products of a backward pass, d1 = a1 b1^T and d2 = a2 b2^T: in one launch where all their 128-wide tiles fit on the SMs, or
+// where one runs on CTA pairs and the other can (the second not split); else one after the other.  One launch pays once for filling and
+// draining the machine and lets the second product's tiles fill the pairs that the first one leaves idle (64 items of 197 K tiles
+// on 74 pairs).  Both together, back to back, in us (rows, columns of X and of dY): 1024, 192, 768 9.6 -> 5.3; 2048, 384, 768
+// 12.7 -> 8.2; 4096, 768, 3072 26.9 -> 21.7; 25216, 384, 1536 41 -> 30; 8192, 2048, 2048 39 -> 33; 50432, 1024, 4096 189 -> 174.
+mxfp4_status_t gemm_two(mxfp4_mat_t a1, mxfp4_mat_t b1, void *d1, int64_t ldd1, int dtype1, mxfp4_mat_t a2, mxfp4_mat_t b2, void *d2, int64_t ldd2, int dtype2,
+                        void *workspace, size_t workspace_bytes, uint32_t *dev_status, cudaStream_t st)
+{
+    mxfp4_status_t s;
+    if ((s = gemm_check(a1, b1, d1, ldd1, dtype1, nullptr, workspace, workspace_bytes, true)) ||
+        (s = gemm_check(a2, b2, d2, ldd2, dtype2, nullptr, workspace, workspace_bytes, true)))
+        return s;
+    if (a1.rows > 0 && b1.rows > 0 && a2.rows > 0 && b2.rows > 0) {
+        const int sms = sm_count();
+        GemmPlan g1 = plan_gemm(a1.rows, b1.rows, a1.cols, sms, true);
+        GemmPlan g2 = plan_gemm(a2.rows, b2.rows, a2.cols, sms, true);
+        const auto single = [](const GemmPlan &g) { return !g.pair && !g.pbs && !g.bs && !g.ck; };
+        const int tiles1 = g1.tiles_m * g1.tiles_n, tiles2 = g2.tiles_m * g2.tiles_n;
+        const bool small = single(g1) && single(g2) && g1.bn == 128 && g2.bn == 128 && g1.splits == 1 && g2.splits == 1 && tiles1 + tiles2 <= sms;
+        // A product on single CTAs joins the other one's pairs, and the second takes the width of the first (192 only where 256 gives as
+        // many columns): its sums stay as they are.  Widths up to 128 and the B-stationary kernels keep their own launch.
+        const int width = g1.pair ? g1.bn : g2.pair && g2.splits == 1 ? g2.bn : 0;
+        const auto join = [&](GemmPlan &g, int64_t n) {
+            if (!(single(g) || g.pair) || g.splits != 1 || n <= 128) return;
+            g.pair = true;
+            g.bn = width;
+            g.tiles_n = (int)ceil_div(n, width);
+        };
+        if (width && !small) {
+            if (!g1.pair) join(g1, b1.rows);
+            join(g2, b2.rows);
+        }
+        if (small || (g1.pair && g2.pair && g1.bn == g2.bn && g2.splits == 1)) {
+            PairJob j1, j2;
+            if (!make_job(j1, g1, a1, b1, d1, ldd1, dtype1, nullptr, workspace, dev_status, kWaitSpinLimit, 0) ||
+                !make_job(j2, g2, a2, b2, d2, ldd2, dtype2, nullptr, nullptr, dev_status, kWaitSpinLimit, 0))
+                return MXFP4_CUDA_ERROR;
+            if (small) return launch_gemm<128, GemmJob>(j1, j2, tiles1 + tiles2, st);
+            const int items = (g1.tiles_m + 1) / 2 * g1.tiles_n * g1.splits + (g2.tiles_m + 1) / 2 * g2.tiles_n, workers = min(sms / 2, items);
+            const bool first = g1.kt_per_split >= g2.kt_per_split;
+            PairJob &a = first ? j1 : j2, &b = first ? j2 : j1;
+            // an item costs its K tiles and, where the epilogue is not hidden, about three more (without the head start
+            // 50432 x 1024 x 4096 takes 183 us)
+            const int tile = g1.bn == 256 ? 3 : 1, ka = a.p.kt_per_split + tile, kb = b.p.kt_per_split + tile;
+            b.p.head = (ka + kb / 2) / kb;
+            if ((s = g1.bn == 256 ? launch_gemm_pair<256>(a, b, 2 * workers, st) : launch_gemm_pair<192>(a, b, 2 * workers, st))) return s;
+            return g1.splits > 1 ? launch_splitk_reduce(g1, workspace, a1.rows, b1.rows, d1, ldd1, dtype1, nullptr, sms, st) : MXFP4_OK;
+        }
     }
-    return MXFP4_OK;
+    if ((s = gemm_impl(a1, b1, d1, ldd1, dtype1, nullptr, workspace, workspace_bytes, dev_status, st, true, kWaitSpinLimit, 0))) return s;
+    return gemm_impl(a2, b2, d2, ldd2, dtype2, nullptr, workspace, workspace_bytes, dev_status, st, true, kWaitSpinLimit, 0);
 }
 
 mxfp4_status_t gemm(mxfp4_mat_t a, mxfp4_mat_t b, void *d, int64_t ldd, int out_dtype, const void *bias, void *workspace,

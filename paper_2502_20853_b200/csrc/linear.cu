@@ -11,6 +11,8 @@ mxfp4_status_t quantize_tile(const void *src_bf16, const mxfp4_mat_t *src_q, int
 mxfp4_status_t quantize_chain_two(const void *x_bf16, int64_t m, int64_t k, int64_t ldx, const mxfp4_mat_t &xq, const mxfp4_mat_t &xq_t, const mxfp4_qparams_t *q6,
                                   const void *w_bf16, int64_t n, const mxfp4_mat_t &wq, const mxfp4_mat_t &wq_t, const mxfp4_qparams_t *q4,
                                   const mxfp4_qparams_t *rne, uint32_t *dev_status, cudaStream_t st);
+mxfp4_status_t gemm_two(mxfp4_mat_t a1, mxfp4_mat_t b1, void *d1, int64_t ldd1, int dtype1, mxfp4_mat_t a2, mxfp4_mat_t b2, void *d2, int64_t ldd2, int dtype2,
+                        void *workspace, size_t workspace_bytes, uint32_t *dev_status, cudaStream_t st);
 mxfp4_status_t gemm(mxfp4_mat_t a, mxfp4_mat_t b, void *d, int64_t ldd, int out_dtype, const void *bias, void *workspace,
                     size_t workspace_bytes, uint32_t *dev_status, cudaStream_t st, bool allow_split);
 mxfp4_status_t gemm_check(mxfp4_mat_t a, mxfp4_mat_t b, const void *d, int64_t ldd, int out_dtype, const void *bias,
@@ -181,9 +183,10 @@ mxfp4_status_t mxfp4_linear_bwd_ex(const void *dy_bf16, int64_t lddy, const mxfp
     // Eq. 5: dW[N,K] = dYq_t[N,M] * Xq_t[K,M]^T ;  Eq. 4: dX[M,K] = dYq[M,N] * Wq_t[K,N]^T.
     // dW first: its output is small, so the tail of Q3(dY) that the quantizer left in L2 is still there when dX reads it
     // (both products take the freshest part of their first operand first: the last K tiles, the last rows).
-    if ((s = gemm(dyq_t, xq_t, dw, lddw, dw_dtype, nullptr, ws + L.gemm_ws, L.gemm_ws_bytes, dev_status, st, true))) return s;
-    if (epi_dx) return gemm_quant(dyq, wq_t, nullptr, epi_dx, dev_status, st);
-    return gemm(dyq, wq_t, dx_bf16, lddx, MXFP4_OUT_BF16, nullptr, ws + L.gemm_ws, L.gemm_ws_bytes, dev_status, st, true);
+    void *const gws = ws + L.gemm_ws;
+    if (!epi_dx) return gemm_two(dyq_t, xq_t, dw, lddw, dw_dtype, dyq, wq_t, dx_bf16, lddx, MXFP4_OUT_BF16, gws, L.gemm_ws_bytes, dev_status, st);
+    if ((s = gemm(dyq_t, xq_t, dw, lddw, dw_dtype, nullptr, gws, L.gemm_ws_bytes, dev_status, st, true))) return s;
+    return gemm_quant(dyq, wq_t, nullptr, epi_dx, dev_status, st);
 }
 
 mxfp4_status_t mxfp4_linear_bwd(const void *dy_bf16, int64_t lddy, const mxfp4_linear_ctx_t *ctx, uint64_t seed,

@@ -5,7 +5,7 @@ import torch
 
 import oracle as orc
 import workloads
-from util import assert_qmat_equal, check_gemm_bound, to_dev_bf16
+from util import assert_qmat_equal, check_gemm_bound, numpy_to_qmat, to_dev_bf16
 
 pytestmark = pytest.mark.gpu
 
@@ -287,3 +287,28 @@ def test_forward_quantizes_activations_and_weight_in_one_launch(mx, M, K, N):
     assert int(st.item()) == mx.DEV_NONFINITE
     for got, want in zip((ctx.xq, ctx.xq_t, ctx.wq, ctx.wq_t), mx.quantize_chain(x, seed=77) + mx.quantize_chain(w, seed=77, stream_id_t=4)):
         assert torch.equal(got.data, want.data) and torch.equal(got.scales, want.scales)
+
+
+# on 148 SMs: one wave of 128-wide tiles in all; CTA pairs with the weight gradient split or not, one or several items per pair, 192
+# and 256 columns wide, ragged in every extent, and with the input gradient's items the longer ones; two launches
+@pytest.mark.parametrize("M,K,N", [(1024, 192, 768), (96, 160, 1120), (2016, 1024, 544), (25216, 384, 1536), (12320, 1024, 1568), (8224, 2080, 2080),
+                                   (2336, 1504, 4128), (1056, 1056, 2848), (4000, 576, 2304), (320, 2048, 512)])
+@pytest.mark.parametrize("dw_dtype", [0, 1])
+def test_products_of_a_backward_pass(mx, M, K, N, dw_dtype):
+    """dX and dW from given operands, as one launch makes them where it does, against the two products of the oracle, within the
+    library's bound for the length of the accumulation chains."""
+    rng = np.random.default_rng(M + K + N + dw_dtype)
+
+    def operand(rows, kc):
+        c = rng.integers(0, 16, size=(rows, kc)).astype(np.uint8)
+        return (c[:, 0::2] | (c[:, 1::2] << 4)).astype(np.uint8), rng.integers(125, 130, size=(rows, kc // 32)).astype(np.uint8)
+
+    dyq, dyq_t, wq_t, xq_t = operand(M, N), operand(N, M), operand(K, N), operand(K, M)
+    ctx = mx.LinearCtx(mx.QMat(M, K), mx.QMat(N, K), numpy_to_qmat(mx, *xq_t), 7, numpy_to_qmat(mx, *wq_t))
+    st = mx.new_status()
+    dx, dw = mx.linear_bwd(None, ctx, 7, dw_dtype=dw_dtype, dev_status=st, dyq=numpy_to_qmat(mx, *dyq), dyq_t=numpy_to_qmat(mx, *dyq_t))
+    torch.cuda.synchronize()
+    assert int(st.item()) == 0
+    for got, a, b, shape, bf16, what in ((dx, dyq, wq_t, (M, K, N), True, "dX"), (dw, dyq_t, xq_t, (N, K, M), dw_dtype == 0, "dW")):
+        want, t = orc.gemm(*a, *b)
+        check_gemm_bound(got.float().cpu().numpy(), want, t, bf16, what, factor=max(1.0, mx.gemm_chain_mmas(*shape) / 8))
