@@ -11,6 +11,8 @@
 //   warps 4-11  epilogue: tcgen05.ld -> (+bias) -> cast -> swizzled staging in shared memory -> TMA store;
 //               two warps share each quarter of the TMEM lanes and split the columns
 // Every mbarrier wait is bounded; on expiry MXFP4_DEV_TIMEOUT is raised and all roles drain.
+#include <algorithm>
+
 #include "common.cuh"
 #include "quant_tile.cuh"
 #include "tma.cuh"
@@ -2709,6 +2711,47 @@ static mxfp4_status_t gemm_impl(mxfp4_mat_t a, mxfp4_mat_t b, void *d, int64_t l
     return launch_splitk_reduce(g, workspace, M, N, d, ldd, out_dtype, bias, sms, st);
 }
 
+enum class TwoKind { kSeparate, kOneWave, kPairs };
+
+// The plans of two products (rows m1, m2, contractions kc1, kc2, n columns each) that may share a launch.
+static TwoKind plan_two(int64_t m1, int64_t kc1, int64_t m2, int64_t kc2, int64_t n, int sms, GemmPlan &g1, GemmPlan &g2)
+{
+    g1 = plan_gemm(m1, n, kc1, sms, true);
+    g2 = plan_gemm(m2, n, kc2, sms, true);
+    const auto single = [](const GemmPlan &g) { return !g.pair && !g.pbs && !g.bs && !g.ck; };
+    if (single(g1) && single(g2) && g1.bn == 128 && g2.bn == 128 && g1.splits == 1 && g2.splits == 1 &&
+        g1.tiles_m * g1.tiles_n + g2.tiles_m * g2.tiles_n <= sms)
+        return TwoKind::kOneWave;
+    const GemmPlan own = g1;
+    if (g1.ck && g2.splits == 1 && (g2.pair || single(g2))) {
+        // CTA pairs with four partial sums in place of the cluster kernel's two pairs of accumulators: chains of the same length, and in one
+        // launch with the other product faster in spite of the sums' way through L2 (both products, in us: 25216, 768, 1536 46.7 -> 35.5;
+        // 6272, 768, 2304 33.9 -> 30.4; 4096, 768, 1536 20.6 -> 16.7; 100352, 768, 2304 182 -> 171; 50432, 768, 2304 89 -> 87)
+        g1.ck = 0;
+        g1.pair = true;
+        g1.bn = g2.pair ? g2.bn : 256;
+        g1.tiles_n = (int)ceil_div(n, g1.bn);
+        g1.kt_per_split = (int)ceil_div(g1.kt_total, 4);
+        g1.splits = (int)ceil_div(g1.kt_total, g1.kt_per_split);
+    }
+    // A product on single CTAs joins the other one's pairs, and the second takes the width of the first (192 only where 256 gives as
+    // many columns): its sums stay as they are.  Widths up to 128 and the B-stationary kernels keep their own launch.
+    const int width = g1.pair ? g1.bn : g2.pair && g2.splits == 1 ? g2.bn : 0;
+    const auto join = [&](GemmPlan &g) {
+        if (!(single(g) || g.pair) || g.splits != 1 || n <= 128) return;
+        g.pair = true;
+        g.bn = width;
+        g.tiles_n = (int)ceil_div(n, width);
+    };
+    if (width) {
+        if (!g1.pair) join(g1);
+        join(g2);
+    }
+    if (g1.pair && g2.pair && g1.bn == g2.bn && g2.splits == 1) return TwoKind::kPairs;
+    g1 = own;
+    return TwoKind::kSeparate;
+}
+
 // The two products of a backward pass, d1 = a1 b1^T and d2 = a2 b2^T: in one launch where all their 128-wide tiles fit on the SMs, or
 // where one runs on CTA pairs and the other can (the second not split); else one after the other.  One launch pays once for filling and
 // draining the machine and lets the second product's tiles fill the pairs that the first one leaves idle (64 items of 197 K tiles
@@ -2723,30 +2766,15 @@ mxfp4_status_t gemm_two(mxfp4_mat_t a1, mxfp4_mat_t b1, void *d1, int64_t ldd1, 
         return s;
     if (a1.rows > 0 && b1.rows > 0 && a2.rows > 0 && b2.rows > 0) {
         const int sms = sm_count();
-        GemmPlan g1 = plan_gemm(a1.rows, b1.rows, a1.cols, sms, true);
-        GemmPlan g2 = plan_gemm(a2.rows, b2.rows, a2.cols, sms, true);
-        const auto single = [](const GemmPlan &g) { return !g.pair && !g.pbs && !g.bs && !g.ck; };
-        const int tiles1 = g1.tiles_m * g1.tiles_n, tiles2 = g2.tiles_m * g2.tiles_n;
-        const bool small = single(g1) && single(g2) && g1.bn == 128 && g2.bn == 128 && g1.splits == 1 && g2.splits == 1 && tiles1 + tiles2 <= sms;
-        // A product on single CTAs joins the other one's pairs, and the second takes the width of the first (192 only where 256 gives as
-        // many columns): its sums stay as they are.  Widths up to 128 and the B-stationary kernels keep their own launch.
-        const int width = g1.pair ? g1.bn : g2.pair && g2.splits == 1 ? g2.bn : 0;
-        const auto join = [&](GemmPlan &g, int64_t n) {
-            if (!(single(g) || g.pair) || g.splits != 1 || n <= 128) return;
-            g.pair = true;
-            g.bn = width;
-            g.tiles_n = (int)ceil_div(n, width);
-        };
-        if (width && !small) {
-            if (!g1.pair) join(g1, b1.rows);
-            join(g2, b2.rows);
-        }
-        if (small || (g1.pair && g2.pair && g1.bn == g2.bn && g2.splits == 1)) {
+        GemmPlan g1, g2;
+        const TwoKind kind = plan_two(a1.rows, a1.cols, a2.rows, a2.cols, b1.rows, sms, g1, g2);
+        if (kind != TwoKind::kSeparate) {
+            if (g1.splits > 1 && workspace_bytes < (size_t)g1.splits * a1.rows * b1.rows * sizeof(float)) return MXFP4_WORKSPACE_TOO_SMALL;
             PairJob j1, j2;
             if (!make_job(j1, g1, a1, b1, d1, ldd1, dtype1, nullptr, workspace, dev_status, kWaitSpinLimit, 0) ||
                 !make_job(j2, g2, a2, b2, d2, ldd2, dtype2, nullptr, nullptr, dev_status, kWaitSpinLimit, 0))
                 return MXFP4_CUDA_ERROR;
-            if (small) return launch_gemm<128, GemmJob>(j1, j2, tiles1 + tiles2, st);
+            if (kind == TwoKind::kOneWave) return launch_gemm<128, GemmJob>(j1, j2, g1.tiles_m * g1.tiles_n + g2.tiles_m * g2.tiles_n, st);
             const int items = (g1.tiles_m + 1) / 2 * g1.tiles_n * g1.splits + (g2.tiles_m + 1) / 2 * g2.tiles_n, workers = min(sms / 2, items);
             const bool first = g1.kt_per_split >= g2.kt_per_split;
             PairJob &a = first ? j1 : j2, &b = first ? j2 : j1;
@@ -2959,6 +2987,17 @@ size_t gemm_workspace_bytes(int64_t m, int64_t n, int64_t kc)
     // the same SM count gemm() plans with (148, the B200's, when no device is current)
     const GemmPlan g = plan_gemm(m, n, kc, sm_count());
     return g.splits > 1 ? (size_t)g.splits * m * n * sizeof(float) : 0;
+}
+
+// Workspace for gemm_two()'s partial sums.
+size_t gemm_two_workspace_bytes(int64_t m1, int64_t kc1, int64_t m2, int64_t kc2, int64_t n)
+{
+    if (m1 <= 0 || kc1 <= 0 || m2 <= 0 || kc2 <= 0 || n <= 0) return 0;
+    GemmPlan g1, g2;
+    const bool pairs = plan_two(m1, kc1, m2, kc2, n, sm_count(), g1, g2) == TwoKind::kPairs;
+    const size_t two = pairs && g1.splits > 1 ? (size_t)g1.splits * m1 * n * sizeof(float) : 0;
+    const size_t w1 = gemm_workspace_bytes(m1, n, kc1), w2 = gemm_workspace_bytes(m2, n, kc2);
+    return std::max(two, std::max(w1, w2));
 }
 
 // The longest chain of MMAs (64 contraction elements each) that gemm() adds into one accumulator for this shape.

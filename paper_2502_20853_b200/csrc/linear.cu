@@ -17,7 +17,7 @@ mxfp4_status_t gemm(mxfp4_mat_t a, mxfp4_mat_t b, void *d, int64_t ldd, int out_
                     size_t workspace_bytes, uint32_t *dev_status, cudaStream_t st, bool allow_split);
 mxfp4_status_t gemm_check(mxfp4_mat_t a, mxfp4_mat_t b, const void *d, int64_t ldd, int out_dtype, const void *bias,
                           const void *workspace, size_t workspace_bytes, bool allow_split);
-size_t gemm_workspace_bytes(int64_t m, int64_t n, int64_t kc);
+size_t gemm_two_workspace_bytes(int64_t m1, int64_t kc1, int64_t m2, int64_t kc2, int64_t n);
 mxfp4_status_t gemm_quant_check(mxfp4_mat_t a, mxfp4_mat_t b, const void *bias, const mxfp4_epilogue_t *epi);
 mxfp4_status_t gemm_quant(mxfp4_mat_t a, mxfp4_mat_t b, const void *bias, const mxfp4_epilogue_t *epi, uint32_t *dev_status, cudaStream_t st);
 
@@ -40,8 +40,7 @@ static BwdLayout bwd_layout(int64_t m, int64_t k, int64_t n)
     L.wqt_s = take(mxfp4_scale_bytes(k, n));
     L.xqt_p = take((size_t)k * m / 2);
     L.xqt_s = take(mxfp4_scale_bytes(k, m));
-    const size_t g1 = gemm_workspace_bytes(m, k, n), g2 = gemm_workspace_bytes(n, k, m);
-    L.gemm_ws_bytes = g1 > g2 ? g1 : g2;
+    L.gemm_ws_bytes = gemm_two_workspace_bytes(n, m, m, n, k);
     L.gemm_ws = take(L.gemm_ws_bytes);
     L.total = o;
     return L;

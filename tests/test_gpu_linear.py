@@ -292,7 +292,7 @@ def test_forward_quantizes_activations_and_weight_in_one_launch(mx, M, K, N):
 # on 148 SMs: one wave of 128-wide tiles in all; CTA pairs with the weight gradient split or not, one or several items per pair, 192
 # and 256 columns wide, ragged in every extent, and with the input gradient's items the longer ones; two launches
 @pytest.mark.parametrize("M,K,N", [(1024, 192, 768), (96, 160, 1120), (2016, 1024, 544), (25216, 384, 1536), (12320, 1024, 1568), (8224, 2080, 2080),
-                                   (2336, 1504, 4128), (1056, 1056, 2848), (4000, 576, 2304), (320, 2048, 512)])
+                                   (2336, 1504, 4128), (1056, 1056, 2848), (4128, 1280, 1280), (5056, 1120, 1184), (4000, 576, 2304), (320, 2048, 512)])
 @pytest.mark.parametrize("dw_dtype", [0, 1])
 def test_products_of_a_backward_pass(mx, M, K, N, dw_dtype):
     """dX and dW from given operands, as one launch makes them where it does, against the two products of the oracle, within the
