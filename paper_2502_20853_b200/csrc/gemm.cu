@@ -207,8 +207,8 @@ __device__ __forceinline__ uint32_t idesc_mxf4(int n, uint32_t a_sf_id, uint32_t
 // fetch it together, a bf16 pair per lane and turn, before the wait for the accumulator (bias_fetch; zero beyond N, where
 // nothing is stored), put it into the warp's own line of shared memory (bias_stage), and read it back as broadcasts, 16 bytes
 // at a time, for the mixed-precision add, which takes bf16 values as they are (add_bias_chunk).  50432 x 4096 x 1024, back to
-// back: 109 us without a bias, 120 with it; passing the pairs round with shuffles instead took 123 to 125 us, every lane
-// fetching every value by itself behind the wait 160.
+// back: 99 us without a bias, 102 with it.  (When the kernel took 109 and 120 us, passing the pairs round with shuffles instead
+// took 123 to 125, every lane fetching every value by itself behind the wait 160.)
 template <int COLS>
 __device__ __forceinline__ void bias_fetch(uint32_t (&w)[(COLS + 63) / 64], const __nv_bfloat16 *bias, int64_t col, int64_t N, int lane)
 {
@@ -2889,8 +2889,8 @@ mxfp4_status_t quantize_gelu_chain(const void *y_bf16, int64_t rows, int64_t col
 // Whether the product and the quantization run as two kernels: when the epilogue is GELU with the double-quantization chain,
 // Y is stored anyway, and there are at least four 128 x 128 tiles per SM.  The fused epilogue has eight warps per SM for the
 // cast, the hook and both passes, and they are the bottleneck; the two kernels read Y back (2 of 5 bytes per element more)
-// but run at the product's and the tile quantizer's own rates: fused / two kernels 84 / 66.3 us at 25216 x 1536 x 384,
-// 396 / 314 at 50432 x 4096 x 1024, 305 / 237 at 401408 x 384 x 96, 33.6 / 31.7 at 8192 x 1536 x 384 (5.2 tiles per SM), but
+// but run at the product's and the tile quantizer's own rates: fused / two kernels 84 / 64.2 us at 25216 x 1536 x 384,
+// 396 / 307 at 50432 x 4096 x 1024, 305 / 226 at 401408 x 384 x 96, 33.6 / 31.7 at 8192 x 1536 x 384 (5.2 tiles per SM), but
 // 20.6 / 22.5 at 4096 x 1536 x 384 (2.6) and 12.3 / 15.3 at 1024 x 768 x 192, where a second launch costs more.
 static bool two_pass(const mxfp4_epilogue_t *epi, int64_t M, int64_t N)
 {
