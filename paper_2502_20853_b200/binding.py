@@ -46,6 +46,7 @@ class CMat(C.Structure):
 
 
 _NO_MAT = CMat(None, None, 0, 0)
+_U64 = 0xFFFFFFFFFFFFFFFF
 
 
 class CQParams(C.Structure):
@@ -219,8 +220,10 @@ class QMat(_host.Mat):
     def device(self):
         return (self._buf if self._buf is not None else self._data).device
 
+    # what hands the contents out also gives up what was made of them (see LinearCtx): they may be written through it
     @property
     def data(self):
+        self._q4 = None
         if self._data is None:
             n = self.rows * (self.cols // 2)
             self._data = self._buf[self._at:self._at + n].view(self.rows, self.cols // 2)
@@ -228,12 +231,14 @@ class QMat(_host.Mat):
 
     @property
     def scales(self):
+        self._q4 = None
         if self._scales is None:
             at = self._at + _align256(self.rows * (self.cols // 2))
             self._scales = self._buf[at:at + max(scale_bytes(self.rows, self.cols), 16)]
         return self._scales
 
     def c(self):
+        self._q4 = None
         return CMat(self.data_addr, self.scales_addr, self.rows, self.cols)
 
     def scales_linear(self):
@@ -247,7 +252,7 @@ class QMat(_host.Mat):
 
 
 def _qp(scale_mode, rounding, seed, stream_id):
-    return CQParams(scale_mode, rounding, seed & 0xFFFFFFFFFFFFFFFF, stream_id, 0)
+    return CQParams(scale_mode, rounding, seed & _U64, stream_id, 0)
 
 
 def _bf16_2d(x):
@@ -422,16 +427,33 @@ class LinearCtx:
     """Forward operands kept for the backward pass.  With ``xq_t`` (a QMat [K, M]) and ``seed`` the forward pass also
     makes the backward operand Q6 of this step in its pass over X.  ``wq_t`` (a QMat [K, N]) is the backward operand Q4:
     made ahead by the caller with ``quantize_t(wq, rounding=ROUND_STOCHASTIC, seed=seed, stream_id=4)``, or written by
-    ``linear_fwd`` itself when that is given the weight ``w`` (one pass over W then makes Q2 and Q4)."""
+    ``linear_fwd`` itself when that is given the weight ``w`` (one pass over W then makes Q2 and Q4).
+
+    A ``wq_t`` that ``linear_fwd`` provided by itself (``_made``) is nothing the caller vouches for: ``wq._q4`` says what it was
+    made with, and is gone as soon as ``wq`` is written again or its contents are handed out; ``linear_bwd`` uses it only
+    where it would make the same Q4, and makes its own otherwise."""
+
+    _made = None
 
     def __init__(self, xq, wq, xq_t=None, seed=0, wq_t=None):
         self.xq, self.wq, self.xq_t, self.seed, self.wq_t = xq, wq, xq_t, seed, wq_t
+
+    def _q4(self, seed, scale_mode, dev_status):
+        """wq_t, or None if linear_fwd made it and it is not the Q4 of a backward pass with these arguments."""
+        if self.wq_t is not self._made or self.wq_t is None:
+            return self.wq_t
+        m = self.wq._q4
+        # (a graph that holds the backward pass alone is replayed with whatever wq holds then; a status word that the forward
+        # pass was not given has not seen Q4's non-finite groups)
+        ok = (m is not None and m[0] is self.wq_t and m[1] == seed & _U64 and m[2] == scale_mode and m[3] == torch.cuda.is_current_stream_capturing()
+              and (m[4] or dev_status is None))
+        return self.wq_t if ok else None
 
 
 def linear_fwd(x, w=None, wq=None, bias=None, scale_mode=SCALE_TRUNCATION_FREE, ctx=None, out=None, dev_status=None,
                bwd_seed=None, epi=None):
     """Y = Q1(X) Q2(W)^T.  Give ``w`` (bf16 [N, K]) or an already quantized ``wq`` (e.g. from qema_quantize).
-    ``bwd_seed``: also make Q6 for the backward pass that will be called with this seed.
+    ``bwd_seed``: also make Q6 for the backward pass that will be called with this seed and, given ``w`` and no ``ctx``, Q4.
     ``x = None``: ``ctx.xq`` (and ``ctx.xq_t``) already hold the quantized input (written by the previous layer's
     epilogue).  ``epi`` (an Epilogue): the product runs with that quantizing epilogue, which names its own outputs;
     the first return value is then ``epi``."""
@@ -455,12 +477,16 @@ def linear_fwd(x, w=None, wq=None, bias=None, scale_mode=SCALE_TRUNCATION_FREE, 
         if bwd_seed is not None:
             xq, xq_t = QMat.two(m, k, k, m, dev)
             ctx = LinearCtx(xq, wq, xq_t, bwd_seed, wq_t)
+            ctx._made = wq_t
         else:
             ctx = LinearCtx(QMat(m, k, dev), wq)
-    elif bwd_seed is not None:
-        ctx.seed = bwd_seed
-        if ctx.xq_t is None:
-            ctx.xq_t = QMat(k, m, dev)
+    else:
+        if bwd_seed is not None:
+            ctx.seed = bwd_seed
+            if ctx.xq_t is None:
+                ctx.xq_t = QMat(k, m, dev)
+        if ctx._made is not None and ctx.wq_t is ctx._made and (w is None or bwd_seed is None):
+            ctx.wq_t = ctx._made = None      # of an earlier pass
     n = ctx.wq.rows
     if epi is None:
         y = out = out if out is not None else _new((m, n), torch.bfloat16, dev)
@@ -474,6 +500,8 @@ def linear_fwd(x, w=None, wq=None, bias=None, scale_mode=SCALE_TRUNCATION_FREE, 
            _host.linear_fwd(lib().at_linear_fwd_ex, _ptr(x), x.stride(0) if x is not None else 0, m, k, _ptr(w), n, _ptr(bias), _ptr(y),
                             y.stride(0) if y is not None else 0, ctx.xq, ctx.wq, ctx.xq_t, ctx.wq_t, ctx.seed, scale_mode,
                             C.addressof(ce) if ce is not None else None, _ptr(dev_status), _stream()))
+    if ctx._made is not None and ctx.wq_t is ctx._made:
+        ctx.wq._q4 = (ctx.wq_t, ctx.seed & _U64, scale_mode, torch.cuda.is_current_stream_capturing(), dev_status is not None)
     return (epi if epi is not None else out), ctx
 
 
@@ -498,7 +526,7 @@ def linear_bwd(dy, ctx, seed, scale_mode=SCALE_TRUNCATION_FREE, dw_dtype=OUT_FP3
         dyq = dyq_t = None
     _check("mxfp4_linear_bwd_ex",
            _host.linear_bwd(lib().at_linear_bwd_ex, _ptr(dy), dy.stride(0) if dy is not None else 0, dyq, dyq_t, ctx.xq, ctx.wq, ctx.xq_t,
-                            ctx.wq_t, ctx.seed, seed, scale_mode, _ptr(dx) if ce is None else None, dx.stride(0) if ce is None else 0,
+                            ctx._q4(seed, scale_mode, dev_status), ctx.seed, seed, scale_mode, _ptr(dx) if ce is None else None, dx.stride(0) if ce is None else 0,
                             dw.data_ptr(), dw.stride(0), dw_dtype, C.addressof(ce) if ce is not None else None, workspace.data_ptr(),
                             workspace.numel(), _ptr(dev_status), _stream()))
     return (epi_dx if epi_dx is not None else dx), dw

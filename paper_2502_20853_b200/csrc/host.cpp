@@ -20,6 +20,7 @@ struct Mat {
     mxfp4_mat_t m;
     PyObject *buf, *data, *scales;   // one buffer for both (data, scales: views of it, made when asked for) or two tensors
     Py_ssize_t at;                   // where the codes start in buf
+    PyObject *q4;                    // what binding.linear_fwd made of it besides (see there); gone once the matrix may have changed
 };
 
 int mat_traverse(PyObject *o, visitproc visit, void *arg)
@@ -28,6 +29,7 @@ int mat_traverse(PyObject *o, visitproc visit, void *arg)
     Py_VISIT(s->buf);
     Py_VISIT(s->data);
     Py_VISIT(s->scales);
+    Py_VISIT(s->q4);
     return 0;
 }
 int mat_clear(PyObject *o)
@@ -36,6 +38,7 @@ int mat_clear(PyObject *o)
     Py_CLEAR(s->buf);
     Py_CLEAR(s->data);
     Py_CLEAR(s->scales);
+    Py_CLEAR(s->q4);
     return 0;
 }
 void mat_dealloc(PyObject *o)
@@ -54,6 +57,7 @@ PyMemberDef mat_members[] = {
     {"_data", T_OBJECT, offsetof(Mat, data), 0, nullptr},
     {"_scales", T_OBJECT, offsetof(Mat, scales), 0, nullptr},
     {"_at", T_PYSSIZET, offsetof(Mat, at), 0, nullptr},
+    {"_q4", T_OBJECT, offsetof(Mat, q4), 0, nullptr},
     {nullptr, 0, 0, 0, nullptr}};
 
 PyTypeObject mat_type = {PyVarObject_HEAD_INIT(nullptr, 0)};
@@ -82,6 +86,13 @@ struct Args {
             bad = true;
         }
         return mxfp4_mat_t{nullptr, nullptr, 0, 0};
+    }
+    // a matrix that the call writes
+    mxfp4_mat_t dst(int i)
+    {
+        const mxfp4_mat_t m = mat(i);
+        if (!bad && given(i)) Py_CLEAR(reinterpret_cast<Mat *>(a[i])->q4);
+        return m;
     }
     // Runs the call without the interpreter lock and returns its status.
     template <class F> PyObject *run(F &&f)
@@ -156,7 +167,7 @@ PyObject *h_linear_fwd(PyObject *, PyObject *const *a, Py_ssize_t n)
     if (!counted("linear_fwd", n, 19)) return nullptr;
     Args r{a};
     const auto f = reinterpret_cast<decltype(&mxfp4_linear_fwd_ex)>(r.ptr(0));
-    mxfp4_linear_ctx_t c{r.mat(10), r.mat(11), r.mat(12), r.u64(14), r.mat(13), r.u64(14)};
+    mxfp4_linear_ctx_t c{r.mat(10), r.given(5) ? r.dst(11) : r.mat(11), r.mat(12), r.u64(14), r.mat(13), r.u64(14)};
     const void *x = r.ptr(1), *w = r.ptr(5), *bias = r.ptr(7);
     void *y = r.ptr(8), *stream = r.ptr(18);
     const int64_t ldx = r.i64(2), m = r.i64(3), k = r.i64(4), nn = r.i64(6), ldy = r.i64(9);
@@ -197,7 +208,7 @@ PyObject *h_quantize(PyObject *, PyObject *const *a, Py_ssize_t n)
     const mxfp4_qparams_t qp{r.i32(6), r.i32(7), r.u64(8), (uint32_t)r.u64(9), 0u};
     const void *x = r.ptr(1);
     const int64_t rows = r.i64(2), cols = r.i64(3), ld = r.i64(4);
-    const mxfp4_mat_t dst = r.mat(5);
+    const mxfp4_mat_t dst = r.dst(5);
     auto *status = r.ptr<uint32_t>(10);
     void *stream = r.ptr(11);
     return r.run([&] { return f(x, rows, cols, ld, dst, &qp, status, stream); });
@@ -212,7 +223,7 @@ PyObject *h_quantize_t(PyObject *, PyObject *const *a, Py_ssize_t n)
     const mxfp4_qparams_t qp{r.i32(7), r.i32(8), r.u64(9), (uint32_t)r.u64(10), 0u};
     const void *x = r.ptr(1);
     const bool given = r.given(2);
-    const mxfp4_mat_t src = r.mat(2), dst = r.mat(6);
+    const mxfp4_mat_t src = r.mat(2), dst = r.dst(6);
     const int64_t rows = r.i64(3), cols = r.i64(4), ld = r.i64(5);
     auto *status = r.ptr<uint32_t>(11);
     void *stream = r.ptr(12);
@@ -231,9 +242,9 @@ PyObject *h_qema(PyObject *, PyObject *const *a, Py_ssize_t n)
     float *ema = r.ptr<float>(2);
     const int32_t update = r.i32(4), mode = r.i32(8);
     const int64_t nn = r.i64(5), k = r.i64(6);
-    const mxfp4_mat_t dst = r.mat(7);
+    const mxfp4_mat_t dst = r.dst(7);
     const bool osc = r.given(9);
-    const mxfp4_osc_state_t o{r.ptr(9), r.mat(10), r.ptr<float>(11), r.ptr<float>(12)};
+    const mxfp4_osc_state_t o{r.ptr(9), r.dst(10), r.ptr<float>(11), r.ptr<float>(12)};
     auto *status = r.ptr<uint32_t>(13);
     void *stream = r.ptr(14);
     return r.run([&] { return f(w, ema, (float)beta, update, nn, k, dst, mode, osc ? &o : nullptr, status, stream); });

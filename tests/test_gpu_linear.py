@@ -312,3 +312,45 @@ def test_products_of_a_backward_pass(mx, M, K, N, dw_dtype):
     for got, a, b, shape, bf16, what in ((dx, dyq, wq_t, (M, K, N), True, "dX"), (dw, dyq_t, xq_t, (N, K, M), dw_dtype == 0, "dW")):
         want, t = orc.gemm(*a, *b)
         check_gemm_bound(got.float().cpu().numpy(), want, t, bf16, what, factor=max(1.0, mx.gemm_chain_mmas(*shape) / 8))
+
+
+@pytest.mark.parametrize("what", ["nothing", "second pass", "second pass, one seed", "weight quantized again", "another weight", "codes written", "scale rule",
+                                  "weight given again", "weight given again without a seed", "status of the backward pass alone"])
+def test_q4_that_the_forward_pass_made_is_used_only_where_it_holds(mx, what):
+    """linear_fwd, given the weight and the backward seed, makes Q4 too.  Whatever happens to the context between the passes, the
+    backward pass gives what it gives with a Q4 made from ctx.wq then, by its own seed and scale rule."""
+    M, K, N = 160, 96, 288
+    g = torch.Generator(device="cuda").manual_seed(3)
+    x, x2 = (torch.randn((M, K), generator=g, device="cuda").to(torch.bfloat16) for _ in range(2))
+    w, w2 = ((torch.randn((N, K), generator=g, device="cuda") * s).to(torch.bfloat16) for s in (0.02, 0.5))
+    dy = torch.randn((M, N), generator=g, device="cuda").to(torch.bfloat16)
+    if what == "status of the backward pass alone":
+        w[5, 7] = float("inf")
+    _, ctx = mx.linear_fwd(x, w, bwd_seed=1)
+    seed, mode, st = 1, mx.SCALE_TRUNCATION_FREE, mx.new_status()
+    if what == "second pass":
+        seed = 2
+        mx.linear_fwd(x2, ctx=ctx, bwd_seed=seed)
+    elif what == "second pass, one seed":
+        mx.quantize(w2, out=ctx.wq)
+        mx.linear_fwd(x2, ctx=ctx, bwd_seed=seed)
+    elif what == "weight quantized again":
+        mx.qema_quantize(w2, w2.float(), out=ctx.wq)
+    elif what == "another weight":
+        ctx.wq = mx.quantize(w2)
+    elif what == "codes written":
+        ctx.wq.data.copy_(mx.quantize(w2).data)
+    elif what == "scale rule":
+        mode = mx.SCALE_FLOOR
+    elif what == "weight given again":
+        seed = 2
+        mx.linear_fwd(x2, w2, ctx=ctx, bwd_seed=seed)
+    elif what == "weight given again without a seed":
+        mx.linear_fwd(x2, w2, ctx=ctx)
+    dx, dw = mx.linear_bwd(dy, ctx, seed, scale_mode=mode, dev_status=st)
+    fresh = mx.LinearCtx(ctx.xq, ctx.wq, xq_t=ctx.xq_t, seed=ctx.seed)
+    st2 = mx.new_status()
+    want_dx, want_dw = mx.linear_bwd(dy, fresh, seed, scale_mode=mode, dev_status=st2)
+    torch.cuda.synchronize()
+    assert torch.equal(dx.view(torch.int16), want_dx.view(torch.int16)) and torch.equal(dw.view(torch.int32), want_dw.view(torch.int32))
+    assert int(st.item()) == int(st2.item())
