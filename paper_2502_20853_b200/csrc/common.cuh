@@ -34,7 +34,9 @@ extern std::atomic<unsigned long long> g_launches;
 // Every kernel of the step is launched with programmatic stream serialization: its blocks may be placed and set up while the
 // kernel before it drains, and wait for it (all of its blocks done, their memory visible) before they touch global memory.
 // Each block calls pdl_wait() before its first access to global memory: a kernel whose blocks could end without having waited
-// would let its successor overtake its predecessor.  The element-wise and tile quantizing kernels call
+// would let its successor overtake its predecessor.  In the GEMM kernels every thread calls it, also in the roles that touch
+// shared and tensor memory alone: their bounded waits for a stage must not start to count before the kernel's inputs exist.
+// The element-wise and tile quantizing kernels call
 // pdl_launch_dependents() first of all (the next kernel may be placed once every block of this one has started); the GEMM
 // kernels do not call it, so that their successor starts when their blocks end: with the call the successor's blocks took
 // over the first free SMs piecemeal, and a step got slower (43.0 against 36.5 us for an evaluation of 19700 tokens on

@@ -86,3 +86,47 @@ def test_selftest_argument_errors(mx):
         mx.gemm_wait_selftest(a, b, mx.new_status(), spin_limit=4)          # below the allowed range
     with pytest.raises(mx.MxError):
         mx.gemm_wait_selftest(a, b, None)                                    # the status word is required
+
+
+@pytest.fixture(scope="module")
+def hold():
+    """A kernel that lets its successor be placed at once and then takes its time (0.6 s, twice the bound of a wait)."""
+    kernel = torch.cuda._compile_kernel(r"""
+        extern "C" __global__ void hold(long long ns)
+        {
+            asm volatile("griddepcontrol.launch_dependents;");
+            unsigned long long t0, t;
+            asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t0));
+            for (int i = 0; i < 2000000; i++) {
+                asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
+                if ((long long)(t - t0) >= ns) break;
+                __nanosleep(1000);
+            }
+        }""", "hold")
+    return lambda: kernel(grid=(1, 1, 1), block=(32, 1, 1), args=[600_000_000])
+
+
+# one tile per CTA, B-stationary, CTA pairs with split K, cluster split-K, CTA pairs with the B block resident
+@pytest.mark.parametrize("M,N,K", [(256, 128, 512), (9600, 384, 512), (1024, 512, 2048), (1280, 768, 4096), (4864, 1536, 1024)])
+def test_waits_count_from_the_inputs_on(mx, hold, M, N, K):
+    """A product whose blocks are in place long before its inputs exist (behind a slow kernel that lets the quantizer be placed,
+    which lets the product be placed) waits for them without its own waits running out."""
+    g = torch.Generator(device="cuda").manual_seed(M)
+    x = torch.randn((M, K), generator=g, device="cuda").to(torch.bfloat16)
+    b = mx.quantize(torch.randn((N, K), generator=g, device="cuda").to(torch.bfloat16))
+    a = mx.QMat(M, K)
+    st, ws = mx.new_status(), torch.empty(max(mx.gemm_workspace_bytes(M, N, K), 16), dtype=torch.uint8, device="cuda")
+    got, want = (torch.full((M, N), float("nan"), dtype=torch.bfloat16, device="cuda") for _ in range(2))
+    zq = [mx.QMat(M, N), mx.QMat(M, N)]
+    torch.cuda.synchronize()
+    for out, z, slow in ((got, zq[0], True), (want, zq[1], False)):
+        for product in (lambda: mx.gemm(a, b, out=out, workspace=ws, dev_status=st), lambda: mx.gemm_quant(a, b, mx.Epilogue(zq=z), dev_status=st)):
+            if slow:
+                a.data.zero_()
+                torch.cuda.synchronize()
+                hold()
+            mx.quantize(x, out=a, dev_status=st)
+            product()
+            torch.cuda.synchronize()
+    assert int(st.item()) == 0
+    assert torch.equal(got, want) and torch.equal(zq[0].data, zq[1].data) and torch.equal(zq[0].scales, zq[1].scales)
