@@ -36,20 +36,16 @@ extern std::atomic<unsigned long long> g_launches;
 // Each block calls pdl_wait() before its first access to global memory: a kernel whose blocks could end without having waited
 // would let its successor overtake its predecessor.  In the GEMM kernels every thread calls it, also in the roles that touch
 // shared and tensor memory alone: their bounded waits for a stage must not start to count before the kernel's inputs exist.
-// The element-wise and tile quantizing kernels call
-// pdl_launch_dependents() first of all (the next kernel may be placed once every block of this one has started); the GEMM
-// kernels do not call it, so that their successor starts when their blocks end: with the call the successor's blocks took
-// over the first free SMs piecemeal, and a step got slower (43.0 against 36.5 us for an evaluation of 19700 tokens on
-// DeiT-Base's qkv, 40.7 with plain launches; 107.9 / 102.6 / 116.0 for DeiT-Small's fc1 step).
+// The element-wise and tile quantizing kernels call pdl_launch_dependents() first of all (the next kernel may be placed once
+// every block of this one has started); the GEMM kernels do not call it, so that their successor starts when their blocks end:
+// with the call the successor's blocks took over the first free SMs piecemeal, and a step got slower (43.0 against 36.5 us for an
+// evaluation of 19700 tokens on DeiT-Base's qkv, 40.7 with plain launches; 107.9 / 102.6 / 116.0 for DeiT-Small's fc1 step).
+//
+// A block may thus be on its SM while its inputs are still being written: nothing may be read through the path for data that is
+// constant for a kernel's lifetime.  Loads are plain ones, and pointers to inputs carry no __restrict__, which would let the
+// compiler take that path (and move a load above the wait).
 __device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-// Pointers to read-only inputs go through this after the wait, so that no load of them can be moved above it.
-template <typename T>
-__device__ __forceinline__ T *after_wait(T *p)
-{
-    asm volatile("" : "+l"(p)::"memory");
-    return p;
-}
 
 template <typename... Params, typename... Args>
 inline cudaError_t launch_pdl(void (*kernel)(Params...), unsigned grid_x, unsigned grid_y, unsigned threads, size_t smem, cudaStream_t st, const Args &...args)
@@ -304,10 +300,10 @@ __device__ __forceinline__ uint32_t absmax_fold(uint32_t acc, uint32_t w)
 }
 __device__ __forceinline__ uint32_t absmax_fold_end(uint32_t acc) { return acc & 0x7FFF7FFFu; }
 
-__device__ __forceinline__ uint4 ld_nc_16(const void *p)
+__device__ __forceinline__ uint4 ld_stream_16(const void *p)
 {
     uint4 v;
-    asm volatile("ld.global.nc.L1::no_allocate.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p));
+    asm volatile("ld.global.L1::no_allocate.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p));
     return v;
 }
 

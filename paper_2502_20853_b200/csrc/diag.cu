@@ -43,7 +43,7 @@ __global__ void __launch_bounds__(256) k_quant_conf_hist(const __nv_bfloat16 *__
         const uint4 *p = reinterpret_cast<const uint4 *>(w + gid * 32);
         uint4 q[4];
 #pragma unroll
-        for (int j = 0; j < 4; j++) q[j] = ld_nc_16(p + j);
+        for (int j = 0; j < 4; j++) q[j] = ld_stream_16(p + j);
         uint32_t am = 0;
 #pragma unroll
         for (int j = 0; j < 4; j++) {
@@ -105,7 +105,7 @@ __global__ void __launch_bounds__(256) k_change_sums(const __nv_bfloat16 *__rest
     float d2 = 0.f, p2 = 0.f;
     const int64_t octs = count / 8;
     for (int64_t i = blockIdx.x * (int64_t)256 + threadIdx.x; i < octs; i += (int64_t)gridDim.x * 256) {
-        const uint4 c = ld_nc_16(reinterpret_cast<const uint4 *>(cur) + i), p = ld_nc_16(reinterpret_cast<const uint4 *>(prev) + i);
+        const uint4 c = ld_stream_16(reinterpret_cast<const uint4 *>(cur) + i), p = ld_stream_16(reinterpret_cast<const uint4 *>(prev) + i);
         const uint32_t cw[4] = {c.x, c.y, c.z, c.w}, pw[4] = {p.x, p.y, p.z, p.w};
 #pragma unroll
         for (int t = 0; t < 4; t++) {

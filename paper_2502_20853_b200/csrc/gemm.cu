@@ -216,7 +216,7 @@ __device__ __forceinline__ void bias_fetch(uint32_t (&w)[(COLS + 63) / 64], cons
     for (int i = 0; i < (COLS + 63) / 64; i++) {
         const int64_t c = col + 64 * i + 2 * lane;
         w[i] = 0u;
-        if (bias != nullptr && c < N) asm volatile("ld.global.nc.u32 %0, [%1];" : "=r"(w[i]) : "l"(bias + c));
+        if (bias != nullptr && c < N) asm volatile("ld.global.u32 %0, [%1];" : "=r"(w[i]) : "l"(bias + c));
     }
 }
 template <int COLS>
@@ -245,7 +245,7 @@ __device__ __forceinline__ uint32_t load_bias_pair(const __nv_bfloat16 *bias, in
 {
     const int64_t c = col + 2 * (lane & 15);
     uint32_t v = 0u;
-    if (bias != nullptr && c < N) asm volatile("ld.global.nc.u32 %0, [%1];" : "=r"(v) : "l"(bias + c));
+    if (bias != nullptr && c < N) asm volatile("ld.global.u32 %0, [%1];" : "=r"(v) : "l"(bias + c));
     return v;
 }
 __device__ __forceinline__ void add_bias_chunk_shfl(uint32_t (&r)[32], uint32_t pair)
@@ -839,7 +839,7 @@ k_gemm_mxf4_q(const __grid_constant__ CUtensorMap map_a, const __grid_constant__
                     } else if (live) {
                         const uint4 *ap = reinterpret_cast<const uint4 *>(e.aux + (int64_t)grow * e.ld_aux + col);
 #pragma unroll
-                        for (int j = 0; j < 4; j++) aw[j] = ld_nc_16(ap + j);
+                        for (int j = 0; j < 4; j++) aw[j] = ld_stream_16(ap + j);
                     }
                     const uint32_t *a32 = reinterpret_cast<const uint32_t *>(aw);
 #pragma unroll
@@ -2284,15 +2284,14 @@ k_gemm_mxf4_pbs(const __grid_constant__ CUtensorMap map_a, const __grid_constant
 // 32.5 -> 24.9 us, 128 x 128 x 50432 9.0 -> 7.9, both with the higher limit on the splits), one where the output fills the
 // machine (384 x 384 x 25216: 11.8 us, 12.9 with eight).
 template <int GROUPS>
-__global__ void __launch_bounds__(256) k_splitk_reduce(const float *__restrict__ part, int splits, int64_t M, int64_t N,
+__global__ void __launch_bounds__(256) k_splitk_reduce(const float *part, int splits, int64_t M, int64_t N,
                                                        void *__restrict__ d, int64_t ldd, int out_fp32,
-                                                       const __nv_bfloat16 *__restrict__ bias)
+                                                       const __nv_bfloat16 *bias)
 {
     constexpr int kCols = 256 / GROUPS;
     __shared__ float4 s_sum[GROUPS][kCols];
     pdl_launch_dependents();
     pdl_wait();
-    part = after_wait(part), bias = after_wait(bias);
     const int64_t total4 = M * N / 4;
     const int c = threadIdx.x % kCols, g = threadIdx.x / kCols;
     for (int64_t i0 = blockIdx.x * (int64_t)kCols; i0 < total4; i0 += (int64_t)gridDim.x * kCols) {
@@ -2300,9 +2299,14 @@ __global__ void __launch_bounds__(256) k_splitk_reduce(const float *__restrict__
         float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
         if (i < total4 && g < splits) {
             acc = *reinterpret_cast<const float4 *>(part + (size_t)g * M * N + e);
-            for (int s = g + GROUPS; s < splits; s += GROUPS) {
-                const float4 v = *reinterpret_cast<const float4 *>(part + (size_t)s * M * N + e);
-                acc.x += v.x; acc.y += v.y; acc.z += v.z; acc.w += v.w;
+            for (int s = g + GROUPS; s < splits; s += 8 * GROUPS) {      // eight loads in flight
+                float4 v[8];
+#pragma unroll
+                for (int j = 0; j < 8; j++)
+                    if (s + j * GROUPS < splits) v[j] = *reinterpret_cast<const float4 *>(part + (size_t)(s + j * GROUPS) * M * N + e);
+#pragma unroll
+                for (int j = 0; j < 8; j++)
+                    if (s + j * GROUPS < splits) acc.x += v[j].x, acc.y += v[j].y, acc.z += v[j].z, acc.w += v[j].w;
             }
         }
         if (GROUPS > 1) {

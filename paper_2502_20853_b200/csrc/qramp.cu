@@ -21,7 +21,7 @@ __device__ __forceinline__ uint32_t ramp_factor(float dw, float dq, float k1, fl
     return (uint32_t)(n < n_max ? n : n_max);
 }
 
-__global__ void __launch_bounds__(256) k_qramp_detect(const float *__restrict__ dist_w, const float *__restrict__ dist_q,
+__global__ void __launch_bounds__(256) k_qramp_detect(const float *dist_w, const float *dist_q,
                                                       int64_t count, float k1, float inv_k1, int k2, int n_max,
                                                       uint8_t *__restrict__ n_w, unsigned long long *oscillating)
 {
@@ -29,7 +29,6 @@ __global__ void __launch_bounds__(256) k_qramp_detect(const float *__restrict__ 
     __shared__ uint32_t s_osc[8];
     pdl_launch_dependents();
     pdl_wait();
-    dist_w = after_wait(dist_w), dist_q = after_wait(dist_q);
     uint32_t osc = 0;
     const int64_t octs = (count + 7) / 8;     // eight elements per thread and turn: 64 bytes of loads in flight
     for (int64_t q = blockIdx.x * (int64_t)256 + threadIdx.x; q < octs; q += (int64_t)gridDim.x * 256) {
@@ -89,13 +88,12 @@ __device__ __forceinline__ bool adamw_one(float &w, float g, float &m, float &v,
 }
 
 __global__ void __launch_bounds__(256) k_qramp_adamw(float *__restrict__ w, __nv_bfloat16 *__restrict__ w_bf16,
-                                                     const float *__restrict__ grad, float *__restrict__ m, float *__restrict__ v,
+                                                     const float *grad, float *__restrict__ m, float *__restrict__ v,
                                                      float *__restrict__ acc, uint8_t *__restrict__ cnt,
-                                                     const uint8_t *__restrict__ n_w, int64_t count, const AdamW h)
+                                                     const uint8_t *n_w, int64_t count, const AdamW h)
 {
     pdl_launch_dependents();
     pdl_wait();
-    grad = after_wait(grad), n_w = after_wait(n_w);
     const int64_t i0 = (blockIdx.x * (int64_t)256 + threadIdx.x) * 4;
     if (i0 + 3 < count) {
         float4 W = *reinterpret_cast<const float4 *>(w + i0), G = *reinterpret_cast<const float4 *>(grad + i0);

@@ -14,7 +14,7 @@ namespace mx {
 // of the 12 and 15 us of the whole quantization with the gaps around it).
 // ------------------------------------------------------------------------------------------------
 template <int ROUNDING>
-__global__ void __launch_bounds__(256) k_quantize_rows(const __nv_bfloat16 *__restrict__ src, int64_t rows, int nblk,
+__global__ void __launch_bounds__(256) k_quantize_rows(const __nv_bfloat16 *src, int64_t rows, int nblk,
                                                        int64_t ld, uint8_t *__restrict__ packed,
                                                        uint8_t *__restrict__ scales, int nblk4, int scale_mode,
                                                        const SrStream sr, uint32_t *dev_status)
@@ -32,7 +32,7 @@ __global__ void __launch_bounds__(256) k_quantize_rows(const __nv_bfloat16 *__re
     const uint4 *p = reinterpret_cast<const uint4 *>(src + row * ld + blk * 32);
     uint4 q[4];
 #pragma unroll
-    for (int j = 0; j < 4; j++) q[j] = ld_nc_16(p + j);
+    for (int j = 0; j < 4; j++) q[j] = ld_stream_16(p + j);
     uint32_t am = 0;
 #pragma unroll
     for (int j = 0; j < 4; j++) am = absmax_u4(am, q[j]);
@@ -73,7 +73,7 @@ __global__ void __launch_bounds__(256) k_quantize_rows(const __nv_bfloat16 *__re
 constexpr int kPitch = 2 * kTile + 16;   // bytes per staged row (16-byte skew against bank conflicts)
 
 template <bool SR_T>
-__global__ void __launch_bounds__(256, 3) k_requantize_tile(const void *__restrict__ src, const uint8_t *__restrict__ src_scales,
+__global__ void __launch_bounds__(256, 3) k_requantize_tile(const void *src, const uint8_t *src_scales,
                                                             int src_nblk4, int rows, int cols, const __grid_constant__ QuantSide tr,
                                                             uint32_t *dev_status)
 {
@@ -92,8 +92,8 @@ __global__ void __launch_bounds__(256, 3) k_requantize_tile(const void *__restri
     {
         // packed source: one thread per (row, 32-element group): 16 bytes of codes + 1 scale byte
         pdl_wait();
-        const uint8_t *s = after_wait(static_cast<const uint8_t *>(src));
-        const uint8_t *sc_chunk = after_wait(src_scales) + ((size_t)(row0 >> 7) * src_nblk4 + (col0 >> 7)) * 512;
+        const uint8_t *s = static_cast<const uint8_t *>(src);
+        const uint8_t *sc_chunk = src_scales + ((size_t)(row0 >> 7) * src_nblk4 + (col0 >> 7)) * 512;
 #pragma unroll
         for (int it = 0; it < 2; it++) {
             const int item = it * 256 + tid;
@@ -102,7 +102,7 @@ __global__ void __launch_bounds__(256, 3) k_requantize_tile(const void *__restri
             uint32_t w[4] = {0, 0, 0, 0};
             uint32_t sc2 = 0u;
             if (gr < rows && gc < cols) {
-                const uint4 q = ld_nc_16(s + (int64_t)gr * (cols >> 1) + (gc >> 1));
+                const uint4 q = ld_stream_16(s + (int64_t)gr * (cols >> 1) + (gc >> 1));
                 w[0] = q.x; w[1] = q.y; w[2] = q.z; w[3] = q.w;
                 const uint32_t sb = sc_chunk[(r & 31) * 16 + (r >> 5) * 4 + g];
                 // a 0xFF scale marks a non-finite group of the first quantizer: propagate NaN
@@ -389,14 +389,13 @@ __device__ __forceinline__ float qema_target(float v, float ve)
 // Four consecutive lanes share a 32-element group: a thread owns 8 consecutive elements (the weight is contiguous).  The grid
 // covers the scale buffer with its padding entries, as in the row-wise quantizer.
 template <bool OSC>
-__global__ void __launch_bounds__(256) k_qema(const __nv_bfloat16 *__restrict__ w, float *__restrict__ ema, float beta,
+__global__ void __launch_bounds__(256) k_qema(const __nv_bfloat16 *w, float *__restrict__ ema, float beta,
                                               int update_ema, int64_t n, int nblk, uint8_t *__restrict__ packed,
                                               uint8_t *__restrict__ scales, int nblk4, int scale_mode, OscPtrs osc,
                                               uint32_t *dev_status)
 {
     pdl_launch_dependents();
     pdl_wait();
-    w = after_wait(w);
     const uint64_t gid = blockIdx.x * (uint64_t)256 + threadIdx.x, grp_pad = gid >> 2;
     const uint32_t nb_pad = (uint32_t)nblk4 * 4u;
     const int64_t row_pad = (grp_pad >> 32) ? (int64_t)(grp_pad / nb_pad) : (int64_t)((uint32_t)grp_pad / nb_pad);
@@ -499,12 +498,11 @@ __global__ void __launch_bounds__(256) k_qema(const __nv_bfloat16 *__restrict__ 
 // ------------------------------------------------------------------------------------------------
 // Exact dequantization, one thread per group.
 // ------------------------------------------------------------------------------------------------
-__global__ void __launch_bounds__(256) k_dequantize(const uint8_t *__restrict__ packed, const uint8_t *__restrict__ scales,
+__global__ void __launch_bounds__(256) k_dequantize(const uint8_t *packed, const uint8_t *scales,
                                                     int64_t rows, int nblk, int nblk4, float *__restrict__ dst, int64_t ld)
 {
     pdl_launch_dependents();
     pdl_wait();
-    packed = after_wait(packed), scales = after_wait(scales);
     const int64_t gid = blockIdx.x * (int64_t)256 + threadIdx.x;
     if (gid >= rows * nblk) return;
     const int64_t row = gid / nblk;
