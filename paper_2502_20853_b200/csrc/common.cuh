@@ -36,6 +36,8 @@ extern std::atomic<unsigned long long> g_launches;
 // Each block calls pdl_wait() before its first access to global memory: a kernel whose blocks could end without having waited
 // would let its successor overtake its predecessor.  In the GEMM kernels every thread calls it, also in the roles that touch
 // shared and tensor memory alone: their bounded waits for a stage must not start to count before the kernel's inputs exist.
+// (Each role calls it for itself: one call for the whole block ahead of the roles took 63.7 instead of 62.4 us for Swin's stage-4
+// qkv step, 97.9 instead of 97.3 for DeiT-Small's fc2 step.)
 // The element-wise and tile quantizing kernels call pdl_launch_dependents() first of all (the next kernel may be placed once
 // every block of this one has started); the GEMM kernels do not call it, so that their successor starts when their blocks end:
 // with the call the successor's blocks took over the first free SMs piecemeal, and a step got slower (43.0 against 36.5 us for an

@@ -435,6 +435,7 @@ __device__ __forceinline__ void gemm_feed_roles(int warp, uint32_t smem_base, ui
             const bool operands = warp == 0;
             uint32_t stage = 0, phase = 0;
             bool alive = true;
+            pdl_wait();
             for (int item = block; item < items && alive; item += blocks) {
                 const int tile = p.by_splits.div(item), split = item - tile * p.splits;
                 const int mb = p.by_tiles_n.div(tile), nb = tile - mb * p.tiles_n;
@@ -473,6 +474,7 @@ __device__ __forceinline__ void gemm_feed_roles(int warp, uint32_t smem_base, ui
         }
     } else if (warp == 2) {
         // ================= scale copier =================
+        pdl_wait();
         // Stage s of the ring owns TMEM columns kSfCol + s * kSfSlot ..: they are free again exactly when the stage's
         // shared memory is (the producer refills it only after the MMAs that read both have completed).
         {
@@ -510,6 +512,7 @@ __device__ __forceinline__ void gemm_feed_roles(int warp, uint32_t smem_base, ui
         }
     } else if (warp == 1) {
         // ================= MMA issuer =================
+        pdl_wait();
         // This warp's loop is the serial chain that bounds short and medium K loops (with every load, copy and store
         // taken out the kernel ran no faster), so it is kept short: one wait per stage (the scale copier has seen the
         // operands land before its copies, and its commit orders them before this warp's MMAs), and the barrier of the
@@ -610,7 +613,6 @@ k_gemm_mxf4(const __grid_constant__ GemmJob one, const __grid_constant__ Job2 tw
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem_base = *tmem_slot;
-    pdl_wait();
 
     const int items = p.tiles_m * p.tiles_n * p.splits;
 
@@ -618,6 +620,7 @@ k_gemm_mxf4(const __grid_constant__ GemmJob one, const __grid_constant__ Job2 tw
         gemm_feed_roles<C, BN>(warp, smem_base, bar_full, bar_sf_full, bar_empty, bar_acc_full, bar_acc_empty, tmem_base, abort_flag, job.a, job.b, p, block, blocks);
     } else if (warp >= kEpiWarp0) {
         // ================= epilogue (warps 4..11) =================
+        pdl_wait();
         const int ew = warp - kEpiWarp0;
         const int quarter = warp & 3;            // TMEM lanes 32*quarter .. +31 are the ones this warp may read
         const int chalf = ew >> 2;               // which half of the tile's columns this warp stores
@@ -757,13 +760,13 @@ k_gemm_mxf4_q(const __grid_constant__ CUtensorMap map_a, const __grid_constant__
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem_base = *tmem_slot;
-    pdl_wait();
 
     if (warp < kEpiWarp0) {
         gemm_feed_roles<C, BN>(warp, smem_base, bar_full, bar_sf_full, bar_empty, bar_acc_full, bar_acc_empty, tmem_base, abort_flag, map_a, map_b, p, blockIdx.x,
                                gridDim.x);
     } else {
         // ================= quantizing epilogue (warps 4..11 = 256 threads) =================
+        pdl_wait();
         const int et = (int)threadIdx.x - 32 * kEpiWarp0;
         const int quarter = warp & 3, chalf = (warp - kEpiWarp0) >> 2;
         const int M = (int)p.M, N = (int)p.N;
@@ -981,7 +984,6 @@ k_gemm_mxf4_bs(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem_base = *tmem_slot;
-    pdl_wait();
 
     const Walk walk = walk_begin(p, blockIdx.x);
     const int ktn = p.kt_total;
@@ -991,6 +993,7 @@ k_gemm_mxf4_bs(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
         const bool leader = elect_one() && !p.withhold_loads;
         uint32_t stage = 0, phase = 0;
         bool alive = true;
+        pdl_wait();
         for (int i = 0; i < walk.count && alive; i++) {
             const int mb = walk_item(p, walk, i).row;
             for (int kt = 0; kt < ktn; kt++) {
@@ -1011,6 +1014,7 @@ k_gemm_mxf4_bs(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
         // ================= B producer: the block of a column, once per run of tiles in that column =================
         const bool leader = elect_one() && !p.withhold_loads;
         uint32_t runs = 0;
+        pdl_wait();
         for (int i = 0; i < walk.count; i++) {
             const WalkItem x = walk_item(p, walk, i);
             if (!x.first) continue;
@@ -1038,6 +1042,7 @@ k_gemm_mxf4_bs(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
         }
     } else if (warp == 2) {
         // ================= scale copier: B scales once per column, A scales per stage =================
+        pdl_wait();
         const bool leader = elect_one();
         uint32_t stage = 0, phase = 0, runs = 0;
         bool alive = true;
@@ -1077,6 +1082,7 @@ k_gemm_mxf4_bs(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
         }
     } else if (warp == 1) {
         // ================= MMA issuer =================
+        pdl_wait();
         const bool leader = elect_one();
         uint32_t stage = 0, phase = 0, acc = 0, acc_phase = 0, runs = 0;
         const int nmma_last = (int)((p.Kc - (int64_t)(ktn - 1) * kBKElems + 63) / 64);   // MMAs of the last K tile
@@ -1126,6 +1132,7 @@ k_gemm_mxf4_bs(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
         }
     } else if (warp >= kEpiWarp0) {
         // ================= epilogue (warps 4..11) =================
+        pdl_wait();
         const int ew = warp - kEpiWarp0;
         const int quarter = warp & 3;
         const int chalf = ew >> 2;
@@ -1740,7 +1747,6 @@ k_gemm_mxf4_pair(const __grid_constant__ PairJob one, const __grid_constant__ Jo
     cluster_sync_all();     // both CTAs have their barriers and TMEM before anyone signals across
     tc_fence_after();
     const uint32_t tmem_base = *tmem_slot;
-    pdl_wait();
 
     const PairWalk walk = pair_walk<kTwo>(one.p, job2->p);
 
@@ -1753,6 +1759,7 @@ k_gemm_mxf4_pair(const __grid_constant__ PairJob one, const __grid_constant__ Jo
         const bool operands = warp == 0;
         uint32_t stage = 0, phase = 0;
         bool alive = true;
+        pdl_wait();
         for (int i = 0; alive; i++) {
             const PairItem x = pair_item<kTwo>(one.p, job2->p, walk, i);
             if (x.done) break;
@@ -1785,6 +1792,7 @@ k_gemm_mxf4_pair(const __grid_constant__ PairJob one, const __grid_constant__ Jo
         }
     } else if (warp == 2) {
         // ================= scale copier (leader CTA only; each copy acts on both CTAs) =================
+        pdl_wait();
         if (rank == 0) {
             const bool leader = elect_one();
             uint32_t stage = 0, phase = 0;
@@ -1821,6 +1829,7 @@ k_gemm_mxf4_pair(const __grid_constant__ PairJob one, const __grid_constant__ Jo
         }
     } else if (warp == 1) {
         // ================= MMA issuer (leader CTA only) =================
+        pdl_wait();
         if (rank == 0) {
             const bool leader = elect_one();
             uint32_t stage = 0, phase = 0, acc = 0, acc_phase = 0;
@@ -1868,6 +1877,7 @@ k_gemm_mxf4_pair(const __grid_constant__ PairJob one, const __grid_constant__ Jo
         }
     } else if (warp >= kEpiWarp0) {
         // ================= epilogue (warps 4..11 of both CTAs: own 128 rows x BN columns) =================
+        pdl_wait();
         const int ew = warp - kEpiWarp0;
         const int quarter = warp & 3;
         const int chalf = ew >> 2;
@@ -2089,7 +2099,6 @@ k_gemm_mxf4_pbs(const __grid_constant__ CUtensorMap map_a, const __grid_constant
     cluster_sync_all();     // both CTAs have their barriers and TMEM before anyone signals across
     tc_fence_after();
     const uint32_t tmem_base = *tmem_slot;
-    pdl_wait();
 
     const Walk walk = walk_begin(p, blockIdx.x >> 1);   // pair tiles: 256 rows x 192 columns
     const int ktn = p.kt_total;
@@ -2100,6 +2109,7 @@ k_gemm_mxf4_pbs(const __grid_constant__ CUtensorMap map_a, const __grid_constant
         const bool leader = elect_one() && !p.withhold_loads;
         uint32_t stage = 0, phase = 0, runs = 0;
         int nb = 0;
+        pdl_wait();
         bool alive = true;
         auto load_block = [&]() -> bool {
             // the MMAs of the previous column have finished reading the block (multicast commits reach both CTAs)
@@ -2139,6 +2149,7 @@ k_gemm_mxf4_pbs(const __grid_constant__ CUtensorMap map_a, const __grid_constant
         }
     } else if (warp == 2) {
         // ===== scale copier (leader only; each copy acts on both CTAs): B scales once per column, A scales per stage =====
+        pdl_wait();
         if (rank == 0) {
             const bool leader = elect_one();
             uint32_t stage = 0, phase = 0, runs = 0;
@@ -2179,6 +2190,7 @@ k_gemm_mxf4_pbs(const __grid_constant__ CUtensorMap map_a, const __grid_constant
         }
     } else if (warp == 1 || warp == 3) {
         // ===== MMA issuers (leader only): warp 1 takes this pair's even tiles into accumulator 0, warp 3 the odd ones
+        pdl_wait();
         // into accumulator 1.  One issuing thread needs about 350 cycles per stage (a barrier query, four MMAs, a commit)
         // and several hundred per tile, more than the tensor pipe needs for the stage; two of them leave it waiting for
         // nothing but operands.  Both walk over EVERY stage and every column in order and wait on each barrier phase
@@ -2241,6 +2253,7 @@ k_gemm_mxf4_pbs(const __grid_constant__ CUtensorMap map_a, const __grid_constant
         }
     } else if (warp >= kEpiWarp0) {
         // ===== epilogue (warps 4..11 of both CTAs: own 128 rows x 192 columns) =====
+        pdl_wait();
         const int ew = warp - kEpiWarp0;
         const int quarter = warp & 3;
         const int chalf = ew >> 2;
