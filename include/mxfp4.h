@@ -114,7 +114,8 @@ size_t mxfp4_scale_offset(int64_t row, int64_t block, int64_t cols);
  * launch sites).  For benchmarks that report how many launches a step takes. */
 uint64_t mxfp4_launch_count(void);
 
-/* Scratch bytes mxfp4_gemm needs for an [M, N] output with contraction length kc (0 if none). */
+/* Scratch bytes mxfp4_gemm makes use of for an [M, N] output with contraction length kc (0 if none): up to 64 partial
+ * sums of the output, where it has few tiles and kc is long.  Room for 32 of them is enough. */
 size_t mxfp4_gemm_workspace_bytes(int64_t m, int64_t n, int64_t kc);
 
 /* The longest chain of tensor-core MMAs (64 contraction elements each) that mxfp4_gemm adds into one FP32
@@ -122,7 +123,10 @@ size_t mxfp4_gemm_workspace_bytes(int64_t m, int64_t n, int64_t kc);
  * the kernels that alternate between two accumulators shorten it. */
 int64_t mxfp4_gemm_chain_mmas(int64_t m, int64_t n, int64_t kc);
 
-/* Scratch bytes mxfp4_linear_bwd needs (backward operands + GEMM scratch). */
+/* Scratch bytes mxfp4_linear_bwd makes use of: the backward operands and the partial sums of a weight gradient that is made
+ * in one launch with the input gradient (four of them where mxfp4_gemm alone would need none: 47 MB at M, K, N = 6272, 768,
+ * 2304, of which 28 MB are sums; 173 and 28 MB at 50432, 768, 2304).  Room for the operands and for what mxfp4_gemm needs for
+ * either product is enough; the products then run one after the other. */
 size_t mxfp4_linear_workspace_bytes(int64_t m, int64_t k, int64_t n);
 
 /* ---- quantizers --------------------------------------------------------------------------- */
@@ -178,7 +182,8 @@ mxfp4_status_t mxfp4_dequantize(mxfp4_mat_t src, float *dst, int64_t ld, void *s
  * cores (the three products of Eq. 3-5 all have this form).  a.cols == b.cols == kc, kc % 32 == 0.
  * d: bf16 or fp32 [M, N] with leading dimension ldd (bytes per row a multiple of 16).
  * bias_bf16: optional [N].  workspace: >= mxfp4_gemm_workspace_bytes(M, N, kc) bytes (may be NULL
- * when that is 0); used for split-K partial sums when M*N is small and kc long.
+ * when that is 0); used for split-K partial sums when M*N is small and kc long.  With less, the contraction is split
+ * into fewer parts, down to 32; below that the call is refused.
  * Accuracy.  The FP4 products are exact; the error is that of the FP32 accumulation.  The tensor core adds
  * each MMA's 64-term sum into its accumulator with truncation, which loses up to one ulp of the running sum
  * per MMA, always in the same direction.  With c = mxfp4_gemm_chain_mmas(M, N, kc) MMAs chained into one
@@ -234,7 +239,8 @@ mxfp4_status_t mxfp4_gemm_quant(mxfp4_mat_t a, mxfp4_mat_t b, const void *bias_b
  * that loads the library carries that array until the process ends.
  *   - Same arguments and results as mxfp4_gemm, without workspace / workspace_bytes.  The function
  *     calls no cudaMalloc, cudaFree or allocating library routine.
- *   - Shapes whose mxfp4_gemm_workspace_bytes(M, N, kc) exceeds MXFP4_STATIC_SCRATCH_BYTES are
+ *   - Where mxfp4_gemm would split the contraction into more parts than the array holds sums of, it is split
+ *     into as many as fit; shapes for which that would be fewer than 32 and fewer than mxfp4_gemm makes are
  *     refused with MXFP4_WORKSPACE_TOO_SMALL and nothing is enqueued.
  *   - The first call on each device looks up the array's device address (the device must be
  *     current); make that first call before any stream capture begins.

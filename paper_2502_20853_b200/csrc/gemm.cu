@@ -2421,8 +2421,9 @@ struct GemmPlan {
 // An MMA takes the same time for any width up to 256, so wide tiles are cheaper per flop; but only tiles up to 192
 // wide leave room in TMEM for a second accumulator, which hides the epilogue behind the next K loop.  For long K
 // loops the product is limited by operand delivery from L2, and pairs of CTAs sharing the B tile cut that by a third.
-// Split K when the output has too few tiles to fill the machine.
-static GemmPlan plan_gemm(int64_t m, int64_t n, int64_t kc, int sms, bool allow_split = true)
+// Split K when the output has too few tiles to fill the machine, beyond a least number of parts only as far as their sums fit into
+// `scratch` bytes.
+static GemmPlan plan_gemm(int64_t m, int64_t n, int64_t kc, int sms, bool allow_split = true, size_t scratch = SIZE_MAX)
 {
     GemmPlan g;
     g.kt_total = (int)ceil_div(kc, kBKElems);
@@ -2510,6 +2511,13 @@ static GemmPlan plan_gemm(int64_t m, int64_t n, int64_t kc, int sms, bool allow_
     if (allow_split && units * 2 <= workers && g.kt_total >= 8) {
         splits = min(workers / units, g.kt_total / 4);
         splits = max(1, min(splits, 64));   // (at 32, three tiles of 384 x 96 x 401408 left 52 of 148 SMs idle: 26.2 us with the reduction, now 24.6)
+        // what a caller has to bring room for: 32 parts, or what tiles of 192 on single CTAs would be split into where those are the
+        // natural ones (widths that a 256-wide tile does not fill), or none where K is split only because of the narrower tiles
+        int least = one_wave ? 1 : min(splits, 32);
+        if ((n > 192 && n < 256) || (kc <= 2304 && n % 192 == 0 && n % 256 != 0))
+            least = min(least, tiles192 * 2 <= sms ? max(1, min((int)(sms / tiles192), g.kt_total / 4)) : 1);
+        const size_t part = (size_t)m * n * sizeof(float);
+        if (splits > least && splits * part > scratch) splits = (int)max((size_t)least, scratch / part);
     }
     g.kt_per_split = (int)ceil_div(g.kt_total, splits);
     g.splits = (int)ceil_div(g.kt_total, g.kt_per_split);
@@ -2616,7 +2624,7 @@ mxfp4_status_t gemm_check(mxfp4_mat_t a, mxfp4_mat_t b, const void *d, int64_t l
     if (M == 0 || N == 0) return MXFP4_OK;
     if (!ensure_device_ok()) return MXFP4_UNSUPPORTED_DEVICE;
     if (Kc == 0) return MXFP4_BAD_SHAPE;
-    const GemmPlan g = plan_gemm(M, N, Kc, sm_count(), allow_split);
+    const GemmPlan g = plan_gemm(M, N, Kc, sm_count(), allow_split, workspace ? workspace_bytes : 0);
     const size_t need = g.splits > 1 ? (size_t)g.splits * M * N * sizeof(float) : 0;
     if (need > 0 && (!workspace || workspace_bytes < need)) return MXFP4_WORKSPACE_TOO_SMALL;
     if (need > 0 && (reinterpret_cast<uintptr_t>(workspace) & 15u)) return MXFP4_MISALIGNED;
@@ -2701,7 +2709,7 @@ static mxfp4_status_t gemm_impl(mxfp4_mat_t a, mxfp4_mat_t b, void *d, int64_t l
     const int64_t M = a.rows, N = b.rows;
     if (M == 0 || N == 0) return MXFP4_OK;
     const int sms = sm_count();
-    const GemmPlan g = plan_gemm(M, N, a.cols, sms, allow_split);
+    const GemmPlan g = plan_gemm(M, N, a.cols, sms, allow_split, workspace ? workspace_bytes : 0);
     PairJob job;
     if (!make_job(job, g, a, b, d, ldd, out_dtype, bias, workspace, dev_status, spin_limit, withhold_loads)) return MXFP4_CUDA_ERROR;
     GemmParams &p = job.p;
@@ -2725,11 +2733,12 @@ static mxfp4_status_t gemm_impl(mxfp4_mat_t a, mxfp4_mat_t b, void *d, int64_t l
 
 enum class TwoKind { kSeparate, kOneWave, kPairs };
 
-// The plans of two products (rows m1, m2, contractions kc1, kc2, n columns each) that may share a launch.
-static TwoKind plan_two(int64_t m1, int64_t kc1, int64_t m2, int64_t kc2, int64_t n, int sms, GemmPlan &g1, GemmPlan &g2)
+// The plans of two products (rows m1, m2, contractions kc1, kc2, n columns each) that may share a launch, if its partial sums fit into
+// `scratch` bytes.
+static TwoKind plan_two(int64_t m1, int64_t kc1, int64_t m2, int64_t kc2, int64_t n, int sms, size_t scratch, GemmPlan &g1, GemmPlan &g2)
 {
-    g1 = plan_gemm(m1, n, kc1, sms, true);
-    g2 = plan_gemm(m2, n, kc2, sms, true);
+    g1 = plan_gemm(m1, n, kc1, sms, true, scratch);
+    g2 = plan_gemm(m2, n, kc2, sms, true, scratch);
     const auto single = [](const GemmPlan &g) { return !g.pair && !g.pbs && !g.bs && !g.ck; };
     if (single(g1) && single(g2) && g1.bn == 128 && g2.bn == 128 && g1.splits == 1 && g2.splits == 1 &&
         g1.tiles_m * g1.tiles_n + g2.tiles_m * g2.tiles_n <= sms)
@@ -2759,7 +2768,8 @@ static TwoKind plan_two(int64_t m1, int64_t kc1, int64_t m2, int64_t kc2, int64_
         if (!g1.pair) join(g1);
         join(g2);
     }
-    if (g1.pair && g2.pair && g1.bn == g2.bn && g2.splits == 1) return TwoKind::kPairs;
+    if (g1.pair && g2.pair && g1.bn == g2.bn && g2.splits == 1 && (g1.splits == 1 || (size_t)g1.splits * m1 * n * sizeof(float) <= scratch))
+        return TwoKind::kPairs;
     g1 = own;
     return TwoKind::kSeparate;
 }
@@ -2779,9 +2789,8 @@ mxfp4_status_t gemm_two(mxfp4_mat_t a1, mxfp4_mat_t b1, void *d1, int64_t ldd1, 
     if (a1.rows > 0 && b1.rows > 0 && a2.rows > 0 && b2.rows > 0) {
         const int sms = sm_count();
         GemmPlan g1, g2;
-        const TwoKind kind = plan_two(a1.rows, a1.cols, a2.rows, a2.cols, b1.rows, sms, g1, g2);
+        const TwoKind kind = plan_two(a1.rows, a1.cols, a2.rows, a2.cols, b1.rows, sms, workspace ? workspace_bytes : 0, g1, g2);
         if (kind != TwoKind::kSeparate) {
-            if (g1.splits > 1 && workspace_bytes < (size_t)g1.splits * a1.rows * b1.rows * sizeof(float)) return MXFP4_WORKSPACE_TOO_SMALL;
             PairJob j1, j2;
             if (!make_job(j1, g1, a1, b1, d1, ldd1, dtype1, nullptr, workspace, dev_status, kWaitSpinLimit, 0) ||
                 !make_job(j2, g2, a2, b2, d2, ldd2, dtype2, nullptr, nullptr, dev_status, kWaitSpinLimit, 0))
@@ -2993,22 +3002,23 @@ mxfp4_status_t gemm_quant(mxfp4_mat_t a, mxfp4_mat_t b, const void *bias, const 
 #undef MX_Q_CASE
 }
 
-size_t gemm_workspace_bytes(int64_t m, int64_t n, int64_t kc)
+// scratch: what there is; the result may be more (then gemm() refuses it) or less.
+size_t gemm_workspace_bytes(int64_t m, int64_t n, int64_t kc, size_t scratch)
 {
     if (m <= 0 || n <= 0 || kc <= 0) return 0;
     // the same SM count gemm() plans with (148, the B200's, when no device is current)
-    const GemmPlan g = plan_gemm(m, n, kc, sm_count());
+    const GemmPlan g = plan_gemm(m, n, kc, sm_count(), true, scratch);
     return g.splits > 1 ? (size_t)g.splits * m * n * sizeof(float) : 0;
 }
 
-// Workspace for gemm_two()'s partial sums.
-size_t gemm_two_workspace_bytes(int64_t m1, int64_t kc1, int64_t m2, int64_t kc2, int64_t n)
+// Workspace for gemm_two()'s partial sums (scratch = 0: the least it takes).
+size_t gemm_two_workspace_bytes(int64_t m1, int64_t kc1, int64_t m2, int64_t kc2, int64_t n, size_t scratch)
 {
     if (m1 <= 0 || kc1 <= 0 || m2 <= 0 || kc2 <= 0 || n <= 0) return 0;
     GemmPlan g1, g2;
-    const bool pairs = plan_two(m1, kc1, m2, kc2, n, sm_count(), g1, g2) == TwoKind::kPairs;
+    const bool pairs = plan_two(m1, kc1, m2, kc2, n, sm_count(), scratch, g1, g2) == TwoKind::kPairs;
     const size_t two = pairs && g1.splits > 1 ? (size_t)g1.splits * m1 * n * sizeof(float) : 0;
-    const size_t w1 = gemm_workspace_bytes(m1, n, kc1), w2 = gemm_workspace_bytes(m2, n, kc2);
+    const size_t w1 = gemm_workspace_bytes(m1, n, kc1, scratch), w2 = gemm_workspace_bytes(m2, n, kc2, scratch);
     return std::max(two, std::max(w1, w2));
 }
 
@@ -3049,7 +3059,7 @@ mxfp4_status_t mxfp4_mma_issue_ceiling(int32_t bn, int32_t iters, uint32_t *dev_
     return MXFP4_OK;
 }
 
-size_t mxfp4_gemm_workspace_bytes(int64_t m, int64_t n, int64_t kc) { return mx::gemm_workspace_bytes(m, n, kc); }
+size_t mxfp4_gemm_workspace_bytes(int64_t m, int64_t n, int64_t kc) { return mx::gemm_workspace_bytes(m, n, kc, SIZE_MAX); }
 
 mxfp4_status_t mxfp4_gemm_quant(mxfp4_mat_t a, mxfp4_mat_t b, const void *bias_bf16, const mxfp4_epilogue_t *epi, uint32_t *dev_status,
                                 void *stream)

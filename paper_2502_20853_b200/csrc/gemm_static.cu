@@ -12,7 +12,7 @@
 namespace mx {
 mxfp4_status_t gemm(mxfp4_mat_t a, mxfp4_mat_t b, void *d, int64_t ldd, int out_dtype, const void *bias, void *workspace,
                     size_t workspace_bytes, uint32_t *dev_status, cudaStream_t st, bool allow_split);
-size_t gemm_workspace_bytes(int64_t m, int64_t n, int64_t kc);
+size_t gemm_workspace_bytes(int64_t m, int64_t n, int64_t kc, size_t scratch);
 }  // namespace mx
 
 // The scratch itself.  It exists once per GPU that loads this library and stays until the process
@@ -45,7 +45,7 @@ mxfp4_status_t scratch_on_current_device(void **out)
 extern "C" mxfp4_status_t mxfp4_gemm_static(mxfp4_mat_t a, mxfp4_mat_t b, void *d, int64_t ldd, int32_t out_dtype,
                                             const void *bias_bf16, uint32_t *dev_status, void *stream)
 {
-    const size_t need = mx::gemm_workspace_bytes(a.rows, b.rows, a.cols);
+    const size_t need = mx::gemm_workspace_bytes(a.rows, b.rows, a.cols, MXFP4_STATIC_SCRATCH_BYTES);
     if (need > (size_t)MXFP4_STATIC_SCRATCH_BYTES) return MXFP4_WORKSPACE_TOO_SMALL;
     void *scratch = nullptr;
     if (need > 0) {

@@ -17,7 +17,7 @@ mxfp4_status_t gemm(mxfp4_mat_t a, mxfp4_mat_t b, void *d, int64_t ldd, int out_
                     size_t workspace_bytes, uint32_t *dev_status, cudaStream_t st, bool allow_split);
 mxfp4_status_t gemm_check(mxfp4_mat_t a, mxfp4_mat_t b, const void *d, int64_t ldd, int out_dtype, const void *bias,
                           const void *workspace, size_t workspace_bytes, bool allow_split);
-size_t gemm_two_workspace_bytes(int64_t m1, int64_t kc1, int64_t m2, int64_t kc2, int64_t n);
+size_t gemm_two_workspace_bytes(int64_t m1, int64_t kc1, int64_t m2, int64_t kc2, int64_t n, size_t scratch);
 mxfp4_status_t gemm_quant_check(mxfp4_mat_t a, mxfp4_mat_t b, const void *bias, const mxfp4_epilogue_t *epi);
 mxfp4_status_t gemm_quant(mxfp4_mat_t a, mxfp4_mat_t b, const void *bias, const mxfp4_epilogue_t *epi, uint32_t *dev_status, cudaStream_t st);
 
@@ -40,7 +40,7 @@ static BwdLayout bwd_layout(int64_t m, int64_t k, int64_t n)
     L.wqt_s = take(mxfp4_scale_bytes(k, n));
     L.xqt_p = take((size_t)k * m / 2);
     L.xqt_s = take(mxfp4_scale_bytes(k, m));
-    L.gemm_ws_bytes = gemm_two_workspace_bytes(n, m, m, n, k);
+    L.gemm_ws_bytes = gemm_two_workspace_bytes(n, m, m, n, k, SIZE_MAX);
     L.gemm_ws = take(L.gemm_ws_bytes);
     L.total = o;
     return L;
@@ -130,8 +130,12 @@ mxfp4_status_t mxfp4_linear_bwd_ex(const void *dy_bf16, int64_t lddy, const mxfp
     if (ctx->wq.cols != k) return MXFP4_BAD_SHAPE;
     if (m % 32 != 0 || n % 32 != 0 || k % 32 != 0) return MXFP4_BAD_SHAPE;
     if (reinterpret_cast<uintptr_t>(workspace) & 255u) return MXFP4_MISALIGNED;
-    const BwdLayout L = bwd_layout(m, k, n);
-    if (workspace_bytes < L.total) return MXFP4_WORKSPACE_TOO_SMALL;
+    BwdLayout L = bwd_layout(m, k, n);
+    if (workspace_bytes < L.total) {
+        // room for the partial sums of separate launches, 32 parts each at most, is enough
+        if (workspace_bytes < align256(L.gemm_ws + gemm_two_workspace_bytes(n, m, m, n, k, 0))) return MXFP4_WORKSPACE_TOO_SMALL;
+        L.gemm_ws_bytes = workspace_bytes - L.gemm_ws;
+    }
     uint8_t *ws = static_cast<uint8_t *>(workspace);
     mxfp4_mat_t dyq = {ws + L.dyq_p, ws + L.dyq_s, m, n};
     mxfp4_mat_t dyq_t = {ws + L.dyqt_p, ws + L.dyqt_s, n, m};

@@ -245,3 +245,38 @@ def test_mma_issue_ceiling_loop_runs(mx):
         assert rate > 2000.0, (bn, rate)
     with pytest.raises(mx.MxError):
         mx.mma_issue_ceiling(bn=64)
+
+
+# (M, N, kc, least): a caller may bring less than mxfp4_gemm_workspace_bytes: 32 parts or fewer, those of 192-wide tiles for widths that
+# 256-wide ones do not fill, or none where only the narrow tiles of one wave have K split
+@pytest.mark.parametrize("M,N,K,least", [(384, 96, 401408, 4718592), (128, 128, 50432, 1900544), (256, 512, 50432, 15204352), (1016, 248, 74816, 9070848),
+                                         (4624, 368, 3744, 0)])
+def test_gemm_takes_a_smaller_workspace(mx, M, N, K, least):
+    assert mx.gemm_workspace_bytes(M, N, K) > least
+    rng = np.random.default_rng(M + N)
+
+    def operand(rows):
+        q = mx.QMat(rows, K)
+        q.data.copy_(torch.from_numpy(rng.integers(0, 256, size=tuple(q.data.shape)).astype(np.uint8)))
+        q.scales.copy_(torch.from_numpy(rng.integers(125, 130, size=tuple(q.scales.shape)).astype(np.uint8)))
+        return q
+
+    a, b = operand(M), operand(N)
+    st = mx.new_status()
+    da, db = mx.dequantize(a).double(), mx.dequantize(b).double()
+    want, t = (da @ db.T).cpu().numpy(), (da.abs() @ db.abs().T).cpu().numpy()
+    parts = max(1, least // (4 * M * N))
+    chain = -(-(-(-K // 256)) // parts) * 4     # MMAs in a chain: K tiles of a part, four each
+    for out_dtype in (0, 1):
+        for size in (least, least + 4 * M * N, mx.gemm_workspace_bytes(M, N, K)):
+            guard = torch.full((size + 256,), 0x5A, dtype=torch.uint8, device="cuda")
+            guard[:size] = 0xFF                 # NaN
+            got = mx.gemm(a, b, out_dtype=out_dtype, workspace=guard[:size], dev_status=st)
+            torch.cuda.synchronize()
+            assert int(st.item()) == 0 and bool((guard[size:] == 0x5A).all())
+            check_gemm_bound(got.float().cpu().numpy(), want, t, out_dtype == 0, "%d bytes" % size, factor=max(1.0, chain / 8))
+    if not least:
+        return
+    with pytest.raises(mx.MxError) as e:
+        mx.gemm(a, b, workspace=torch.empty(least - 16, dtype=torch.uint8, device="cuda"))
+    assert e.value.status == 4

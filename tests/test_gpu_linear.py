@@ -354,3 +354,26 @@ def test_q4_that_the_forward_pass_made_is_used_only_where_it_holds(mx, what):
     torch.cuda.synchronize()
     assert torch.equal(dx.view(torch.int16), want_dx.view(torch.int16)) and torch.equal(dw.view(torch.int32), want_dw.view(torch.int32))
     assert int(st.item()) == int(st2.item())
+
+
+# (M, K, N, bytes of the backward operands and the two products' own partial sums, 32 at most)
+@pytest.mark.parametrize("M,K,N,least", [(4096, 768, 1536, 8982528), (6272, 768, 2304, 18852864), (401408, 96, 384, 189386240)])
+def test_backward_pass_takes_a_smaller_workspace(mx, M, K, N, least):
+    """With less than mxfp4_linear_workspace_bytes the products run one after the other, with their own numbers of parts."""
+    assert least < mx.linear_workspace_bytes(M, K, N)
+    g = torch.Generator(device="cuda").manual_seed(M)
+    x, w = torch.randn((M, K), generator=g, device="cuda").to(torch.bfloat16), torch.randn((N, K), generator=g, device="cuda").to(torch.bfloat16)
+    dy = torch.randn((M, N), generator=g, device="cuda").to(torch.bfloat16)
+    st = mx.new_status()
+    _, ctx = mx.linear_fwd(x, w, bwd_seed=3, dev_status=st)
+    dyq, dyq_t = mx.quantize_2axis(dy, (0, 1, 3, 3), (0, 1, 3, 5))
+    wq_t = mx.quantize_t(ctx.wq, rounding=1, seed=3, stream_id=4)
+    buf = torch.full((least + 256,), 0x5A, dtype=torch.uint8, device="cuda")
+    dx, dw = mx.linear_bwd(dy, ctx, 3, workspace=buf[:least], dev_status=st)
+    torch.cuda.synchronize()
+    assert int(st.item()) == 0 and bool((buf[least:] == 0x5A).all())
+    small = torch.empty(32 * N * K * 4, dtype=torch.uint8, device="cuda")
+    assert torch.equal(dx, mx.gemm(dyq, wq_t, workspace=small)) and torch.equal(dw, mx.gemm(dyq_t, ctx.xq_t, out_dtype=1, workspace=small))
+    with pytest.raises(mx.MxError) as e:
+        mx.linear_bwd(dy, ctx, 3, workspace=buf[:least - 16])
+    assert e.value.status == 4

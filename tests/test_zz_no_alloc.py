@@ -11,6 +11,8 @@ import numpy as np
 import pytest
 import torch
 
+from util import check_gemm_bound
+
 pytestmark = pytest.mark.gpu
 
 
@@ -78,3 +80,21 @@ def test_static_scratch_gemm_refuses_what_does_not_fit(mx):
     with pytest.raises(mx.MxError) as e:
         mx.gemm_static(a, b, out, out_dtype=1)
     assert e.value.status == 4  # MXFP4_WORKSPACE_TOO_SMALL
+
+
+# shapes whose partial sums fill the array: with as many parts as mxfp4_gemm makes of them they would not fit
+@pytest.mark.parametrize("M,N,K", [(256, 512, 37888), (512, 256, 37888), (256, 512, 50432), (128, 1024, 50432)])
+def test_static_scratch_gemm_makes_as_many_parts_as_fit(mx, M, N, K):
+    assert mx.gemm_workspace_bytes(M, N, K) > mx.STATIC_SCRATCH_BYTES
+    a, b = _operand(mx, M, K, 7), _operand(mx, N, K, 8)
+    st = mx.new_status()
+    for out_dtype in (0, 1):
+        got = torch.full((M, N), float("nan"), dtype=torch.float32 if out_dtype else torch.bfloat16, device="cuda")
+        mx.gemm_static(a, b, got, out_dtype=out_dtype, dev_status=st)
+        torch.cuda.synchronize()
+        assert int(st.item()) == 0
+        da, db = mx.dequantize(a).double(), mx.dequantize(b).double()
+        want, t = (da @ db.T).cpu().numpy(), (da.abs() @ db.abs().T).cpu().numpy()
+        # at most 32 parts: ceil(ceil(K / 256) / 32) K tiles of four MMAs each in a chain
+        chain = -(-(-(-K // 256)) // 32) * 4
+        check_gemm_bound(got.float().cpu().numpy(), want, t, out_dtype == 0, "static", factor=max(1.0, chain / 8))
