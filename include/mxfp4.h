@@ -202,7 +202,8 @@ mxfp4_status_t mxfp4_gemm(mxfp4_mat_t a, mxfp4_mat_t b, void *d, int64_t ldd, in
  * product reads quantized; "Double Quantization" for the operand along the other axis).  Per output tile:
  *     Y  = bf16(deq(A) deq(B)^T + bias)                              the layer's result
  *     Z  = bf16(hook(Y))                                             hook: identity, GELU (0.5 y (1 + erf(y / sqrt 2)),
- *                                                                    in FP32, absolute error below 1e-6 |y|), or
+ *                                                                    in FP32, error below 2e-7 |y|, and below 1.1 % of the
+ *                                                                    result itself down to 2^-125), or
  *                                                                    Y * aux elementwise (exact before the rounding)
  *     Zq   = Q(Z; qp_row)      [M, N], groups along N                (the next product's row operand, e.g. Q1 or Q3)
  *     Zq_t = Q(Z^T; qp_t)      [N, M], groups along M                (its transposed operand, e.g. Q5), or with

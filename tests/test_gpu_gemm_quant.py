@@ -198,3 +198,34 @@ def test_gemm_quant_argument_errors(mx):
     with pytest.raises(mx.MxError) as e:
         mx.gemm_quant(a, mx.QMat(72, 64), mx.Epilogue(zq=mx.QMat(128, 72)))  # N must be a multiple of 32
     assert e.value.status == 2
+
+
+# one tile row (the fused epilogue) and two (two kernels, from four tiles per SM on)
+@pytest.mark.parametrize("M", [32, 160])
+def test_gelu_of_every_bf16_value(mx, M):
+    """Every finite bf16 value as Y.  Z is the rounding to bf16 (2^-8 of the result at most) of a value within 1.1 % of GELU(Y) down to
+    2^-125, and within 2e-7 |y|."""
+    from scipy.special import erfc
+    y = torch.arange(65536, dtype=torch.int32).to(torch.int16).view(torch.bfloat16).cuda()
+    y = torch.where(torch.isnan(y), torch.zeros_like(y), y)
+    N = y.numel()
+    a, b = mx.QMat(M, 32), mx.QMat(N, 32)
+    for q in (a, b):
+        q.data.zero_()
+        q.scales.fill_(127)
+    out_y, z = torch.empty((M, N), dtype=torch.bfloat16, device="cuda"), torch.empty((M, N), dtype=torch.bfloat16, device="cuda")
+    st = mx.new_status()
+    epi = mx.Epilogue(hook=mx.HOOK_GELU, y=out_y, z=z, zq=mx.QMat(M, N), zq_t=mx.QMat(N, M), qp_t=(0, 0, 0, 0), chain=True)
+    mx.gemm_quant(a, b, epi, bias=y, dev_status=st)
+    torch.cuda.synchronize()
+    assert int(st.item()) == mx.DEV_NONFINITE      # of the two infinities
+    assert torch.equal(out_y, (y + 0.0).expand(M, N))
+    assert torch.equal(z.view(torch.int16), z[:1].view(torch.int16).expand(M, N))
+    yv, zv = y.double().cpu().numpy(), z[0].double().cpu().numpy()
+    assert zv[yv == np.inf] == np.inf and np.isnan(zv[yv == -np.inf])
+    fin = np.isfinite(yv)
+    yv, zv = yv[fin], zv[fin]
+    want = 0.5 * yv * erfc(-yv * np.sqrt(0.5))
+    assert (np.signbit(zv) == (yv < 0)).all()
+    assert (np.abs(zv - want) <= np.abs(want) * (2.0 ** -8 + 0.011 * (1 + 2.0 ** -8)) + 2.0 ** -125).all()
+    assert (np.abs(zv - want) <= (np.abs(want) + 2e-7 * np.abs(yv)) * 2.0 ** -8 + 2e-7 * np.abs(yv) + 2.0 ** -125).all()
