@@ -4,6 +4,7 @@ serving step makes are marshalled by the native module ``_host`` (csrc/host.cpp)
 torch is used for device memory and streams.  The library must be present (built in-tree by
 ``paper_2502_20853_b200.build``); there is no fallback path of any kind.
 """
+import copyreg
 import ctypes as C
 import os
 
@@ -193,9 +194,7 @@ def _align256(n):
 class QMat(_host.Mat):
     """A quantized matrix in device memory: packed E2M1 codes + E8M0 scales in tiled order.  Codes and scales that the
     binding allocates itself share one buffer (an allocation costs a call 1.7 us); ``data`` and ``scales`` are views of it,
-    made when they are asked for."""
-
-    __slots__ = ()
+    made when they are asked for.  As state (copies, pickles) it is its rows, cols, data and scales."""
 
     def __init__(self, rows, cols, device="cuda", data=None, scales=None):
         rows, cols = int(rows), int(cols)
@@ -206,7 +205,6 @@ class QMat(_host.Mat):
         self.rows, self.cols = rows, cols
         self._data = data if data is not None else _new((rows, cols // 2), torch.uint8, device)
         self._scales = scales if scales is not None else _new((max(scale_bytes(rows, cols), 16),), torch.uint8, device)
-        self.data_addr, self.scales_addr = self._data.data_ptr(), self._scales.data_ptr()
 
     @staticmethod
     def two(r0, c0, r1, c1, device):
@@ -216,26 +214,45 @@ class QMat(_host.Mat):
         buf = torch.empty(_host.nbytes(r0, c0, r1, c1), dtype=torch.uint8, device=device)
         return _host.place(QMat, buf, buf.data_ptr(), r0, c0, r1, c1)
 
+    def __reduce_ex__(self, protocol):
+        return copyreg.__newobj__, (type(self),), dict(vars(self), rows=self.rows, cols=self.cols, data=self.data, scales=self.scales)
+
+    def __setstate__(self, state):
+        for name, value in state.items():
+            setattr(self, name, value)
+
+    def _open(self):
+        # what hands the contents out also gives up what was made of them (see LinearCtx): they may be written through it
+        self._q4 = None
+        if self._data is None and self._buf is not None:
+            n = self.rows * (self.cols // 2)
+            at = self._at + _align256(n)
+            self._data = self._buf[self._at:self._at + n].view(self.rows, self.cols // 2)
+            self._scales = self._buf[at:at + max(scale_bytes(self.rows, self.cols), 16)]
+
     @property
     def device(self):
-        return (self._buf if self._buf is not None else self._data).device
+        return (self._data if self._data is not None else self._buf).device
 
-    # what hands the contents out also gives up what was made of them (see LinearCtx): they may be written through it
     @property
     def data(self):
-        self._q4 = None
-        if self._data is None:
-            n = self.rows * (self.cols // 2)
-            self._data = self._buf[self._at:self._at + n].view(self.rows, self.cols // 2)
+        self._open()
         return self._data
+
+    @data.setter
+    def data(self, t):
+        self._open()
+        self._data = t
 
     @property
     def scales(self):
-        self._q4 = None
-        if self._scales is None:
-            at = self._at + _align256(self.rows * (self.cols // 2))
-            self._scales = self._buf[at:at + max(scale_bytes(self.rows, self.cols), 16)]
+        self._open()
         return self._scales
+
+    @scales.setter
+    def scales(self, t):
+        self._open()
+        self._scales = t
 
     def c(self):
         self._q4 = None

@@ -48,11 +48,36 @@ void mat_dealloc(PyObject *o)
     Py_TYPE(o)->tp_free(o);
 }
 
+PyObject *g_data_ptr;   // the name of the tensors' method
+
+// Once the tensors of a matrix have been handed out (or came from the caller), its addresses are theirs: a program may give a
+// tensor another storage.
+bool refresh(Mat *s)
+{
+    if (s->data && s->data != Py_None) {
+        PyObject *a = PyObject_CallMethodNoArgs(s->data, g_data_ptr);
+        if (!a) return false;
+        s->m.data = reinterpret_cast<void *>((uintptr_t)PyLong_AsUnsignedLongLongMask(a));
+        Py_DECREF(a);
+    }
+    if (s->scales && s->scales != Py_None) {
+        PyObject *a = PyObject_CallMethodNoArgs(s->scales, g_data_ptr);
+        if (!a) return false;
+        s->m.scales = reinterpret_cast<uint8_t *>((uintptr_t)PyLong_AsUnsignedLongLongMask(a));
+        Py_DECREF(a);
+    }
+    return !PyErr_Occurred();
+}
+PyObject *mat_address(PyObject *o, void *scales)
+{
+    Mat *s = reinterpret_cast<Mat *>(o);
+    return refresh(s) ? PyLong_FromVoidPtr(scales ? (void *)s->m.scales : s->m.data) : nullptr;
+}
+PyGetSetDef mat_getset[] = {{"data_addr", mat_address, nullptr, nullptr, nullptr}, {"scales_addr", mat_address, nullptr, nullptr, (void *)1}, {nullptr, nullptr, nullptr, nullptr, nullptr}};
+
 PyMemberDef mat_members[] = {
     {"rows", T_LONGLONG, offsetof(Mat, m.rows), 0, nullptr},
     {"cols", T_LONGLONG, offsetof(Mat, m.cols), 0, nullptr},
-    {"data_addr", T_ULONGLONG, offsetof(Mat, m.data), 0, nullptr},
-    {"scales_addr", T_ULONGLONG, offsetof(Mat, m.scales), 0, nullptr},
     {"_buf", T_OBJECT, offsetof(Mat, buf), 0, nullptr},
     {"_data", T_OBJECT, offsetof(Mat, data), 0, nullptr},
     {"_scales", T_OBJECT, offsetof(Mat, scales), 0, nullptr},
@@ -80,7 +105,11 @@ struct Args {
     bool given(int i) const { return a[i] != Py_None; }
     mxfp4_mat_t mat(int i)
     {
-        if (PyObject_TypeCheck(a[i], &mat_type)) return reinterpret_cast<Mat *>(a[i])->m;
+        if (PyObject_TypeCheck(a[i], &mat_type)) {
+            Mat *s = reinterpret_cast<Mat *>(a[i]);
+            if (!bad && !refresh(s)) bad = true;
+            return s->m;
+        }
         if (given(i) && !bad) {
             PyErr_SetString(PyExc_TypeError, "a quantized matrix (QMat) is expected");
             bad = true;
@@ -154,6 +183,8 @@ PyObject *h_place(PyObject *, PyObject *const *a, Py_ssize_t n)
         Mat *s = reinterpret_cast<Mat *>(o);
         s->m = mxfp4_mat_t{p + at, p + at + ((rows * (cols / 2) + 255) & ~int64_t(255)), rows, cols};
         Py_XSETREF(s->buf, Py_NewRef(a[1]));
+        Py_CLEAR(s->data);
+        Py_CLEAR(s->scales);
         s->at = at;
         at += mat_bytes(rows, cols);
         if (!one) PyTuple_SET_ITEM(all, i, o);
@@ -267,6 +298,8 @@ PyMODINIT_FUNC PyInit__host()
     mat_type.tp_traverse = mat_traverse;
     mat_type.tp_clear = mat_clear;
     mat_type.tp_members = mat_members;
+    mat_type.tp_getset = mat_getset;
+    if (!g_data_ptr && !(g_data_ptr = PyUnicode_InternFromString("data_ptr"))) return nullptr;
     if (PyType_Ready(&mat_type) < 0) return nullptr;
     PyObject *m = PyModule_Create(&module);
     if (m && PyModule_AddObjectRef(m, "Mat", reinterpret_cast<PyObject *>(&mat_type)) < 0) Py_CLEAR(m);

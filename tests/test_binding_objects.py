@@ -1,0 +1,90 @@
+"""The binding's objects as plain Python objects: what a program does with them besides passing them to the library.  No GPU."""
+import copy
+import gc
+import io
+import pickle
+import weakref
+
+import pytest
+import torch
+
+import paper_2502_20853_b200 as mx
+
+
+def _filled(rows=96, cols=64, given=False):
+    if given:
+        q = mx.QMat(rows, cols, "cpu", torch.empty((rows, cols // 2), dtype=torch.uint8), torch.empty(mx.scale_bytes(rows, cols), dtype=torch.uint8))
+    else:
+        q = mx.QMat(rows, cols, "cpu")
+    q.data.copy_(torch.arange(q.data.numel()).view(q.data.shape) % 251)
+    q.scales.copy_(torch.arange(q.scales.numel()) % 241)
+    return q
+
+
+def _same(a, b):
+    return type(a) is type(b) and (a.rows, a.cols) == (b.rows, b.cols) and torch.equal(a.data, b.data) and torch.equal(a.scales, b.scales)
+
+
+@pytest.mark.parametrize("given", [False, True])
+def test_matrix_is_copied_pickled_and_saved(given):
+    q = _filled(given=given)
+    q.note = "of layer 3"
+    assert copy.copy(q).data.data_ptr() == q.data.data_ptr() and _same(copy.copy(q), q)
+    for proto in range(pickle.HIGHEST_PROTOCOL + 1):
+        assert _same(pickle.loads(pickle.dumps(q, proto)), q)
+    f = io.BytesIO()
+    osc = mx.OscState(torch.zeros(2, 2), q, torch.ones(2), torch.ones(3))
+    torch.save(dict(osc=osc, ctx=mx.LinearCtx(q, q, seed=5)), f)
+    f.seek(0)
+    state = torch.load(f, weights_only=False)
+    assert _same(state["osc"].wq_prev, q) and state["osc"].wq_prev.note == "of layer 3" and _same(state["ctx"].xq, q)
+    for r in (copy.deepcopy(q), pickle.loads(pickle.dumps(q)), state["ctx"].wq):
+        assert _same(r, q) and r.note == q.note and r.device == q.device
+        r.data.zero_()
+        r.scales.zero_()
+        assert not _same(r, q) and q.data.any() and q.scales.any()
+        assert (r.c().data, r.c().scales) == (r.data.data_ptr(), r.scales.data_ptr())
+
+
+def test_matrix_saved_as_a_plain_object_is_loaded():
+    """Objects pickled when the class was a plain one: its attributes are rows, cols, data and scales."""
+    q = _filled()
+    old = copy.copy(q)
+    state = dict(rows=96, cols=64, data=q.data.clone(), scales=q.scales.clone())
+    new = mx.QMat.__new__(mx.QMat)
+    (new.__setstate__ if hasattr(new, "__setstate__") else new.__dict__.update)(state)
+    assert _same(new, old) and new.c().data == state["data"].data_ptr() and new.device.type == "cpu"
+
+
+def test_matrix_takes_other_tensors_and_attributes():
+    q, other = _filled(), _filled(given=True)
+    other.data.add_(1)
+    q.data, q.scales = other.data, other.scales
+    q.tag = 7
+    assert _same(q, other) and q.tag == 7 and (q.c().data, q.c().scales) == (other.data.data_ptr(), other.scales.data_ptr())
+    q.rows, q.cols = 48, 128
+    assert (q.c().rows, q.c().cols) == (48, 128)
+    w = weakref.ref(q)
+    del q
+    gc.collect()
+    assert w() is None
+
+
+def test_calls_follow_a_tensor_whose_storage_is_replaced():
+    import ctypes as C
+    seen = []
+    entry = C.CFUNCTYPE(C.c_int32, C.c_void_p, C.c_int64, C.c_int64, C.c_int64, mx.binding.CMat, C.c_void_p, C.c_void_p, C.c_void_p)(
+        lambda x, rows, cols, ld, dst, qp, status, stream: seen.append((dst.data, dst.scales)) or 0)
+    address = C.cast(entry, C.c_void_p).value
+
+    def call(q):
+        assert mx.binding._host.quantize(address, None, q.rows, q.cols, q.cols, q, 0, 0, 0, 0, None, None) == 0
+        return seen[-1]
+
+    for q in (_filled(), _filled(given=True)):
+        assert call(q) == (q.data.data_ptr(), q.scales.data_ptr())
+        q.data.data = q.data.clone()            # e.g. moved elsewhere and back
+        q.scales.set_(q.scales.clone())
+        assert call(q) == (q.data.data_ptr(), q.scales.data_ptr()) == (q.c().data, q.c().scales) == (q.data_addr, q.scales_addr)
+    q = mx.QMat(96, 64, "cpu")                  # nothing handed out yet
+    assert call(q) == (q.data.data_ptr(), q.scales.data_ptr())
