@@ -337,6 +337,9 @@ class OscState:
     def __init__(self, w_prev, wq_prev, dist_w, dist_q):
         self.w_prev, self.wq_prev, self.dist_w, self.dist_q = w_prev, wq_prev, dist_w, dist_q
 
+    def c(self):
+        return COsc(self.w_prev.data_ptr(), self.wq_prev.c(), self.dist_w.data_ptr(), self.dist_q.data_ptr())
+
 
 def qema_quantize(w, ema, beta=0.998, update_ema=True, scale_mode=SCALE_TRUNCATION_FREE, osc=None, out=None,
                   dev_status=None):
@@ -454,6 +457,11 @@ class LinearCtx:
 
     def __init__(self, xq, wq, xq_t=None, seed=0, wq_t=None):
         self.xq, self.wq, self.xq_t, self.seed, self.wq_t = xq, wq, xq_t, seed, wq_t
+
+    def c(self):
+        t, wt = self.xq_t, self.wq_t if self.wq_t is not self._made else None
+        sd = self.seed & _U64
+        return CCtx(self.xq.c(), self.wq.c(), t.c() if t is not None else _NO_MAT, sd, wt.c() if wt is not None else _NO_MAT, sd)
 
     def _q4(self, seed, scale_mode, dev_status):
         """wq_t, or None if linear_fwd made it and it is not the Q4 of a backward pass with these arguments."""

@@ -88,3 +88,15 @@ def test_calls_follow_a_tensor_whose_storage_is_replaced():
         assert call(q) == (q.data.data_ptr(), q.scales.data_ptr()) == (q.c().data, q.c().scales) == (q.data_addr, q.scales_addr)
     q = mx.QMat(96, 64, "cpu")                  # nothing handed out yet
     assert call(q) == (q.data.data_ptr(), q.scales.data_ptr())
+
+
+def test_c_structures_of_a_context_and_of_the_oscillation_state():
+    xq, wq, xq_t, wq_t = (_filled() for _ in range(4))
+    c = mx.LinearCtx(xq, wq, xq_t, -1, wq_t).c()
+    assert [m.data for m in (c.xq, c.wq, c.xq_t, c.wq_t)] == [q.data.data_ptr() for q in (xq, wq, xq_t, wq_t)]
+    assert c.xq_t_seed == c.wq_t_seed == 2 ** 64 - 1
+    c = mx.LinearCtx(xq, wq).c()
+    assert not c.xq_t.data and not c.wq_t.data and c.wq.rows == 96
+    w, dw, dq = torch.zeros(3), torch.ones(3), torch.ones(4)
+    c = mx.OscState(w, wq, dw, dq).c()
+    assert (c.w_prev, c.wq_prev.scales, c.dist_w, c.dist_q) == (w.data_ptr(), wq.scales.data_ptr(), dw.data_ptr(), dq.data_ptr())
