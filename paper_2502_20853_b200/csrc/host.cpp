@@ -94,14 +94,13 @@ struct Args {
 
     uint64_t u64(int i)
     {
-        if (a[i] == Py_None) return 0;
         const unsigned long long v = PyLong_AsUnsignedLongLongMask(a[i]);
         if (v == (unsigned long long)-1 && PyErr_Occurred()) bad = true;
         return v;
     }
     int64_t i64(int i) { return (int64_t)u64(i); }
     int32_t i32(int i) { return (int32_t)u64(i); }
-    template <class T = void> T *ptr(int i) { return reinterpret_cast<T *>((uintptr_t)u64(i)); }
+    template <class T = void> T *ptr(int i) { return given(i) ? reinterpret_cast<T *>((uintptr_t)u64(i)) : nullptr; }
     bool given(int i) const { return a[i] != Py_None; }
     mxfp4_mat_t mat(int i)
     {

@@ -100,3 +100,37 @@ def test_c_structures_of_a_context_and_of_the_oscillation_state():
     w, dw, dq = torch.zeros(3), torch.ones(3), torch.ones(4)
     c = mx.OscState(w, wq, dw, dq).c()
     assert (c.w_prev, c.wq_prev.scales, c.dist_w, c.dist_q) == (w.data_ptr(), wq.scales.data_ptr(), dw.data_ptr(), dq.data_ptr())
+
+
+# every whole-number argument of every native call: None is no number
+@pytest.mark.parametrize("name,numbers,pointers,matrices,n", [
+    ("linear_fwd", (2, 3, 4, 6, 9, 14, 15), (1, 5, 7, 8, 16, 17, 18), (10, 11, 12, 13), 19),
+    ("linear_bwd", (2, 9, 10, 11, 13, 15, 16, 19), (1, 12, 14, 17, 18, 20, 21), (3, 4, 5, 6, 7, 8), 22),
+    ("quantize", (2, 3, 4, 6, 7, 8, 9), (1, 10, 11), (5,), 12),
+    ("quantize_t", (3, 4, 5, 7, 8, 9, 10), (1, 11, 12), (2, 6), 13),
+    ("qema_quantize", (4, 5, 6, 8), (1, 2, 9, 11, 12, 13, 14), (7, 10), 15)])
+def test_native_calls_refuse_none_for_a_number(name, numbers, pointers, matrices, n):
+    import ctypes as C
+    called = []
+    entry = C.CFUNCTYPE(C.c_int32)(lambda: called.append(1) or 0)
+    fn, q = getattr(mx.binding._host, name), _filled()
+
+    def call(**other):
+        args = [0] * n
+        args[0] = C.cast(entry, C.c_void_p).value
+        for i in pointers:
+            args[i] = None
+        for i in matrices:
+            args[i] = q
+        if name == "qema_quantize":
+            args[3] = 0.5
+        for i, v in other.items():
+            args[int(i[1:])] = v
+        return fn(*args)
+
+    assert call() == 0 and called
+    for i in numbers:
+        for bad in (None, 1.5, "1"):
+            with pytest.raises(TypeError):
+                call(**{"_%d" % i: bad})
+    assert len(called) == 1
