@@ -1,8 +1,8 @@
 """Binding of libmxfp4.so: argument marshalling only — every step runs in the CUDA kernels.  The calls that a training or
 serving step makes are marshalled by the native module ``_host`` (csrc/host.cpp), all others by ctypes.
 
-torch is used for device memory and streams.  The library must be present (built in-tree by
-``paper_2502_20853_b200.build``); there is no fallback path of any kind.
+torch is used for device memory and streams.  The library and the module must be present (built in-tree by
+``paper_2502_20853_b200.build``); there is no fallback path of any kind, and the first use says what is missing.
 """
 import copyreg
 import ctypes as C
@@ -10,12 +10,22 @@ import os
 
 import torch
 
+
+class _NotBuilt:
+    """In the place of the native module until it has been built (build.py then loads this module again)."""
+
+    Mat = object
+
+    def __getattr__(self, name):
+        raise RuntimeError("the module _host is missing or of another build: run `python -m paper_2502_20853_b200.build`")
+
+
 try:
     from . import _host
-except ImportError:      # not built yet: it takes the host compiler alone, and the class QMat needs it
-    from .build import build_host
-    build_host()
-    from . import _host
+    if getattr(_host, "interface", 0) != 2:      # what the calls below expect of it
+        _host = _NotBuilt()
+except ImportError:
+    _host = _NotBuilt()
 
 _HERE = os.path.dirname(os.path.abspath(__file__))
 LIB_PATH = os.path.join(_HERE, "libmxfp4.so")

@@ -1,4 +1,5 @@
-"""Compile the CUDA sources into the in-tree shared library libmxfp4.so (sm_100a only) and the binding's host module _host.so."""
+"""Compile the CUDA sources into the in-tree shared library libmxfp4.so (sm_100a only) and the binding's host module _host."""
+import importlib
 import os
 import subprocess
 import sys
@@ -13,12 +14,22 @@ NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", 
               "-Xcompiler", "-fPIC", "--expt-relaxed-constexpr"]
 
 
-HOST = os.path.join(_HERE, "_host.so")
+HOST = os.path.join(_HERE, "_host" + sysconfig.get_config_var("EXT_SUFFIX"))   # for this interpreter alone
 HOST_SOURCE = os.path.join(CSRC, "host.cpp")
 
 
 def build_host(force: bool = False) -> str:
-    """Build _host.so if missing or stale; return its path."""
+    """Build the host module if missing or stale and load the binding again if it was loaded without it; return its path."""
+    path = _build_host(force)
+    binding, package = (sys.modules.get(__package__ + s) for s in (".binding", "")) if __package__ else (None, None)
+    if binding is not None and isinstance(binding._host, binding._NotBuilt):
+        importlib.invalidate_caches()
+        importlib.reload(binding)
+        importlib.reload(package)
+    return path
+
+
+def _build_host(force):
     header = os.path.join(os.path.dirname(_HERE), "include", "mxfp4.h")
     if not force and os.path.exists(HOST) and os.path.getmtime(HOST) >= max(os.path.getmtime(HOST_SOURCE), os.path.getmtime(header)):
         return HOST
@@ -38,7 +49,7 @@ def _newest_source_mtime():
 
 
 def build(force: bool = False, verbose: bool = False, extra_flags=()) -> str:
-    """Build libmxfp4.so and _host.so if missing or stale; return the former's path.  nvcc cross-compiles without a GPU."""
+    """Build libmxfp4.so and _host if missing or stale; return the former's path.  nvcc cross-compiles without a GPU."""
     build_host(force)
     if not force and os.path.exists(LIB) and os.path.getmtime(LIB) >= _newest_source_mtime():
         return LIB

@@ -301,6 +301,6 @@ PyMODINIT_FUNC PyInit__host()
     if (!g_data_ptr && !(g_data_ptr = PyUnicode_InternFromString("data_ptr"))) return nullptr;
     if (PyType_Ready(&mat_type) < 0) return nullptr;
     PyObject *m = PyModule_Create(&module);
-    if (m && PyModule_AddObjectRef(m, "Mat", reinterpret_cast<PyObject *>(&mat_type)) < 0) Py_CLEAR(m);
+    if (m && (PyModule_AddObjectRef(m, "Mat", reinterpret_cast<PyObject *>(&mat_type)) < 0 || PyModule_AddIntConstant(m, "interface", 2) < 0)) Py_CLEAR(m);
     return m;
 }

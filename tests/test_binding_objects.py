@@ -9,6 +9,12 @@ import pytest
 import torch
 
 import paper_2502_20853_b200 as mx
+from paper_2502_20853_b200 import build
+
+
+@pytest.fixture(scope="module", autouse=True)
+def built():
+    build.build()
 
 
 def _filled(rows=96, cols=64, given=False):
