@@ -218,10 +218,12 @@ class QMat(_host.Mat):
 
     @staticmethod
     def two(r0, c0, r1, c1, device):
-        """Two QMats in one buffer: operands that live and die together."""
-        if ALLOC_HOOK is not None:
+        """Two QMats, in one buffer up to 1 MiB: there the allocation is a tenth of a step, and whoever keeps one of the two keeps little
+        of the other's memory."""
+        n = _host.nbytes(r0, c0, r1, c1)
+        if n > 1 << 20 or ALLOC_HOOK is not None:
             return QMat(r0, c0, device), QMat(r1, c1, device)
-        buf = torch.empty(_host.nbytes(r0, c0, r1, c1), dtype=torch.uint8, device=device)
+        buf = torch.empty(n, dtype=torch.uint8, device=device)
         return _host.place(QMat, buf, buf.data_ptr(), r0, c0, r1, c1)
 
     def __reduce_ex__(self, protocol):

@@ -140,3 +140,13 @@ def test_native_calls_refuse_none_for_a_number(name, numbers, pointers, matrices
             with pytest.raises(TypeError):
                 call(**{"_%d" % i: bad})
     assert len(called) == 1
+
+
+@pytest.mark.parametrize("rows,cols,shared", [(1024, 192, True), (2048, 768, False), (25216, 384, False)])
+def test_matrices_of_a_call_share_memory_only_while_it_is_little(rows, cols, shared):
+    """The two operands made from one tensor may be kept for different times: keeping one of them keeps no more than 1 MiB of the
+    other's memory."""
+    a, b = mx.QMat.two(rows, cols, cols, rows, "cpu")
+    assert (a._buf is b._buf) == shared and a._buf.numel() <= (1 << 20 if shared else rows * cols)
+    assert (a.rows, a.cols, b.rows, b.cols) == (rows, cols, cols, rows)
+    assert a.data.shape == (rows, cols // 2) and b.scales.numel() >= mx.scale_bytes(cols, rows)
