@@ -175,9 +175,16 @@ def _check(fn, status):
         raise MxError(fn, status)
 
 
-def _stream():
+try:
     # the raw handle of the current stream, without the Stream object that torch.cuda.current_stream() builds (3 us)
-    return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
+    _raw_stream, _device = torch._C._cuda_getCurrentRawStream, torch._C._cuda_getDevice
+
+    def _stream():
+        return _raw_stream(_device())
+except AttributeError:      # they are internal to torch
+
+    def _stream():
+        return torch.cuda.current_stream().cuda_stream
 
 
 def _ptr(t):

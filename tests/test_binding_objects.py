@@ -150,3 +150,16 @@ def test_matrices_of_a_call_share_memory_only_while_it_is_little(rows, cols, sha
     assert (a._buf is b._buf) == shared and a._buf.numel() <= (1 << 20 if shared else rows * cols)
     assert (a.rows, a.cols, b.rows, b.cols) == (rows, cols, cols, rows)
     assert a.data.shape == (rows, cols // 2) and b.scales.numel() >= mx.scale_bytes(cols, rows)
+
+
+def test_stream_without_the_private_calls(monkeypatch):
+    """A torch without the two internal functions: the public call gives the handle."""
+    import importlib
+    import types
+    for name in ("_cuda_getCurrentRawStream", "_cuda_getDevice"):
+        monkeypatch.delattr(torch._C, name, raising=False)
+    monkeypatch.setattr(torch.cuda, "current_stream", lambda: types.SimpleNamespace(cuda_stream=5))
+    spec = importlib.util.spec_from_file_location("paper_2502_20853_b200._binding_again", mx.binding.__file__)
+    again = importlib.util.module_from_spec(spec)
+    spec.loader.exec_module(again)
+    assert again._stream() == 5
