@@ -294,7 +294,7 @@ __device__ __forceinline__ void stage_line_wide(uint8_t *line, int row, const ui
 // The warp owns TMEM lanes (= tile rows) row0 .. row0 + 31 and BN / 2 accumulator columns starting at `taddr`
 // (global column `colbase`).  bf16: the whole share is read and packed first, the accumulator is handed back (an
 // arrive on `acc_empty_bar`), then the rows go through 64B-swizzled staging buffers to TMA stores clipped at M, N.
-// `map_w` (bf16 only, may be null): the same output with boxes of 64 columns and 128B swizzle; pairs of chunks then
+// `map_w` (bf16 only): the same output with boxes of 64 columns and 128B swizzle; pairs of chunks then
 // leave through one store instead of two (issuing a store costs its thread about 150 cycles).
 // Arrive on a barrier of another CTA of the cluster (a shared::cluster address).  Used to hand an accumulator back: what
 // the arrive has to order are this warp's accumulator reads, which tcgen05.wait::ld has already completed, so the default
@@ -353,9 +353,10 @@ __device__ __forceinline__ void epilogue_tile(const CUtensorMap *map_d, const CU
             }
         }
         release_acc();
-        if (BUFS >= kChunks && map_w != nullptr) {
-            // as below, with each pair of chunks staged as one 128-byte-wide box (two staging buffers are contiguous)
-            if (lane == 0) bulk_wait_read<0>();
+        if (BUFS >= kChunks) {
+            // a staging buffer per chunk: stage everything, each pair of chunks as one 128-byte-wide box (two staging buffers are
+            // contiguous), make it visible once, then issue all the stores
+            if (lane == 0) bulk_wait_read<0>();   // the stores of the previous tile have long been read
             __syncwarp();
 #pragma unroll
             for (int cc = 0; cc < kChunks; cc += 2) {
@@ -371,22 +372,6 @@ __device__ __forceinline__ void epilogue_tile(const CUtensorMap *map_d, const CU
                 for (int cc = 0; cc < kChunks; cc += 2)
                     if (colbase + cc * 32 < p.N && row0 < p.M)
                         tma_store_3d(cc + 1 < kChunks ? map_w : map_d, colbase + cc * 32, row0, split, smem_u32(staging + cc * kStagingBytes));
-                bulk_commit();
-            }
-        } else if (BUFS >= kChunks) {
-            // a staging buffer per chunk: stage everything, make it visible once, then issue all the stores
-            if (lane == 0) bulk_wait_read<0>();   // the stores of the previous tile have long been read
-            __syncwarp();
-#pragma unroll
-            for (int cc = 0; cc < kChunks; cc++)
-                if (colbase + cc * 32 < p.N && row0 < p.M) stage_line(staging + cc * kStagingBytes + lane * 64, lane, pk[cc]);
-            fence_async_smem();
-            __syncwarp();
-            if (lane == 0) {
-#pragma unroll
-                for (int cc = 0; cc < kChunks; cc++)
-                    if (colbase + cc * 32 < p.N && row0 < p.M)
-                        tma_store_3d(map_d, colbase + cc * 32, row0, split, smem_u32(staging + cc * kStagingBytes));
                 bulk_commit();
             }
         } else {
@@ -642,7 +627,7 @@ k_gemm_mxf4(const __grid_constant__ GemmJob one, const __grid_constant__ Job2 tw
             const int colbase = nb * BN + chalf * kHalfCols;
             const uint32_t taddr = tmem_base + ((uint32_t)(quarter * 32) << 16) + acc * BN + chalf * kHalfCols;
             if (p.bias != nullptr) bias_stage<kHalfCols>(bias, bias_line, lane);
-            epilogue_tile<BN, C::kStagingBufs>(&job.d, p.out_fp32 ? nullptr : &job.dw, p, taddr, row0, colbase, split, staging, sbuf, lane,
+            epilogue_tile<BN, C::kStagingBufs>(&job.d, &job.dw, p, taddr, row0, colbase, split, staging, sbuf, lane,
                                                bar_acc_empty + 8 * acc, bias_line);
             if (++acc == C::kAccStages) { acc = 0; acc_phase ^= 1u; }
         }
@@ -1152,7 +1137,7 @@ k_gemm_mxf4_bs(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
             const int colbase = nb * BN + chalf * kHalfCols;
             const uint32_t taddr = tmem_base + ((uint32_t)(quarter * 32) << 16) + acc * BN + chalf * kHalfCols;
             if (p.bias != nullptr) bias_stage<kHalfCols>(bias, bias_line, lane);
-            epilogue_tile<BN, C::kStagingBufs>(&map_d, p.out_fp32 ? nullptr : &map_dw, p, taddr, row0, colbase, 0, staging, sbuf, lane,
+            epilogue_tile<BN, C::kStagingBufs>(&map_d, &map_dw, p, taddr, row0, colbase, 0, staging, sbuf, lane,
                                                bar_acc_empty + 8 * acc, bias_line);
             if (++acc == 2) { acc = 0; acc_phase ^= 1u; }
         }
@@ -1882,12 +1867,11 @@ k_gemm_mxf4_pair(const __grid_constant__ PairJob one, const __grid_constant__ Jo
         const int quarter = warp & 3;
         const int chalf = ew >> 2;
         uint8_t *staging = smem + C::kStagingOff + ew * C::kStagingBufs * kStagingBytes;
-        uint32_t sbuf = 0;
         constexpr int kHalfCols = BN / 2;
         constexpr int kChunks = kHalfCols / 32;
         if constexpr (BN == 192) {
             const uint32_t bias_line = smem_base + C::kBiasOff + ew * (BN / 2) * 2;
-            uint32_t acc = 0, acc_phase = 0;
+            uint32_t sbuf = 0, acc = 0, acc_phase = 0;
             for (int i = 0;; i++) {
                 const PairItem x = pair_item<kTwo>(one.p, job2->p, walk, i);
                 if (x.done) break;
@@ -1899,7 +1883,7 @@ k_gemm_mxf4_pair(const __grid_constant__ PairJob one, const __grid_constant__ Jo
                 if (!mbar_wait_warp(bar_acc_full + 8 * acc, acc_phase, abort_flag, p0.dev_status, p0.spin_limit)) break;
                 tc_fence_after();
                 if (p.bias != nullptr) bias_stage<kHalfCols>(bias, bias_line, lane);
-                epilogue_tile<BN, C::kStagingBufs, true>(&job.d, p.out_fp32 ? nullptr : &job.dw, p,
+                epilogue_tile<BN, C::kStagingBufs, true>(&job.d, &job.dw, p,
                                                          tmem_base + ((uint32_t)(quarter * 32) << 16) + acc * BN + chalf * kHalfCols, mb * kBM + quarter * 32,
                                                          nb * BN + chalf * kHalfCols, x.split, staging, sbuf, lane, map_to_cta(bar_acc_empty + 8 * acc, 0), bias_line);
                 if (++acc == C::kAccStages) { acc = 0; acc_phase ^= 1u; }
@@ -1924,17 +1908,15 @@ k_gemm_mxf4_pair(const __grid_constant__ PairJob one, const __grid_constant__ Jo
             const uint32_t taddr = tmem_base + ((uint32_t)(quarter * 32) << 16) + chalf * kHalfCols;
             const bool use_bias = p.bias != nullptr && p.splits == 1;
             auto store_box = [&](const uint32_t *w, int col0) {
-                if (lane == 0) bulk_wait_read<C::kStagingBufs - 1>();
+                if (lane == 0) bulk_wait_read<0>();     // the one staging buffer has been read
                 __syncwarp();
-                uint8_t *buf = staging + sbuf * kStagingBytes;
-                stage_line(buf + lane * 64, lane, w);
+                stage_line(staging + lane * 64, lane, w);
                 fence_async_smem();
                 __syncwarp();
                 if (lane == 0) {
-                    tma_store_3d(&job.d, col0, row0, x.split, smem_u32(buf));
+                    tma_store_3d(&job.d, col0, row0, x.split, smem_u32(staging));
                     bulk_commit();
                 }
-                sbuf = (sbuf + 1) % C::kStagingBufs;
             };
             auto release_acc = [&]() {
                 tc_fence_before();
@@ -1955,27 +1937,10 @@ k_gemm_mxf4_pair(const __grid_constant__ PairJob one, const __grid_constant__ Jo
                     }
                 }
                 release_acc();
-                if (C::kStagingBufs >= kChunks) {
-                    if (lane == 0) bulk_wait_read<0>();
-                    __syncwarp();
 #pragma unroll
-                    for (int cc = 0; cc < kChunks; cc++)
-                        if (colbase + cc * 32 < p.N && row0 < p.M) stage_line(staging + cc * kStagingBytes + lane * 64, lane, pk[cc]);
-                    fence_async_smem();
-                    __syncwarp();
-                    if (lane == 0) {
-#pragma unroll
-                        for (int cc = 0; cc < kChunks; cc++)
-                            if (colbase + cc * 32 < p.N && row0 < p.M)
-                                tma_store_3d(&job.d, colbase + cc * 32, row0, x.split, smem_u32(staging + cc * kStagingBytes));
-                        bulk_commit();
-                    }
-                } else {
-#pragma unroll
-                    for (int cc = 0; cc < kChunks; cc++) {
-                        const int col = colbase + cc * 32;
-                        if (col < p.N && row0 < p.M) store_box(pk[cc], col);
-                    }
+                for (int cc = 0; cc < kChunks; cc++) {
+                    const int col = colbase + cc * 32;
+                    if (col < p.N && row0 < p.M) store_box(pk[cc], col);
                 }
             } else {
 #pragma unroll 1
@@ -2273,7 +2238,7 @@ k_gemm_mxf4_pbs(const __grid_constant__ CUtensorMap map_a, const __grid_constant
             const int colbase = nb * BN + chalf * kHalfCols;
             const uint32_t taddr = tmem_base + ((uint32_t)(quarter * 32) << 16) + acc * BN + chalf * kHalfCols;
             if (p.bias != nullptr) bias_stage<kHalfCols>(bias, bias_line, lane);
-            epilogue_tile<BN, C::kStagingBufs, true>(&map_d, p.out_fp32 ? nullptr : &map_dw, p, taddr, row0, colbase, 0, staging, sbuf, lane,
+            epilogue_tile<BN, C::kStagingBufs, true>(&map_d, &map_dw, p, taddr, row0, colbase, 0, staging, sbuf, lane,
                                                      map_to_cta(bar_acc_empty + 8 * acc, 0), bias_line);
             if (++acc == 2) { acc = 0; acc_phase ^= 1u; }
         }
@@ -2290,7 +2255,6 @@ k_gemm_mxf4_pbs(const __grid_constant__ CUtensorMap map_a, const __grid_constant
     }
 }
 
-// Split-K: sum the FP32 partials in a fixed order, add the bias, cast.
 // Sum of the split-K partial tiles in a fixed order, + bias, cast.  GROUPS threads share four output columns: each adds every
 // GROUPS-th partial, then the sums meet in shared memory in rising order: eight where one thread per output would leave most
 // SMs without a block and each with a long chain of loads (products with their reductions, back to back: 96 x 288 x 401408
@@ -2438,7 +2402,7 @@ static GemmPlan plan_gemm(int64_t m, int64_t n, int64_t kc, int sms, bool allow_
         // part (cudaOccupancyMaxActiveClusters; 33 times for four, 45 for three), and with fewer, longer K loops the
         // two-kernel path below (CTA pairs on 256 x 256 tiles, partial sums through L2) was measured faster.
         const int units = (int)(ceil_div(m, kBM) * ceil_div(n, 192));
-        if (units * 2 <= sms && units * 4 >= sms && g.kt_total >= 8) g.ck = 2;
+        if (units * 2 <= sms && units * 4 >= sms) g.ck = 2;
     }
     if (g.ck) {
         g.bn = 192;
@@ -2658,8 +2622,7 @@ static void set_walk(GemmParams &p, int workers = 1, int rows = 1)
     p.extra = rest_workers ? (int)(rest % rest_workers) : 0;
 }
 
-// spin_limit / withhold_loads: see GemmParams (normal use: kWaitSpinLimit, 0).
-// The maps and parameters of one product with plan g.
+// The maps and parameters of one product with plan g.  spin_limit / withhold_loads: see GemmParams (normal use: kWaitSpinLimit, 0).
 static bool make_job(PairJob &job, const GemmPlan &g, mxfp4_mat_t a, mxfp4_mat_t b, void *d, int64_t ldd, int out_dtype, const void *bias, void *workspace,
                      uint32_t *dev_status, uint32_t spin_limit, int withhold_loads)
 {
