@@ -267,7 +267,8 @@ mxfp4_status_t mxfp4_mma_issue_ceiling(int32_t bn, int32_t iters, uint32_t *dev_
  * thread block leave its loop; the block then synchronises, frees its tensor memory and returns, so the context
  * stays usable.  In normal use the bound (about 0.3 s) is never reached.  These two calls exercise that path
  * without any fault: they launch the very kernels mxfp4_gemm / mxfp4_quantize_2axis would launch for these
- * arguments, with the operand loads withheld and the bound set to `spin_limit` polls (128 .. 65536), so that the
+ * arguments, and those that make two products (a backward pass: this one, and the same with a contraction cut to 1536, if
+ * they would share a launch) or quantize two matrices (a forward pass: twice this one), with the operand loads withheld and the bound set to `spin_limit` polls (128 .. 65536), so that the
  * first wait of every block runs out within milliseconds.  Nothing is computed; the outputs (and the workspace)
  * are left undefined; *dev_status (required) has MXFP4_DEV_TIMEOUT set when the kernels have finished.  All waits
  * stay bounded: the calls return like any other and the next call on the stream runs normally. */

@@ -455,7 +455,7 @@ STATIC_SCRATCH_BYTES = 16 << 20
 
 def gemm_static(a, b, out, out_dtype=OUT_BF16, bias=None, dev_status=None):
     """gemm() for callers that must not allocate: ``out`` is required, the split-K scratch is the
-    library's own fixed device array (STATIC_SCRATCH_BYTES; larger needs raise WORKSPACE_TOO_SMALL).
+    library's own fixed device array (STATIC_SCRATCH_BYTES; as many parts as fit, WORKSPACE_TOO_SMALL where those are too few).
     Nothing is allocated here or in the library.  Calls on one GPU share the array: do not overlap them."""
     _check("mxfp4_gemm_static", lib().mxfp4_gemm_static(a.c(), b.c(), _ptr(out), out.stride(0), out_dtype, _ptr(bias),
                                                         _ptr(dev_status), _stream()))

@@ -67,6 +67,8 @@ inline cudaError_t launch_pdl(void (*kernel)(Params...), unsigned grid_x, unsign
     return e;
 }
 
+constexpr uint32_t kWaitSpinLimit = 1u << 22;   // x ~64 ns backoff  =>  ~0.3 s before a bounded wait gives up
+
 __host__ __device__ inline int64_t ceil_div(int64_t a, int64_t b) { return (a + b - 1) / b; }
 
 // Offset of scale (row, block) in the 128x4 tiled order; nblk4 = ceil(nblk / 4).

@@ -2742,8 +2742,10 @@ static TwoKind plan_two(int64_t m1, int64_t kc1, int64_t m2, int64_t kc2, int64_
 // draining the machine and lets the second product's tiles fill the pairs that the first one leaves idle (64 items of 197 K tiles
 // on 74 pairs).  Both together, back to back, in us (rows, columns of X and of dY): 1024, 192, 768 9.6 -> 5.3; 2048, 384, 768
 // 12.7 -> 8.2; 4096, 768, 3072 26.9 -> 21.7; 25216, 384, 1536 41 -> 30; 8192, 2048, 2048 39 -> 33; 50432, 1024, 4096 189 -> 174.
-mxfp4_status_t gemm_two(mxfp4_mat_t a1, mxfp4_mat_t b1, void *d1, int64_t ldd1, int dtype1, mxfp4_mat_t a2, mxfp4_mat_t b2, void *d2, int64_t ldd2, int dtype2,
-                        void *workspace, size_t workspace_bytes, uint32_t *dev_status, cudaStream_t st)
+// spin_limit / withhold_loads: see GemmParams; the self-test runs the joint launch alone.
+static mxfp4_status_t gemm_two_impl(mxfp4_mat_t a1, mxfp4_mat_t b1, void *d1, int64_t ldd1, int dtype1, mxfp4_mat_t a2, mxfp4_mat_t b2, void *d2, int64_t ldd2,
+                                    int dtype2, void *workspace, size_t workspace_bytes, uint32_t *dev_status, cudaStream_t st, uint32_t spin_limit,
+                                    int withhold_loads)
 {
     mxfp4_status_t s;
     if ((s = gemm_check(a1, b1, d1, ldd1, dtype1, nullptr, workspace, workspace_bytes, true)) ||
@@ -2755,8 +2757,8 @@ mxfp4_status_t gemm_two(mxfp4_mat_t a1, mxfp4_mat_t b1, void *d1, int64_t ldd1, 
         const TwoKind kind = plan_two(a1.rows, a1.cols, a2.rows, a2.cols, b1.rows, sms, workspace ? workspace_bytes : 0, g1, g2);
         if (kind != TwoKind::kSeparate) {
             PairJob j1, j2;
-            if (!make_job(j1, g1, a1, b1, d1, ldd1, dtype1, nullptr, workspace, dev_status, kWaitSpinLimit, 0) ||
-                !make_job(j2, g2, a2, b2, d2, ldd2, dtype2, nullptr, nullptr, dev_status, kWaitSpinLimit, 0))
+            if (!make_job(j1, g1, a1, b1, d1, ldd1, dtype1, nullptr, workspace, dev_status, spin_limit, withhold_loads) ||
+                !make_job(j2, g2, a2, b2, d2, ldd2, dtype2, nullptr, nullptr, dev_status, spin_limit, withhold_loads))
                 return MXFP4_CUDA_ERROR;
             if (kind == TwoKind::kOneWave) return launch_gemm<128, GemmJob>(j1, j2, g1.tiles_m * g1.tiles_n + g2.tiles_m * g2.tiles_n, st);
             const int items = (g1.tiles_m + 1) / 2 * g1.tiles_n * g1.splits + (g2.tiles_m + 1) / 2 * g2.tiles_n, workers = min(sms / 2, items);
@@ -2767,11 +2769,18 @@ mxfp4_status_t gemm_two(mxfp4_mat_t a1, mxfp4_mat_t b1, void *d1, int64_t ldd1, 
             const int tile = g1.bn == 256 ? 3 : 1, ka = a.p.kt_per_split + tile, kb = b.p.kt_per_split + tile;
             b.p.head = (ka + kb / 2) / kb;
             if ((s = g1.bn == 256 ? launch_gemm_pair<256>(a, b, 2 * workers, st) : launch_gemm_pair<192>(a, b, 2 * workers, st))) return s;
-            return g1.splits > 1 ? launch_splitk_reduce(g1, workspace, a1.rows, b1.rows, d1, ldd1, dtype1, nullptr, sms, st) : MXFP4_OK;
+            return g1.splits > 1 && !withhold_loads ? launch_splitk_reduce(g1, workspace, a1.rows, b1.rows, d1, ldd1, dtype1, nullptr, sms, st) : MXFP4_OK;
         }
     }
+    if (withhold_loads) return MXFP4_OK;
     if ((s = gemm_impl(a1, b1, d1, ldd1, dtype1, nullptr, workspace, workspace_bytes, dev_status, st, true, kWaitSpinLimit, 0))) return s;
     return gemm_impl(a2, b2, d2, ldd2, dtype2, nullptr, workspace, workspace_bytes, dev_status, st, true, kWaitSpinLimit, 0);
+}
+
+mxfp4_status_t gemm_two(mxfp4_mat_t a1, mxfp4_mat_t b1, void *d1, int64_t ldd1, int dtype1, mxfp4_mat_t a2, mxfp4_mat_t b2, void *d2, int64_t ldd2, int dtype2,
+                        void *workspace, size_t workspace_bytes, uint32_t *dev_status, cudaStream_t st)
+{
+    return gemm_two_impl(a1, b1, d1, ldd1, dtype1, a2, b2, d2, ldd2, dtype2, workspace, workspace_bytes, dev_status, st, kWaitSpinLimit, 0);
 }
 
 mxfp4_status_t gemm(mxfp4_mat_t a, mxfp4_mat_t b, void *d, int64_t ldd, int out_dtype, const void *bias, void *workspace,
@@ -3034,8 +3043,12 @@ mxfp4_status_t mxfp4_gemm_wait_selftest(mxfp4_mat_t a, mxfp4_mat_t b, void *d, i
                                         size_t workspace_bytes, uint32_t spin_limit, uint32_t *dev_status, void *stream)
 {
     if (!dev_status || spin_limit < 128u || spin_limit > (1u << 16)) return MXFP4_INVALID_ARG;
-    return mx::gemm_impl(a, b, d, ldd, out_dtype, nullptr, workspace, workspace_bytes, dev_status, static_cast<cudaStream_t>(stream), true,
-                         spin_limit, 1);
+    cudaStream_t st = static_cast<cudaStream_t>(stream);
+    const mxfp4_status_t s = mx::gemm_impl(a, b, d, ldd, out_dtype, nullptr, workspace, workspace_bytes, dev_status, st, true, spin_limit, 1);
+    if (s) return s;
+    mxfp4_mat_t a2 = a, b2 = b;
+    a2.cols = b2.cols = std::min<int64_t>(a.cols, 1536);     // short enough not to be split
+    return mx::gemm_two_impl(a, b, d, ldd, out_dtype, a2, b2, d, ldd, out_dtype, workspace, workspace_bytes, dev_status, st, spin_limit, 1);
 }
 
 mxfp4_status_t mxfp4_gemm(mxfp4_mat_t a, mxfp4_mat_t b, void *d, int64_t ldd, int32_t out_dtype, const void *bias_bf16,

@@ -10,7 +10,7 @@ mxfp4_status_t quantize_tile(const void *src_bf16, const mxfp4_mat_t *src_q, int
                              const mxfp4_qparams_t *qp_t, uint32_t *dev_status, cudaStream_t st, bool chain);
 mxfp4_status_t quantize_chain_two(const void *x_bf16, int64_t m, int64_t k, int64_t ldx, const mxfp4_mat_t &xq, const mxfp4_mat_t &xq_t, const mxfp4_qparams_t *q6,
                                   const void *w_bf16, int64_t n, const mxfp4_mat_t &wq, const mxfp4_mat_t &wq_t, const mxfp4_qparams_t *q4,
-                                  const mxfp4_qparams_t *rne, uint32_t *dev_status, cudaStream_t st);
+                                  const mxfp4_qparams_t *rne, uint32_t *dev_status, cudaStream_t st, uint32_t spin_limit, int withhold_loads);
 mxfp4_status_t gemm_two(mxfp4_mat_t a1, mxfp4_mat_t b1, void *d1, int64_t ldd1, int dtype1, mxfp4_mat_t a2, mxfp4_mat_t b2, void *d2, int64_t ldd2, int dtype2,
                         void *workspace, size_t workspace_bytes, uint32_t *dev_status, cudaStream_t st);
 mxfp4_status_t gemm(mxfp4_mat_t a, mxfp4_mat_t b, void *d, int64_t ldd, int out_dtype, const void *bias, void *workspace,
@@ -96,7 +96,7 @@ mxfp4_status_t mxfp4_linear_fwd_ex(const void *x_bf16, int64_t ldx, int64_t m, i
     const bool make_q6 = x_bf16 && ctx->xq_t.data;
     if (make_q6 && make_q4 && m > 0 && n > 0 && k > 0) {
         if (scale_mode != MXFP4_SCALE_TRUNCATION_FREE && scale_mode != MXFP4_SCALE_FLOOR) return MXFP4_INVALID_ARG;
-        s = quantize_chain_two(x_bf16, m, k, ldx, ctx->xq, ctx->xq_t, &q6, w_bf16, n, ctx->wq, ctx->wq_t, &q4, &qp, dev_status, st);
+        s = quantize_chain_two(x_bf16, m, k, ldx, ctx->xq, ctx->xq_t, &q6, w_bf16, n, ctx->wq, ctx->wq_t, &q4, &qp, dev_status, st, kWaitSpinLimit, 0);
         if (s) return s;
     } else {
         if (make_q6) s = quantize_tile(x_bf16, nullptr, m, k, ldx, &ctx->xq, &qp, ctx->xq_t, &q6, dev_status, st, true);

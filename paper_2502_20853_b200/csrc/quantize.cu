@@ -713,13 +713,13 @@ mxfp4_status_t quantize_gelu_chain(const void *y_bf16, int64_t rows, int64_t col
 // then stochastic double quantization).  The caller has checked every argument; m, n and k are multiples of 32.
 mxfp4_status_t quantize_chain_two(const void *x_bf16, int64_t m, int64_t k, int64_t ldx, const mxfp4_mat_t &xq, const mxfp4_mat_t &xq_t, const mxfp4_qparams_t *q6,
                                   const void *w_bf16, int64_t n, const mxfp4_mat_t &wq, const mxfp4_mat_t &wq_t, const mxfp4_qparams_t *q4,
-                                  const mxfp4_qparams_t *rne, uint32_t *dev_status, cudaStream_t st)
+                                  const mxfp4_qparams_t *rne, uint32_t *dev_status, cudaStream_t st, uint32_t spin_limit, int withhold_loads)
 {
     if (m == 0 || n == 0 || k == 0) return MXFP4_BAD_SHAPE;
     if (qs_tiles(m, k) + qs_tiles(n, k) > 0x7FFFFFFF || m > 0x7FFFFF80 || n > 0x7FFFFF80 || k > 0x7FFFFF80) return MXFP4_BAD_SHAPE;
     QsJob x, w;
     if (!make_job(&x, x_bf16, m, k, ldx, &xq, rne, xq_t, q6) || !make_job(&w, w_bf16, n, k, k, &wq, rne, wq_t, q4)) return MXFP4_CUDA_ERROR;
-    return launch_stream<true, false, true, true, false, QsJob>(st, x, dev_status, kWaitSpinLimit, 0, nullptr, 0, w, qs_tiles(n, k));
+    return launch_stream<true, false, true, true, false, QsJob>(st, x, dev_status, spin_limit, withhold_loads, nullptr, 0, w, qs_tiles(n, k));
 }
 
 std::atomic<unsigned long long> g_launches{0};
@@ -737,8 +737,10 @@ mxfp4_status_t mxfp4_quantize_wait_selftest(const void *src_bf16, int64_t rows, 
 {
     if (!src_bf16 || !dev_status || spin_limit < 128u || spin_limit > (1u << 16)) return MXFP4_INVALID_ARG;
     const mxfp4_qparams_t qp = {MXFP4_SCALE_TRUNCATION_FREE, MXFP4_ROUND_NEAREST, 0, 0, 0};
-    return quantize_tile_ex(src_bf16, nullptr, rows, cols, ld, &dst, &qp, dst_t, &qp, dev_status, static_cast<cudaStream_t>(stream), false,
-                            spin_limit, 1);
+    cudaStream_t st = static_cast<cudaStream_t>(stream);
+    const mxfp4_status_t s = quantize_tile_ex(src_bf16, nullptr, rows, cols, ld, &dst, &qp, dst_t, &qp, dev_status, st, false, spin_limit, 1);
+    if (s || rows == 0 || cols == 0) return s;
+    return quantize_chain_two(src_bf16, rows, cols, ld, dst, dst_t, &qp, src_bf16, rows, dst, dst_t, &qp, &qp, dev_status, st, spin_limit, 1);
 }
 
 size_t mxfp4_scale_bytes(int64_t rows, int64_t cols)

@@ -130,3 +130,45 @@ def test_waits_count_from_the_inputs_on(mx, hold, M, N, K):
             torch.cuda.synchronize()
     assert int(st.item()) == 0
     assert torch.equal(got, want) and torch.equal(zq[0].data, zq[1].data) and torch.equal(zq[0].scales, zq[1].scales)
+
+
+# the launches of two products: one wave of 128-wide tiles, CTA pairs 256 wide without and with split K, and 192 wide
+@pytest.mark.parametrize("M,N,K", [(256, 128, 512), (9600, 512, 1536), (1024, 512, 8192), (384, 384, 8192)])
+def test_waits_of_two_products_in_a_launch_run_out(mx, M, N, K):
+    """The joint launch of a backward pass drains like a single product's; afterwards a backward pass of the same shapes is right."""
+    rng = np.random.default_rng(M)
+    a, b = (numpy_to_qmat(mx, *rand_operand(rng, r, K)) for r in (M, N))
+    st = mx.new_status()
+    before = mx.launch_count()
+    mx.gemm_wait_selftest(a, b, st, spin_limit=2048)
+    assert mx.launch_count() - before == 2
+    torch.cuda.synchronize()
+    assert int(st.item()) & mx.DEV_TIMEOUT
+    st.zero_()
+    # dW [M, N] over K tokens, dX [K, N] over M channels
+    dyq_t, xq_t, dyq, wq_t = a, b, numpy_to_qmat(mx, *rand_operand(rng, K, M)), numpy_to_qmat(mx, *rand_operand(rng, N, M))
+    ctx = mx.LinearCtx(mx.QMat(K, N), mx.QMat(M, N), xq_t, 7, wq_t)
+    dx, dw = mx.linear_bwd(None, ctx, 7, dyq=dyq, dyq_t=dyq_t, dev_status=st)
+    torch.cuda.synchronize()
+    assert int(st.item()) == 0
+    for got, p, q, shape in ((dw, dyq_t, xq_t, (M, N, K)), (dx, dyq, wq_t, (K, N, M))):
+        da, db = mx.dequantize(p).double(), mx.dequantize(q).double()
+        check_gemm_bound(got.float().cpu().numpy(), (da @ db.T).cpu().numpy(), (da.abs() @ db.abs().T).cpu().numpy(), got.dtype == torch.bfloat16, "after",
+                         factor=max(1.0, mx.gemm_chain_mmas(*shape) / 8))
+
+
+def test_waits_of_two_matrices_in_a_launch_run_out(mx):
+    """The forward pass's quantizer of activations and weight drains too (test_quantizer_waits... launches it behind the two-axis one)."""
+    x = torch.randn((384, 320), device="cuda").to(torch.bfloat16)
+    st = mx.new_status()
+    before = mx.launch_count()
+    mx.quantize_wait_selftest(x, st, spin_limit=2048)
+    assert mx.launch_count() - before == 2
+    torch.cuda.synchronize()
+    assert int(st.item()) & mx.DEV_TIMEOUT
+    st.zero_()
+    _, ctx = mx.linear_fwd(x, x, bwd_seed=9, dev_status=st)
+    torch.cuda.synchronize()
+    assert int(st.item()) == 0
+    for got, want in zip((ctx.xq, ctx.xq_t, ctx.wq, ctx.wq_t), mx.quantize_chain(x, seed=9) + mx.quantize_chain(x, seed=9, stream_id_t=4)):
+        assert torch.equal(got.data, want.data) and torch.equal(got.scales, want.scales)
