@@ -5,11 +5,11 @@ One "step" = the whole hot path over one batch of a workload's layers: per layer
 EMA update, or round to nearest) and Q4, Q1 + Q6 + GEMM-1 (forward), Q3/Q5 (one pass over dY), GEMM-2, GEMM-3
 (backward).  Metric: useful TFLOP/s = 6*M*N*K per layer / time.  The headline is config 4 (ViT-Large MLP, 50432
 tokens: the largest workload that the method's configurations name); the other configurations are timed in the same
-run and reported under "configs".
+run and reported under "configs"; what does not fit a line (the per-kernel tables, notes) goes to standard error as a second one.
 
   python bench.py [--gpus N] [--steps K] [--warmup W] [--impl ours|reference] [--config 4] [--others 1,2,3,5,6]
 
-Prints ONE JSON line (rank 0).  `--impl reference` times the CPU oracle on a bounded sample instead.
+Prints ONE JSON line (rank 0) to standard output.  `--impl reference` times the CPU oracle on a bounded sample instead.
 """
 import argparse
 import json
@@ -41,7 +41,7 @@ def source_digest():
     import hashlib
     h = hashlib.sha256()
     d = os.path.join(ROOT, "paper_2502_20853_b200", "csrc")
-    for f in ("common.cuh", "gemm.cu", "quantize.cu"):
+    for f in ("common.cuh", "tma.cuh", "quant_tile.cuh", "gemm.cu", "quantize.cu"):
         with open(os.path.join(d, f), "rb") as fh:
             h.update(fh.read())
     return h.hexdigest()[:16]
@@ -722,7 +722,7 @@ def run_ours(args):
                              ms_per_step=total_e2e / args.steps * 1e3,
                              note="steps timed as one block; every step copies all inputs in from pinned host memory and all "
                                   "results out; copies of neighbouring steps overlap on their own streams"),
-                    gpu_launches=launches, roofline=roof, kernels=kernels)
+                    gpu_launches=launches, roofline=roof)
     del run
     torch.cuda.empty_cache()
 
@@ -772,8 +772,11 @@ def run_ours(args):
     if rank == 0:
         sampler.stop()
         cpu = time_oracle(args.config, CPU_SAMPLE_ROWS, args.cpu_passes, 0)
-        line["configs"] = configs
-        line["mlp_pair"] = mlp_pair
+        print(json.dumps(dict(kernels=kernels, configs=configs, mlp_pair=mlp_pair)), file=sys.stderr, flush=True)
+        line["configs"] = {c: {k: d[k] for k in ("ms_per_step", "tflops", "dominant_kernel", "dominant_frac", "sm_mhz")} for c, d in configs.items()}
+        if "block" in configs.get("5", {}):
+            line["configs"]["5"]["block_ms"] = configs["5"]["block"]["ms_per_step"]
+        line["mlp_pair"] = {c: {k: d[k] for k in ("unfused_ms", "fused_ms")} for c, d in mlp_pair.items()}
         line["cpu_baseline"] = dict(value=cpu["value"], unit=UNIT, cores=cpu["cores"], kind="oracle",
                                     sample=oracle_sample_text(args.config, CPU_SAMPLE_ROWS) + "; %d passes" % args.cpu_passes)
         line["peaks"] = dict(measure_stream_rates(torch), hbm_gbs=peaks["hbm"], bf16_tflops=peaks["bf16"], bf16_tflops_sustained=peaks["bf16_sustained"],
