@@ -211,7 +211,8 @@ mxfp4_status_t mxfp4_gemm(mxfp4_mat_t a, mxfp4_mat_t b, void *d, int64_t ldd, in
  * Zq and Zq_t are bit for bit what mxfp4_quantize_2axis / mxfp4_quantize_chain give on Z (same rounding rules, same
  * random stream by (seed, stream_id, position in the output)).  Every output is optional (data / pointer NULL = not
  * written), at least one must be asked for; chain needs both Zq and Zq_t.  N % 32 == 0; M % 32 == 0 when Zq_t is
- * asked for; y, z, aux: bf16 [M, N], 16-byte aligned, leading dimensions multiples of 8.  No workspace: the
+ * asked for; y, z, aux: bf16 [M, N], 16-byte aligned, leading dimensions multiples of 8.  Normally one kernel; GELU with
+ * chain and a stored Y on at least four 128 x 128 tiles per SM runs as two, the second of which reads Y back.  No workspace: the
  * contraction is never split (see mxfp4_gemm for the accuracy bound with c = ceil(kc / 64)). */
 enum { MXFP4_HOOK_IDENTITY = 0, MXFP4_HOOK_GELU = 1, MXFP4_HOOK_MULTIPLY = 2 };
 typedef struct {
@@ -267,8 +268,9 @@ mxfp4_status_t mxfp4_mma_issue_ceiling(int32_t bn, int32_t iters, uint32_t *dev_
  * thread block leave its loop; the block then synchronises, frees its tensor memory and returns, so the context
  * stays usable.  In normal use the bound (about 0.3 s) is never reached.  These two calls exercise that path
  * without any fault: they launch the very kernels mxfp4_gemm / mxfp4_quantize_2axis would launch for these
- * arguments, and those that make two products (a backward pass: this one, and the same with a contraction cut to 1536, if
- * they would share a launch) or quantize two matrices (a forward pass: twice this one), with the operand loads withheld and the bound set to `spin_limit` polls (128 .. 65536), so that the
+ * arguments, and those that make two products (a backward pass: this one, and the same with a contraction cut to
+ * 1536, if they would share a launch) or quantize two matrices (a forward pass: twice this one), with the operand
+ * loads withheld and the bound set to `spin_limit` polls (128 .. 65536), so that the
  * first wait of every block runs out within milliseconds.  Nothing is computed; the outputs (and the workspace)
  * are left undefined; *dev_status (required) has MXFP4_DEV_TIMEOUT set when the kernels have finished.  All waits
  * stay bounded: the calls return like any other and the next call on the stream runs normally. */
@@ -345,6 +347,8 @@ mxfp4_status_t mxfp4_change_sums_q(mxfp4_mat_t cur, mxfp4_mat_t prev, double *ou
  * mxfp4_qema_quantize, once per optimizer step).  If ctx->xq_t.data != NULL (needs M % 32 == 0), the same
  * kernel that makes Q1(X) also writes Q6 = Q(deq(Q1(X))^T; stochastic, seed ctx->xq_t_seed, stream 6) into
  * it, which saves the backward pass its second read of Q1(X).
+ * If w_bf16 != NULL, ctx->wq_t.data != NULL and N % 32 == 0, Q4 = Q(deq(Q2(W))^T; stochastic, seed ctx->wq_t_seed,
+ * stream 4) is written into ctx->wq_t in the same way.
  * The forward pass takes no workspace: its product never splits the contraction (for a small M with a very long
  * K, mxfp4_gemm with a workspace has more parallelism).  All arguments are checked before the first launch. */
 mxfp4_status_t mxfp4_linear_fwd(const void *x_bf16, int64_t ldx, int64_t m, int64_t k,
@@ -356,7 +360,9 @@ mxfp4_status_t mxfp4_linear_fwd(const void *x_bf16, int64_t ldx, int64_t m, int6
  * all four quantizers stochastic with Philox streams 3, 4, 5, 6 of `seed`.
  * dy bf16 [M, N] (lddy); dx bf16 [M, K] (lddx); dw [N, K] (lddw) in dw_dtype (MXFP4_OUT_*).
  * If ctx->xq_t.data != NULL and ctx->xq_t_seed == seed, ctx->xq_t is used as Q6 instead of being recomputed
- * (the result is the same either way); likewise ctx->wq_t with ctx->wq_t_seed == seed is used as Q4.
+ * (the result is the same either way, provided it was made from ctx->xq); likewise ctx->wq_t with ctx->wq_t_seed == seed is
+ * used as Q4 (made from ctx->wq).  The two products may run at the same time: dx and dw must not overlap each other, the
+ * operands or the workspace.
  * workspace: >= mxfp4_linear_workspace_bytes(M, K, N). */
 mxfp4_status_t mxfp4_linear_bwd(const void *dy_bf16, int64_t lddy, const mxfp4_linear_ctx_t *ctx,
                                 uint64_t seed, int32_t scale_mode, void *dx_bf16, int64_t lddx,
