@@ -377,3 +377,32 @@ def test_backward_pass_takes_a_smaller_workspace(mx, M, K, N, least):
     with pytest.raises(mx.MxError) as e:
         mx.linear_bwd(dy, ctx, 3, workspace=buf[:least - 16])
     assert e.value.status == 4
+
+
+@pytest.mark.parametrize("whole", [True, False])
+def test_backward_pass_in_a_graph_after_a_forward_pass_that_made_q4(mx, whole):
+    """A graph of both passes uses the Q4 of its own forward pass.  A graph of the backward pass alone makes Q4 from what ctx.wq holds
+    at each replay."""
+    M, K, N = 160, 96, 288
+    g = torch.Generator(device="cuda").manual_seed(4)
+    x, dy = (torch.randn((M, c), generator=g, device="cuda").to(torch.bfloat16) for c in (K, N))
+    w, w2 = ((torch.randn((N, K), generator=g, device="cuda") * s).to(torch.bfloat16) for s in (0.02, 0.5))
+    ws = torch.empty(mx.linear_workspace_bytes(M, K, N), dtype=torch.uint8, device="cuda")
+    dx, dw = torch.empty((M, K), dtype=torch.bfloat16, device="cuda"), torch.empty((N, K), device="cuda")
+    ctx = mx.linear_fwd(x, w, bwd_seed=1)[1]
+    mx.linear_bwd(dy, ctx, 1, dx=dx, dw=dw, workspace=ws)
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        if whole:
+            ctx = mx.linear_fwd(x, w, bwd_seed=1)[1]
+        mx.linear_bwd(dy, ctx, 1, dx=dx, dw=dw, workspace=ws)
+    for weight in (w, w2):
+        if whole:
+            w.copy_(weight)
+        else:
+            mx.quantize(weight, out=ctx.wq)
+        graph.replay()
+        torch.cuda.synchronize()
+        xq, xq_t = mx.quantize_chain(x, seed=1)
+        want_dx, want_dw = mx.linear_bwd(dy, mx.LinearCtx(xq, mx.quantize(weight), xq_t=xq_t, seed=1), 1)
+        assert torch.equal(dx, want_dx) and torch.equal(dw, want_dw)
