@@ -140,8 +140,7 @@ __device__ __forceinline__ uint32_t rne_x8(float v0, float v1, float v2, float v
 }
 
 // ---- packed bf16 arithmetic ---------------------------------------------------------------------
-// Product of two bf16 pairs.  One factor is always a power of two here, so the product is exact unless it falls
-// below the normal range, where it is far too small to round to anything but (signed) zero on the E2M1 grid.
+// Product of two bf16 pairs, rounded once to nearest (subnormal results too): what the product in FP32, which is exact, rounds to.
 __device__ __forceinline__ uint32_t mul_bf16x2(uint32_t a, uint32_t b)
 {
     uint32_t d;

@@ -651,8 +651,12 @@ k_gemm_mxf4(const __grid_constant__ GemmJob one, const __grid_constant__ Job2 tw
 // through plain stores.  Then the same 256 threads run the row pass (codes of Z with groups along N, the forward /
 // gradient operand of the next product) and the column pass (groups along M, stored transposed; with DQ it
 // re-quantizes the dequantized result of the row pass: double quantization).  The results are bit for bit those of the
-// stand-alone quantizers applied to Z.  Two accumulators: the next tile's K loop runs during this long epilogue.
-template <bool WITH_Y>   // WITH_Y: a third tile for Y (stored beside a Z that differs from it) at the price of one ring stage
+// stand-alone quantizers applied to Z.  Two accumulators: the next tile's K loop runs during this long epilogue, and a second group
+// of epilogue warps may take every other tile (two_groups).
+// GROUPS = 2: two groups of eight epilogue warps take the tiles in turn, each with an accumulator, tiles and staging of its own, on a
+// ring of two stages.  TILES: 32 KB tiles per group: Z, and one each for the hook's second factor or the dequantized row codes beside
+// a Z that is stored, and for a Y that is stored beside a Z that differs from it.
+template <int GROUPS, int TILES>
 struct GemmQCfg {
     static constexpr int BN = 128;
     static constexpr int kRB = 1;
@@ -661,19 +665,18 @@ struct GemmQCfg {
     static constexpr int kSfaBytes = 2 * kSfChunk;
     static constexpr int kSfbBytes = 2 * kSfChunk;
     static constexpr int kStageBytes = kABytes + kBBytes + kSfaBytes + kSfbBytes;   // 34 KB
-    static constexpr int kStages = WITH_Y ? 3 : 4;
+    static constexpr int kStages = GROUPS == 2 ? 2 : TILES == 3 ? 3 : 4;
     static constexpr int kAccStages = 2;
     static constexpr int kSfCol = kAccStages * BN;
     static constexpr int kSfSlot = 16;
     static constexpr int kTmemCols = 512;
-    static constexpr int kTileOff = kStages * kStageBytes;           // Z, 32 KB
-    static constexpr int kTile2Off = kTileOff + kTileBytes;          // DQ: dequantized row codes for the column pass; else: the hook's second factor
-    static constexpr int kTileYOff = kTile2Off + kTileBytes;         // Y, when it is wanted beside a Z that differs from it
-    static constexpr int kStagingOff = kTileYOff + (WITH_Y ? kTileBytes : 0);   // 2 x (transposed codes 8 KB + two scale chunks)
+    static constexpr int kThreads = 32 * (kEpiWarp0 + GROUPS * kEpiWarps);
+    static constexpr int kTileOff = kStages * kStageBytes;           // per group: TILES tiles
+    static constexpr int kStagingOff = kTileOff + GROUPS * TILES * kTileBytes;   // transposed codes 8 KB + two scale chunks: two for one group, else one per group
     static constexpr int kStagingBytes = kTile * 64 + 1024;
     static constexpr int kBarOff = kStagingOff + 2 * kStagingBytes;
     static constexpr int kBiasOff = kBarOff + 256;                   // a line of 64 bf16 per epilogue warp
-    static constexpr int kSmemBytes = kBiasOff + kEpiWarps * 128 + 1024 /*align*/;
+    static constexpr int kSmemBytes = kBiasOff + GROUPS * kEpiWarps * 128 + 1024 /*align*/;
     static_assert(kSfCol + kStages * kSfSlot <= 512, "TMEM budget");
     static_assert(kStageBytes % 1024 == 0 && kStagingBytes % 1024 == 0, "alignment");
     static_assert(kSmemBytes <= 232448, "shared memory budget");
@@ -690,22 +693,23 @@ struct QuantEpilogue {
     int aux_tma;                  // the hook's second factor arrives through map_aux (otherwise per-thread loads)
 };
 
-// named barrier of the 256 epilogue threads (barrier 0 belongs to __syncthreads)
-__device__ __forceinline__ void epi_sync() { asm volatile("bar.sync 1, 256;" ::: "memory"); }
-__device__ __forceinline__ bool epi_any(bool x)
+// named barriers of the 256 threads of an epilogue group (barrier 0 belongs to __syncthreads)
+__device__ __forceinline__ void epi_sync(int id) { asm volatile("bar.sync %0, 256;" ::"r"(id) : "memory"); }
+__device__ __forceinline__ bool epi_any(int id, bool x)
 {
     uint32_t r;
-    asm volatile("{\n\t.reg .pred p, q;\n\tsetp.ne.u32 q, %1, 0;\n\tbar.red.or.pred p, 1, 256, q;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(r) : "r"((uint32_t)x) : "memory");
+    asm volatile("{\n\t.reg .pred p, q;\n\tsetp.ne.u32 q, %1, 0;\n\tbar.red.or.pred p, %2, 256, q;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(r) : "r"((uint32_t)x), "r"(id) : "memory");
     return r != 0;
 }
 
-template <bool SR_ROW, bool SR_T, bool DQ, bool WITH_Y>
-__global__ void __launch_bounds__(kGemmThreads, 1)
+template <bool SR_ROW, bool SR_T, bool DQ, bool WITH_Y, int GROUPS>
+__global__ void __launch_bounds__(32 * (kEpiWarp0 + GROUPS * kEpiWarps), 1)
 k_gemm_mxf4_q(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b,
               const __grid_constant__ CUtensorMap map_y, const __grid_constant__ CUtensorMap map_z, const __grid_constant__ CUtensorMap map_aux,
               const __grid_constant__ CUtensorMap map_t, const GemmParams p, const __grid_constant__ QuantEpilogue e)
 {
-    using C = GemmQCfg<WITH_Y>;
+    constexpr int kTiles = WITH_Y && GROUPS == 1 ? 3 : 2;
+    using C = GemmQCfg<GROUPS, kTiles>;
     constexpr int BN = C::BN;
     extern __shared__ uint8_t smem_raw[];
     uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
@@ -717,7 +721,7 @@ k_gemm_mxf4_q(const __grid_constant__ CUtensorMap map_a, const __grid_constant__
     const uint32_t bar_acc_empty = bar_acc_full + 8 * C::kAccStages;
     uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(bars + 3 * C::kStages + 2 * C::kAccStages);
     volatile uint32_t *abort_flag = tmem_slot + 1;
-    const uint32_t bar_aux = smem_u32(bars + 3 * C::kStages + 2 * C::kAccStages + 1);   // the hook's second factor has landed
+    const uint32_t bar_aux0 = smem_u32(bars + 3 * C::kStages + 2 * C::kAccStages + 1);   // per group: the hook's second factor has landed
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const uint32_t smem_base = smem_u32(smem);
@@ -733,7 +737,7 @@ k_gemm_mxf4_q(const __grid_constant__ CUtensorMap map_a, const __grid_constant__
             mbar_init(bar_acc_full + 8 * a, 1);
             mbar_init(bar_acc_empty + 8 * a, kEpiWarps);
         }
-        mbar_init(bar_aux, 1);
+        for (int g = 0; g < GROUPS; g++) mbar_init(bar_aux0 + 8 * g, 1);
         *abort_flag = 0u;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
@@ -750,14 +754,17 @@ k_gemm_mxf4_q(const __grid_constant__ CUtensorMap map_a, const __grid_constant__
         gemm_feed_roles<C, BN>(warp, smem_base, bar_full, bar_sf_full, bar_empty, bar_acc_full, bar_acc_empty, tmem_base, abort_flag, map_a, map_b, p, blockIdx.x,
                                gridDim.x);
     } else {
-        // ================= quantizing epilogue (warps 4..11 = 256 threads) =================
+        // ================= quantizing epilogue (warps 4..11, and 12..19 of a second group: 256 threads each) =================
         pdl_wait();
-        const int et = (int)threadIdx.x - 32 * kEpiWarp0;
-        const int quarter = warp & 3, chalf = (warp - kEpiWarp0) >> 2;
+        const int group = GROUPS == 1 ? 0 : (warp - kEpiWarp0) / kEpiWarps, sync_id = 1 + group;
+        const int et = (int)threadIdx.x - 32 * (kEpiWarp0 + group * kEpiWarps);
+        const int quarter = warp & 3, chalf = et >> 7;
+        const uint32_t bar_aux = bar_aux0 + 8 * group;
         const int M = (int)p.M, N = (int)p.N;
         const QsGeom g = qs_geom(et, M, N, e.rw.packed);
         const uint32_t tfa_r2 = tf_add_of(e.rw.scale_mode) * 0x00010001u, tfa_t2 = tf_add_of(e.tr.scale_mode) * 0x00010001u;
-        const uint32_t t_base = smem_base + C::kTileOff, t2_base = smem_base + C::kTile2Off, ty_base = smem_base + C::kTileYOff;
+        const uint32_t t_base = smem_base + C::kTileOff + group * kTiles * kTileBytes, t2_base = t_base + kTileBytes, ty_base = t_base + (kTiles - 1) * kTileBytes;
+        const uint32_t dq_base = e.store_z ? t2_base : t_base;       // a Z that is stored keeps its tile until it has left
         const int trow = quarter * 32 + lane;                        // this thread's row of the tile
         const uint32_t row_off = (uint32_t)(chalf * (kTileBytes / 2) + trow * 128);
         const uint32_t t_row = t_base + row_off;
@@ -769,24 +776,25 @@ k_gemm_mxf4_q(const __grid_constant__ CUtensorMap map_a, const __grid_constant__
             tma_load_2d(t2_base, &map_aux, nb * BN, mb * kBM, bar_aux);
             tma_load_2d(t2_base + kTileBytes / 2, &map_aux, nb * BN + 64, mb * kBM, bar_aux);
         };
-        if (aux_tma && et == 0 && !p.withhold_loads && (int)blockIdx.x < p.tiles_m * p.tiles_n) issue_aux(blockIdx.x);
+        const int items = p.tiles_m * p.tiles_n, step = GROUPS * (int)gridDim.x, item0 = (int)blockIdx.x + group * (int)gridDim.x;
+        if (aux_tma && et == 0 && !p.withhold_loads && item0 < items) issue_aux(item0);
         const bool use_bias = p.bias != nullptr;
         const uint32_t bias_line = smem_base + C::kBiasOff + (warp - kEpiWarp0) * 128;
         uint32_t nonfinite = 0;
-        uint32_t acc = 0, acc_phase = 0;
-        const int items = p.tiles_m * p.tiles_n;
-        int it = 0;
-        for (int item = blockIdx.x; item < items; item += gridDim.x, it++) {
+        int it = 0;            // turn of the group; the block's tiles take the accumulators in turn
+        for (int item = item0; item < items; item += step, it++) {
+            const uint32_t acc = GROUPS == 1 ? it & 1 : group, acc_phase = GROUPS == 1 ? (it >> 1) & 1 : it & 1;
             const int mb = p.by_tiles_n.div(item), nb = item - mb * p.tiles_n;
             const int row0 = mb * kBM, col0 = nb * BN;
             uint32_t bias[1];
             bias_fetch<64>(bias, p.bias, col0 + chalf * 64, N, lane);
             bool ok = mbar_wait(bar_acc_full + 8 * acc, acc_phase, abort_flag, p.dev_status, p.spin_limit);
             if (aux_tma) ok = mbar_wait(bar_aux, (uint32_t)it & 1u, abort_flag, p.dev_status, p.spin_limit) && ok;
-            if (epi_any(!ok)) break;      // a wait ran out in one of the eight warps: all of them leave together
+            if (GROUPS == 2 && et == 0) bulk_wait_read<0>();   // the codes of the group's last tile have left its staging tile
+            if (epi_any(sync_id, !ok)) break;      // a wait ran out in one of the eight warps: all of them leave together
             tc_fence_after();
             if (use_bias) bias_stage<64>(bias, bias_line, lane);
-            uint8_t *staging = smem + C::kStagingOff + (it & 1) * C::kStagingBytes;
+            uint8_t *staging = smem + C::kStagingOff + (GROUPS == 1 ? it & 1 : group) * C::kStagingBytes;
             uint8_t *s_sc_row = staging + kTile * 64, *s_sc_t = s_sc_row + 512;
             const uint32_t taddr = tmem_base + ((uint32_t)(quarter * 32) << 16) + acc * BN + chalf * 64;
             const int grow = row0 + trow;
@@ -832,9 +840,7 @@ k_gemm_mxf4_q(const __grid_constant__ CUtensorMap map_a, const __grid_constant__
                     const uint32_t *a32 = reinterpret_cast<const uint32_t *>(aw);
 #pragma unroll
                     for (int j = 0; j < 16; j++) {
-                        // the product of two bf16 values is exact in FP32: one rounding, to bf16
-                        const __nv_bfloat162 h = __floats2bfloat162_rn(bf16lo(yw[j]) * bf16lo(a32[j]), bf16hi(yw[j]) * bf16hi(a32[j]));
-                        zw[j] = *reinterpret_cast<const uint32_t *>(&h);
+                        zw[j] = mul_bf16x2(yw[j], a32[j]);       // one rounding, as of the FP32 product, which is exact
                     }
                 } else {
 #pragma unroll
@@ -850,7 +856,7 @@ k_gemm_mxf4_q(const __grid_constant__ CUtensorMap map_a, const __grid_constant__
                                  "r"(t_row + (uint32_t)((((cc * 4 + j) ^ (trow & 7))) << 4)) : "memory");
             }
             fence_async_smem();
-            epi_sync();                                   // the tile is complete, the second factor has been read
+            epi_sync(sync_id);                            // the tile is complete, the second factor has been read
             if (et == 0) {
                 if (e.store_z) {
                     tma_store_2d(&map_z, col0, row0, t_base);
@@ -861,13 +867,13 @@ k_gemm_mxf4_q(const __grid_constant__ CUtensorMap map_a, const __grid_constant__
                     tma_store_2d(&map_y, col0 + 64, row0, ty_base + kTileBytes / 2);
                 }
                 bulk_commit();
-                if (aux_tma && item + (int)gridDim.x < items) issue_aux(item + gridDim.x);
+                if (aux_tma && item + step < items) issue_aux(item + step);
             }
-            qs_tile<SR_ROW, SR_T, DQ>(g, t_base, t2_base, row0, col0, M, N, e.emit_row, e.emit_t, e.rw, e.tr, tfa_r2, tfa_t2, staging, s_sc_row, s_sc_t,
+            qs_tile<SR_ROW, SR_T, DQ>(g, t_base, dq_base, row0, col0, M, N, e.emit_row, e.emit_t, e.rw, e.tr, tfa_r2, tfa_t2, staging, s_sc_row, s_sc_t,
                                       nonfinite);
             fence_async_smem();
             if (et == 0) bulk_wait_read<0>();             // Z has left the tile, the previous tile's codes their staging buffer
-            epi_sync();
+            epi_sync(sync_id);
             if (et == 0) {
                 if (e.emit_t) {
                     tma_store_2d(&map_t, row0 >> 1, col0, smem_u32(staging));
@@ -876,7 +882,6 @@ k_gemm_mxf4_q(const __grid_constant__ CUtensorMap map_a, const __grid_constant__
                 if (e.emit_row) bulk_store(e.rw.scales + ((size_t)(row0 >> 7) * e.rw.nblk4 + (col0 >> 7)) * 512, smem_u32(s_sc_row), 512);
                 bulk_commit();
             }
-            if (++acc == C::kAccStages) { acc = 0; acc_phase ^= 1u; }
         }
         if (et == 0) bulk_wait_read<0>();
         if (nonfinite && p.dev_status) atomicOr(p.dev_status, MXFP4_DEV_NONFINITE);
@@ -2827,15 +2832,15 @@ static QuantSide make_quant_side(const mxfp4_mat_t &m, const mxfp4_qparams_t &qp
     return s;
 }
 
-template <bool SR_ROW, bool SR_T, bool DQ, bool WITH_Y>
+template <bool SR_ROW, bool SR_T, bool DQ, bool WITH_Y, int GROUPS>
 static mxfp4_status_t launch_gemm_q(const CUtensorMap &ma, const CUtensorMap &mb, const CUtensorMap &my, const CUtensorMap &mz,
                                     const CUtensorMap &mx_, const CUtensorMap &mt, const GemmParams &p, const QuantEpilogue &e, int grid,
                                     cudaStream_t st)
 {
-    using C = GemmQCfg<WITH_Y>;
+    using C = GemmQCfg<GROUPS, WITH_Y && GROUPS == 1 ? 3 : 2>;
     static bool attr_set[kMaxDevices];
-    MX_CHECK_CUDA(set_smem_once(attr_set, k_gemm_mxf4_q<SR_ROW, SR_T, DQ, WITH_Y>, C::kSmemBytes));
-    MX_CHECK_CUDA(launch_pdl(k_gemm_mxf4_q<SR_ROW, SR_T, DQ, WITH_Y>, (unsigned)grid, 1, kGemmThreads, C::kSmemBytes, st, ma, mb, my, mz, mx_, mt, p, e));
+    MX_CHECK_CUDA(set_smem_once(attr_set, k_gemm_mxf4_q<SR_ROW, SR_T, DQ, WITH_Y, GROUPS>, C::kSmemBytes));
+    MX_CHECK_CUDA(launch_pdl(k_gemm_mxf4_q<SR_ROW, SR_T, DQ, WITH_Y, GROUPS>, (unsigned)grid, 1, C::kThreads, C::kSmemBytes, st, ma, mb, my, mz, mx_, mt, p, e));
     return MXFP4_OK;
 }
 
@@ -2879,16 +2884,31 @@ mxfp4_status_t gemm_quant_check(mxfp4_mat_t a, mxfp4_mat_t b, const void *bias, 
 mxfp4_status_t quantize_gelu_chain(const void *y_bf16, int64_t rows, int64_t cols, int64_t ldy, void *z_bf16, int64_t ldz, mxfp4_mat_t dst,
                                    const mxfp4_qparams_t *qp_row, mxfp4_mat_t dst_t, const mxfp4_qparams_t *qp_t, uint32_t *dev_status, cudaStream_t st);
 
+// Whether two groups of epilogue warps take the tiles in turn.  The epilogue is bound by the instructions it issues, and eight warps
+// with their waits for the accumulator and for one another do not fill the SM.  The second group's tiles and staging cost the ring two
+// of its four stages, so the contraction has to be short, and shorter where the epilogue is (no hook); they have to fit (GemmQCfg); and
+// a block needs a second tile.  One group / two, back to back, in us, multiply with Q3 + Q5: 25216 x 1536 x 384 52.9 / 47.5,
+// 50432 x 4096 x 1024 264 / 248, 401408 x 384 x 96 197 / 177, 2048 x 1536 x 384 (1.3 tiles per SM) 9.8 / 9.6, but 1024 x 768 x 192 6.5 / 7.0
+// and 8192 x 4096 x 2048 54 / 80; identity with Z kept: 25216 x 1536 x 384 50.2 / 45.7, 16384 x 1024 x 256 22.4 / 22.3, 50432 x 4096 x 1024
+// 249 / 269; GELU and the chain with Y kept: 4096 x 1536 x 384 16.2 / 15.6.
+static bool two_groups(const mxfp4_epilogue_t *epi, int64_t M, int64_t N, int64_t Kc)
+{
+    const bool identity = epi->hook == MXFP4_HOOK_IDENTITY, y = epi->y_bf16 && !(identity && !epi->z_bf16), z = epi->z_bf16 || (identity && epi->y_bf16);
+    const int tiles = 1 + (epi->hook == MXFP4_HOOK_MULTIPLY && !epi->chain) + (epi->chain && z) + y;
+    return tiles <= 2 && ceil_div(M, kBM) * ceil_div(N, 128) > sm_count() && Kc <= (identity ? 2 : 4) * kBKElems;
+}
+
 // Whether the product and the quantization run as two kernels: when the epilogue is GELU with the double-quantization chain,
-// Y is stored anyway, and there are at least four 128 x 128 tiles per SM.  The fused epilogue has eight warps per SM for the
-// cast, the hook and both passes, and they are the bottleneck; the two kernels read Y back (2 of 5 bytes per element more)
-// but run at the product's and the tile quantizer's own rates: fused / two kernels 84 / 64.2 us at 25216 x 1536 x 384,
-// 396 / 307 at 50432 x 4096 x 1024, 305 / 226 at 401408 x 384 x 96, 33.6 / 31.7 at 8192 x 1536 x 384 (5.2 tiles per SM), but
-// 20.6 / 22.5 at 4096 x 1536 x 384 (2.6) and 12.3 / 15.3 at 1024 x 768 x 192, where a second launch costs more.
-static bool two_pass(const mxfp4_epilogue_t *epi, int64_t M, int64_t N)
+// Y is stored anyway, and there are many 128 x 128 tiles per SM.  The fused epilogue's passes are the bottleneck; the two kernels read
+// Y back (2 of 5 bytes per element more) but run at the product's and the tile quantizer's own rates.  With one group of epilogue
+// warps the line lies at four tiles per SM: fused / two kernels 84 / 64.2 us at 25216 x 1536 x 384, 396 / 307 at 50432 x 4096 x 1024,
+// 33.6 / 31.7 at 8192 x 1536 x 384 (5.2 tiles per SM), but 20.6 / 22.5 at 4096 x 1536 x 384 (2.6) and 12.3 / 15.3 at 1024 x 768 x 192,
+// where a second launch costs more.  With two groups (back to back) it lies at about twelve: 25.3 / 26.9 at 8192 x 1536 x 384, 30.1 / 32.9 at
+// 16384 x 1024 x 256 (6.9 tiles per SM), 62.0 / 61.0 at 25216 x 1536 x 384 (16), 320 / 309 at 50432 x 4096 x 1024, 235 / 225 at 401408 x 384 x 96.
+static bool two_pass(const mxfp4_epilogue_t *epi, int64_t M, int64_t N, int64_t Kc)
 {
     return epi->hook == MXFP4_HOOK_GELU && epi->chain && epi->y_bf16 && epi->y_bf16 != epi->z_bf16 &&
-           ceil_div(M, kBM) * ceil_div(N, 128) >= 4 * (int64_t)sm_count();
+           ceil_div(M, kBM) * ceil_div(N, 128) >= (two_groups(epi, M, N, Kc) ? 12 : 4) * (int64_t)sm_count();
 }
 
 mxfp4_status_t gemm_quant(mxfp4_mat_t a, mxfp4_mat_t b, const void *bias, const mxfp4_epilogue_t *epi, uint32_t *dev_status, cudaStream_t st)
@@ -2898,7 +2918,7 @@ mxfp4_status_t gemm_quant(mxfp4_mat_t a, mxfp4_mat_t b, const void *bias, const 
     const int64_t M = a.rows, N = b.rows, Kc = a.cols;
     if (M == 0 || N == 0) return MXFP4_OK;
     const bool row = epi->zq.data != nullptr, tr = epi->zq_t.data != nullptr;
-    if (two_pass(epi, M, N)) {
+    if (two_pass(epi, M, N, Kc)) {
         // Y by the product's own kernels (the contraction is not split), then the tile quantizer reads it back
         mxfp4_status_t s = gemm(a, b, epi->y_bf16, epi->ldy, MXFP4_OUT_BF16, bias, nullptr, 0, dev_status, st, false);
         if (s) return s;
@@ -2952,7 +2972,9 @@ mxfp4_status_t gemm_quant(mxfp4_mat_t a, mxfp4_mat_t b, const void *bias, const 
     const int grid = items < sms ? items : sms;
     const bool sr_r = row && epi->qp_row.rounding == MXFP4_ROUND_STOCHASTIC, sr_t = tr && epi->qp_t.rounding == MXFP4_ROUND_STOCHASTIC;
     const int sel = (e.store_y ? 8 : 0) | (epi->chain ? 4 : 0) | (sr_r ? 2 : 0) | (sr_t ? 1 : 0);
-#define MX_Q_CASE(i, a_, b_, c_, d_) case i: return launch_gemm_q<a_, b_, c_, d_>(ma, mb, my, mz, mx_, mt, p, e, grid, st)
+    const bool two = two_groups(epi, M, N, Kc);
+#define MX_Q_CASE(i, a_, b_, c_, d_) \
+    case i: return two ? launch_gemm_q<a_, b_, c_, d_, 2>(ma, mb, my, mz, mx_, mt, p, e, grid, st) : launch_gemm_q<a_, b_, c_, d_, 1>(ma, mb, my, mz, mx_, mt, p, e, grid, st)
     switch (sel) {
     MX_Q_CASE(0, false, false, false, false);
     MX_Q_CASE(1, false, true, false, false);
@@ -2969,7 +2991,8 @@ mxfp4_status_t gemm_quant(mxfp4_mat_t a, mxfp4_mat_t b, const void *bias, const 
     MX_Q_CASE(12, false, false, true, true);
     MX_Q_CASE(13, false, true, true, true);
     MX_Q_CASE(14, true, false, true, true);
-    default: return launch_gemm_q<true, true, true, true>(ma, mb, my, mz, mx_, mt, p, e, grid, st);
+    MX_Q_CASE(15, true, true, true, true);
+    default: return MXFP4_INVALID_ARG;
     }
 #undef MX_Q_CASE
 }

@@ -187,6 +187,40 @@ def test_quantizing_epilogue_equals_the_standalone_quantizers(mx):
         assert torch.equal(epi.zq_t.data, qt.data) and torch.equal(epi.zq_t.scales, qt.scales)
 
 
+# more tiles than SMs and a short contraction: two groups of epilogue warps.  298 tiles (two blocks have a third), 171 (23 blocks
+# have a second), 225, all with ragged last tiles; contractions of one, two and four K tiles
+@pytest.mark.parametrize("M,N,K", [(18976, 160, 96), (2400, 1056, 384), (9504, 288, 1024)])
+@pytest.mark.parametrize("hook", ["gelu", "multiply"])
+def test_two_groups_of_epilogue_warps(mx, M, N, K, hook):
+    _, a, b = operands(mx, M, N, K, M + N + K)
+    g = torch.Generator(device="cuda").manual_seed(M)
+    aux = torch.randn((M, N), generator=g, device="cuda").to(torch.bfloat16)
+    bias = torch.randn(N, generator=g, device="cuda").to(torch.bfloat16)
+    # Y and Z in pieces that have no more tiles than SMs (one group; held against the oracle above): the same bits
+    y, z = (torch.empty((M, N), dtype=torch.bfloat16, device="cuda") for _ in range(2))
+    for r in range(0, M, 1280):
+        rows = slice(r, min(r + 1280, M))
+        n = rows.stop - r
+        part = mx.QMat(n, K, data=a.data[rows].contiguous(), scales=a.scales[r // 128 * ((K // 32 + 3) // 4) * 512:].clone())
+        kw = dict(hook=mx.HOOK_GELU) if hook == "gelu" else dict(hook=mx.HOOK_MULTIPLY, aux=aux[rows])
+        mx.gemm_quant(part, b, mx.Epilogue(y=y[rows], z=z[rows], zq=mx.QMat(n, N), zq_t=mx.QMat(N, n), chain=True, **kw), bias=bias)
+    st = mx.new_status()
+    seed = 77 + K
+    got_y, got_z = (torch.zeros((M, N), dtype=torch.bfloat16, device="cuda") for _ in range(2))
+    if hook == "gelu":
+        epi = mx.Epilogue(hook=mx.HOOK_GELU, y=got_y, zq=mx.QMat(M, N), zq_t=mx.QMat(N, M), qp_t=(0, 1, seed, 6), chain=True)
+        zq, zq_t = mx.quantize_chain(z, seed)
+    else:
+        epi = mx.Epilogue(hook=mx.HOOK_MULTIPLY, aux=aux, z=got_z, zq=mx.QMat(M, N), qp_row=(0, 1, seed, 3), zq_t=mx.QMat(N, M), qp_t=(0, 1, seed, 5))
+        zq, zq_t = mx.quantize_2axis(z, (0, 1, seed, 3), (0, 1, seed, 5))
+    mx.gemm_quant(a, b, epi, bias=bias, dev_status=st)
+    torch.cuda.synchronize()
+    assert int(st.item()) == 0
+    assert torch.equal(got_y, y) if hook == "gelu" else torch.equal(got_z, z)
+    for got, want in ((epi.zq, zq), (epi.zq_t, zq_t)):
+        assert torch.equal(got.data, want.data) and torch.equal(got.scales, want.scales)
+
+
 def test_gemm_quant_argument_errors(mx):
     a, b = mx.QMat(128, 64), mx.QMat(128, 64)
     with pytest.raises(mx.MxError) as e:
