@@ -1444,6 +1444,186 @@ k_gemm_mxf4_ck(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
     }
 }
 
+// ---- the kernel of a small forward pass -------------------------------------------------------------------
+// Y = Q1(X) Q2(W)^T for a batch whose 128 x 128 tiles all fit on the SMs at once, X in bf16: one launch quantizes X and multiplies.
+// Such a call is bound by the host and by the latency of its launches, so the quantizer as a launch of its own is a fifth of it.
+// The CTAs of a cluster have the same 128 rows of X and share their quantization: each takes every cluster-size-th group of 32, rounds it
+// as k_quantize_rows does, and writes codes and scale into the shared memory of all of them, in the layout the tensor core reads.  The B
+// tile and its scales, the whole contraction of them, travel meanwhile.  The cluster that has the first columns also stores the
+// codes and scales of X, padding included: the backward pass reads them.
+constexpr int kXQuantThreads = kGemmThreads - 32;   // all warps but the one that loads B
+constexpr int kXMaxKt = 2;
+struct XSource {
+    const __nv_bfloat16 *x;
+    int64_t ldx;
+    uint8_t *codes, *scales;
+    int scale_mode, cluster;
+};
+constexpr int x_staging_off(int kt) { return kt * (2 * kBM * kBKBytes + 4 * kSfChunk); }
+constexpr int x_smem_bytes(int kt) { return x_staging_off(kt) + kEpiWarps * 2 * kStagingBytes + 256 + kEpiWarps * 128 + 1024; }
+constexpr int kXSmemBytes = 120 << 10;   // one CTA per SM: a CTA that waited for tensor memory would keep its cluster waiting
+static_assert(x_smem_bytes(kXMaxKt) <= kXSmemBytes, "shared memory budget");
+
+__global__ void __launch_bounds__(kGemmThreads, 1)
+k_gemm_mxf4_x(const __grid_constant__ CUtensorMap map_b, const __grid_constant__ CUtensorMap map_d, const __grid_constant__ CUtensorMap map_dw,
+              const __grid_constant__ GemmParams p, const XSource x)
+{
+    constexpr int BN = 128, kTmemCols = 256, kSfaCol = BN, kSfbCol = BN + 8 * kXMaxKt;   // 8 columns of scales per K tile
+    extern __shared__ uint8_t smem_raw[];
+    uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
+    const int ktn = p.kt_total;
+    const uint32_t smem_base = smem_u32(smem);
+    const uint32_t sA = smem_base, sB = sA + ktn * kBM * kBKBytes, sSFA = sB + ktn * kBM * kBKBytes, sSFB = sSFA + ktn * 2 * kSfChunk;
+    uint8_t *staging0 = smem + x_staging_off(ktn);
+    uint64_t *bars = reinterpret_cast<uint64_t *>(staging0 + kEpiWarps * 2 * kStagingBytes);
+    const uint32_t bar_b = smem_u32(bars), bar_acc_full = bar_b + 8 * kXMaxKt, bar_acc_empty = bar_acc_full + 8;   // bar_b: one per K tile
+    uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(bars + kXMaxKt + 2);
+    volatile uint32_t *abort_flag = tmem_slot + 1;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int mb = p.by_tiles_n.div(blockIdx.x), nb = (int)blockIdx.x - mb * p.tiles_n;
+    const uint32_t rank = ck_cluster_rank();
+
+    if (threadIdx.x == 0) {
+        prefetch_map(&map_b);
+        for (int k = 0; k < ktn; k++) mbar_init(bar_b + 8 * k, 1);
+        mbar_init(bar_acc_full, 1);
+        mbar_init(bar_acc_empty, kEpiWarps);
+        *abort_flag = 0u;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    if (warp == 1) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)), "r"(kTmemCols) : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    }
+    tc_fence_before();
+    __syncthreads();
+    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");   // this CTA is there: its shared memory may be written
+    tc_fence_after();
+    const uint32_t tmem_base = *tmem_slot;
+    const int ew = warp - kEpiWarp0, quarter = warp & 3, chalf = ew >> 2;   // epilogue warps
+    pdl_wait();
+    uint32_t bias[1];
+    if (warp >= kEpiWarp0) bias_fetch<BN / 2>(bias, p.bias, (int64_t)nb * BN + chalf * (BN / 2), p.N, lane);
+
+    if (warp == 0) {
+        if (elect_one() && !p.withhold_loads) {
+            for (int kt = 0; kt < ktn; kt++) {
+                const int nch = min(2, p.nblk4 - 2 * kt);
+                mbar_expect_tx(bar_b + 8 * kt, (uint32_t)(kBM * kBKBytes + nch * kSfChunk));
+                tma_load_2d(sB + kt * kBM * kBKBytes, &map_b, kt * kBKBytes, nb * BN, bar_b + 8 * kt);
+                bulk_load(sSFB + kt * 2 * kSfChunk, p.sfb + ((size_t)nb * p.nblk4 + 2 * kt) * kSfChunk, (uint32_t)(nch * kSfChunk), bar_b + 8 * kt);
+            }
+        }
+        __syncwarp();
+        asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+    } else {
+        // ================= this CTA's share of Q1(X) =================
+        const int nblk = (int)(p.Kc / 32), nb_pad = p.nblk4 * 4, total = kBM * nb_pad;
+        const uint32_t tf_add = tf_add_of(x.scale_mode);
+        bool nonfinite = false, there = false;
+        // (the condition is that of the warp's first lane: the warp stays together for the barrier)
+        for (int e = ((int)threadIdx.x - 32) * x.cluster + (int)rank; e - lane * x.cluster < total; e += kXQuantThreads * x.cluster) {
+            const int row = e / nb_pad, blk = e - row * nb_pad;
+            const int64_t grow = (int64_t)mb * kBM + row;
+            const bool in = e < total && grow < p.M && blk < nblk;
+            uint4 q[4] = {make_uint4(0, 0, 0, 0), make_uint4(0, 0, 0, 0), make_uint4(0, 0, 0, 0), make_uint4(0, 0, 0, 0)};
+            if (in) {
+                const uint4 *src = reinterpret_cast<const uint4 *>(x.x + grow * x.ldx + blk * 32);
+#pragma unroll
+                for (int j = 0; j < 4; j++) q[j] = ld_stream_16(src + j);
+            }
+            uint32_t byte;
+            const uint4 codes = rne_group(q, tf_add, byte);
+            if (!in) byte = 0x7Fu;
+            nonfinite |= byte == 0xFFu;
+            if (!there) {                                       // before the first store into another CTA; the whole warp, once
+                __syncwarp();
+                asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+                there = true;
+            }
+            if (e < total) {
+                const uint32_t at = sA + (uint32_t)((blk >> 3) * kBM * kBKBytes + row * kBKBytes + (((blk & 7) ^ (row & 7)) << 4));
+                const uint32_t sc = sSFA + (uint32_t)((blk >> 2) * kSfChunk + (row & 31) * 16 + (row >> 5) * 4 + (blk & 3));
+                for (int t = 0; t < x.cluster; t++) {
+                    if (blk < nblk)
+                        asm volatile("st.shared::cluster.v4.u32 [%0], {%1, %2, %3, %4};" ::"r"(ck_map(at, t)), "r"(codes.x), "r"(codes.y), "r"(codes.z), "r"(codes.w) : "memory");
+                    asm volatile("st.shared::cluster.u8 [%0], %1;" ::"r"(ck_map(sc, t)), "r"(byte) : "memory");
+                }
+            }
+        }
+        __syncwarp();
+        if (!there) asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+        if (nonfinite && p.dev_status) atomicOr(p.dev_status, MXFP4_DEV_NONFINITE);
+        asm volatile("fence.proxy.async.shared::cluster;" ::: "memory");   // the stores above, before the tensor core reads them
+        __syncwarp();
+    }
+    ck_cluster_sync();                                          // all of Q1(X) is in place
+
+    if (warp == 1) {
+        // ================= scale copies and MMAs, from one thread: they run in order =================
+        asm volatile("fence.proxy.async.shared::cluster;" ::: "memory");
+        const bool leader = elect_one();
+        bool alive = true;
+        for (int kt = 0; kt < ktn; kt++) {
+            if (!mbar_wait_warp(bar_b + 8 * kt, 0u, abort_flag, p.dev_status, p.spin_limit)) { alive = false; break; }
+            tc_fence_after();
+            const int64_t left = p.Kc - (int64_t)kt * kBKElems;
+            const uint32_t t_sfa = tmem_base + kSfaCol + 8 * kt, t_sfb = tmem_base + kSfbCol + 8 * kt;
+            const uint64_t adesc = desc_operand_sw128(sA + kt * kBM * kBKBytes), bdesc = desc_operand_sw128(sB + kt * kBM * kBKBytes);
+            if (leader) {
+#pragma unroll
+                for (int c = 0; c < 2; c++) {
+                    if (left > 128 * c) {
+                        tc_cp_sf(t_sfa + 4 * c, desc_sf(sSFA + (2 * kt + c) * kSfChunk));
+                        tc_cp_sf(t_sfb + 4 * c, desc_sf(sSFB + (2 * kt + c) * kSfChunk));
+                    }
+                }
+#pragma unroll
+                for (int k = 0; k < 4; k++) {
+                    if (left > 64 * k) {
+                        const uint32_t sf_id = (uint32_t)(k & 1) * 2u;
+                        tc_mma_mxf4(tmem_base, adesc + (uint64_t)(k * (kMmaKBytes >> 4)), bdesc + (uint64_t)(k * (kMmaKBytes >> 4)), idesc_mxf4(BN, sf_id, sf_id),
+                                    t_sfa + 4 * (k >> 1), t_sfb + 4 * (k >> 1), (kt > 0 || k > 0) ? 1u : 0u);
+                    }
+                }
+            }
+            __syncwarp();
+        }
+        if (alive && leader) tc_commit(bar_acc_full);
+        __syncwarp();
+    } else if (warp < kEpiWarp0 && nb < x.cluster) {
+        // ================= codes and scales of X, by the row block's first cluster =================
+        // (behind the cluster's barrier: a barrier that releases stores to global memory waits for them)
+        const int nblk = (int)(p.Kc / 32), nb_pad = p.nblk4 * 4, total = kBM * nb_pad, me = warp == 0 ? lane : 32 * (warp - 1) + lane;
+        for (int e = me * x.cluster + (int)rank; e < total; e += 96 * x.cluster) {
+            const int row = e / nb_pad, blk = e - row * nb_pad;
+            const int64_t grow = (int64_t)mb * kBM + row;
+            const uint32_t at = (uint32_t)((blk >> 3) * kBM * kBKBytes + row * kBKBytes + (((blk & 7) ^ (row & 7)) << 4));
+            const uint32_t sc = (sSFA - smem_base) + (uint32_t)((blk >> 2) * kSfChunk + (row & 31) * 16 + (row >> 5) * 4 + (blk & 3));
+            if (grow < p.M && blk < nblk) *reinterpret_cast<uint4 *>(x.codes + grow * (p.Kc / 2) + blk * 16) = *reinterpret_cast<const uint4 *>(smem + at);
+            x.scales[scale_offset(grow, blk, p.nblk4)] = smem[sc];
+        }
+    } else if (warp >= kEpiWarp0) {
+        // ================= epilogue =================
+        const uint32_t bias_line = smem_u32(staging0) + kEpiWarps * 2 * kStagingBytes + 256 + ew * 128;
+        uint32_t sbuf = 0;
+        if (mbar_wait(bar_acc_full, 0u, abort_flag, p.dev_status, p.spin_limit)) {
+            tc_fence_after();
+            if (p.bias != nullptr) bias_stage<BN / 2>(bias, bias_line, lane);
+            epilogue_tile<BN, 2>(&map_d, &map_dw, p, tmem_base + ((uint32_t)(quarter * 32) << 16) + chalf * (BN / 2), mb * kBM + quarter * 32,
+                                 nb * BN + chalf * (BN / 2), 0, staging0 + ew * 2 * kStagingBytes, sbuf, lane, bar_acc_empty, bias_line);
+        }
+        if (lane == 0) bulk_wait_read<0>();   // the stores of this warp have read their staging buffers: the shared memory may go
+    }
+
+    tc_fence_before();
+    __syncthreads();
+    if (warp == 1) {
+        tc_fence_after();
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(kTmemCols) : "memory");
+    }
+}
+
 // ---- MMA issue ceiling -----------------------------------------------------------------------------------
 // What the tensor pipe takes when nothing else is in the way: one CTA per SM, operands and scales resident in shared
 // memory / TMEM, one warp issuing kind::mxf4 MMAs of 128 x BN x 64 back to back into one accumulator, no loads, no
@@ -2714,6 +2894,72 @@ static mxfp4_status_t gemm_impl(mxfp4_mat_t a, mxfp4_mat_t b, void *d, int64_t l
                                            : launch_gemm<128>(job, NoJob{}, grid, st);
     if (s || g.splits == 1 || withhold_loads) return s;
     return launch_splitk_reduce(g, workspace, M, N, d, ldd, out_dtype, bias, sms, st);
+}
+
+// The CTAs that share the quantization of a row block, for a forward pass in one launch; 0: not in one launch.  All tiles on the SMs at once,
+// a contraction of two K tiles, at most three groups of X per thread (a chain of loads), and not while a graph is captured: replayed, a
+// second launch costs nothing, and the two kernels are the faster ones on the device.  Two launches / one, in us, eager calls in a row:
+// 197 x 1536 x 384 12.8 / 10.1; from the call to its synchronized result: 21.7 / 20.7 there, 21.2 / 18.3 at 2000 x 768 x 256, but 17.5 / 19.5 at
+// 32 x 768 x 768 and 18.4 / 24.0 at 128 x 4096 x 1024; replayed 5.2 / 7.2.  Clusters of three or four: 7.2 and 7.6 us of device time at 197 x 1536 x 384,
+// 8.4 with one CTA, 7.7 with six.  They do not fit everywhere on a full machine (four whole SMs each: room for 33), and a second wave
+// costs more than they save.
+static int x_cluster(int64_t m, int64_t n, int64_t kc, int sms)
+{
+    const int64_t tiles_n = ceil_div(n, 128), tiles = ceil_div(m, kBM) * tiles_n;
+    if (m <= 0 || n <= 0 || kc <= 0 || kc > kXMaxKt * kBKElems || tiles > sms) return 0;
+    int c = tiles <= 112 ? 4 : 2;
+    while (tiles_n % c) c--;
+    return kBM * ceil_div(kc, 128) * 4 <= 3 * kXQuantThreads * c ? c : 0;
+}
+bool gemm_from_x_fits(int64_t m, int64_t n, int64_t kc, cudaStream_t st)
+{
+    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+    return x_cluster(m, n, kc, sm_count()) > 0 && cudaStreamIsCapturing(st, &capture) == cudaSuccess && capture == cudaStreamCaptureStatusNone;
+}
+
+// Y = Q1(X) b^T in one launch; xq receives Q1(X).  The caller has checked every argument, and that it fits.
+mxfp4_status_t gemm_from_x(const void *x, int64_t ldx, const mxfp4_mat_t &xq, const mxfp4_mat_t &b, void *y, int64_t ldy, const void *bias, int scale_mode,
+                           uint32_t *dev_status, cudaStream_t st, uint32_t spin_limit, int withhold_loads)
+{
+    const int64_t M = xq.rows, N = b.rows, Kc = xq.cols;
+    GemmParams p;
+    p.sfa = nullptr; p.sfb = b.scales;
+    p.M = M; p.N = N; p.Kc = Kc;
+    p.nblk4 = (int)ceil_div(Kc / 32, 4);
+    p.rbA = (int)ceil_div(M, 128); p.rbB = (int)ceil_div(N, 128);
+    p.tiles_m = p.rbA; p.tiles_n = p.rbB; p.splits = 1;
+    p.kt_total = p.kt_per_split = (int)ceil_div(Kc, kBKElems);
+    p.head = 0;
+    p.out_fp32 = 0;
+    p.bias = static_cast<const __nv_bfloat16 *>(bias);
+    p.dev_status = dev_status;
+    p.d = y;
+    p.ldd = ldy;
+    p.spin_limit = spin_limit;
+    p.withhold_loads = withhold_loads;
+    set_walk(p);
+    CUtensorMap mb, md, mdw;
+    if (!make_operand_map(&mb, b.data, N, Kc, 128) || !make_output_map(&md, y, M, N, ldy, 1, false) || !make_output_map_wide(&mdw, y, M, N, ldy)) return MXFP4_CUDA_ERROR;
+    const XSource x_ = {static_cast<const __nv_bfloat16 *>(x), ldx, static_cast<uint8_t *>(xq.data), xq.scales, scale_mode, x_cluster(M, N, Kc, sm_count())};
+    static bool attr_set[kMaxDevices];
+    MX_CHECK_CUDA(set_smem_once(attr_set, k_gemm_mxf4_x, kXSmemBytes));
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)(p.tiles_m * p.tiles_n));
+    cfg.blockDim = dim3(kGemmThreads);
+    cfg.dynamicSmemBytes = kXSmemBytes;
+    cfg.stream = st;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = (unsigned)x_.cluster;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[1].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 2;
+    MX_CHECK_CUDA(cudaLaunchKernelEx(&cfg, k_gemm_mxf4_x, mb, md, mdw, p, x_));
+    MX_LAUNCHED();
+    return MXFP4_OK;
 }
 
 enum class TwoKind { kSeparate, kOneWave, kPairs };

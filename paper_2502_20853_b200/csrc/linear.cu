@@ -15,6 +15,9 @@ mxfp4_status_t gemm_two(mxfp4_mat_t a1, mxfp4_mat_t b1, void *d1, int64_t ldd1, 
                         void *workspace, size_t workspace_bytes, uint32_t *dev_status, cudaStream_t st);
 mxfp4_status_t gemm(mxfp4_mat_t a, mxfp4_mat_t b, void *d, int64_t ldd, int out_dtype, const void *bias, void *workspace,
                     size_t workspace_bytes, uint32_t *dev_status, cudaStream_t st, bool allow_split);
+bool gemm_from_x_fits(int64_t m, int64_t n, int64_t kc, cudaStream_t st);
+mxfp4_status_t gemm_from_x(const void *x, int64_t ldx, const mxfp4_mat_t &xq, const mxfp4_mat_t &b, void *y, int64_t ldy, const void *bias, int scale_mode,
+                           uint32_t *dev_status, cudaStream_t st, uint32_t spin_limit, int withhold_loads);
 mxfp4_status_t gemm_check(mxfp4_mat_t a, mxfp4_mat_t b, const void *d, int64_t ldd, int out_dtype, const void *bias,
                           const void *workspace, size_t workspace_bytes, bool allow_split);
 size_t gemm_two_workspace_bytes(int64_t m1, int64_t kc1, int64_t m2, int64_t kc2, int64_t n, size_t scratch);
@@ -94,6 +97,11 @@ mxfp4_status_t mxfp4_linear_fwd_ex(const void *x_bf16, int64_t ldx, int64_t m, i
     const mxfp4_qparams_t q6 = {scale_mode, MXFP4_ROUND_STOCHASTIC, ctx->xq_t_seed, 6, 0};
     const mxfp4_qparams_t q4 = {scale_mode, MXFP4_ROUND_STOCHASTIC, ctx->wq_t_seed, 4, 0};
     const bool make_q6 = x_bf16 && ctx->xq_t.data;
+    // a small batch on a weight that is quantized already: one launch
+    if (x_bf16 && !make_q6 && !w_bf16 && !epi && gemm_from_x_fits(m, n, k, st)) {
+        if (scale_mode != MXFP4_SCALE_TRUNCATION_FREE && scale_mode != MXFP4_SCALE_FLOOR) return MXFP4_INVALID_ARG;
+        return gemm_from_x(x_bf16, ldx, ctx->xq, ctx->wq, y_bf16, ldy, bias_bf16, scale_mode, dev_status, st, kWaitSpinLimit, 0);
+    }
     if (make_q6 && make_q4 && m > 0 && n > 0 && k > 0) {
         if (scale_mode != MXFP4_SCALE_TRUNCATION_FREE && scale_mode != MXFP4_SCALE_FLOOR) return MXFP4_INVALID_ARG;
         s = quantize_chain_two(x_bf16, m, k, ldx, ctx->xq, ctx->xq_t, &q6, w_bf16, n, ctx->wq, ctx->wq_t, &q4, &qp, dev_status, st, kWaitSpinLimit, 0);

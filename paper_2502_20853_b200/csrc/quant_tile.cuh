@@ -90,6 +90,19 @@ __device__ __forceinline__ uint32_t absmax_u4(uint32_t acc, const uint4 &q)
     return absmax2(acc, q.w);
 }
 
+// The 16 bytes of codes of one 32-element group, round to nearest, and its scale byte (0xFF for a group with Inf / NaN, codes 0).
+__device__ __forceinline__ uint4 rne_group(const uint4 (&q)[4], uint32_t tf_add, uint32_t &byte)
+{
+    uint32_t am = 0;
+#pragma unroll
+    for (int j = 0; j < 4; j++) am = absmax_u4(am, q[j]);
+    am = hmax_halves(am);
+    byte = 0xFFu;
+    if (am >= 0x7F80u) return make_uint4(0, 0, 0, 0);
+    byte = scale_byte_from_amax(am, tf_add);
+    const uint32_t inv = inv_scale_bf16x2(byte);
+    return make_uint4(rne8(q[0], inv), rne8(q[1], inv), rne8(q[2], inv), rne8(q[3], inv));
+}
 
 // Two FP32 values in one 64-bit register: an FMA of such pairs takes one issue slot (the passes are bound by issue).
 __device__ __forceinline__ uint64_t f32x2(float a, float b)

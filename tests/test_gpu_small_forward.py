@@ -1,0 +1,73 @@
+"""GPU parity of the forward pass of a small batch, which quantizes X and multiplies in one launch: codes, scales and product are the
+bits of the row-wise quantizer and the product as launches of their own (each held against the oracle elsewhere)."""
+import pytest
+import torch
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def mx():
+    import paper_2502_20853_b200 as m
+    m.lib()
+    return m
+
+
+# one row to several row blocks, ragged everywhere; contractions of one group up to two whole K tiles; column tiles that divide into
+# clusters of 1, 2, 3 and 4 CTAs, three of them in a grid too wide for clusters above two
+@pytest.mark.parametrize("M,N,K", [(1, 8, 32), (197, 1536, 384), (31, 384, 96), (128, 1000, 512), (129, 136, 160), (300, 640, 256), (64, 896, 224), (33, 1280, 416),
+                                   (2048, 1152, 256), (1792, 1280, 64), (2300, 1024, 480)])
+@pytest.mark.parametrize("form", ["plain", "bias_strided_floor"])
+def test_forward_in_one_launch(mx, M, N, K, form):
+    g = torch.Generator(device="cuda").manual_seed(M + N + K)
+    x = torch.randn((M, K + 24), generator=g, device="cuda").to(torch.bfloat16)
+    x = x[:, :K] if form != "plain" else x[:, :K].contiguous()
+    mode = mx.SCALE_TRUNCATION_FREE if form == "plain" else mx.SCALE_FLOOR
+    x[:, : K // 2] *= 0.01
+    x[M // 2, -32:] = 0.0
+    wq = mx.quantize((torch.randn((N, K), generator=g, device="cuda") * 0.02).to(torch.bfloat16))
+    bias = torch.randn(N, generator=g, device="cuda").to(torch.bfloat16) if form != "plain" else None
+    st = mx.new_status()
+    want_q = mx.quantize(x, scale_mode=mode)
+    want = mx.gemm(want_q, wq, bias=bias)
+    big = torch.full((M, N + 8), 7.0, dtype=torch.bfloat16, device="cuda")
+    n0 = mx.launch_count()
+    y, ctx = mx.linear_fwd(x, wq=wq, bias=bias, scale_mode=mode, out=big[:, :N], dev_status=st)
+    assert mx.launch_count() == n0 + 1
+    torch.cuda.synchronize()
+    assert int(st.item()) == 0
+    assert torch.equal(y, want) and (big[:, N:] == 7.0).all()
+    assert torch.equal(ctx.xq.data, want_q.data) and torch.equal(ctx.xq.scales, want_q.scales)
+
+
+def test_nonfinite_groups_and_a_scale_rule_that_does_not_exist(mx):
+    x = torch.ones((40, 128), device="cuda", dtype=torch.bfloat16)
+    x[3, 40], x[17, 5] = float("nan"), float("inf")
+    wq = mx.quantize(torch.ones((256, 128), device="cuda", dtype=torch.bfloat16))
+    st = mx.new_status()
+    y, ctx = mx.linear_fwd(x, wq=wq, dev_status=st)
+    want = mx.quantize(x)
+    torch.cuda.synchronize()
+    assert int(st.item()) == mx.DEV_NONFINITE
+    assert torch.equal(ctx.xq.data, want.data) and torch.equal(ctx.xq.scales, want.scales)
+    bad = torch.isnan(y).any(dim=1).nonzero().flatten().tolist()
+    assert bad == [3, 17] and torch.isnan(y[bad]).all()
+    n0 = mx.launch_count()
+    with pytest.raises(RuntimeError, match="INVALID_ARG"):
+        mx.linear_fwd(x, wq=wq, scale_mode=5)
+    assert mx.launch_count() == n0
+
+
+def test_two_launches_in_a_graph(mx):
+    x = torch.randn((197, 384), device="cuda").to(torch.bfloat16)
+    wq = mx.quantize(torch.randn((1536, 384), device="cuda").to(torch.bfloat16))
+    y, ctx = mx.linear_fwd(x, wq=wq)
+    torch.cuda.synchronize()
+    n0 = mx.launch_count()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        y2, ctx2 = mx.linear_fwd(x, wq=wq)
+    assert mx.launch_count() == n0 + 2
+    graph.replay()
+    torch.cuda.synchronize()
+    assert torch.equal(y2, y) and torch.equal(ctx2.xq.data, ctx.xq.data) and torch.equal(ctx2.xq.scales, ctx.xq.scales)
