@@ -2445,74 +2445,57 @@ k_gemm_mxf4_pbs(const __grid_constant__ CUtensorMap map_a, const __grid_constant
 // SMs without a block and each with a long chain of loads (products with their reductions, back to back: 96 x 288 x 401408
 // 32.5 -> 24.9 us, 128 x 128 x 50432 9.0 -> 7.9, both with the higher limit on the splits), one where the output fills the
 // machine (384 x 384 x 25216: 11.8 us, 12.9 with eight).
-// With one thread per output each takes two of them, so that a 2304 x 768 gradient with four partials is one round of blocks instead of one
-// and a half, and indices are 32-bit: in a step the sum takes 6.5 -> 4.7 us there, 9.1 -> 8.1 behind a large input gradient, 3.5 -> 2.9 for
-// 384 x 96 x 401408 with eight.
 template <int GROUPS>
 __global__ void __launch_bounds__(256) k_splitk_reduce(const float *part, int splits, int64_t M, int64_t N,
                                                        void *__restrict__ d, int64_t ldd, int out_fp32,
                                                        const __nv_bfloat16 *bias)
 {
-    constexpr int kCols = 256 / GROUPS, kPer = GROUPS == 1 ? 2 : 1, kFlight = 8 / kPer;
+    constexpr int kCols = 256 / GROUPS;
     __shared__ float4 s_sum[GROUPS][kCols];
     pdl_launch_dependents();
     pdl_wait();
-    const uint32_t n4 = (uint32_t)(N / 4), total4 = (uint32_t)M * n4;   // K is split where the output has few tiles: far below 2^32
+    const int64_t total4 = M * N / 4;
     const int c = threadIdx.x % kCols, g = threadIdx.x / kCols;
-    const float4 *const part4 = reinterpret_cast<const float4 *>(part);
-    for (uint32_t i0 = blockIdx.x * (uint32_t)(kCols * kPer); i0 < total4; i0 += gridDim.x * (uint32_t)(kCols * kPer)) {
-        float4 acc[kPer];
+    for (int64_t i0 = blockIdx.x * (int64_t)kCols; i0 < total4; i0 += (int64_t)gridDim.x * kCols) {
+        const int64_t i = i0 + c, e = i * 4, row = e / N, col = e - row * N;
+        float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (i < total4 && g < splits) {
+            acc = *reinterpret_cast<const float4 *>(part + (size_t)g * M * N + e);
+            for (int s = g + GROUPS; s < splits; s += 8 * GROUPS) {      // eight loads in flight
+                float4 v[8];
 #pragma unroll
-        for (int u = 0; u < kPer; u++) {
-            const uint32_t i = i0 + u * kCols + c;
-            acc[u] = i < total4 && g < splits ? part4[(size_t)g * total4 + i] : make_float4(0.f, 0.f, 0.f, 0.f);
-        }
-        for (int s = g + GROUPS; s < splits; s += kFlight * GROUPS) {      // eight loads in flight
-            float4 v[kPer][kFlight];
+                for (int j = 0; j < 8; j++)
+                    if (s + j * GROUPS < splits) v[j] = *reinterpret_cast<const float4 *>(part + (size_t)(s + j * GROUPS) * M * N + e);
 #pragma unroll
-            for (int u = 0; u < kPer; u++)
-#pragma unroll
-                for (int j = 0; j < kFlight; j++)
-                    if (s + j * GROUPS < splits && i0 + u * kCols + c < total4) v[u][j] = part4[(size_t)(s + j * GROUPS) * total4 + i0 + u * kCols + c];
-#pragma unroll
-            for (int u = 0; u < kPer; u++)
-#pragma unroll
-                for (int j = 0; j < kFlight; j++)
-                    if (s + j * GROUPS < splits && i0 + u * kCols + c < total4)
-                        acc[u].x += v[u][j].x, acc[u].y += v[u][j].y, acc[u].z += v[u][j].z, acc[u].w += v[u][j].w;
+                for (int j = 0; j < 8; j++)
+                    if (s + j * GROUPS < splits) acc.x += v[j].x, acc.y += v[j].y, acc.z += v[j].z, acc.w += v[j].w;
+            }
         }
         if (GROUPS > 1) {
-            s_sum[g][c] = acc[0];
+            s_sum[g][c] = acc;
             __syncthreads();
             if (g == 0) {
 #pragma unroll
                 for (int q = 1; q < GROUPS; q++) {
                     const float4 v = s_sum[q][c];
-                    acc[0].x += v.x; acc[0].y += v.y; acc[0].z += v.z; acc[0].w += v.w;
+                    acc.x += v.x; acc.y += v.y; acc.z += v.z; acc.w += v.w;
                 }
             }
             __syncthreads();
         }
-        if (g != 0) continue;
-#pragma unroll
-        for (int u = 0; u < kPer; u++) {
-            const uint32_t i = i0 + u * kCols + c;
-            if (i >= total4) continue;
-            const int64_t row = i / n4, col = (int64_t)(i % n4) * 4;
-            float4 o4 = acc[u];
-            if (bias) {
-                o4.x += __bfloat162float(bias[col]); o4.y += __bfloat162float(bias[col + 1]);
-                o4.z += __bfloat162float(bias[col + 2]); o4.w += __bfloat162float(bias[col + 3]);
-            }
-            if (out_fp32) {
-                *reinterpret_cast<float4 *>(static_cast<float *>(d) + row * ldd + col) = o4;
-            } else {
-                __nv_bfloat162 lo = __floats2bfloat162_rn(o4.x, o4.y), hi = __floats2bfloat162_rn(o4.z, o4.w);
-                uint2 o;
-                o.x = *reinterpret_cast<uint32_t *>(&lo);
-                o.y = *reinterpret_cast<uint32_t *>(&hi);
-                *reinterpret_cast<uint2 *>(static_cast<__nv_bfloat16 *>(d) + row * ldd + col) = o;
-            }
+        if (g != 0 || i >= total4) continue;
+        if (bias) {
+            acc.x += __bfloat162float(bias[col]); acc.y += __bfloat162float(bias[col + 1]);
+            acc.z += __bfloat162float(bias[col + 2]); acc.w += __bfloat162float(bias[col + 3]);
+        }
+        if (out_fp32) {
+            *reinterpret_cast<float4 *>(static_cast<float *>(d) + row * ldd + col) = acc;
+        } else {
+            __nv_bfloat162 lo = __floats2bfloat162_rn(acc.x, acc.y), hi = __floats2bfloat162_rn(acc.z, acc.w);
+            uint2 o;
+            o.x = *reinterpret_cast<uint32_t *>(&lo);
+            o.y = *reinterpret_cast<uint32_t *>(&hi);
+            *reinterpret_cast<uint2 *>(static_cast<__nv_bfloat16 *>(d) + row * ldd + col) = o;
         }
     }
 }
@@ -2858,7 +2841,7 @@ static mxfp4_status_t launch_splitk_reduce(const GemmPlan &g, const void *worksp
                                            const void *bias, int sms, cudaStream_t st)
 {
     const int groups = g.splits >= 8 && M * N / 4 < 64 * 256 ? 8 : 1;   // fewer than 64 blocks otherwise
-    const int64_t nb4 = ceil_div(M * N / 4, groups == 8 ? 32 : 512);
+    const int64_t nb4 = ceil_div(M * N / 4, 256 / groups);
     const unsigned blocks = (unsigned)(nb4 < (int64_t)sms * 8 ? nb4 : (int64_t)sms * 8);
     MX_CHECK_CUDA(launch_pdl(groups == 8 ? k_splitk_reduce<8> : k_splitk_reduce<1>, blocks, 1, 256, 0, st, static_cast<const float *>(workspace),
                              g.splits, M, N, d, ldd, (int)(out_dtype == MXFP4_OUT_FP32), static_cast<const __nv_bfloat16 *>(bias)));
