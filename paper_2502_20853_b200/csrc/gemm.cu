@@ -2880,16 +2880,16 @@ static mxfp4_status_t gemm_impl(mxfp4_mat_t a, mxfp4_mat_t b, void *d, int64_t l
 }
 
 // The CTAs that share the quantization of a row block, for a forward pass in one launch; 0: not in one launch.  All tiles on the SMs at once,
-// a contraction of two K tiles, at most three groups of X per thread (a chain of loads), and not while a graph is captured: replayed, a
+// a contraction of at most 384, at most three groups of X per thread (a chain of loads), and not while a graph is captured: replayed, a
 // second launch costs nothing, and the two kernels are the faster ones on the device.  Two launches / one, in us, eager calls in a row:
-// 197 x 1536 x 384 12.8 / 10.1; from the call to its synchronized result: 21.7 / 20.7 there, 21.2 / 18.3 at 2000 x 768 x 256, but 17.5 / 19.5 at
-// 32 x 768 x 768 and 18.4 / 24.0 at 128 x 4096 x 1024; replayed 5.2 / 7.2.  Clusters of three or four: 7.2 and 7.6 us of device time at 197 x 1536 x 384,
+// 197 x 1536 x 384 12.8 / 10.1; from the call to its synchronized result: 21.7 / 20.7 there, 21.2 / 18.3 at 2000 x 768 x 256, but 18.1 / 19.2 at
+// 33 x 1280 x 416, 18.4 / 21.9 at 128 x 1024 x 512 and 17.5 / 19.5 at 32 x 768 x 768; replayed 5.2 / 7.2.  Clusters of three or four: 7.2 and 7.6 us of device time at 197 x 1536 x 384,
 // 8.4 with one CTA, 7.7 with six.  They do not fit everywhere on a full machine (four whole SMs each: room for 33), and a second wave
 // costs more than they save.
 static int x_cluster(int64_t m, int64_t n, int64_t kc, int sms)
 {
     const int64_t tiles_n = ceil_div(n, 128), tiles = ceil_div(m, kBM) * tiles_n;
-    if (m <= 0 || n <= 0 || kc <= 0 || kc > kXMaxKt * kBKElems || tiles > sms) return 0;
+    if (m <= 0 || n <= 0 || kc <= 0 || kc > 384 || tiles > sms) return 0;
     int c = tiles <= 112 ? 4 : 2;
     while (tiles_n % c) c--;
     return kBM * ceil_div(kc, 128) * 4 <= 3 * kXQuantThreads * c ? c : 0;
