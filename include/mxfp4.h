@@ -350,7 +350,8 @@ mxfp4_status_t mxfp4_change_sums_q(mxfp4_mat_t cur, mxfp4_mat_t prev, double *ou
  * If w_bf16 != NULL, ctx->wq_t.data != NULL and N % 32 == 0, Q4 = Q(deq(Q2(W))^T; stochastic, seed ctx->wq_t_seed,
  * stream 4) is written into ctx->wq_t in the same way.
  * The forward pass takes no workspace: its product never splits the contraction (for a small M with a very long
- * K, mxfp4_gemm with a workspace has more parallelism).  All arguments are checked before the first launch. */
+ * K, mxfp4_gemm with a workspace has more parallelism).  All arguments are checked before the first launch.
+ * y may lie over x in any way: all of x is read before anything of y is written. */
 mxfp4_status_t mxfp4_linear_fwd(const void *x_bf16, int64_t ldx, int64_t m, int64_t k,
                                 const void *w_bf16, int64_t n, const void *bias_bf16, void *y_bf16,
                                 int64_t ldy, mxfp4_linear_ctx_t *ctx, int32_t scale_mode,

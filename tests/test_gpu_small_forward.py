@@ -40,6 +40,26 @@ def test_forward_in_one_launch(mx, M, N, K, form):
     assert torch.equal(ctx.xq.data, want_q.data) and torch.equal(ctx.xq.scales, want_q.scales)
 
 
+# Y in the memory of X: as its first columns, at the same address row by row, shifted by rows, and with as many columns; the last three:
+# neighbours that share nothing (one launch; the columns beside X lie between its first and last bytes and count as shared)
+@pytest.mark.parametrize("M,N,K,x_at,ldx,y_at,ldy,launches", [
+    (197, 1536, 384, 0, 1536, 0, 1536, 2), (197, 1536, 384, 0, 384, 0, 1536, 2), (300, 640, 256, 128 * 256, 256, 0, 640, 2), (160, 160, 160, 0, 160, 0, 160, 2),
+    (33, 256, 256, 32 * 256 + 248, 256, 0, 256, 2), (197, 1152, 384, 0, 1536, 384, 1536, 2), (197, 1536, 384, 0, 384, 197 * 384, 1536, 1),
+    (33, 256, 256, 33 * 256, 256, 0, 256, 1), (33, 256, 96, 32 * 264 + 256, 96, 0, 264, 1)])
+def test_y_over_x(mx, M, N, K, x_at, ldx, y_at, ldy, launches):
+    g = torch.Generator(device="cuda").manual_seed(M + N)
+    size = max(x_at + (M - 1) * ldx + K, y_at + (M - 1) * ldy + N)
+    buf = torch.randn(size, generator=g, device="cuda").to(torch.bfloat16)
+    x, out = buf.as_strided((M, K), (ldx, 1), x_at), buf.as_strided((M, N), (ldy, 1), y_at)
+    wq = mx.quantize((torch.randn((N, K), generator=g, device="cuda") * 0.02).to(torch.bfloat16))
+    want, want_ctx = mx.linear_fwd(x.clone(), wq=wq)
+    n0 = mx.launch_count()
+    y, ctx = mx.linear_fwd(x, wq=wq, out=out)
+    assert mx.launch_count() == n0 + launches
+    assert torch.equal(y, want)
+    assert torch.equal(ctx.xq.data, want_ctx.xq.data) and torch.equal(ctx.xq.scales, want_ctx.xq.scales)
+
+
 def test_nonfinite_groups_and_a_scale_rule_that_does_not_exist(mx):
     x = torch.ones((40, 128), device="cuda", dtype=torch.bfloat16)
     x[3, 40], x[17, 5] = float("nan"), float("inf")
