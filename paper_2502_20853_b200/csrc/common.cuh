@@ -31,6 +31,14 @@ extern std::atomic<unsigned long long> g_launches;
         MX_LAUNCHED();                          \
     } while (0)
 
+// The memory of an operand, from its first byte to behind its last (between the columns of a strided matrix too).
+struct Span {
+    uintptr_t lo, hi;
+};
+inline Span span_of(const void *p, int64_t bytes) { return {reinterpret_cast<uintptr_t>(p), reinterpret_cast<uintptr_t>(p) + (uintptr_t)bytes}; }
+inline Span span_of_bf16(const void *p, int64_t ld, int64_t rows, int64_t cols) { return span_of(p, p ? 2 * ((rows - 1) * ld + cols) : 0); }
+inline bool meet(const Span &a, const Span &b) { return a.lo < b.hi && b.lo < a.hi; }
+
 // Every kernel of the step is launched with programmatic stream serialization: its blocks may be placed and set up while the
 // kernel before it drains, and wait for it (all of its blocks done, their memory visible) before they touch global memory.
 // Each block calls pdl_wait() before its first access to global memory: a kernel whose blocks could end without having waited

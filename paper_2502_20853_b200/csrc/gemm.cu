@@ -3144,6 +3144,19 @@ static bool two_groups(const mxfp4_epilogue_t *epi, int64_t M, int64_t N, int64_
     return tiles <= 2 && ceil_div(M, kBM) * ceil_div(N, 128) > sm_count() && Kc <= (identity ? 2 : 4) * kBKElems;
 }
 
+// Whether what the quantization writes lies in memory that the product reads.
+static bool over_operands(const mxfp4_epilogue_t *epi, const mxfp4_mat_t &a, const mxfp4_mat_t &b, const void *bias)
+{
+    const auto codes = [](const mxfp4_mat_t &q) { return span_of(q.data, q.data ? q.rows * (q.cols / 2) : 0); };
+    const auto scales = [](const mxfp4_mat_t &q) { return span_of(q.scales, q.data ? (int64_t)mxfp4_scale_bytes(q.rows, q.cols) : 0); };
+    const Span in[] = {codes(a), scales(a), codes(b), scales(b), span_of_bf16(bias, 0, 1, b.rows)};
+    const Span out[] = {codes(epi->zq), scales(epi->zq), codes(epi->zq_t), scales(epi->zq_t), span_of_bf16(epi->z_bf16, epi->ldz, a.rows, b.rows)};
+    for (const Span &i : in)
+        for (const Span &o : out)
+            if (meet(i, o)) return true;
+    return false;
+}
+
 // Whether the product and the quantization run as two kernels: when the epilogue is GELU with the double-quantization chain,
 // Y is stored anyway, and there are many 128 x 128 tiles per SM.  The fused epilogue's passes are the bottleneck; the two kernels read
 // Y back (2 of 5 bytes per element more) but run at the product's and the tile quantizer's own rates.  With one group of epilogue
@@ -3151,10 +3164,12 @@ static bool two_groups(const mxfp4_epilogue_t *epi, int64_t M, int64_t N, int64_
 // 33.6 / 31.7 at 8192 x 1536 x 384 (5.2 tiles per SM), but 20.6 / 22.5 at 4096 x 1536 x 384 (2.6) and 12.3 / 15.3 at 1024 x 768 x 192,
 // where a second launch costs more.  With two groups (back to back) it lies at about twelve: 25.3 / 26.9 at 8192 x 1536 x 384, 30.1 / 32.9 at
 // 16384 x 1024 x 256 (6.9 tiles per SM), 62.0 / 61.0 at 25216 x 1536 x 384 (16), 320 / 309 at 50432 x 4096 x 1024, 235 / 225 at 401408 x 384 x 96.
-static bool two_pass(const mxfp4_epilogue_t *epi, int64_t M, int64_t N, int64_t Kc)
+// Outputs of the quantization in the operands' memory are in time behind a product of its own: from four tiles per SM on they get one.
+static bool two_pass(const mxfp4_epilogue_t *epi, const mxfp4_mat_t &a, const mxfp4_mat_t &b, const void *bias)
 {
-    return epi->hook == MXFP4_HOOK_GELU && epi->chain && epi->y_bf16 && epi->y_bf16 != epi->z_bf16 &&
-           ceil_div(M, kBM) * ceil_div(N, 128) >= (two_groups(epi, M, N, Kc) ? 12 : 4) * (int64_t)sm_count();
+    const int64_t tiles = ceil_div(a.rows, kBM) * ceil_div(b.rows, 128), sms = sm_count();
+    return epi->hook == MXFP4_HOOK_GELU && epi->chain && epi->y_bf16 && epi->y_bf16 != epi->z_bf16 && tiles >= 4 * sms &&
+           (tiles >= 12 * sms || !two_groups(epi, a.rows, b.rows, a.cols) || over_operands(epi, a, b, bias));
 }
 
 mxfp4_status_t gemm_quant(mxfp4_mat_t a, mxfp4_mat_t b, const void *bias, const mxfp4_epilogue_t *epi, uint32_t *dev_status, cudaStream_t st)
@@ -3164,7 +3179,7 @@ mxfp4_status_t gemm_quant(mxfp4_mat_t a, mxfp4_mat_t b, const void *bias, const 
     const int64_t M = a.rows, N = b.rows, Kc = a.cols;
     if (M == 0 || N == 0) return MXFP4_OK;
     const bool row = epi->zq.data != nullptr, tr = epi->zq_t.data != nullptr;
-    if (two_pass(epi, M, N, Kc)) {
+    if (two_pass(epi, a, b, bias)) {
         // Y by the product's own kernels (the contraction is not split), then the tile quantizer reads it back
         mxfp4_status_t s = gemm(a, b, epi->y_bf16, epi->ldy, MXFP4_OUT_BF16, bias, nullptr, 0, dev_status, st, false);
         if (s) return s;

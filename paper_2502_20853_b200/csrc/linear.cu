@@ -24,13 +24,6 @@ size_t gemm_two_workspace_bytes(int64_t m1, int64_t kc1, int64_t m2, int64_t kc2
 mxfp4_status_t gemm_quant_check(mxfp4_mat_t a, mxfp4_mat_t b, const void *bias, const mxfp4_epilogue_t *epi);
 mxfp4_status_t gemm_quant(mxfp4_mat_t a, mxfp4_mat_t b, const void *bias, const mxfp4_epilogue_t *epi, uint32_t *dev_status, cudaStream_t st);
 
-// Whether two bf16 matrices share bytes, or might: what lies between their first and last elements is compared.
-static bool overlap(const void *a, int64_t lda, int64_t rows_a, int64_t cols_a, const void *b, int64_t ldb, int64_t rows_b, int64_t cols_b)
-{
-    const uintptr_t a0 = reinterpret_cast<uintptr_t>(a), b0 = reinterpret_cast<uintptr_t>(b);
-    return a0 < b0 + 2 * (uintptr_t)((rows_b - 1) * ldb + cols_b) && b0 < a0 + 2 * (uintptr_t)((rows_a - 1) * lda + cols_a);
-}
-
 static size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
 
 struct BwdLayout {
@@ -106,7 +99,8 @@ mxfp4_status_t mxfp4_linear_fwd_ex(const void *x_bf16, int64_t ldx, int64_t m, i
     const bool make_q6 = x_bf16 && ctx->xq_t.data;
     // a small batch on a weight that is quantized already: one launch, unless Y may lie over X (its blocks would write Y while others
     // still read X; two launches have read all of X first)
-    if (x_bf16 && !make_q6 && !w_bf16 && !epi && gemm_from_x_fits(m, n, k, st) && !overlap(x_bf16, ldx, m, k, y_bf16, ldy, m, n)) {
+    if (x_bf16 && !make_q6 && !w_bf16 && !epi && gemm_from_x_fits(m, n, k, st) &&
+        !meet(span_of_bf16(x_bf16, ldx, m, k), span_of_bf16(y_bf16, ldy, m, n))) {
         if (scale_mode != MXFP4_SCALE_TRUNCATION_FREE && scale_mode != MXFP4_SCALE_FLOOR) return MXFP4_INVALID_ARG;
         return gemm_from_x(x_bf16, ldx, ctx->xq, ctx->wq, y_bf16, ldy, bias_bf16, scale_mode, dev_status, st, kWaitSpinLimit, 0);
     }

@@ -187,6 +187,23 @@ def test_quantizing_epilogue_equals_the_standalone_quantizers(mx):
         assert torch.equal(epi.zq_t.data, qt.data) and torch.equal(epi.zq_t.scales, qt.scales)
 
 
+def test_gelu_chain_over_its_operands(mx):
+    """Between four and twelve tiles per SM, where one kernel does it all, codes written over the product's operands still wait for
+    all of the product: two kernels, and the results of buffers of their own."""
+    M, N = 128 * 148, 512
+    _, a, b = operands(mx, M, N, N, 12)
+    bufs = [mx.QMat(M, N), mx.QMat(N, M)]
+    ys = [torch.empty((M, N), dtype=torch.bfloat16, device="cuda") for _ in range(2)]
+    for y, zq, launches in ((ys[0], bufs[0], 1), (ys[1], a, 2)):
+        n0 = mx.launch_count()
+        mx.gemm_quant(a, b, mx.Epilogue(hook=mx.HOOK_GELU, y=y, zq=zq, zq_t=bufs[1], qp_t=(0, 1, 5, 6), chain=True))
+        assert mx.launch_count() == n0 + launches
+        if launches == 1:
+            want_t = bufs[1].data.clone()
+    assert torch.equal(ys[0], ys[1])
+    assert torch.equal(a.data, bufs[0].data) and torch.equal(a.scales_linear(), bufs[0].scales_linear()) and torch.equal(bufs[1].data, want_t)
+
+
 # more tiles than SMs and a short contraction: two groups of epilogue warps.  298 tiles (two blocks have a third), 171 (23 blocks
 # have a second), 225, all with ragged last tiles; contractions of one, two and four K tiles
 @pytest.mark.parametrize("M,N,K", [(18976, 160, 96), (2400, 1056, 384), (9504, 288, 1024)])
