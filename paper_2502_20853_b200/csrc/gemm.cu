@@ -3130,18 +3130,34 @@ mxfp4_status_t gemm_quant_check(mxfp4_mat_t a, mxfp4_mat_t b, const void *bias, 
 mxfp4_status_t quantize_gelu_chain(const void *y_bf16, int64_t rows, int64_t cols, int64_t ldy, void *z_bf16, int64_t ldz, mxfp4_mat_t dst,
                                    const mxfp4_qparams_t *qp_row, mxfp4_mat_t dst_t, const mxfp4_qparams_t *qp_t, uint32_t *dev_status, cudaStream_t st);
 
-// Whether two groups of epilogue warps take the tiles in turn.  The epilogue is bound by the instructions it issues, and eight warps
+// Whether two groups of epilogue warps take the tiles in turn.  Where the epilogue is bound by the instructions it issues, eight warps
 // with their waits for the accumulator and for one another do not fill the SM.  The second group's tiles and staging cost the ring two
-// of its four stages, so the contraction has to be short, and shorter where the epilogue is (no hook); they have to fit (GemmQCfg); and
-// a block needs a second tile.  One group / two, back to back, in us, multiply with Q3 + Q5: 25216 x 1536 x 384 52.9 / 47.5,
-// 50432 x 4096 x 1024 264 / 248, 401408 x 384 x 96 197 / 177, 2048 x 1536 x 384 (1.3 tiles per SM) 9.8 / 9.6, but 1024 x 768 x 192 6.5 / 7.0
-// and 8192 x 4096 x 2048 54 / 80; identity with Z kept: 25216 x 1536 x 384 50.2 / 45.7, 16384 x 1024 x 256 22.4 / 22.3, 50432 x 4096 x 1024
-// 249 / 269; GELU and the chain with Y kept: 4096 x 1536 x 384 16.2 / 15.6.
+// of its four stages, so the contraction has to be short, and the shorter the less the epilogue does; the groups have to fit (GemmQCfg),
+// and a block needs a second tile.  K tiles of 256 up to which two groups are taken, with one group / two, back to back, in us:
+//   GELU: 4.  Chain and Y 25216 x 1536 x 384 72.0 / 60.0, x 1024 75.6 / 64.1, 2400 x 1024 x 1024 12.0 / 11.8; 3 where Y or Z is stored and at
+//     most one pass is made: Y and a row pass 25216 x 1536 x 768 50.2 / 46.0, x 1024 51.5 / 54.7, Z alone x 1024 46.9 / 49.1.
+//   Multiply: 2, as the second factor is loaded too.  A nearest row pass 25216 x 1536 x 512 32.6 / 28.9, x 768 34.2 / 39.4; Z alone
+//     49.4 / 36.6, x 1024 49.3 / 55.2.  With both passes stochastic 3 from four tiles per SM on: 25216 x 1536 x 768 51.9 / 46.8,
+//     6272 x 1536 x 768 (4.0 per SM) 15.5 / 14.7, 3136 x 2048 x 768 (2.7) 12.5 / 12.6; without Z and from 3072 columns on, where the SMs share
+//     more of the rows that they read, 4: 50432 x 4096 x 1024 273 / 256, 50432 x 3072 x 1024 198 / 187, 50432 x 1536 x 1024 100.3 / 101.1,
+//     50432 x 768 x 1024 53.6 / 55.6.  With the chain, whose passes are the longest, 4: 25216 x 1536 x 1024 107 / 101.
+//   Identity: 2.  Q3 + Q5 25216 x 1536 x 512 47.9 / 42.9, a nearest row pass 26.7 / 21.9 (x 768 27.7 / 28.4).  None where Z is stored and at
+//     most one pass is made, the stores being the bound: 25216 x 1536 x 384 29.0 / 31.6.
+// Beyond: multiply with Q3 + Q5 8192 x 4096 x 2048 54 / 80.  No second tile: 1024 x 768 x 192 6.5 / 7.0.
 static bool two_groups(const mxfp4_epilogue_t *epi, int64_t M, int64_t N, int64_t Kc)
 {
     const bool identity = epi->hook == MXFP4_HOOK_IDENTITY, y = epi->y_bf16 && !(identity && !epi->z_bf16), z = epi->z_bf16 || (identity && epi->y_bf16);
-    const int tiles = 1 + (epi->hook == MXFP4_HOOK_MULTIPLY && !epi->chain) + (epi->chain && z) + y;
-    return tiles <= 2 && ceil_div(M, kBM) * ceil_div(N, 128) > sm_count() && Kc <= (identity ? 2 : 4) * kBKElems;
+    const int smem_tiles = 1 + (epi->hook == MXFP4_HOOK_MULTIPLY && !epi->chain) + (epi->chain && z) + y;
+    const int64_t tiles = ceil_div(M, kBM) * ceil_div(N, 128), sms = sm_count();
+    if (smem_tiles > 2 || tiles <= sms) return false;
+    const bool stored = y || z, row = epi->zq.data != nullptr, tr = epi->zq_t.data != nullptr;
+    const bool stochastic = row && tr && epi->qp_row.rounding == MXFP4_ROUND_STOCHASTIC && epi->qp_t.rounding == MXFP4_ROUND_STOCHASTIC;
+    int kt;
+    if (epi->hook == MXFP4_HOOK_GELU) kt = (row && tr) || !stored ? 4 : 3;
+    else if (identity) kt = (row && tr) || !stored ? 2 : 0;
+    else if (epi->chain) kt = 4;
+    else kt = !stochastic || tiles < 4 * sms ? 2 : stored || N < 3072 ? 3 : 4;
+    return Kc <= kt * kBKElems;
 }
 
 // Whether what the quantization writes lies in memory that the product reads.
@@ -3162,8 +3178,9 @@ static bool over_operands(const mxfp4_epilogue_t *epi, const mxfp4_mat_t &a, con
 // Y back (2 of 5 bytes per element more) but run at the product's and the tile quantizer's own rates.  With one group of epilogue
 // warps the line lies at four tiles per SM: fused / two kernels 84 / 64.2 us at 25216 x 1536 x 384, 396 / 307 at 50432 x 4096 x 1024,
 // 33.6 / 31.7 at 8192 x 1536 x 384 (5.2 tiles per SM), but 20.6 / 22.5 at 4096 x 1536 x 384 (2.6) and 12.3 / 15.3 at 1024 x 768 x 192,
-// where a second launch costs more.  With two groups (back to back) it lies at about twelve: 25.3 / 26.9 at 8192 x 1536 x 384, 30.1 / 32.9 at
-// 16384 x 1024 x 256 (6.9 tiles per SM), 62.0 / 61.0 at 25216 x 1536 x 384 (16), 320 / 309 at 50432 x 4096 x 1024, 235 / 225 at 401408 x 384 x 96.
+// where a second launch costs more.  With two groups the two ways are within 2 % of each other from eight to sixteen tiles per SM, at all
+// contractions up to 1024, and the line is in the middle (back to back): 24.5 / 27.6 at 9472 x 1536 x 384 (6.0 tiles per SM), 35.3 / 35.3 at 12672
+// (8.0), 45.9 / 47.2 at 18944 (12.0), 60.2 / 60.0 at 25216 (16), 91.8 / 88.9 at 38016 (24); x 1024 49.8 / 50.9 (12.0) and 94.5 / 94.2 (24).
 // Outputs of the quantization in the operands' memory are in time behind a product of its own: from four tiles per SM on they get one.
 static bool two_pass(const mxfp4_epilogue_t *epi, const mxfp4_mat_t &a, const mxfp4_mat_t &b, const void *bias)
 {

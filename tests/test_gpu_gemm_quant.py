@@ -205,15 +205,16 @@ def test_gelu_chain_over_its_operands(mx):
 
 
 # more tiles than SMs and a short contraction: two groups of epilogue warps.  298 tiles (two blocks have a third), 171 (23 blocks
-# have a second), 225, all with ragged last tiles; contractions of one, two and four K tiles
-@pytest.mark.parametrize("M,N,K", [(18976, 160, 96), (2400, 1056, 384), (9504, 288, 1024)])
+# have a second), 225, 600, 625, all with ragged last tiles; contractions of one to four K tiles (multiply: with three from 592 tiles
+# on, with four from 3072 columns on; 225 tiles are one group's there)
+@pytest.mark.parametrize("M,N,K", [(18976, 160, 96), (2400, 1056, 384), (9504, 288, 1024), (12768, 736, 704), (3168, 3104, 992)])
 @pytest.mark.parametrize("hook", ["gelu", "multiply"])
 def test_two_groups_of_epilogue_warps(mx, M, N, K, hook):
     _, a, b = operands(mx, M, N, K, M + N + K)
     g = torch.Generator(device="cuda").manual_seed(M)
     aux = torch.randn((M, N), generator=g, device="cuda").to(torch.bfloat16)
     bias = torch.randn(N, generator=g, device="cuda").to(torch.bfloat16)
-    # Y and Z in pieces that have no more tiles than SMs (one group; held against the oracle above): the same bits
+    # Y and Z in pieces, chained and both kept: always one group (held against the oracle above).  The same bits
     y, z = (torch.empty((M, N), dtype=torch.bfloat16, device="cuda") for _ in range(2))
     for r in range(0, M, 1280):
         rows = slice(r, min(r + 1280, M))
