@@ -2879,19 +2879,24 @@ static mxfp4_status_t gemm_impl(mxfp4_mat_t a, mxfp4_mat_t b, void *d, int64_t l
     return launch_splitk_reduce(g, workspace, M, N, d, ldd, out_dtype, bias, sms, st);
 }
 
-// The CTAs that share the quantization of a row block, for a forward pass in one launch; 0: not in one launch.  All tiles on the SMs at once,
-// a contraction of at most 384, at most three groups of X per thread (a chain of loads), and not while a graph is captured: replayed, a
-// second launch costs nothing, and the two kernels are the faster ones on the device.  Two launches / one, in us, eager calls in a row:
-// 197 x 1536 x 384 12.8 / 10.1; from the call to its synchronized result: 21.7 / 20.7 there, 21.2 / 18.3 at 2000 x 768 x 256, but 18.1 / 19.2 at
-// 33 x 1280 x 416, 18.4 / 21.9 at 128 x 1024 x 512 and 17.5 / 19.5 at 32 x 768 x 768; replayed 5.2 / 7.2.  Clusters of three or four: 7.2 and 7.6 us of device time at 197 x 1536 x 384,
-// 8.4 with one CTA, 7.7 with six.  They do not fit everywhere on a full machine (four whole SMs each: room for 33), and a second wave
-// costs more than they save.
+// The CTAs that share the quantization of a row block, for a forward pass in one launch; 0: not in one launch.  What one launch saves is
+// host time, so it is for eager calls: in a row 13.0-13.3 us with two launches, 10.4 with one, at all sizes here.  The kernel itself is
+// slower than the two it replaces, and a graph takes those two.  Two launches / one, from the call to its synchronized result and (device
+// time) of calls that queue behind other work, in us, clusters of c:
+//   197 x 1536 x 384 22.6 / 23.0 (5.8 / 7.2) c = 3, 23.5 (7.6) c = 4, 23.5 (7.7) c = 2, 24.4 (8.5) c = 1
+//   1 x 1536 x 384 22.1 / 21.6 (5.0 / 5.6) c = 3, 22.8 (6.9) c = 1;  128 x 1024 x 384 22.5 / 23.5 (5.8 / 7.6) c = 2
+//   197 x 1152 x 256 22.2 / 21.8 (5.3 / 6.0) c = 3;  300 x 640 x 256 22.2 / 22.6 (5.4 / 6.8) c = 1, x 128 21.5 (5.3 / 5.6)
+//   3136 x 384 x 96 22.7 / 21.4 (5.9 / 5.4) c = 3
+// Beyond: 197 x 1536 x 448 22.7 / 23.6 (5.9 / 7.6), x 512 22.7 / 23.8 (5.8 / 7.8), both c = 3, 128 x 1024 x 512 22.6 / 24.3 (5.6 / 8.5) c = 2.  Taken while
+// a synchronized call loses no more than a microsecond: contractions of at most 384 and three groups of X per thread (a chain of loads).
+// Three CTAs share best.  Clusters of three fit on the GPU 45 at once (the SMs left over in its partitions make none): a second wave costs
+// 27.8 (11.7) instead of 23.1 (7.0) at 2048 x 1152 x 256 (144 tiles), so they are taken up to six sevenths of the SMs (126 tiles: 784 x 2304 x 384 23.4,
+// c = 2 23.9).  Pairs fit on all SMs.
 static int x_cluster(int64_t m, int64_t n, int64_t kc, int sms)
 {
     const int64_t tiles_n = ceil_div(n, 128), tiles = ceil_div(m, kBM) * tiles_n;
     if (m <= 0 || n <= 0 || kc <= 0 || kc > 384 || tiles > sms) return 0;
-    int c = tiles <= 112 ? 4 : 2;
-    while (tiles_n % c) c--;
+    const int c = tiles_n % 3 == 0 && 7 * tiles <= 6 * sms ? 3 : tiles_n % 2 == 0 ? 2 : 1;
     return kBM * ceil_div(kc, 128) * 4 <= 3 * kXQuantThreads * c ? c : 0;
 }
 bool gemm_from_x_fits(int64_t m, int64_t n, int64_t kc, cudaStream_t st)

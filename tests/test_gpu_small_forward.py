@@ -14,7 +14,7 @@ def mx():
 
 
 # one row to several row blocks, ragged everywhere; contractions of one group up to the longest, 384; column tiles that divide into
-# clusters of 1, 2, 3 and 4 CTAs, three of them in a grid too wide for clusters above two
+# clusters of 1, 2 and 3 CTAs, one of them in a grid too wide for clusters of three
 @pytest.mark.parametrize("M,N,K", [(1, 8, 32), (197, 1536, 384), (31, 384, 96), (128, 1000, 384), (129, 136, 160), (300, 640, 256), (64, 896, 224), (33, 1280, 352),
                                    (2048, 1152, 256), (1792, 1280, 64), (2300, 1024, 320)])
 @pytest.mark.parametrize("form", ["plain", "bias_strided_floor"])
@@ -38,6 +38,22 @@ def test_forward_in_one_launch(mx, M, N, K, form):
     assert int(st.item()) == 0
     assert torch.equal(y, want) and (big[:, N:] == 7.0).all()
     assert torch.equal(ctx.xq.data, want_q.data) and torch.equal(ctx.xq.scales, want_q.scales)
+
+
+# on either side of the lines: contractions of 384 and 416, 148 tiles and 149, two CTAs to share the groups of a row block of 384 and one,
+# clusters of three in a grid of 126 and pairs and single CTAs in wider ones
+@pytest.mark.parametrize("M,N,K,launches", [(40, 1280, 384, 1), (40, 1280, 416, 2), (18944, 96, 64, 1), (18945, 96, 64, 2), (64, 1280, 384, 1),
+                                            (64, 640, 384, 2), (64, 640, 256, 1), (1792, 1152, 384, 1), (1800, 1152, 384, 2), (1800, 1152, 224, 1), (1792, 1272, 384, 1)])
+def test_lines_of_one_launch(mx, M, N, K, launches):
+    g = torch.Generator(device="cuda").manual_seed(M + N + K)
+    x = torch.randn((M, K), generator=g, device="cuda").to(torch.bfloat16)
+    wq = mx.quantize((torch.randn((N, K), generator=g, device="cuda") * 0.02).to(torch.bfloat16))
+    want_q = mx.quantize(x)
+    want = mx.gemm(want_q, wq)
+    n0 = mx.launch_count()
+    y, ctx = mx.linear_fwd(x, wq=wq)
+    assert mx.launch_count() == n0 + launches
+    assert torch.equal(y, want) and torch.equal(ctx.xq.data, want_q.data) and torch.equal(ctx.xq.scales, want_q.scales)
 
 
 # Y in the memory of X: as its first columns, at the same address row by row, shifted by rows, and with as many columns; the last three:
