@@ -106,18 +106,23 @@ def test_quantizing_epilogue_gelu_with_bias_keeps_y(mx):
     assert_qmat_equal(epi.zq_t, pt, s_t, "Q6 of the next layer")
 
 
-@pytest.mark.parametrize("M,N,with_z", [(4128, 2336, True), (18944, 512, False), (18912, 512, False)])
-def test_gelu_chain_of_many_tiles(mx, M, N, with_z):
-    """From four tiles per SM on the product and the quantization behind GELU run as two kernels: sizes on both sides of that
-    line (592 and 591 tiles of the 592 on 148 SMs) and partial tiles, Y with a leading dimension of its own."""
-    K = 64
+# one kernel or two, by 128 x 128 tiles on 148 SMs.  Y and Z stored: two from four per SM on (627; 592 with ragged last tiles; 588: one).  Y
+# alone: two from twelve per SM on (1776, also ragged; 1764: one; 592: one), and from four on where the contraction is longer than 1024
+@pytest.mark.parametrize("M,N,K,with_z,launches", [
+    (4128, 2336, 64, True, 2), (18912, 480, 64, True, 2), (18784, 480, 64, True, 1), (18944, 512, 64, False, 1), (18912, 512, 64, False, 1),
+    (18944, 1536, 64, False, 2), (18912, 1504, 64, False, 2), (18784, 1504, 64, False, 1), (18912, 480, 1056, False, 2)])
+def test_gelu_chain_of_many_tiles(mx, M, N, K, with_z, launches):
+    """The product and the quantization behind GELU in one kernel or in two, which reads Y back: sizes on both sides of the lines
+    and partial tiles, Y with a leading dimension of its own."""
     ops, a, b = operands(mx, M, N, K, 11)
     big = torch.full((M, N + 16), 7.0, dtype=torch.bfloat16, device="cuda")
     y = big[:, :N]
     z = torch.empty((M, N), dtype=torch.bfloat16, device="cuda") if with_z else None
     epi = mx.Epilogue(hook=mx.HOOK_GELU, y=y, z=z, zq=mx.QMat(M, N), zq_t=mx.QMat(N, M), qp_t=(0, 1, 5, 6), chain=True)
     st = mx.new_status()
+    n0 = mx.launch_count()
     mx.gemm_quant(a, b, epi, dev_status=st)
+    assert mx.launch_count() == n0 + launches
     torch.cuda.synchronize()
     assert int(st.item()) == 0 and bool((big[:, N:] == 7.0).all())
     assert torch.equal(y, mx.gemm(a, b))
@@ -185,6 +190,41 @@ def test_quantizing_epilogue_equals_the_standalone_quantizers(mx):
             q, qt = mx.quantize_2axis(z, qp_row, qp_t)
         assert torch.equal(epi.zq.data, q.data) and torch.equal(epi.zq.scales, q.scales)
         assert torch.equal(epi.zq_t.data, qt.data) and torch.equal(epi.zq_t.scales, qt.scales)
+
+
+@pytest.mark.parametrize("M,N", [(384, 256), (6400, 384)])   # one group of epilogue warps, two (150 tiles)
+def test_multiply_by_any_bf16_value(mx, M, N):
+    """Z = bf16(Y * aux), exact before its one rounding, over all bf16 values of aux (subnormal ones, infinities, NaN) and Y over
+    many binades: products that are subnormal, tie at the smallest ones, vanish, overflow, or are no number."""
+    rng = np.random.default_rng(N)
+    c = rng.integers(0, 16, size=(M, 32)).astype(np.uint8)
+    unit = np.zeros((N, 32), np.uint8)
+    unit[np.arange(N), np.arange(N) % 32] = 2                       # 1.0: Y[m, n] = A[m, n % 32]
+    pack = lambda v: (v[:, 0::2] | (v[:, 1::2] << 4)).astype(np.uint8)  # noqa: E731
+    a = numpy_to_qmat(mx, pack(c), rng.integers(8, 247, size=(M, 1)).astype(np.uint8))
+    b = numpy_to_qmat(mx, pack(unit), np.full((N, 1), 127, np.uint8))
+    bits = rng.integers(0, 1 << 16, size=(M, N)).astype(np.int32)
+    bits[:, ::7] = rng.choice([0, 0x8000, 1, 0x8001, 0x7F, 0x80, 0x7F7F, 0xFF7F, 0x7F80, 0xFF80, 0x7FC0, 0xFF81], size=bits[:, ::7].shape)
+    aux = torch.from_numpy(bits.astype(np.uint16).view(np.int16)).view(torch.bfloat16).cuda()
+    y = mx.gemm(a, b)
+    z = torch.empty((M, N), dtype=torch.bfloat16, device="cuda")
+    epi = mx.Epilogue(hook=mx.HOOK_MULTIPLY, aux=aux, z=z, zq=mx.QMat(M, N), qp_row=(0, 1, 9, 3), zq_t=mx.QMat(N, M), qp_t=(0, 1, 9, 5))
+    st = mx.new_status()
+    mx.gemm_quant(a, b, epi, dev_status=st)
+    torch.cuda.synchronize()
+    assert int(st.item()) == mx.DEV_NONFINITE
+    with np.errstate(invalid="ignore", over="ignore"):
+        p = y.double().cpu().numpy() * aux.double().cpu().numpy()   # 16 bits: exact
+        ulp = np.ldexp(1.0, np.maximum(np.frexp(p)[1] - 1, -126) - 7)
+        want = np.where(np.isfinite(p), np.rint(p / ulp) * ulp, p)
+        want[np.abs(want) >= 2.0 ** 128] *= np.inf
+    zf = z.double().cpu().numpy()
+    assert (((np.abs(want) < 2.0 ** -126) & (want != 0)).sum() > 100 and (want == 0).sum() > 100 and (np.isinf(want) & np.isfinite(p)).sum() > 100 and
+            np.isnan(want).sum() > 100)
+    assert np.array_equal(zf, want, equal_nan=True)
+    q, qt = mx.quantize_2axis(z, (0, 1, 9, 3), (0, 1, 9, 5))
+    for got, ref in ((epi.zq, q), (epi.zq_t, qt)):
+        assert torch.equal(got.data, ref.data) and torch.equal(got.scales, ref.scales)
 
 
 def test_gelu_chain_over_its_operands(mx):
