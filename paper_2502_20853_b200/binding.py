@@ -43,7 +43,8 @@ EXPORTS = ["mxfp4_launch_count", "mxfp4_scale_bytes", "mxfp4_scale_offset", "mxf
            "mxfp4_linear_workspace_bytes", "mxfp4_quantize", "mxfp4_quantize_t", "mxfp4_quantize_2axis", "mxfp4_quantize_chain",
            "mxfp4_qema_quantize", "mxfp4_dequantize", "mxfp4_gemm", "mxfp4_gemm_quant", "mxfp4_gemm_static", "mxfp4_linear_fwd",
            "mxfp4_linear_bwd", "mxfp4_linear_fwd_ex", "mxfp4_linear_bwd_ex", "mxfp4_qramp_adamw", "mxfp4_qramp_detect", "mxfp4_quant_conf_hist", "mxfp4_change_sums",
-           "mxfp4_change_sums_q", "mxfp4_mma_issue_ceiling", "mxfp4_gemm_wait_selftest", "mxfp4_quantize_wait_selftest"]
+           "mxfp4_change_sums_q", "mxfp4_mma_issue_ceiling", "mxfp4_gemm_wait_selftest", "mxfp4_quantize_wait_selftest",
+           "mxfp4_forward_wait_selftest"]
 
 
 class MxError(RuntimeError):
@@ -146,6 +147,8 @@ def lib():
     L.mxfp4_gemm_wait_selftest.argtypes = [CMat, CMat, vp, i64, i32, vp, sz, C.c_uint32, vp, vp]
     L.mxfp4_quantize_wait_selftest.restype = i32
     L.mxfp4_quantize_wait_selftest.argtypes = [vp, i64, i64, i64, CMat, CMat, C.c_uint32, vp, vp]
+    L.mxfp4_forward_wait_selftest.restype = i32
+    L.mxfp4_forward_wait_selftest.argtypes = [vp, i64, i64, i64, i64, vp, i64, C.POINTER(CCtx), C.POINTER(CEpilogue), C.c_uint32, vp, vp]
     L.mxfp4_linear_fwd_ex.restype = i32
     L.mxfp4_linear_fwd_ex.argtypes = [vp, i64, i64, i64, vp, i64, vp, vp, i64, C.POINTER(CCtx), i32, C.POINTER(CEpilogue), vp, vp]
     L.mxfp4_linear_bwd_ex.restype = i32
@@ -448,6 +451,21 @@ def quantize_wait_selftest(x, dev_status, spin_limit=2048):
     out, out_t = QMat(rows, cols, x.device), QMat(cols, rows, x.device)
     _check("mxfp4_quantize_wait_selftest", lib().mxfp4_quantize_wait_selftest(_ptr(x), rows, cols, x.stride(0), out.c(), out_t.c(), spin_limit,
                                                                               _ptr(dev_status), _stream()))
+
+
+def forward_wait_selftest(x, wq, dev_status, epi=None, spin_limit=2048):
+    """The one kernel of linear_fwd(x, wq=wq) or, with ``epi`` and a QMat x, of gemm_quant(x, wq, epi), with its loads withheld: see
+    gemm_wait_selftest."""
+    if epi is None:
+        x = _bf16_2d(x)
+        (m, k), n = x.shape, wq.rows
+        y, ce = _new((m, n), torch.bfloat16, x.device), None
+        ctx = LinearCtx(QMat(m, k, x.device), wq)
+    else:
+        m, k, n, y, ce, ctx, x = x.rows, x.cols, wq.rows, None, epi.c(), LinearCtx(x, wq), None
+    _check("mxfp4_forward_wait_selftest",
+           lib().mxfp4_forward_wait_selftest(_ptr(x), x.stride(0) if x is not None else 0, m, k, n, _ptr(y), n, C.byref(ctx.c()),
+                                             C.byref(ce) if ce is not None else None, spin_limit, _ptr(dev_status), _stream()))
 
 
 STATIC_SCRATCH_BYTES = 16 << 20

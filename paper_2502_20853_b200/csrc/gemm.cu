@@ -3194,7 +3194,9 @@ static bool two_pass(const mxfp4_epilogue_t *epi, const mxfp4_mat_t &a, const mx
            (tiles >= 12 * sms || !two_groups(epi, a.rows, b.rows, a.cols) || over_operands(epi, a, b, bias));
 }
 
-mxfp4_status_t gemm_quant(mxfp4_mat_t a, mxfp4_mat_t b, const void *bias, const mxfp4_epilogue_t *epi, uint32_t *dev_status, cudaStream_t st)
+// spin_limit / withhold_loads: see GemmParams; the self-test runs the quantizing kernel alone.
+mxfp4_status_t gemm_quant(mxfp4_mat_t a, mxfp4_mat_t b, const void *bias, const mxfp4_epilogue_t *epi, uint32_t *dev_status, cudaStream_t st,
+                          uint32_t spin_limit, int withhold_loads)
 {
     const mxfp4_status_t chk = gemm_quant_check(a, b, bias, epi);
     if (chk) return chk;
@@ -3202,6 +3204,7 @@ mxfp4_status_t gemm_quant(mxfp4_mat_t a, mxfp4_mat_t b, const void *bias, const 
     if (M == 0 || N == 0) return MXFP4_OK;
     const bool row = epi->zq.data != nullptr, tr = epi->zq_t.data != nullptr;
     if (two_pass(epi, a, b, bias)) {
+        if (withhold_loads) return MXFP4_BAD_SHAPE;
         // Y by the product's own kernels (the contraction is not split), then the tile quantizer reads it back
         mxfp4_status_t s = gemm(a, b, epi->y_bf16, epi->ldy, MXFP4_OUT_BF16, bias, nullptr, 0, dev_status, st, false);
         if (s) return s;
@@ -3225,8 +3228,8 @@ mxfp4_status_t gemm_quant(mxfp4_mat_t a, mxfp4_mat_t b, const void *bias, const 
     p.dev_status = dev_status;
     p.d = nullptr;
     p.ldd = 0;
-    p.spin_limit = kWaitSpinLimit;
-    p.withhold_loads = 0;
+    p.spin_limit = spin_limit;
+    p.withhold_loads = withhold_loads;
     set_walk(p);
 
     QuantEpilogue e;
@@ -3342,7 +3345,7 @@ size_t mxfp4_gemm_workspace_bytes(int64_t m, int64_t n, int64_t kc) { return mx:
 mxfp4_status_t mxfp4_gemm_quant(mxfp4_mat_t a, mxfp4_mat_t b, const void *bias_bf16, const mxfp4_epilogue_t *epi, uint32_t *dev_status,
                                 void *stream)
 {
-    return mx::gemm_quant(a, b, bias_bf16, epi, dev_status, static_cast<cudaStream_t>(stream));
+    return mx::gemm_quant(a, b, bias_bf16, epi, dev_status, static_cast<cudaStream_t>(stream), mx::kWaitSpinLimit, 0);
 }
 
 mxfp4_status_t mxfp4_gemm_wait_selftest(mxfp4_mat_t a, mxfp4_mat_t b, void *d, int64_t ldd, int32_t out_dtype, void *workspace,

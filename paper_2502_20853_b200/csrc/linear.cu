@@ -22,7 +22,8 @@ mxfp4_status_t gemm_check(mxfp4_mat_t a, mxfp4_mat_t b, const void *d, int64_t l
                           const void *workspace, size_t workspace_bytes, bool allow_split);
 size_t gemm_two_workspace_bytes(int64_t m1, int64_t kc1, int64_t m2, int64_t kc2, int64_t n, size_t scratch);
 mxfp4_status_t gemm_quant_check(mxfp4_mat_t a, mxfp4_mat_t b, const void *bias, const mxfp4_epilogue_t *epi);
-mxfp4_status_t gemm_quant(mxfp4_mat_t a, mxfp4_mat_t b, const void *bias, const mxfp4_epilogue_t *epi, uint32_t *dev_status, cudaStream_t st);
+mxfp4_status_t gemm_quant(mxfp4_mat_t a, mxfp4_mat_t b, const void *bias, const mxfp4_epilogue_t *epi, uint32_t *dev_status, cudaStream_t st,
+                          uint32_t spin_limit, int withhold_loads);
 
 static size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
 
@@ -61,9 +62,10 @@ size_t mxfp4_linear_workspace_bytes(int64_t m, int64_t k, int64_t n)
     return bwd_layout(m, k, n).total;
 }
 
-mxfp4_status_t mxfp4_linear_fwd_ex(const void *x_bf16, int64_t ldx, int64_t m, int64_t k, const void *w_bf16, int64_t n,
-                                   const void *bias_bf16, void *y_bf16, int64_t ldy, mxfp4_linear_ctx_t *ctx, int32_t scale_mode,
-                                   const mxfp4_epilogue_t *epi, uint32_t *dev_status, void *stream)
+// withhold_loads (self-test of the drain path): the one launch of a small batch, or a quantizing epilogue's product alone
+static mxfp4_status_t linear_fwd(const void *x_bf16, int64_t ldx, int64_t m, int64_t k, const void *w_bf16, int64_t n, const void *bias_bf16, void *y_bf16,
+                                 int64_t ldy, mxfp4_linear_ctx_t *ctx, int32_t scale_mode, const mxfp4_epilogue_t *epi, uint32_t *dev_status, void *stream,
+                                 uint32_t spin_limit, int withhold_loads)
 {
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     if (!ctx || (!epi && !y_bf16)) return MXFP4_INVALID_ARG;
@@ -102,8 +104,9 @@ mxfp4_status_t mxfp4_linear_fwd_ex(const void *x_bf16, int64_t ldx, int64_t m, i
     if (x_bf16 && !make_q6 && !w_bf16 && !epi && gemm_from_x_fits(m, n, k, st) &&
         !meet(span_of_bf16(x_bf16, ldx, m, k), span_of_bf16(y_bf16, ldy, m, n))) {
         if (scale_mode != MXFP4_SCALE_TRUNCATION_FREE && scale_mode != MXFP4_SCALE_FLOOR) return MXFP4_INVALID_ARG;
-        return gemm_from_x(x_bf16, ldx, ctx->xq, ctx->wq, y_bf16, ldy, bias_bf16, scale_mode, dev_status, st, kWaitSpinLimit, 0);
+        return gemm_from_x(x_bf16, ldx, ctx->xq, ctx->wq, y_bf16, ldy, bias_bf16, scale_mode, dev_status, st, spin_limit, withhold_loads);
     }
+    if (withhold_loads && (x_bf16 || w_bf16 || !epi)) return MXFP4_BAD_SHAPE;
     if (make_q6 && make_q4 && m > 0 && n > 0 && k > 0) {
         if (scale_mode != MXFP4_SCALE_TRUNCATION_FREE && scale_mode != MXFP4_SCALE_FLOOR) return MXFP4_INVALID_ARG;
         s = quantize_chain_two(x_bf16, m, k, ldx, ctx->xq, ctx->xq_t, &q6, w_bf16, n, ctx->wq, ctx->wq_t, &q4, &qp, dev_status, st, kWaitSpinLimit, 0);
@@ -116,8 +119,22 @@ mxfp4_status_t mxfp4_linear_fwd_ex(const void *x_bf16, int64_t ldx, int64_t m, i
         else s = w_bf16 ? quantize_rows(w_bf16, n, k, k, ctx->wq, &qp, dev_status, st) : MXFP4_OK;
         if (s) return s;
     }
-    if (epi) return gemm_quant(ctx->xq, ctx->wq, bias_bf16, epi, dev_status, st);
+    if (epi) return gemm_quant(ctx->xq, ctx->wq, bias_bf16, epi, dev_status, st, spin_limit, withhold_loads);
     return gemm(ctx->xq, ctx->wq, y_bf16, ldy, MXFP4_OUT_BF16, bias_bf16, nullptr, 0, dev_status, st, false);
+}
+
+mxfp4_status_t mxfp4_linear_fwd_ex(const void *x_bf16, int64_t ldx, int64_t m, int64_t k, const void *w_bf16, int64_t n,
+                                   const void *bias_bf16, void *y_bf16, int64_t ldy, mxfp4_linear_ctx_t *ctx, int32_t scale_mode,
+                                   const mxfp4_epilogue_t *epi, uint32_t *dev_status, void *stream)
+{
+    return linear_fwd(x_bf16, ldx, m, k, w_bf16, n, bias_bf16, y_bf16, ldy, ctx, scale_mode, epi, dev_status, stream, kWaitSpinLimit, 0);
+}
+
+mxfp4_status_t mxfp4_forward_wait_selftest(const void *x_bf16, int64_t ldx, int64_t m, int64_t k, int64_t n, void *y_bf16, int64_t ldy, mxfp4_linear_ctx_t *ctx,
+                                           const mxfp4_epilogue_t *epi, uint32_t spin_limit, uint32_t *dev_status, void *stream)
+{
+    if (!dev_status || spin_limit < 128u || spin_limit > (1u << 16)) return MXFP4_INVALID_ARG;
+    return linear_fwd(x_bf16, ldx, m, k, nullptr, n, nullptr, y_bf16, ldy, ctx, MXFP4_SCALE_TRUNCATION_FREE, epi, dev_status, stream, spin_limit, 1);
 }
 
 mxfp4_status_t mxfp4_linear_fwd(const void *x_bf16, int64_t ldx, int64_t m, int64_t k, const void *w_bf16, int64_t n,
@@ -199,7 +216,7 @@ mxfp4_status_t mxfp4_linear_bwd_ex(const void *dy_bf16, int64_t lddy, const mxfp
     void *const gws = ws + L.gemm_ws;
     if (!epi_dx) return gemm_two(dyq_t, xq_t, dw, lddw, dw_dtype, dyq, wq_t, dx_bf16, lddx, MXFP4_OUT_BF16, gws, L.gemm_ws_bytes, dev_status, st);
     if ((s = gemm(dyq_t, xq_t, dw, lddw, dw_dtype, nullptr, gws, L.gemm_ws_bytes, dev_status, st, true))) return s;
-    return gemm_quant(dyq, wq_t, nullptr, epi_dx, dev_status, st);
+    return gemm_quant(dyq, wq_t, nullptr, epi_dx, dev_status, st, kWaitSpinLimit, 0);
 }
 
 mxfp4_status_t mxfp4_linear_bwd(const void *dy_bf16, int64_t lddy, const mxfp4_linear_ctx_t *ctx, uint64_t seed,

@@ -1,6 +1,6 @@
 """The drain path of the bounded waits, exercised without any fault.
 
-Every wait on a barrier in the GEMM kernels and in the two-axis quantizer gives up after a bounded number of polls,
+Every wait on a barrier in the GEMM kernels, the quantizing epilogue and the two-axis quantizer gives up after a bounded number of polls,
 raises MXFP4_DEV_TIMEOUT, and makes every role of its thread block leave; the block then frees its tensor memory and
 returns.  The self-test entry points launch the real kernels with their loads withheld and the bound at a few
 thousand polls, so that path runs within milliseconds: no trap, no endless loop, no bad address.  Afterwards the same
@@ -172,3 +172,82 @@ def test_waits_of_two_matrices_in_a_launch_run_out(mx):
     assert int(st.item()) == 0
     for got, want in zip((ctx.xq, ctx.xq_t, ctx.wq, ctx.wq_t), mx.quantize_chain(x, seed=9) + mx.quantize_chain(x, seed=9, stream_id_t=4)):
         assert torch.equal(got.data, want.data) and torch.equal(got.scales, want.scales)
+
+
+# the forward pass of a small batch: clusters of three CTAs, of two, single ones; one and two K tiles
+@pytest.mark.parametrize("M,N,K", [(197, 1536, 384), (129, 136, 160), (300, 640, 128)])
+def test_waits_of_a_small_forward_pass_run_out(mx, M, N, K):
+    g = torch.Generator(device="cuda").manual_seed(M)
+    x = torch.randn((M, K), generator=g, device="cuda").to(torch.bfloat16)
+    wq = mx.quantize(torch.randn((N, K), generator=g, device="cuda").to(torch.bfloat16))
+    want = mx.gemm(mx.quantize(x), wq)
+    st = mx.new_status()
+    before = mx.launch_count()
+    mx.forward_wait_selftest(x, wq, st)
+    assert mx.launch_count() - before == 1
+    torch.cuda.synchronize()
+    assert int(st.item()) & mx.DEV_TIMEOUT
+    st.zero_()
+    for _ in range(2):
+        y, _ = mx.linear_fwd(x, wq=wq, dev_status=st)
+    torch.cuda.synchronize()
+    assert int(st.item()) == 0 and torch.equal(y, want)
+
+
+# one group of epilogue warps, and two (171 tiles); with the second factor (a wait of its own) and without
+@pytest.mark.parametrize("M,N,K", [(384, 256, 128), (2400, 1056, 384)])
+@pytest.mark.parametrize("hook", ["gelu", "multiply"])
+def test_waits_of_the_quantizing_epilogue_run_out(mx, M, N, K, hook):
+    rng = np.random.default_rng(M)
+    a, b = (numpy_to_qmat(mx, *rand_operand(rng, r, K)) for r in (M, N))
+    aux = torch.randn((M, N), generator=torch.Generator(device="cuda").manual_seed(N), device="cuda").to(torch.bfloat16)
+    y = torch.empty((M, N), dtype=torch.bfloat16, device="cuda")
+    q = [mx.QMat(M, N), mx.QMat(N, M)]
+    if hook == "gelu":
+        epi = mx.Epilogue(hook=mx.HOOK_GELU, y=y, zq=q[0], zq_t=q[1], qp_t=(0, 1, 5, 6), chain=True)
+    else:
+        epi = mx.Epilogue(hook=mx.HOOK_MULTIPLY, aux=aux, z=y, zq=q[0], qp_row=(0, 1, 5, 3), zq_t=q[1], qp_t=(0, 1, 5, 5))
+    st = mx.new_status()
+    before = mx.launch_count()
+    mx.forward_wait_selftest(a, b, st, epi=epi)
+    assert mx.launch_count() - before == 1
+    torch.cuda.synchronize()
+    assert int(st.item()) & mx.DEV_TIMEOUT
+    st.zero_()
+    for _ in range(2):
+        mx.gemm_quant(a, b, epi, dev_status=st)
+    torch.cuda.synchronize()
+    assert int(st.item()) == 0
+    product = mx.gemm(a, b)
+    if hook == "gelu":
+        assert torch.equal(y, product) and torch.equal(q[1].data, mx.quantize_t(q[0], rounding=1, seed=5, stream_id=6).data)
+    else:
+        assert torch.equal(y, product * aux)
+        for got, want in zip(q, mx.quantize_2axis(y, (0, 1, 5, 3), (0, 1, 5, 5))):
+            assert torch.equal(got.data, want.data) and torch.equal(got.scales, want.scales)
+
+
+def test_forward_selftest_is_for_one_kernel(mx):
+    x, wq, st = torch.ones((128, 512), dtype=torch.bfloat16, device="cuda"), mx.QMat(128, 512), mx.new_status()
+    before = mx.launch_count()
+    with pytest.raises(mx.MxError):
+        mx.forward_wait_selftest(x, wq, st)                                  # two launches
+    with pytest.raises(mx.MxError):
+        mx.forward_wait_selftest(x[:, :128].contiguous(), mx.QMat(128, 128), st, spin_limit=4)
+    assert mx.launch_count() == before
+
+
+@pytest.mark.parametrize("M,N,K", [(197, 1536, 384), (300, 640, 128)])
+def test_waits_of_a_small_forward_pass_count_from_the_inputs_on(mx, hold, M, N, K):
+    """Its blocks are in place behind a slow kernel, twice as long as the bound of a wait."""
+    x = torch.randn((M, K), device="cuda").to(torch.bfloat16)
+    wq = mx.quantize(torch.randn((N, K), device="cuda").to(torch.bfloat16))
+    st = mx.new_status()
+    want, _ = mx.linear_fwd(x, wq=wq)
+    before = mx.launch_count()
+    torch.cuda.synchronize()
+    hold()
+    y, _ = mx.linear_fwd(x, wq=wq, dev_status=st)
+    assert mx.launch_count() - before == 1
+    torch.cuda.synchronize()
+    assert int(st.item()) == 0 and torch.equal(y, want)
