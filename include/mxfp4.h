@@ -212,7 +212,8 @@ mxfp4_status_t mxfp4_gemm(mxfp4_mat_t a, mxfp4_mat_t b, void *d, int64_t ldd, in
  * random stream by (seed, stream_id, position in the output)).  Every output is optional (data / pointer NULL = not
  * written), at least one must be asked for; chain needs both Zq and Zq_t.  N % 32 == 0; M % 32 == 0 when Zq_t is
  * asked for; y, z, aux: bf16 [M, N], 16-byte aligned, leading dimensions multiples of 8.  Normally one kernel; GELU with
- * chain and a stored Y on at least four 128 x 128 tiles per SM runs as two, the second of which reads Y back.  No workspace: the
+ * chain and a stored Y on many 128 x 128 tiles per SM (twelve; four where Z is stored too, the contraction is longer than
+ * 1024, or an output lies over an operand) runs as two, the second of which reads Y back.  No workspace: the
  * contraction is never split (see mxfp4_gemm for the accuracy bound with c = ceil(kc / 64)). */
 enum { MXFP4_HOOK_IDENTITY = 0, MXFP4_HOOK_GELU = 1, MXFP4_HOOK_MULTIPLY = 2 };
 typedef struct {

@@ -5,7 +5,8 @@
 
 Kernels: quantize, quantize_sr, quantize_t, quantize_t_sr, quantize_2axis, quantize_chain, requant (double quantization), qema,
 qema_osc, qramp_detect, qramp_adamw (all elements update every step), qramp_adamw_ramped (a tenth of the elements
-accumulate over 6 steps), quant_conf_hist, change_sums, mma_ceiling (MMA-only loop, --n = tile width), gemm.  Prints one line with the mean time and the algorithmic GB/s or TFLOP/s.
+accumulate over 6 steps), quant_conf_hist, change_sums, mma_ceiling (MMA-only loop, --n = tile width), gemm, linear_fwd,
+gemm_quant_gelu_chain, gemm_quant_mul_2axis, gemm_quant_chain.  Prints one line with the mean time and the algorithmic GB/s or TFLOP/s.
 """
 import argparse
 
@@ -59,6 +60,12 @@ def main():
             out_bytes = 2 + 2 * Q          # the second factor read, two sets of codes written
         fn = lambda: mx.gemm_quant(A, B, epi, dev_status=st)  # noqa: E731
         nbytes = Q * a.k * (a.m + a.n) + out_bytes * a.m * a.n
+        flops = 2.0 * a.m * a.n * a.k
+    elif a.kernel == "linear_fwd":
+        # the forward pass on a weight that is quantized already: for a small batch one kernel
+        x, wq = torch.randn((a.m, a.k), device="cuda").to(torch.bfloat16), mx.quantize((torch.randn((a.n, a.k), device="cuda") * 0.02).to(torch.bfloat16))
+        fn = lambda: mx.linear_fwd(x, wq=wq)  # noqa: E731
+        nbytes = 2 * a.m * (a.k + a.n) + Q * a.n * a.k
         flops = 2.0 * a.m * a.n * a.k
     elif a.kernel == "gemm":
         A, B = mx.QMat(a.m, a.k), mx.QMat(a.n, a.k)
