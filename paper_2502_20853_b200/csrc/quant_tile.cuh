@@ -90,13 +90,19 @@ __device__ __forceinline__ uint32_t absmax_u4(uint32_t acc, const uint4 &q)
     return absmax2(acc, q.w);
 }
 
-// The 16 bytes of codes of one 32-element group, round to nearest, and its scale byte (0xFF for a group with Inf / NaN, codes 0).
-__device__ __forceinline__ uint4 rne_group(const uint4 (&q)[4], uint32_t tf_add, uint32_t &byte)
+// The largest magnitude of a 32-element group, as bf16 bits (0x7F80 and above: it holds Inf / NaN).
+__device__ __forceinline__ uint32_t group_amax(const uint4 (&q)[4])
 {
     uint32_t am = 0;
 #pragma unroll
     for (int j = 0; j < 4; j++) am = absmax_u4(am, q[j]);
-    am = hmax_halves(am);
+    return hmax_halves(am);
+}
+
+// The 16 bytes of codes of one 32-element group, round to nearest, and its scale byte (0xFF for a group with Inf / NaN, codes 0).
+__device__ __forceinline__ uint4 rne_group(const uint4 (&q)[4], uint32_t tf_add, uint32_t &byte)
+{
+    const uint32_t am = group_amax(q);
     byte = 0xFFu;
     if (am >= 0x7F80u) return make_uint4(0, 0, 0, 0);
     byte = scale_byte_from_amax(am, tf_add);

@@ -33,20 +33,18 @@ __global__ void __launch_bounds__(256) k_quantize_rows(const __nv_bfloat16 *src,
     uint4 q[4];
 #pragma unroll
     for (int j = 0; j < 4; j++) q[j] = ld_stream_16(p + j);
-    uint4 out;
+    const uint32_t am = group_amax(q);
+    uint4 out = make_uint4(0, 0, 0, 0);
     uint32_t byte;
-    if (ROUNDING == MXFP4_ROUND_NEAREST) {
-        out = rne_group(q, tf_add_of(scale_mode), byte);
-    } else {
-        uint32_t am = 0;
-#pragma unroll
-        for (int j = 0; j < 4; j++) am = absmax_u4(am, q[j]);
-        am = hmax_halves(am);
-        out = make_uint4(0, 0, 0, 0);
+    if (am >= 0x7F80u) {
         byte = 0xFFu;
-        if (am < 0x7F80u) {
-            byte = scale_byte_from_amax(am, tf_add_of(scale_mode));
-            const uint32_t inv = inv_scale_bf16x2(byte);
+        if (dev_status) atomicOr(dev_status, MXFP4_DEV_NONFINITE);
+    } else {
+        byte = scale_byte_from_amax(am, tf_add_of(scale_mode));
+        const uint32_t inv = inv_scale_bf16x2(byte);
+        if (ROUNDING == MXFP4_ROUND_NEAREST) {
+            out = make_uint4(rne8(q[0], inv), rne8(q[1], inv), rne8(q[2], inv), rne8(q[3], inv));
+        } else {
             const uint64_t q0 = ((uint64_t)row * ((uint64_t)nblk * 32) + (uint64_t)blk * 32) >> 4;
             uint4 ra, rb;
             sr_words_two(sr, q0, q0 + 1, ra, rb);
@@ -56,7 +54,6 @@ __global__ void __launch_bounds__(256) k_quantize_rows(const __nv_bfloat16 *src,
             out.w = sr8(q[3], inv, rb.z, rb.w);
         }
     }
-    if (byte == 0xFFu && dev_status) atomicOr(dev_status, MXFP4_DEV_NONFINITE);
     *reinterpret_cast<uint4 *>(packed + row * ((int64_t)nblk * 16) + blk * 16) = out;
     scales[scale_offset(row, blk, nblk4)] = (uint8_t)byte;
 }
