@@ -758,13 +758,13 @@ k_gemm_mxf4_q(const __grid_constant__ CUtensorMap map_a, const __grid_constant__
         pdl_wait();
         const int group = GROUPS == 1 ? 0 : (warp - kEpiWarp0) / kEpiWarps, sync_id = 1 + group;
         const int et = (int)threadIdx.x - 32 * (kEpiWarp0 + group * kEpiWarps);
-        const int quarter = warp & 3, chalf = et >> 7;
+        const int quarter = warp & 3, chalf = GROUPS == 1 ? (warp - kEpiWarp0) >> 2 : et >> 7;
         const uint32_t bar_aux = bar_aux0 + 8 * group;
         const int M = (int)p.M, N = (int)p.N;
         const QsGeom g = qs_geom(et, M, N, e.rw.packed);
         const uint32_t tfa_r2 = tf_add_of(e.rw.scale_mode) * 0x00010001u, tfa_t2 = tf_add_of(e.tr.scale_mode) * 0x00010001u;
         const uint32_t t_base = smem_base + C::kTileOff + group * kTiles * kTileBytes, t2_base = t_base + kTileBytes, ty_base = t_base + (kTiles - 1) * kTileBytes;
-        const uint32_t dq_base = e.store_z ? t2_base : t_base;       // a Z that is stored keeps its tile until it has left
+        const uint32_t dq_base = GROUPS == 1 || e.store_z ? t2_base : t_base;   // a Z that is stored keeps its tile until it has left
         const int trow = quarter * 32 + lane;                        // this thread's row of the tile
         const uint32_t row_off = (uint32_t)(chalf * (kTileBytes / 2) + trow * 128);
         const uint32_t t_row = t_base + row_off;
@@ -800,61 +800,65 @@ k_gemm_mxf4_q(const __grid_constant__ CUtensorMap map_a, const __grid_constant__
             const int grow = row0 + trow;
 
             // ---- accumulator -> Y (bf16) -> hook -> Z (bf16) -> the tile in shared memory ----
+            // One group has this code once per hook: beside the packed multiplication a common one took 1-4 % longer than before it where
+            // there is no hook (25216 x 1536 x 1024, Q3 + Q5 48.1, 49.9 us, so 45.4); with the 96 registers of two groups that would spill.
+            const auto fill = [&](auto hook) {
 #pragma unroll
-            for (int cc = 0; cc < 2; cc++) {
-                const int col = col0 + chalf * 64 + cc * 32;
-                const bool live = grow < M && col < N;     // N is a multiple of 32: a chunk is inside the matrix or outside it
-                uint32_t r[32];
-                tc_ld32(taddr + cc * 32, r);
-                tc_wait_ld();
-                if (cc == 1) {
-                    tc_fence_before();
-                    __syncwarp();
-                    if (lane == 0) mbar_arrive(bar_acc_empty + 8 * acc);   // the accumulator goes back to the MMA issuer
-                }
-                if (use_bias) add_bias_chunk(r, bias_line + 64u * cc);
-                uint32_t yw[16];
-                pack_row_bf16(r, yw);
-                if (WITH_Y && e.store_y) {
+                for (int cc = 0; cc < 2; cc++) {
+                    const int col = col0 + chalf * 64 + cc * 32;
+                    const bool live = grow < M && col < N;     // N is a multiple of 32: a chunk is inside the matrix or outside it
+                    uint32_t r[32];
+                    tc_ld32(taddr + cc * 32, r);
+                    tc_wait_ld();
+                    if (cc == 1) {
+                        tc_fence_before();
+                        __syncwarp();
+                        if (lane == 0) mbar_arrive(bar_acc_empty + 8 * acc);   // the accumulator goes back to the MMA issuer
+                    }
+                    if (use_bias) add_bias_chunk(r, bias_line + 64u * cc);
+                    uint32_t yw[16];
+                    pack_row_bf16(r, yw);
+                    if (WITH_Y && e.store_y) {
+#pragma unroll
+                        for (int j = 0; j < 4; j++)
+                            asm volatile("st.shared.v4.u32 [%4], {%0,%1,%2,%3};" ::"r"(yw[4 * j]), "r"(yw[4 * j + 1]), "r"(yw[4 * j + 2]), "r"(yw[4 * j + 3]),
+                                         "r"(ty_base + row_off + (uint32_t)((((cc * 4 + j) ^ (trow & 7))) << 4)) : "memory");
+                    }
+                    if (hook != MXFP4_HOOK_IDENTITY) {
+                        if (hook == MXFP4_HOOK_GELU) {
+#pragma unroll
+                            for (int j = 0; j < 16; j++) yw[j] = gelu_bf16x2(yw[j]);
+                        } else {
+                            uint4 aw[4] = {make_uint4(0, 0, 0, 0), make_uint4(0, 0, 0, 0), make_uint4(0, 0, 0, 0), make_uint4(0, 0, 0, 0)};
+                            if (aux_tma) {
+#pragma unroll
+                                for (int j = 0; j < 4; j++)
+                                    asm volatile("ld.shared.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(aw[j].x), "=r"(aw[j].y), "=r"(aw[j].z), "=r"(aw[j].w)
+                                                 : "r"(t2_base + row_off + (uint32_t)((((cc * 4 + j) ^ (trow & 7))) << 4)));
+                            } else if (live) {
+                                const uint4 *ap = reinterpret_cast<const uint4 *>(e.aux + (int64_t)grow * e.ld_aux + col);
+#pragma unroll
+                                for (int j = 0; j < 4; j++) aw[j] = ld_stream_16(ap + j);
+                            }
+                            const uint32_t *a32 = reinterpret_cast<const uint32_t *>(aw);
+#pragma unroll
+                            for (int j = 0; j < 16; j++) yw[j] = mul_bf16x2(yw[j], a32[j]);   // one rounding, as of the FP32 product, which is exact
+                        }
+                    }
+                    if (!live) {
+#pragma unroll
+                        for (int j = 0; j < 16; j++) yw[j] = 0u;   // outside the matrix the tile holds zeros, as a TMA load would leave them
+                    }
 #pragma unroll
                     for (int j = 0; j < 4; j++)
                         asm volatile("st.shared.v4.u32 [%4], {%0,%1,%2,%3};" ::"r"(yw[4 * j]), "r"(yw[4 * j + 1]), "r"(yw[4 * j + 2]), "r"(yw[4 * j + 3]),
-                                     "r"(ty_base + row_off + (uint32_t)((((cc * 4 + j) ^ (trow & 7))) << 4)) : "memory");
+                                     "r"(t_row + (uint32_t)((((cc * 4 + j) ^ (trow & 7))) << 4)) : "memory");
                 }
-                uint32_t zw[16];
-                if (e.hook == MXFP4_HOOK_GELU) {
-#pragma unroll
-                    for (int j = 0; j < 16; j++) zw[j] = gelu_bf16x2(yw[j]);
-                } else if (e.hook == MXFP4_HOOK_MULTIPLY) {
-                    uint4 aw[4] = {make_uint4(0, 0, 0, 0), make_uint4(0, 0, 0, 0), make_uint4(0, 0, 0, 0), make_uint4(0, 0, 0, 0)};
-                    if (aux_tma) {
-#pragma unroll
-                        for (int j = 0; j < 4; j++)
-                            asm volatile("ld.shared.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(aw[j].x), "=r"(aw[j].y), "=r"(aw[j].z), "=r"(aw[j].w)
-                                         : "r"(t2_base + row_off + (uint32_t)((((cc * 4 + j) ^ (trow & 7))) << 4)));
-                    } else if (live) {
-                        const uint4 *ap = reinterpret_cast<const uint4 *>(e.aux + (int64_t)grow * e.ld_aux + col);
-#pragma unroll
-                        for (int j = 0; j < 4; j++) aw[j] = ld_stream_16(ap + j);
-                    }
-                    const uint32_t *a32 = reinterpret_cast<const uint32_t *>(aw);
-#pragma unroll
-                    for (int j = 0; j < 16; j++) {
-                        zw[j] = mul_bf16x2(yw[j], a32[j]);       // one rounding, as of the FP32 product, which is exact
-                    }
-                } else {
-#pragma unroll
-                    for (int j = 0; j < 16; j++) zw[j] = yw[j];
-                }
-                if (!live) {
-#pragma unroll
-                    for (int j = 0; j < 16; j++) zw[j] = 0u;       // outside the matrix the tile holds zeros, as a TMA load would leave them
-                }
-#pragma unroll
-                for (int j = 0; j < 4; j++)
-                    asm volatile("st.shared.v4.u32 [%4], {%0,%1,%2,%3};" ::"r"(zw[4 * j]), "r"(zw[4 * j + 1]), "r"(zw[4 * j + 2]), "r"(zw[4 * j + 3]),
-                                 "r"(t_row + (uint32_t)((((cc * 4 + j) ^ (trow & 7))) << 4)) : "memory");
-            }
+            };
+            if (GROUPS == 2) fill(e.hook);
+            else if (e.hook == MXFP4_HOOK_IDENTITY) fill(std::integral_constant<int, MXFP4_HOOK_IDENTITY>());
+            else if (e.hook == MXFP4_HOOK_GELU) fill(std::integral_constant<int, MXFP4_HOOK_GELU>());
+            else fill(std::integral_constant<int, MXFP4_HOOK_MULTIPLY>());
             fence_async_smem();
             epi_sync(sync_id);                            // the tile is complete, the second factor has been read
             if (et == 0) {
@@ -3139,29 +3143,32 @@ mxfp4_status_t quantize_gelu_chain(const void *y_bf16, int64_t rows, int64_t col
 // with their waits for the accumulator and for one another do not fill the SM.  The second group's tiles and staging cost the ring two
 // of its four stages, so the contraction has to be short, and the shorter the less the epilogue does; the groups have to fit (GemmQCfg),
 // and a block needs a second tile.  K tiles of 256 up to which two groups are taken, with one group / two, back to back, in us:
-//   GELU: 4.  Chain and Y 25216 x 1536 x 384 72.0 / 60.0, x 1024 75.6 / 64.1, 2400 x 1024 x 1024 12.0 / 11.8; 3 where Y or Z is stored and at
-//     most one pass is made: Y and a row pass 25216 x 1536 x 768 50.2 / 46.0, x 1024 51.5 / 54.7, Z alone x 1024 46.9 / 49.1.
-//   Multiply: 2, as the second factor is loaded too.  A nearest row pass 25216 x 1536 x 512 32.6 / 28.9, x 768 34.2 / 39.4; Z alone
-//     49.4 / 36.6, x 1024 49.3 / 55.2.  With both passes stochastic 3 from four tiles per SM on: 25216 x 1536 x 768 51.9 / 46.8,
-//     6272 x 1536 x 768 (4.0 per SM) 15.5 / 14.7, 3136 x 2048 x 768 (2.7) 12.5 / 12.6; without Z and from 3072 columns on, where the SMs share
-//     more of the rows that they read, 4: 50432 x 4096 x 1024 273 / 256, 50432 x 3072 x 1024 198 / 187, 50432 x 1536 x 1024 100.3 / 101.1,
-//     50432 x 768 x 1024 53.6 / 55.6.  With the chain, whose passes are the longest, 4: 25216 x 1536 x 1024 107 / 101.
-//   Identity: 2.  Q3 + Q5 25216 x 1536 x 512 47.9 / 42.9, a nearest row pass 26.7 / 21.9 (x 768 27.7 / 28.4).  None where Z is stored and at
-//     most one pass is made, the stores being the bound: 25216 x 1536 x 384 29.0 / 31.6.
-// Beyond: multiply with Q3 + Q5 8192 x 4096 x 2048 54 / 80.  No second tile: 1024 x 768 x 192 6.5 / 7.0.
+//   GELU: 4.  Chain and Y 25216 x 1536 x 384 66.6 / 59.4, x 1024 69.5 / 64.4.  3 where Y and Z are stored, or one of them without a
+//     stochastic column pass behind a row pass: Y and a row pass 25216 x 1536 x 768 48.6 / 45.9, x 1024 49.9 / 54.7, Z alone x 1024 45.7 / 50.5.
+//   Multiply: 2, as the second factor is loaded too.  A nearest row pass 25216 x 1536 x 512 31.9 / 27.4, x 768 33.7 / 38.4; Z alone
+//     48.7 / 36.1, x 1024 48.8 / 54.9.  With both passes stochastic 3: 25216 x 1536 x 768 50.6 / 47.4, x 1024 51.2 / 54.2; without Z, on wide
+//     outputs (the SMs share more of the rows that they read) of very many tiles 4: 50432 x 4096 x 1024 271 / 259, 50432 x 3072 x 1024
+//     196 / 192, but 12544 x 4096 x 896 (21 tiles per SM) 67.8 / 68.0, 50432 x 768 x 1024 51.2 / 55.0.  With the chain, the longest passes, 4:
+//     25216 x 1536 x 1024 99.8 / 97.9.
+//   Identity: 2.  Q3 + Q5 25216 x 1536 x 384 43.2 / 42.1, a nearest row pass 25.3 / 21.7, x 768 26.3 / 28.1.  None where Z is stored and at
+//     most one pass is made, the stores being the bound: 25216 x 1536 x 384 28.2 / 31.8.
+// The short epilogues of these two take one group between two and four tiles per SM, where one of the groups often has a tile more than
+// the other: Q3 + Q5 4096 x 1536 x 384 (2.6) 11.7 / 11.9 and 10.9 / 11.1, the chain without a hook 10.8 / 11.2; but 2400 x 1024 x 256 (1.03)
+// 8.5 / 8.1 and 7.9 / 7.7, multiply 6272 x 3072 x 768 (8.3) 26.7 / 25.0.
 static bool two_groups(const mxfp4_epilogue_t *epi, int64_t M, int64_t N, int64_t Kc)
 {
     const bool identity = epi->hook == MXFP4_HOOK_IDENTITY, y = epi->y_bf16 && !(identity && !epi->z_bf16), z = epi->z_bf16 || (identity && epi->y_bf16);
     const int smem_tiles = 1 + (epi->hook == MXFP4_HOOK_MULTIPLY && !epi->chain) + (epi->chain && z) + y;
     const int64_t tiles = ceil_div(M, kBM) * ceil_div(N, 128), sms = sm_count();
     if (smem_tiles > 2 || tiles <= sms) return false;
-    const bool stored = y || z, row = epi->zq.data != nullptr, tr = epi->zq_t.data != nullptr;
-    const bool stochastic = row && tr && epi->qp_row.rounding == MXFP4_ROUND_STOCHASTIC && epi->qp_t.rounding == MXFP4_ROUND_STOCHASTIC;
+    const bool row = epi->zq.data != nullptr, tr = epi->zq_t.data != nullptr, both = row && tr;
+    const bool sr_row = row && epi->qp_row.rounding == MXFP4_ROUND_STOCHASTIC, sr_t = tr && epi->qp_t.rounding == MXFP4_ROUND_STOCHASTIC;
     int kt;
-    if (epi->hook == MXFP4_HOOK_GELU) kt = (row && tr) || !stored ? 4 : 3;
-    else if (identity) kt = (row && tr) || !stored ? 2 : 0;
-    else if (epi->chain) kt = 4;
-    else kt = !stochastic || tiles < 4 * sms ? 2 : stored || N < 3072 ? 3 : 4;
+    if (epi->hook == MXFP4_HOOK_GELU) kt = !(y || z) || (both && sr_t && !(y && z)) ? 4 : 3;
+    else if (epi->hook == MXFP4_HOOK_MULTIPLY && epi->chain) kt = 4;
+    else if (tiles > 2 * sms && tiles < 4 * sms) kt = 0;
+    else if (identity) kt = both || !(y || z) ? 2 : 0;
+    else kt = !(sr_row && sr_t) || tiles <= sms * 2 ? 2 : z || N < 3072 || tiles < 32 * sms ? 3 : 4;
     return Kc <= kt * kBKElems;
 }
 

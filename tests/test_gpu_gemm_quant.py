@@ -244,10 +244,10 @@ def test_gelu_chain_over_its_operands(mx):
     assert torch.equal(a.data, bufs[0].data) and torch.equal(a.scales_linear(), bufs[0].scales_linear()) and torch.equal(bufs[1].data, want_t)
 
 
-# more tiles than SMs and a short contraction: two groups of epilogue warps.  298 tiles (two blocks have a third), 171 (23 blocks
-# have a second), 225, 600, 625, all with ragged last tiles; contractions of one to four K tiles (multiply: with three from 592 tiles
-# on, with four from 3072 columns on; 225 tiles are one group's there)
-@pytest.mark.parametrize("M,N,K", [(18976, 160, 96), (2400, 1056, 384), (9504, 288, 1024), (12768, 736, 704), (3168, 3104, 992)])
+# more tiles than SMs and a short contraction: two groups of epilogue warps, with ragged last tiles.  GELU: 298 tiles (two blocks have a
+# third), 171 (23 blocks have a second), 225, 600, contractions of one, two, four and three K tiles.  Multiply: 171, 600 and 4950 tiles, two, three
+# and four K tiles (298 and 225 are one group's there, as 4950 is two kernels' behind GELU)
+@pytest.mark.parametrize("M,N,K", [(18976, 160, 96), (2400, 1056, 384), (9504, 288, 1024), (12768, 736, 704), (25248, 3104, 992)])
 @pytest.mark.parametrize("hook", ["gelu", "multiply"])
 def test_two_groups_of_epilogue_warps(mx, M, N, K, hook):
     _, a, b = operands(mx, M, N, K, M + N + K)
